@@ -238,6 +238,7 @@ struct MorState {
   bool hess_res = false;
   int hess_qn = 0;
   DBuf<cplx> hH, hb, hc, hA1, hA2, hRB, hV;
+  DBuf<cplx> hHr, hbr;             // hH and hb by rows (the evaluation's order)
   DBuf<double> htau;
   double last_max_err = -1.0;
   void reset() {
@@ -250,7 +251,7 @@ struct MorState {
     solve_iters = 0; solve_cols = 0;
     ++version;
     hess_version = -1;
-    for (DBuf<cplx>* b : {&hH, &hb, &hc, &hA1, &hA2, &hRB, &hV}) b->release();
+    for (DBuf<cplx>* b : {&hH, &hb, &hc, &hA1, &hA2, &hRB, &hV, &hHr, &hbr}) b->release();
     htau.release();
     m = 0; m_cap = 0; qn = 0; q_cap = 0;
     for (DBuf<cplx>* b : {&S, &Z, &Hh, &bh, &ch, &Q, &RS, &RZ, &RB}) b->release();

@@ -11,8 +11,8 @@
 // * Reduced model: Hhat = S^H Z, bhat = S^H b, chat = c^T S, updated incrementally.
 // * Evaluation at many frequencies: Hhat is reduced once to upper Hessenberg form by Householder
 //   reflections (applied alongside to bhat, chat and the residual coefficients); each frequency is
-//   then an O(m^2) shifted Hessenberg solve (one CTA per frequency, partial pivoting between adjacent
-//   rows). Ghat_pq = chat_q^T yhat_p for all frequencies is one complex GEMM, and A = -(1/pi) sum_p
+//   then an O(m^2 np) shifted Hessenberg solve (partial pivoting between adjacent rows, then a blocked back
+//   substitution). Ghat_pq = chat_q^T yhat_p for all frequencies is one complex GEMM, and A = -(1/pi) sum_p
 //   Im Ghat_pp.
 // * Residual estimate for refinement: the columns of [B, S, Z] are kept as coefficients in an
 //   orthonormal basis Q of their span (extended with every new block), so that the residual
@@ -177,22 +177,26 @@ __global__ void house_rows_kernel(cplx* __restrict__ Y, long long ldy, long long
   }
 }
 
-// ---- per-frequency shifted Hessenberg solve --------------------------------------------------------
+// ---- per-frequency shifted Hessenberg solves -------------------------------------------------------
+// (w - i eta + H) y_p = b_p for every frequency w and right-hand side p in two kernels: the elimination,
+// one CTA per frequency, leaves U (double-float, in 32 x 32 tiles) and the transformed right-hand sides;
+// the back substitution, one CTA per frequency and group of right-hand sides, is a blocked triangular solve.
 struct EvalArgs {
   int m, np, nw;
-  const cplx* H;      // m x m col-major (ld m), upper Hessenberg
-  const cplx* bw;     // m x np col-major (ld m)
+  const cplx* H;      // m x m row-major, upper Hessenberg
+  const cplx* b;      // m x np row-major; null: the right-hand sides are in Y (per frequency), solved in place
   const double* omegas;
   double eta;
-  cplx* scratch;      // per CTA: U (m(m+1)/2) | rows (2m)
-  long long scratch_per_cta;
+  float4* U;          // per frequency: tiles (J, K), J <= K, of 32 x 32 entries at (K(K+1)/2 + J) * 1024
+  cplx* dU;           // per frequency: the diagonal of U in FP64 (m)
   cplx* Y;            // solutions: Y[k * ldy + w * np + p] = yhat_p(w)[k]
   long long ldy;
   int* singular;
-  int rhs_in_Y = 0;   // 1: the right-hand sides are already in Y (per frequency), solved in place
 };
-
-__device__ __forceinline__ double cabs2(cplx a) { return a.x * a.x + a.y * a.y; }
+constexpr int ET = 32;   // tile edge of U
+__host__ __device__ constexpr long long eval_tiles(int m) {
+  return (long long)((m + ET - 1) / ET) * ((m + ET - 1) / ET + 1) / 2;
+}
 
 // ---- double-float arithmetic (value = h + l, two FP32 numbers) ------------------------------------
 // GB300 issues FP32 operations at many times its FP64 rate, so the O(m^2 np) back substitution runs
@@ -249,149 +253,365 @@ __device__ __forceinline__ float4 dfc_sub_mul(float4 c, float4 u, float4 y) {
   return make_float4(r.h, r.l, i.h, i.l);
 }
 
-// One CTA per frequency (grid-stride): LU of (w - i eta + H) with partial pivoting between adjacent
-// rows (the only pivots a Hessenberg matrix needs), applied to the np right-hand sides, in FP64 (O(m^2
-// + m np) work); then the back substitution (O(m^2 np)) in double-float, P right-hand sides at a time
-// held in shared memory, with U stored column by column. Everything after the solves (Ghat, A,
-// residual norms) is a GEMM over all frequencies at once and runs outside this kernel.
-// Scratch per CTA (16-byte units): U (m(m+1)/2, double-float, column j at j(j+1)/2) | two FP64 rows
-// (2m) | the FP64 diagonal of U (m). Dynamic shared memory: m P double-float complex values.
-template <int P>
-__global__ void __launch_bounds__(256) eval_solve_kernel(EvalArgs a) {
-  static_assert(256 % P == 0, "P divides the block");
-  extern __shared__ float4 Rs[];   // [m][P]
-  const int m = a.m, np = a.np;
-  float4* Ud = reinterpret_cast<float4*>(a.scratch + blockIdx.x * a.scratch_per_cta);
-  cplx* rowA = reinterpret_cast<cplx*>(Ud + (long long)m * (m + 1) / 2);
-  cplx* rowB = rowA + m;
-  cplx* dU = rowB + m;
-  const long long ldr = a.ldy;
-  __shared__ int s_swap;
-  __shared__ cplx s_l;
-  for (int w = blockIdx.x; w < a.nw; w += gridDim.x) {
-    const cplx sig = make_cuDoubleComplex(a.omegas[w], -a.eta);
-    cplx* R = a.Y + (long long)w * np;   // R[k * ldr + p]
-    if (!a.rhs_in_Y) {
-      for (long long t = threadIdx.x; t < (long long)m * np; t += blockDim.x) {
-        int k = (int)(t / np), p = (int)(t % np);
-        R[k * ldr + p] = a.bw[k + (long long)p * m];
-      }
+// df_from without FP64 arithmetic: h is x rounded to 24 bits (half up), l the rest rounded to 24 bits, both cut
+// out of the bit pattern (the same split up to the direction of exact ties). Outside the range of normal
+// FP32 numbers x is converted alone.
+__device__ __forceinline__ df2 df_split(double x) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFULL;
+  const int e = (int)(b >> 52);
+  if (e < 897 || e > 1149) return {(float)x, 0.f};
+  const unsigned long long r = (b + 0x10000000ULL) & ~0x1FFFFFFFULL;   // rounded to 23 mantissa bits
+  const int low = (int)(long long)(b - r);                             // in [-2^28, 2^28), times 2^(e - 1075)
+  const unsigned sign = (unsigned)((unsigned long long)__double_as_longlong(x) >> 32) & 0x80000000u;
+  const unsigned hb = (unsigned)(r >> 29) - (896u << 23);
+  const int k = (e - 1075) >> 1;   // the scale in two factors, each a normal number
+  const float l = (float)low * __uint_as_float((unsigned)(k + 127) << 23) *
+                  __uint_as_float((unsigned)(e - 1075 - k + 127) << 23);
+  return {__uint_as_float(hb | sign), __uint_as_float(__float_as_uint(l) ^ sign)};
+}
+__device__ __forceinline__ float4 dfc_split(cplx z) {
+  const df2 r = df_split(z.x), i = df_split(z.y);
+  return make_float4(r.h, r.l, i.h, i.l);
+}
+// a b (complex double-float)
+__device__ __forceinline__ float4 dfc_mul(float4 a, float4 b) {
+  const df2 z{0.f, 0.f}, ar{a.x, a.y}, ai{a.z, a.w}, nai{-a.z, -a.w}, br{b.x, b.y}, bi{b.z, b.w};
+  const df2 r = df_dot2(z, ar, br, nai, bi), i = df_dot2(z, ar, bi, ai, br);
+  return make_float4(r.h, r.l, i.h, i.l);
+}
+// (h, l) -= a b without renormalising: the leading product exactly (fma), its sum with h exactly (two-sum),
+// the rest added to l in FP32. The caller renormalises every few terms, which keeps l small enough that
+// its own rounding stays at the 2^-48 level.
+__device__ __forceinline__ void df_acc(float& h, float& l, float ah, float al, float bh, float bl) {
+  const float p = __fmul_rn(ah, bh);
+  const float e = __fmaf_rn(ah, bh, -p);
+  const df2 s = two_sum(h, -p);
+  h = s.h;
+  l = __fadd_rn(l, __fsub_rn(s.l, e));
+  l = __fmaf_rn(-ah, bl, l);
+  l = __fmaf_rn(-al, bh, l);
+}
+__device__ __forceinline__ void dfc_acc(float4& c, const float4& u, const float4& y) {   // c -= u y
+  df_acc(c.x, c.y, u.x, u.y, y.x, y.y);
+  df_acc(c.x, c.y, -u.z, -u.w, y.z, y.w);
+  df_acc(c.z, c.w, u.x, u.y, y.z, y.w);
+  df_acc(c.z, c.w, u.z, u.w, y.x, y.y);
+}
+__device__ __forceinline__ void dfc_renorm(float4& c) {
+  const df2 r = fast_two_sum(c.x, c.y), i = fast_two_sum(c.z, c.w);
+  c = make_float4(r.h, r.l, i.h, i.l);
+}
+
+__device__ __forceinline__ void cp_async16(void* smem, const void* gmem, bool on) {
+  const uint32_t d = (uint32_t)__cvta_generic_to_shared(smem);
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(gmem), "r"(on ? 16 : 0) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+// bits of max(|re|, |im|): non-negative doubles order like their bit patterns
+__device__ __forceinline__ unsigned long long max_bits(cplx z) {
+  const unsigned long long a = (unsigned long long)__double_as_longlong(z.x) & 0x7FFFFFFFFFFFFFFFULL;
+  const unsigned long long b = (unsigned long long)__double_as_longlong(z.y) & 0x7FFFFFFFFFFFFFFFULL;
+  return a > b ? a : b;
+}
+// x / p for the elimination: x conj(p) / |p|^2 with p scaled to order one by a power of two and the reciprocal by
+// two Newton steps from an FP32 seed. 15 FP64 operations in a chain of 10, where the library's complex division
+// is two FP64 divisions one after the other: an FP64 instruction holds a scheduler for 75 clocks on this
+// GPU (measured 1.7 lanes per clock and SM) and the division is the serial part of every elimination step.
+__device__ __forceinline__ cplx cdiv_newton(cplx x, cplx p) {
+  const int e = (int)(max_bits(p) >> 52);
+  if (e < 100 || e > 1946) return cuCdiv(x, p);   // near the ends of the exponent range
+  const double s = __longlong_as_double((long long)(2046 - e) << 52);   // 2^(1023 - e)
+  const double a = p.x * s, b = p.y * s;
+  const double d = fma(a, a, b * b);   // in [1, 8)
+  double r = (double)(1.0f / (float)d);
+  r = fma(r, fma(-d, r, 1.0), r);
+  r = fma(r, fma(-d, r, 1.0), r);
+  r *= s;
+  return make_cuDoubleComplex(fma(x.x, a, x.y * b) * r, fma(x.y, a, -(x.x * b)) * r);
+}
+
+// Elimination, one CTA per frequency: LU of (w - i eta + H) with partial pivoting between adjacent rows
+// (the only pivots a Hessenberg matrix needs), in FP64, the np right-hand sides carried along as np more
+// columns. Only one row is carried from step to step (in shared memory, every thread owning the columns
+// it alone reads and writes), and the rows still to come arrive by cp.async EF_RING - 1 steps ahead. The
+// chain of a step is the pivot of its owner thread (an FP64 division) and one barrier; everything else
+// (two FP64 multiply-adds per column, the split to double-float) is in its shadow. RING = false (rows too
+// long for shared memory) reads each row when it is needed and carries the row in global memory (the
+// tail of the frequency's dU block).
+constexpr int EF_T = 128, EF_RING = 4;
+template <bool RING>
+__global__ void __launch_bounds__(EF_T) eval_factor_kernel(EvalArgs a, int w0, cplx* __restrict__ rows) {
+  extern __shared__ float4 ef_sm[];
+  __shared__ cplx s_l[2];
+  __shared__ int s_swap[2];
+  const int m = a.m, np = a.np, n = m + np, f = blockIdx.x, w = w0 + f, tid = threadIdx.x;
+  const cplx sig = make_cuDoubleComplex(a.omegas[w], -a.eta);
+  cplx* cur = RING ? reinterpret_cast<cplx*>(ef_sm) : rows + (long long)f * n;
+  cplx* ring = reinterpret_cast<cplx*>(ef_sm) + n;
+  cplx* R = a.Y + (long long)w * np;   // row k at R[k * ldy]
+  float4* U = a.U + (long long)f * eval_tiles(m) * (ET * ET);
+  cplx* dU = a.dU + (long long)f * m;
+  auto src = [&](int r, int col) -> const cplx* {
+    if (col < m) return a.H + (long long)r * m + col;
+    return a.b ? a.b + (long long)r * np + (col - m) : R + (long long)r * a.ldy + (col - m);
+  };
+  // the thread's own columns of row r (columns before r - 1 are zero and never read)
+  auto issue = [&](int r) {
+    if (RING && r < m) {
+      cplx* d = ring + (long long)(r % EF_RING) * n;
+      for (int col = tid; col < n; col += EF_T)
+        if (col >= r - 1) cp_async16(d + col, src(r, col), true);
     }
-    for (int col = threadIdx.x; col < m; col += blockDim.x) {
-      cplx h = a.H[(long long)col * m + 0];
-      if (col == 0) h = cuCadd(h, sig);
-      rowA[col] = h;
+    cp_async_commit();
+  };
+  auto next = [&](int r, int col) { return RING ? ring[(long long)(r % EF_RING) * n + col] : *src(r, col); };
+  // pivot of step j from the carried row's entry c: swap and multiplier (owner of column j)
+  auto pivot = [&](int j, cplx c) {
+    cplx l = cz();
+    int swap = 0;
+    if (j + 1 < m) {
+      const cplx x = next(j + 1, j);
+      swap = max_bits(x) > max_bits(c);
+      const cplx piv = swap ? x : c;
+      if (piv.x == 0.0 && piv.y == 0.0) atomicExch(a.singular, 1);
+      else l = cdiv_newton(swap ? c : x, piv);
     }
+    s_l[j & 1] = l;
+    s_swap[j & 1] = swap;
+  };
+  for (int r = 1; r < EF_RING; ++r) issue(r);   // rows 1 .. EF_RING - 1
+  for (int col = tid; col < n; col += EF_T) {
+    cplx h = *src(0, col);
+    if (col == 0) h = cuCadd(h, sig);
+    cur[col] = h;
+  }
+  cp_async_wait<EF_RING - 2>();   // row 1
+  if (tid == 0) pivot(0, cur[0]);
+  for (int j = 0; j < m; ++j) {
     __syncthreads();
-    cplx* cur = rowA;
-    cplx* nxt = rowB;
-    for (int j = 0; j < m; ++j) {
-      if (j + 1 < m) {
-        for (int col = j + threadIdx.x; col < m; col += blockDim.x) {
-          cplx h = a.H[(long long)col * m + (j + 1)];
-          if (col == j + 1) h = cuCadd(h, sig);
-          nxt[col] = h;
-        }
+    const cplx l = s_l[j & 1];
+    const int swap = s_swap[j & 1];
+    const bool last = j + 1 == m;
+    cp_async_wait<EF_RING - 3>();   // row j + 2 (the next pivot); row j + 1 arrived a step ago
+    const int J = j / ET;
+    // the new carried value of a column and its entry of U (or of the transformed right-hand sides)
+    auto step = [&](int col, cplx x) {
+      const cplx c = cur[col];
+      const cplx u = swap ? x : c, low = swap ? c : x;
+      if (!last)
+        cur[col] = make_cuDoubleComplex(fma(-l.x, u.x, fma(l.y, u.y, low.x)),
+                                        fma(-l.x, u.y, fma(-l.y, u.x, low.y)));
+      if (col < m) {
+        const int K = col / ET;
+        U[((long long)K * (K + 1) / 2 + J) * (ET * ET) + (j % ET) * ET + col % ET] = dfc_split(u);
+        if (col == j) dU[j] = u;
+      } else {
+        R[(long long)j * a.ldy + (col - m)] = u;
       }
-      __syncthreads();
-      if (threadIdx.x == 0) {
-        s_swap = (j + 1 < m && cabs2(nxt[j]) > cabs2(cur[j])) ? 1 : 0;
-      }
-      __syncthreads();
-      if (s_swap) {
-        cplx* tmp = cur; cur = nxt; nxt = tmp;
-        for (int p = threadIdx.x; p < np; p += blockDim.x) {
-          cplx t0 = R[j * ldr + p];
-          R[j * ldr + p] = R[(j + 1) * ldr + p];
-          R[(j + 1) * ldr + p] = t0;
-        }
-      }
-      __syncthreads();
-      // row j of U: U(j, col) at column col's offset col(col+1)/2 + j
-      for (int col = j + threadIdx.x; col < m; col += blockDim.x)
-        Ud[(long long)col * (col + 1) / 2 + j] = dfc_from(cur[col]);
-      if (threadIdx.x == 0) dU[j] = cur[j];
-      if (j + 1 < m) {
-        if (threadIdx.x == 0) {
-          cplx piv = cur[j];
-          if (piv.x == 0.0 && piv.y == 0.0) { atomicExch(a.singular, 1); s_l = cz(); }
-          else s_l = cuCdiv(nxt[j], piv);
-        }
-        __syncthreads();
-        const cplx l = s_l;
-        for (int col = j + 1 + threadIdx.x; col < m; col += blockDim.x) nxt[col] = cuCsub(nxt[col], cuCmul(l, cur[col]));
-        for (int p = threadIdx.x; p < np; p += blockDim.x)
-          R[(j + 1) * ldr + p] = cuCsub(R[(j + 1) * ldr + p], cuCmul(l, R[j * ldr + p]));
-        __syncthreads();
-        cplx* tmp = cur; cur = nxt; nxt = tmp;
-      }
+    };
+    int col = j + ((tid - j) & (EF_T - 1));   // the thread's first column >= j
+    if (!last && col == j + 1) {              // the next pivot first: the next step waits for nothing else
+      step(col, cuCadd(next(j + 1, col), sig));
+      pivot(col, cur[col]);
+      col += EF_T;
     }
-    __syncthreads();
-    // back substitution, column oriented, P right-hand sides at a time: y_j = R_j / U_jj (FP64);
-    // R_i -= U_ij y_j for i < j (double-float)
-    const int p = threadIdx.x % P, i0 = threadIdx.x / P;
-    constexpr int ISTEP = 256 / P;
-    for (int pc0 = 0; pc0 < np; pc0 += P) {
-      const int pn = min(P, np - pc0);
-      for (int t = threadIdx.x; t < m * P; t += blockDim.x) {
-        const int i = t / P, pp = t % P;
-        Rs[t] = pp < pn ? dfc_from(R[i * ldr + pc0 + pp]) : make_float4(0.f, 0.f, 0.f, 0.f);
-      }
-      __syncthreads();
-      for (int j = m - 1; j >= 0; --j) {
-        if (threadIdx.x < pn) {
-          const cplx d = dU[j];
-          const cplx y = (d.x == 0.0 && d.y == 0.0) ? cz() : cuCdiv(dfc_to(Rs[j * P + threadIdx.x]), d);
-          Rs[j * P + threadIdx.x] = dfc_from(y);
-        }
-        __syncthreads();
-        if (p < pn) {
-          const float4 yj = Rs[j * P + p];
-          const float4* Uc = Ud + (long long)j * (j + 1) / 2;
-          for (int i = i0; i < j; i += ISTEP) Rs[i * P + p] = dfc_sub_mul(Rs[i * P + p], Uc[i], yj);
-        }
-        __syncthreads();
-      }
-      for (int t = threadIdx.x; t < m * P; t += blockDim.x) {
-        const int i = t / P, pp = t % P;
-        if (pp < pn) R[i * ldr + pc0 + pp] = dfc_to(Rs[t]);
-      }
-      __syncthreads();
-    }
+    for (; col < n; col += EF_T) step(col, last ? cz() : next(j + 1, col));
+    issue(j + EF_RING);   // into the slot of row j, which this thread has consumed
   }
 }
 
-// scratch per CTA of eval_solve_kernel (16-byte units)
-long long eval_scratch_per_cta(int m) { return (long long)m * (m + 1) / 2 + 3LL * m + 64; }
-
-// CTAs per SM of the evaluation solves: the steps of one solve are a chain of barriers and memory
-// round trips, so several solves share each SM
-constexpr int EVAL_CTAS_PER_SM = 4;
-// launch with the widest right-hand-side chunk whose double-float block lets EVAL_CTAS_PER_SM CTAs
-// share an SM (narrower chunks, down to one column, for large models)
-void launch_eval_solve(const EvalArgs& ea, int grid, cudaStream_t s) {
-  const size_t cap = std::max<size_t>(200 * 1024 / EVAL_CTAS_PER_SM, sizeof(float4) * (size_t)ea.m);
-  GFCC_CHECK(cap <= 200 * 1024, GFCC_ERR_ARG, "reduced model too large for the evaluation kernel");
-  auto go = [&](auto Pc) {
-    constexpr int P = decltype(Pc)::value;
-    const size_t bytes = sizeof(float4) * (size_t)ea.m * P;
-    static bool attr[64] = {};   // per instantiation, once per device (attributes live in each context)
-    int dev = 0;
-    GFCC_CUDA(cudaGetDevice(&dev));
-    GFCC_CHECK(dev >= 0 && dev < 64, GFCC_ERR_ARG, "device ordinal above 63");
-    if (!attr[dev]) {
-      GFCC_CUDA(cudaFuncSetAttribute(eval_solve_kernel<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
-      attr[dev] = true;
+// Back substitution, one CTA per (frequency, group of P = 8 C right-hand sides), by blocks of 32 rows from
+// the bottom: acc = R_J - sum_{K > J} U_JK Y_K in double-float with 2 x C register tiles, then the 32 x 32
+// triangular solve by four lanes per right-hand side with one warp barrier per row. U and Y arrive by
+// cp.async in steps of 16 columns of U, double-buffered: per step a thread takes 2 + C shared loads for 2 C
+// complex multiply-adds of 48 FP32 operations, so the FP32 pipe is what bounds it; 34-43 KB of shared memory
+// and 128 threads whatever P keep four CTAs (one warp each per scheduler) on an SM. Solved blocks are kept
+// in Y as double-float and converted to FP64 at the end.
+constexpr int EB_T = 128, EK = ET / 2;
+template <int C>
+__global__ void __launch_bounds__(EB_T, 4) eval_backsub_kernel(EvalArgs a, int w0) {
+  constexpr int P = 8 * C, US = EK + 1;    // padded U row: rows of a column on different banks
+  extern __shared__ float4 eb_sm[];
+  float4* sU = eb_sm;                      // [2][ET][US]: a half tile each; both halves of the diagonal tile
+  float4* sY = sU + 2 * ET * US;           // [2][EK][P]; the block's right-hand sides during its solve
+  float4* sD = sY + 2 * EK * P;            // [ET] reciprocal diagonal
+  const int m = a.m, np = a.np, tid = threadIdx.x, f = blockIdx.x, w = w0 + f;
+  const int p0 = blockIdx.y * P, pn = min(P, np - p0);
+  const float4* U = a.U + (long long)f * eval_tiles(m) * (ET * ET);
+  const cplx* dU = a.dU + (long long)f * m;
+  cplx* R = a.Y + (long long)w * np + p0;
+  const int T = (m + ET - 1) / ET;
+  const int tx = tid & 7, ty = tid >> 3;   // columns tx + 8 i, rows 2 ty + r
+  // half h of tile (J, K) into buffer h; columns of U beyond m as zeros
+  auto load_u = [&](int J, int K, int h) {
+    const float4* s = U + ((long long)K * (K + 1) / 2 + J) * (ET * ET) + h * EK;
+    for (int t = tid; t < ET * EK; t += EB_T) {
+      const int r = t / EK, k = t % EK;
+      cp_async16(sU + (h * ET + r) * US + k, s + r * ET + k, K * ET + h * EK + k < m);
     }
-    eval_solve_kernel<P><<<grid, 256, bytes, s>>>(ea);
   };
-  const size_t row = sizeof(float4) * (size_t)ea.m;
-  if (row * 16 <= cap) go(std::integral_constant<int, 16>{});
-  else if (row * 8 <= cap) go(std::integral_constant<int, 8>{});
-  else if (row * 4 <= cap) go(std::integral_constant<int, 4>{});
-  else if (row * 2 <= cap) go(std::integral_constant<int, 2>{});
-  else go(std::integral_constant<int, 1>{});
-  GFCC_LAUNCH_CHECK();
+  auto load_y = [&](int K, int h) {
+    for (int t = tid; t < EK * P; t += EB_T) {
+      const int k = K * ET + h * EK + t / P, p = t % P;
+      const bool on = k < m && p < pn;
+      cp_async16(sY + h * EK * P + t, on ? R + (long long)k * a.ldy + p : R, on);
+    }
+  };
+  for (int J = T - 1; J >= 0; --J) {
+    if (J < T - 1) {
+      load_u(J, T - 1, 0);
+      load_y(T - 1, 0);
+      cp_async_commit();
+    }
+    float4 acc[2][C];
+#pragma unroll
+    for (int r = 0; r < 2; ++r)
+#pragma unroll
+      for (int i = 0; i < C; ++i) {
+        const int row = J * ET + 2 * ty + r, p = tx + 8 * i;
+        acc[r][i] = (row < m && p < pn) ? dfc_from(R[(long long)row * a.ldy + p]) : make_float4(0.f, 0.f, 0.f, 0.f);
+      }
+    for (int K = T - 1; K > J; --K) {
+#pragma unroll 1
+      for (int h = 0; h < 2; ++h) {
+        // the next half tile: the second half of this one, the first of the next; after the last the diagonal
+        // tile is loaded below
+        if (h == 0 || K - 1 > J) {
+          load_u(J, h == 0 ? K : K - 1, h ^ 1);
+          load_y(h == 0 ? K : K - 1, h ^ 1);
+        }
+        cp_async_commit();
+        cp_async_wait<1>();
+        __syncthreads();
+        const float4* u = sU + (h * ET + 2 * ty) * US;
+        const float4* y = sY + h * EK * P + tx;
+#pragma unroll 1
+        for (int k0 = 0; k0 < EK; k0 += 8) {
+#pragma unroll 2
+          for (int k = k0; k < k0 + 8; ++k) {
+            const float4 u0 = u[k], u1 = u[US + k];
+#pragma unroll
+            for (int i = 0; i < C; ++i) {
+              const float4 yy = y[k * P + 8 * i];
+              dfc_acc(acc[0][i], u0, yy);
+              dfc_acc(acc[1][i], u1, yy);
+            }
+          }
+#pragma unroll
+          for (int r = 0; r < 2; ++r)
+#pragma unroll
+            for (int i = 0; i < C; ++i) dfc_renorm(acc[r][i]);
+        }
+        __syncthreads();
+      }
+    }
+    load_u(J, J, 0);
+    load_u(J, J, 1);
+    cp_async_commit();
+    float4* sR = sY;   // [ET][P]
+#pragma unroll
+    for (int r = 0; r < 2; ++r)
+#pragma unroll
+      for (int i = 0; i < C; ++i) sR[(2 * ty + r) * P + tx + 8 * i] = acc[r][i];
+    if (tid < ET && J * ET + tid < m) {
+      const cplx d = dU[J * ET + tid];
+      sD[tid] = (d.x == 0.0 && d.y == 0.0) ? make_float4(0.f, 0.f, 0.f, 0.f)
+                                           : dfc_from(cuCdiv(make_cuDoubleComplex(1.0, 0.0), d));
+    }
+    cp_async_wait<0>();
+    __syncthreads();
+    {
+      // lanes 8 g .. 8 g + 7 hold eight right-hand sides and take the rows i = g (mod 4)
+      const int g = (tid & 31) >> 3;
+      for (int c8 = tid >> 5; c8 < C; c8 += EB_T / 32) {
+        const int p = c8 * 8 + (tid & 7);
+        for (int j = min(ET, m - J * ET) - 1; j >= 0; --j) {
+          const float4* u = sU + (j / EK) * ET * US + j % EK;
+          const float4 y = dfc_mul(sR[j * P + p], sD[j]);
+          for (int i = g; i < j; i += 4) sR[i * P + p] = dfc_sub_mul(sR[i * P + p], u[i * US], y);
+          __syncwarp();
+          if (g == 0) sR[j * P + p] = y;
+        }
+      }
+    }
+    __syncthreads();
+    for (int t = tid; t < ET * P; t += EB_T) {
+      const int row = J * ET + t / P, p = t % P;
+      if (row < m && p < pn) *reinterpret_cast<float4*>(R + (long long)row * a.ldy + p) = sR[t];
+    }
+    __syncthreads();
+  }
+  for (int t = tid; t < m * P; t += EB_T) {
+    const int p = t % P;
+    cplx* q = R + (long long)(t / P) * a.ldy + p;
+    if (p < pn) *q = dfc_to(*reinterpret_cast<const float4*>(q));
+  }
+}
+
+// width of the right-hand-side groups: the one that pads np least (the widest of equals: U is read once
+// per group)
+int eval_group(int np) {
+  int best = 8;
+  for (int P : {8, 16, 24, 32, 40, 48})
+    if ((np + P - 1) / P * P <= (np + best - 1) / best * best) best = P;
+  return best;
+}
+struct EvalScratch {   // U tiles and diagonals of the frequencies in flight
+  DBuf<float4> U;
+  DBuf<cplx> dU, rows;
+  int nf = 0;          // frequencies they hold
+};
+// Frequencies in flight: U of all of them in at most 4 GB and an eighth of the free memory.
+void eval_scratch_alloc(EvalScratch& e, int m, int np, int nw) {
+  const long long per = eval_tiles(m) * ET * ET * (long long)sizeof(float4) + 16LL * m;
+  long long budget = 1LL << 30;
+  if (per * nw > budget) {
+    size_t freeb = device_free_bytes();
+    if (freeb == 0) freeb = 8ull << 30;
+    budget = std::min<long long>(4LL << 30, (long long)(freeb / 8));
+  }
+  e.nf = (int)std::max<long long>(1, std::min<long long>({(long long)nw, budget / per, 65535LL}));
+  e.U.alloc(eval_tiles(m) * ET * ET * e.nf);
+  e.dU.alloc((long long)m * e.nf);
+  if (sizeof(cplx) * (size_t)(EF_RING + 1) * (m + np) > 200 * 1024) e.rows.alloc((long long)(m + np) * e.nf);
+}
+void launch_eval_solve(EvalArgs ea, EvalScratch& es, cudaStream_t s) {
+  const size_t fbytes = sizeof(cplx) * (size_t)(EF_RING + 1) * (ea.m + ea.np);
+  const bool ring = fbytes <= 200 * 1024;
+  int dev = 0;
+  GFCC_CUDA(cudaGetDevice(&dev));
+  GFCC_CHECK(dev >= 0 && dev < 64, GFCC_ERR_ARG, "device ordinal above 63");
+  ea.U = es.U.p;
+  ea.dU = es.dU.p;
+  auto backsub = [&](auto Cc, int w0, int nf) {
+    constexpr int C = decltype(Cc)::value;   // at most 43 KB of shared memory: no attribute needed
+    constexpr size_t bytes = sizeof(float4) * (2 * ET * (EK + 1) + 2 * EK * 8 * C + ET);
+    static_assert(bytes <= 48 * 1024, "default shared memory");
+    eval_backsub_kernel<C><<<dim3(nf, (ea.np + 8 * C - 1) / (8 * C)), EB_T, bytes, s>>>(ea, w0);
+  };
+  static bool attr_f[64] = {};
+  if (!attr_f[dev]) {
+    GFCC_CUDA(cudaFuncSetAttribute(eval_factor_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
+    attr_f[dev] = true;
+  }
+  for (int w0 = 0; w0 < ea.nw; w0 += es.nf) {
+    const int nf = std::min(es.nf, ea.nw - w0);
+    if (ring) eval_factor_kernel<true><<<nf, EF_T, fbytes, s>>>(ea, w0, nullptr);
+    else eval_factor_kernel<false><<<nf, EF_T, 0, s>>>(ea, w0, es.rows.p);
+    GFCC_LAUNCH_CHECK();
+    switch (eval_group(ea.np)) {
+      case 8: backsub(std::integral_constant<int, 1>{}, w0, nf); break;
+      case 16: backsub(std::integral_constant<int, 2>{}, w0, nf); break;
+      case 24: backsub(std::integral_constant<int, 3>{}, w0, nf); break;
+      case 32: backsub(std::integral_constant<int, 4>{}, w0, nf); break;
+      case 40: backsub(std::integral_constant<int, 5>{}, w0, nf); break;
+      default: backsub(std::integral_constant<int, 6>{}, w0, nf); break;
+    }
+    GFCC_LAUNCH_CHECK();
+  }
 }
 
 // A[w] = -(1/pi) sum_p Im G[w][p][qidx[p]] (p with a matching q only)
@@ -1211,6 +1431,13 @@ static void hessenberg(gfcc_ctx* c, bool want_res) {
                                                                         rows_all * len);
     GFCC_LAUNCH_CHECK();
   }
+  {  // the evaluation reads H and bhat by rows
+    ms.hHr.alloc((long long)m * m);
+    ms.hbr.alloc((long long)m * np);
+    int dh[3] = {m, m, 2}, db[3] = {np, m, 2}, pm[3] = {1, 0, 2};
+    permute(reinterpret_cast<const double*>(Hw), dh, 3, pm, reinterpret_cast<double*>(ms.hHr.p), 1.0, 0.0, s);
+    permute(reinterpret_cast<const double*>(bw), db, 3, pm, reinterpret_cast<double*>(ms.hbr.p), 1.0, 0.0, s);
+  }
   GFCC_CUDA(cudaStreamSynchronize(s));   // wv is released on return
   ms.hess_version = ms.version;
   ms.hess_res = want_res;
@@ -1226,7 +1453,7 @@ void mor_eval(gfcc_ctx* c, const double* omegas_host, int nw, cplx* G_dev, doubl
   GFCC_CHECK(m > 0, GFCC_ERR_STATE, "mor_eval: empty reduced model");
   const bool want_res = maxres_dev != nullptr;
   hessenberg(c, want_res);
-  const cplx *Hw = ms.hH.p, *bw = ms.hb.p, *cw = ms.hc.p;
+  const cplx* cw = ms.hc.p;
   const cplx *A1 = ms.hA1.p, *A2 = ms.hA2.p, *RBw = ms.hRB.p;
   DBuf<double> dbn;
   std::vector<int> qidx(np, -1);
@@ -1242,13 +1469,12 @@ void mor_eval(gfcc_ctx* c, const double* omegas_host, int nw, cplx* G_dev, doubl
   GFCC_CUDA(cudaMemcpyAsync(dbn.p, ms.bnorm.data(), sizeof(double) * np, cudaMemcpyHostToDevice, s));
   // frequencies in batches: solutions Y [m][nb np] of a batch (about 2 GB at most), then Ghat = chat^T Y
   // and the residual coefficients (w - i eta) RS Y + RZ Y - RB as complex GEMMs over the whole batch
-  const long long per = eval_scratch_per_cta(m);
   const long long bw_max = std::max<long long>(1, (2LL << 30) / ((long long)m * np * (long long)sizeof(cplx)));
   const int nbw = (int)std::min<long long>(nw, bw_max);
-  const int ncta = (int)std::min<long long>(nbw, (long long)EVAL_CTAS_PER_SM * 152);
-  DBuf<cplx> scratch, Y, Ys, Cr, Gt, Yd;
+  DBuf<cplx> Y, Ys, Cr, Gt, Yd;
   DBuf<double> rcol;
-  scratch.alloc(per * ncta);
+  EvalScratch es;
+  eval_scratch_alloc(es, m, np, nbw);
   Y.alloc((long long)m * nbw * np);
   const bool want_G = G_dev != nullptr || A_dev != nullptr;
   if (want_G && !G_dev) Gt.alloc((long long)nbw * np * nq);
@@ -1263,13 +1489,12 @@ void mor_eval(gfcc_ctx* c, const double* omegas_host, int nw, cplx* G_dev, doubl
     const long long ldy = (long long)nb * np;
     EvalArgs ea;
     ea.m = m; ea.np = np; ea.nw = nb;
-    ea.H = Hw; ea.bw = bw;
+    ea.H = ms.hHr.p; ea.b = ms.hbr.p;
     ea.omegas = dom.p + w0; ea.eta = ms.eta;
-    ea.scratch = scratch.p; ea.scratch_per_cta = per;
     ea.Y = Y.p; ea.ldy = ldy; ea.singular = dsing.p;
     {
       ProfScope ps(PROF_EVAL_SOLVE, 0.0, s);
-      launch_eval_solve(ea, std::min(ncta, nb), s);
+      launch_eval_solve(ea, es, s);
     }
     if (want_G) {   // G(q, n) = sum_k cw[q][k] Y[k][n], stored at Gb[n nq + q]
       cplx* Gb = G_dev ? G_dev + (long long)w0 * np * nq : Gt.p;
@@ -1289,8 +1514,8 @@ void mor_eval(gfcc_ctx* c, const double* omegas_host, int nw, cplx* G_dev, doubl
       GFCC_CUDA(cudaMemcpyAsync(Yd.p, Y.p, sizeof(cplx) * m * ldy, cudaMemcpyDeviceToDevice, s));
       EvalArgs eb = ea;
       eb.Y = Yd.p;
-      eb.rhs_in_Y = 1;
-      launch_eval_solve(eb, std::min(ncta, nb), s);
+      eb.b = nullptr;
+      launch_eval_solve(eb, es, s);
       ZGemmDesc g;
       g.M = nq; g.N = (int)ldy; g.K = m;
       g.A = cw; g.sam = 1; g.sak = nq;
@@ -1337,23 +1562,21 @@ void mor_extrapolate(gfcc_ctx* c, const double* omegas_host, int nw, cplx* X0) {
   GFCC_CHECK(m > 0, GFCC_ERR_STATE, "mor_extrapolate: empty reduced model");
   const long long N = (long long)nw * np;
   hessenberg(c, false);
-  DBuf<cplx> Y, scratch;
+  DBuf<cplx> Y;
   DBuf<double> dom;
   DBuf<int> dsing;
-  const long long per = eval_scratch_per_cta(m);
-  const int ncta = (int)std::min<long long>(nw, (long long)EVAL_CTAS_PER_SM * 152);
-  scratch.alloc(per * ncta);
+  EvalScratch es;
+  eval_scratch_alloc(es, m, np, nw);
   Y.alloc((long long)m * N);
   dom.alloc(nw); dsing.alloc(1);
   dsing.zero(s);
   GFCC_CUDA(cudaMemcpyAsync(dom.p, omegas_host, sizeof(double) * nw, cudaMemcpyHostToDevice, s));
   EvalArgs ea;
   ea.m = m; ea.np = np; ea.nw = nw;
-  ea.H = ms.hH.p; ea.bw = ms.hb.p;
+  ea.H = ms.hHr.p; ea.b = ms.hbr.p;
   ea.omegas = dom.p; ea.eta = ms.eta;
-  ea.scratch = scratch.p; ea.scratch_per_cta = per;
   ea.Y = Y.p; ea.ldy = N; ea.singular = dsing.p;
-  launch_eval_solve(ea, ncta, s);
+  launch_eval_solve(ea, es, s);
   for (int j = m - 3; j >= 0; --j) {   // yhat = P y_H, P = H_0 H_1 ... (Hermitian reflectors)
     house_rows_kernel<<<(unsigned)((N + 127) / 128), 128, 0, s>>>(Y.p, N, N, j + 1, m - j - 1,
                                                                   ms.hV.p + (long long)j * m, ms.htau.p + j);
