@@ -45,7 +45,7 @@ extern "C" {
 #define GFCC_PREC_FP64 0        /* FP64 everywhere */
 #define GFCC_PREC_TF32 1        /* every sigma GEMM on tcgen05 kind::tf32, FP32 accumulate; FP64 diagonal */
 #define GFCC_PREC_BF16 2        /* every sigma GEMM on tcgen05 kind::f16 with bf16 operands, FP32 accumulate */
-#define GFCC_PREC_FP64_TC 3     /* FP64-accurate: exact integer bf16 slices of the FP64 operands on tcgen05,
+#define GFCC_PREC_FP64_TC 3     /* FP64-accurate: exact integer f16 slices of the FP64 operands on tcgen05,
                                    exact FP32 partial sums recombined in FP64 (Ozaki scheme) */
 
 typedef struct gfcc_ctx* gfcc_t;
@@ -326,7 +326,7 @@ long long gfcc_launch_count(void);
 
 /* Turn per-launch CUDA-event timing of the GEMM kernel classes and of the pipeline phases on
  * (enable = 1) or off, clearing earlier records. Kernel classes: 0 tcgen05 GEMM with tf32/bf16-
- * rounded operands (inner solves); 1 FP64 SIMT GEMM; 2 tcgen05 GEMM on exact bf16 slices
+ * rounded operands (inner solves); 1 FP64 SIMT GEMM; 2 tcgen05 GEMM on exact f16 slices
  * (FP64-accurate products). Phases (whole regions, nested ones counted in both): 3 low-precision
  * sigma; 4 FP64-accurate sigma; 5 Arnoldi orthogonalisation and updates; 6 MOR orthonormalisation
  * and projections; 7 reduced-model evaluation; 8 H-bar build; 9 column-by-column Gram-Schmidt

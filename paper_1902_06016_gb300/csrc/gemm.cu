@@ -316,10 +316,10 @@ void dgemm(const GemmDesc& d, cudaStream_t s) {
 
 void zgemm(const ZGemmDesc& d, cudaStream_t s) {
   // large complex products (the subspace projections of the reduced model) go to the exact-slice
-  // tensor-core GEMM with 7 slices (48 bits per row)
+  // tensor-core GEMM with 6 slices (53 bits per row)
   if (d.batch == 1 && (double)d.M * (double)d.N * (double)d.K >= oz_min_macs() && d.M >= 16 && d.N >= 1 &&
       (double)d.K >= 256) {
-    zgemm_oz(d, 7, s);
+    zgemm_oz(d, 6, s);
     return;
   }
   Args<cplx> a{d.M, d.N, d.K, d.A, d.sam, d.sak, d.bsa, d.conjA, d.B, d.sbk, d.sbn, d.bsb, d.conjB,

@@ -45,7 +45,7 @@ void count_launch();
 enum ProfClass {
   PROF_TC_GEMM = 0,      // tcgen05 GEMM, tf32/bf16-rounded operands
   PROF_F64_GEMM = 1,     // FP64 SIMT GEMM
-  PROF_TC_SLICE = 2,     // tcgen05 GEMM on exact bf16 slices
+  PROF_TC_SLICE = 2,     // tcgen05 GEMM on exact f16 slices
   PROF_SIGMA_LP = 3,     // whole low-precision sigma (operand prep, GEMMs, combine)
   PROF_SIGMA_EX = 4,     // whole FP64-accurate sigma (exact slices or FP64 SIMT)
   PROF_KRYLOV = 5,       // Arnoldi: preconditioner, Gram-Schmidt, norms, Givens, corrections

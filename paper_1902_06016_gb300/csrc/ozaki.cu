@@ -2,7 +2,7 @@
 #include "ozaki.cuh"
 #include "tc_gemm.cuh"
 
-#include <cuda_bf16.h>
+#include <cuda_fp16.h>
 
 #include <algorithm>
 #include <type_traits>
@@ -24,14 +24,15 @@ int grid_for(long long n) {
 __device__ __forceinline__ unsigned long long abs_bits(double x) {
   return (unsigned long long)__double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFULL;
 }
+constexpr int OZ_BITS = 9, OZ_TOP = 8;   // bits per digit; the leading digit's weight is 2^(e - OZ_TOP)
 constexpr int ZERO_ROW = -100000;   // row exponent marker of a zero (or subnormal-only) row
 __device__ __forceinline__ int row_exponent(unsigned long long maxbits) {
   const int ex = (int)(maxbits >> 52);
   return ex == 0 ? ZERO_ROW : ex - 1022;
 }
-// Balanced base-128 digits of x relative to 2^(e - 6):  x ~ 2^(e-6) sum_{i<ns} a_i 2^(-7i), |a_i| <= 64.
-// V = round(|x| 2^(6 - e + 7(ns-1))) is formed exactly from the mantissa (|V| <= 2^(6 + 7(ns-1)) < 2^56);
-// digit i is V / 2^(7(ns-1-i)) rounded half up, V keeps the remainder (|remainder| <= 2^(shift-1)), and
+// Balanced base-512 digits of x relative to 2^(e - 8):  x ~ 2^(e-8) sum_{i<ns} a_i 2^(-9i), |a_i| <= 256.
+// V = round(|x| 2^(8 - e + 9(ns-1))) is formed exactly from the mantissa (|V| <= 2^(8 + 9(ns-1)) <= 2^62);
+// digit i is V / 2^(9(ns-1-i)) rounded half up, V keeps the remainder (|remainder| <= 2^(shift-1)), and
 // the signs of all digits follow x (so -x gives exactly the negated digits). a[i] holds digit i. The slice
 // count NS is a template argument (no predicated iterations, constant shifts).
 template <int NS>
@@ -41,30 +42,30 @@ __device__ __forceinline__ void digits_t(double x, int e, int (&a)[NS]) {
   long long V = 0;
   if (ex != 0 && e != ZERO_ROW) {
     const long long m = (bits & 0xFFFFFFFFFFFFFLL) | 0x10000000000000LL;
-    const int t = ex - 1075 + 6 - e + 7 * (NS - 1);
+    const int t = ex - 1075 + OZ_TOP - e + OZ_BITS * (NS - 1);
     if (t >= 0) V = m << t;
     else if (t > -62) V = (m + (1LL << (-t - 1))) >> (-t);
   }
   const bool neg = bits < 0;
 #pragma unroll
   for (int i = 0; i < NS; ++i) {
-    const int shift = 7 * (NS - 1 - i);
+    const int shift = OZ_BITS * (NS - 1 - i);
     const long long d = (i < NS - 1) ? ((V + (1LL << (shift - 1))) >> shift) : V;
     V -= d << shift;
     a[i] = neg ? -(int)d : (int)d;
   }
 }
-// digits of two adjacent elements of a row, written as one bf16 pair per slot (k even)
+// digits of two adjacent elements of a row, written as one f16 pair per slot (k even)
 template <int NS>
-__device__ __forceinline__ void slice_pair(double x0, double x1, int e, __nv_bfloat16* __restrict__ o, long long kp,
+__device__ __forceinline__ void slice_pair(double x0, double x1, int e, __half* __restrict__ o, long long kp,
                                            int reversed, long long k) {
   int a0[NS], a1[NS];
   digits_t<NS>(x0, e, a0);
   digits_t<NS>(x1, e, a1);
 #pragma unroll
   for (int i = 0; i < NS; ++i)
-    *reinterpret_cast<__nv_bfloat162*>(o + (long long)(reversed ? NS - 1 - i : i) * kp + k) =
-        __halves2bfloat162(__int2bfloat16_rn(a0[i]), __int2bfloat16_rn(a1[i]));
+    *reinterpret_cast<__half2*>(o + (long long)(reversed ? NS - 1 - i : i) * kp + k) =
+        __halves2half2(__int2half_rn(a0[i]), __int2half_rn(a1[i]));
 }
 
 // Real rows (row-major, row stride ldx, K used columns): one block per row (grid-stride) for long
@@ -72,7 +73,7 @@ __device__ __forceinline__ void slice_pair(double x0, double x1, int e, __nv_bfl
 template <int NS>
 __global__ void __launch_bounds__(256) slice_kernel(const double* __restrict__ X, long long ldx, long long rows,
                                                     long long K, long long kp, int reversed,
-                                                    __nv_bfloat16* __restrict__ out, int* __restrict__ expo) {
+                                                    __half* __restrict__ out, int* __restrict__ expo) {
   __shared__ unsigned long long red[8];
   for (long long r = blockIdx.x; r < rows; r += gridDim.x) {
     const double* x = X + r * ldx;
@@ -86,7 +87,7 @@ __global__ void __launch_bounds__(256) slice_kernel(const double* __restrict__ X
     const int e = row_exponent(mx);
     __syncthreads();
     if (threadIdx.x == 0) expo[r] = e == ZERO_ROW ? 0 : e;
-    __nv_bfloat16* o = out + r * (long long)NS * kp;
+    __half* o = out + r * (long long)NS * kp;
     for (long long k = 2LL * threadIdx.x; k < kp; k += 2LL * blockDim.x)
       slice_pair<NS>(k < K ? x[k] : 0.0, k + 1 < K ? x[k + 1] : 0.0, e, o, kp, reversed, k);
   }
@@ -95,7 +96,7 @@ __global__ void __launch_bounds__(256) slice_kernel(const double* __restrict__ X
 template <int NS>
 __global__ void __launch_bounds__(256) slice_rows_warp_kernel(const double* __restrict__ X, long long ldx,
                                                               long long rows, long long K, long long kp, int reversed,
-                                                              __nv_bfloat16* __restrict__ out, int* __restrict__ expo) {
+                                                              __half* __restrict__ out, int* __restrict__ expo) {
   const long long r = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (r >= rows) return;
@@ -105,7 +106,7 @@ __global__ void __launch_bounds__(256) slice_rows_warp_kernel(const double* __re
   for (int off = 16; off > 0; off >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, off));
   const int e = row_exponent(mx);
   if (lane == 0) expo[r] = e == ZERO_ROW ? 0 : e;
-  __nv_bfloat16* o = out + r * (long long)NS * kp;
+  __half* o = out + r * (long long)NS * kp;
   for (long long k = 2LL * lane; k < kp; k += 64)
     slice_pair<NS>(k < K ? x[k] : 0.0, k + 1 < K ? x[k + 1] : 0.0, e, o, kp, reversed, k);
 }
@@ -133,17 +134,17 @@ template <int NS>
 __global__ void __launch_bounds__(256) slice_chunk_kernel(const double* __restrict__ X, long long ldx, long long K,
                                                           long long kp, int reversed,
                                                           const unsigned long long* __restrict__ rowmax,
-                                                          __nv_bfloat16* __restrict__ out, int* __restrict__ expo) {
+                                                          __half* __restrict__ out, int* __restrict__ expo) {
   const long long r = blockIdx.y, k0 = blockIdx.x * SL_CH, k1 = min(kp, k0 + SL_CH);   // SL_CH is even
   const double* x = X + r * ldx;
   const int e = row_exponent(rowmax[r]);
   if (blockIdx.x == 0 && threadIdx.x == 0) expo[r] = e == ZERO_ROW ? 0 : e;
-  __nv_bfloat16* o = out + r * (long long)NS * kp;
+  __half* o = out + r * (long long)NS * kp;
   for (long long k = k0 + 2LL * threadIdx.x; k < k1; k += 2LL * blockDim.x)
     slice_pair<NS>(k < K ? x[k] : 0.0, k + 1 < K ? x[k + 1] : 0.0, e, o, kp, reversed, k);
 }
 
-// the slice count of a launch as a template argument (2..8 slices)
+// the slice count of a launch as a template argument (2..7 slices)
 template <typename F>
 void with_ns(int ns, F&& f) {
   switch (ns) {
@@ -152,8 +153,7 @@ void with_ns(int ns, F&& f) {
     case 4: f(std::integral_constant<int, 4>{}); break;
     case 5: f(std::integral_constant<int, 5>{}); break;
     case 6: f(std::integral_constant<int, 6>{}); break;
-    case 7: f(std::integral_constant<int, 7>{}); break;
-    default: f(std::integral_constant<int, 8>{}); break;
+    default: f(std::integral_constant<int, 7>{}); break;
   }
 }
 
@@ -213,7 +213,7 @@ template <int NS>
 __global__ void __launch_bounds__(256) zslice_kernel(const cplx* __restrict__ Z, long long s_r, long long s_k,
                                                      int conj, long long R, long long K, int mode,
                                                      const unsigned long long* __restrict__ rowmax, long long kp,
-                                                     int reversed, __nv_bfloat16* __restrict__ out,
+                                                     int reversed, __half* __restrict__ out,
                                                      int* __restrict__ expo, int slot_major = 0) {
   constexpr int ns = NS;
   __shared__ cplx tile[ZT_R][ZT_K + 1];
@@ -234,8 +234,8 @@ __global__ void __launch_bounds__(256) zslice_kernel(const cplx* __restrict__ Z,
     const long long b0 = slot_major ? r * kp : r * (long long)ns * kp;
     const long long b1 = slot_major ? (R + r) * kp : (R + r) * (long long)ns * kp;
     const long long sstep = slot_major ? rows_total * kp : kp;
-    __nv_bfloat16* o0 = out + b0;
-    __nv_bfloat16* o1 = out + b1;
+    __half* o0 = out + b0;
+    __half* o1 = out + b1;
     for (int tk = lane; tk < ZT_K; tk += 32) {
       const long long k = k0 + tk;
       if (2 * k >= kp) break;
@@ -248,13 +248,13 @@ __global__ void __launch_bounds__(256) zslice_kernel(const cplx* __restrict__ Z,
         {
           const long long off = (long long)(reversed ? ns - 1 - i : i) * sstep + 2 * k;
           if (mode == 0) {
-            *reinterpret_cast<__nv_bfloat162*>(o0 + off) = __halves2bfloat162(__int2bfloat16_rn(are[i]),
-                                                                               __int2bfloat16_rn(aim[i]));
+            *reinterpret_cast<__half2*>(o0 + off) = __halves2half2(__int2half_rn(are[i]),
+                                                                               __int2half_rn(aim[i]));
           } else {
-            *reinterpret_cast<__nv_bfloat162*>(o0 + off) = __halves2bfloat162(__int2bfloat16_rn(are[i]),
-                                                                               __int2bfloat16_rn(-aim[i]));
-            *reinterpret_cast<__nv_bfloat162*>(o1 + off) = __halves2bfloat162(__int2bfloat16_rn(aim[i]),
-                                                                               __int2bfloat16_rn(are[i]));
+            *reinterpret_cast<__half2*>(o0 + off) = __halves2half2(__int2half_rn(are[i]),
+                                                                               __int2half_rn(-aim[i]));
+            *reinterpret_cast<__half2*>(o1 + off) = __halves2half2(__int2half_rn(aim[i]),
+                                                                               __int2half_rn(are[i]));
           }
         }
       }
@@ -287,19 +287,22 @@ __device__ __forceinline__ double scale_pow2(double x, int k) {
   if (k >= -1022 && k <= 1023) return x * __longlong_as_double((long long)(k + 1023) << 52);
   return ldexp(x, k);
 }
-// sum_d S_d 2^(7 (nd - 1 - d)) for nd <= 8 per-diagonal integer sums |S_d| < 2^40: the first (up to four)
-// and the remaining diagonals are combined exactly in two 64-bit integers (each below 2^62) and joined by
-// one fused multiply-add, instead of an FP64 conversion and multiply-add per diagonal (FP64 is the scarce
-// pipe on this GPU: the output passes were bound by it). The caller scales by 2^(-7 (nd - 1)).
+// sum_d S_d 2^(9 (nd - 1 - d)) for nd <= 7 per-diagonal integer sums |S_d| < 2^43: up to three diagonals at a
+// time are combined exactly in a 64-bit integer (below 2^62) and the two or three integers joined by fused
+// multiply-adds, instead of an FP64 conversion and multiply-add per diagonal (FP64 is the scarce pipe on this
+// GPU: the output passes were bound by it). The caller scales by 2^(-9 (nd - 1)).
+__device__ __forceinline__ double pow2(int k) { return __longlong_as_double((long long)(k + 1023) << 52); }
 __device__ __forceinline__ double diag_combine(const long long* S, int nd) {
-  const int H = nd < 4 ? nd : 4;
-  long long hi = 0, lo = 0;
+  const int H = nd < 3 ? nd : 3, L = nd < 6 ? nd : 6;   // diagonals [0, H), [H, L), [L, nd)
+  long long hi = 0, mid = 0, lo = 0;
 #pragma unroll
   for (int d = 0; d < OZ_SLICES_MAX; ++d) {
-    if (d < H) hi += S[d] * (1LL << (7 * (H - 1 - d)));
-    else if (d < nd) lo += S[d] * (1LL << (7 * (nd - 1 - d)));
+    if (d < H) hi += S[d] * (1LL << (OZ_BITS * (H - 1 - d)));
+    else if (d < L) mid += S[d] * (1LL << (OZ_BITS * (L - 1 - d)));
+    else if (d < nd) lo += S[d];
   }
-  return fma((double)hi, __longlong_as_double((long long)(7 * (nd - H) + 1023) << 52), (double)lo);
+  if (nd <= 6) return fma((double)hi, pow2(OZ_BITS * (nd - H)), (double)mid);
+  return fma((double)hi, pow2(OZ_BITS * (nd - H)), fma((double)mid, pow2(OZ_BITS * (nd - L)), (double)lo));
 }
 // complex output value: alpha (re + i im) + beta C
 __device__ __forceinline__ cplx out_value(const OzOut& o, double re, double im, const cplx* p) {
@@ -345,9 +348,9 @@ __device__ __forceinline__ long long split_sum(const int* __restrict__ p, int zs
   return sum;
 }
 
-// One diagonal of a column chunk (Np real columns): its split sums, weighted by scale = 2^(-7d), are
+// One diagonal of a column chunk (Np real columns): its split sums, weighted by scale = 2^(-9d), are
 // added to the FP64 accumulator acc[m][n'] (MODE 0; first: acc is set), or, on the last diagonal, added
-// to acc, scaled by 2^(ea[m] + eb[n'] - 12) and written to a real (MODE 1) or complex (MODE 2) output.
+// to acc, scaled by 2^(ea[m] + eb[n'] - 16) and written to a real (MODE 1) or complex (MODE 2) output.
 // One thread per element, or (WARP) one warp for outputs too small to occupy the GPU that have many K
 // splits. Only the last diagonal needs the (m, n) of an element; 32-bit division when it fits.
 template <typename I>
@@ -377,7 +380,7 @@ __global__ void __launch_bounds__(256) oz_accumulate_kernel(const int* __restric
       if (!first) a = acc[t] + a;
       long long m, n;
       divmod<I>(t, Np, m, n);
-      const double v = scale_pow2(a, ea[m] + eb[n] - 12);
+      const double v = scale_pow2(a, ea[m] + eb[n] - 2 * OZ_TOP);
       if (writer) {
         double* p = o.out + m * o.ldo + n;
         *p = out_value_real(o, v, p);
@@ -393,7 +396,8 @@ __global__ void __launch_bounds__(256) oz_accumulate_kernel(const int* __restric
         ar = acc[tr] + ar;
         ai = acc[ti] + ai;
       }
-      const double re = scale_pow2(ar, ea[m] + eb[n] - 12), im = scale_pow2(ai, ea[m] + eb[N + n] - 12);
+      const double re = scale_pow2(ar, ea[m] + eb[n] - 2 * OZ_TOP),
+                   im = scale_pow2(ai, ea[m] + eb[N + n] - 2 * OZ_TOP);
       if (writer) {
         cplx* p = o.C + m * o.scm + n * o.scn;
         *p = out_value(o, re, im, p);
@@ -406,10 +410,9 @@ __global__ void __launch_bounds__(256) oz_accumulate_kernel(const int* __restric
 struct OzDiags {
   long long off[OZ_SLICES_MAX];
   int zs[OZ_SLICES_MAX];
-  double scale[OZ_SLICES_MAX];
   int nd;
 };
-// sum_d 2^(-7d) (split sums of diagonal d), times 2^(7 (nd - 1)) (see diag_combine)
+// sum_d 2^(-9d) (split sums of diagonal d), times 2^(9 (nd - 1)) (see diag_combine)
 template <bool WARP>
 __device__ __forceinline__ double diag_total(const int* __restrict__ slabs, const OzDiags& dg, long long stride,
                                              long long t, int lane) {
@@ -434,7 +437,7 @@ __global__ void __launch_bounds__(256) oz_output_kernel(const int* __restrict__ 
     if constexpr (MODE == 1) {
       long long m, n;
       divmod<I>(t, Np, m, n);
-      const double v = scale_pow2(diag_total<WARP>(slabs, dg, stride, t, lane), ea[m] + eb[n] - 12 - 7 * (dg.nd - 1));
+      const double v = scale_pow2(diag_total<WARP>(slabs, dg, stride, t, lane), ea[m] + eb[n] - 2 * OZ_TOP - OZ_BITS * (dg.nd - 1));
       if (writer) {
         double* p = o.out + m * o.ldo + n;
         *p = out_value_real(o, v, p);
@@ -444,7 +447,7 @@ __global__ void __launch_bounds__(256) oz_output_kernel(const int* __restrict__ 
       long long m, n;
       divmod<I>(t, N, m, n);
       const long long tr = m * Np + n;
-      const int sh = -12 - 7 * (dg.nd - 1);
+      const int sh = -2 * OZ_TOP - OZ_BITS * (dg.nd - 1);
       const double re = scale_pow2(diag_total<WARP>(slabs, dg, stride, tr, lane), ea[m] + eb[n] + sh);
       const double im = scale_pow2(diag_total<WARP>(slabs, dg, stride, tr + N, lane), ea[m] + eb[N + n] + sh);
       if (writer) {
@@ -470,7 +473,7 @@ __global__ void __launch_bounds__(256) oz_output1_kernel(const int* __restrict__
       for (int d = 0; d < NS; ++d) v[d] = slabs[dg.off[d] + t];
       long long m, n;
       divmod<I>(t, Np, m, n);
-      const double r = scale_pow2(diag_combine(v, NS), ea[m] + eb[n] - 12 - 7 * (NS - 1));
+      const double r = scale_pow2(diag_combine(v, NS), ea[m] + eb[n] - 2 * OZ_TOP - OZ_BITS * (NS - 1));
       double* p = o.out + m * o.ldo + n;
       *p = out_value_real(o, r, p);
     } else {
@@ -484,7 +487,7 @@ __global__ void __launch_bounds__(256) oz_output1_kernel(const int* __restrict__
         vr[d] = slabs[dg.off[d] + tr];
         vi[d] = slabs[dg.off[d] + ti];
       }
-      const int sh = -12 - 7 * (NS - 1);
+      const int sh = -2 * OZ_TOP - OZ_BITS * (NS - 1);
       const double re = scale_pow2(diag_combine(vr, NS), ea[m] + eb[n] + sh);
       const double im = scale_pow2(diag_combine(vi, NS), ea[m] + eb[N + n] + sh);
       cplx* p = o.C + m * o.scm + n * o.scn;
@@ -501,8 +504,7 @@ void launch_output1(int ns, int grid, cudaStream_t s, const int* slabs, const Oz
     case 4: oz_output1_kernel<4, MODE, I><<<grid, 256, 0, s>>>(slabs, dg, M, Np, ea, eb, o); break;
     case 5: oz_output1_kernel<5, MODE, I><<<grid, 256, 0, s>>>(slabs, dg, M, Np, ea, eb, o); break;
     case 6: oz_output1_kernel<6, MODE, I><<<grid, 256, 0, s>>>(slabs, dg, M, Np, ea, eb, o); break;
-    case 7: oz_output1_kernel<7, MODE, I><<<grid, 256, 0, s>>>(slabs, dg, M, Np, ea, eb, o); break;
-    default: oz_output1_kernel<8, MODE, I><<<grid, 256, 0, s>>>(slabs, dg, M, Np, ea, eb, o); break;
+    default: oz_output1_kernel<7, MODE, I><<<grid, 256, 0, s>>>(slabs, dg, M, Np, ea, eb, o); break;
   }
 }
 
@@ -523,7 +525,6 @@ struct OzStack {
   long long off[OZ_SLICES_MAX];
   long long ncol[OZ_SLICES_MAX];
   int zs[OZ_SLICES_MAX];
-  double scale[OZ_SLICES_MAX];
   int ns;
 };
 template <bool WARP>
@@ -537,7 +538,7 @@ __device__ __forceinline__ double stack_total(const int* __restrict__ slabs, con
       for (int i = 0; i <= d; ++i)
         S[d] += split_sum<WARP>(slabs + st.off[i] + m * st.ncol[i] + (d - i) * Np + col, st.zs[i], M * st.ncol[i], lane);
   }
-  return diag_combine(S, st.ns);   // times 2^(7 (ns - 1))
+  return diag_combine(S, st.ns);   // times 2^(9 (ns - 1))
 }
 // complex output C(m, n) = alpha (re + i im) + beta C (real columns n and N + n of the Np = 2N)
 template <bool WARP, typename I>
@@ -552,7 +553,7 @@ __global__ void __launch_bounds__(256) oz_stack_output_kernel(const int* __restr
   for (long long t = start; t < total; t += step) {
     long long m, n;
     divmod<I>(t, N, m, n);
-    const int sh = -12 - 7 * (st.ns - 1);
+    const int sh = -2 * OZ_TOP - OZ_BITS * (st.ns - 1);
     const double re = scale_pow2(stack_total<WARP>(slabs, st, M, Np, m, n, lane), ea[m] + eb[n] + sh);
     const double im = scale_pow2(stack_total<WARP>(slabs, st, M, Np, m, N + n, lane), ea[m] + eb[N + n] + sh);
     if (!WARP || lane == 0) {
@@ -590,7 +591,7 @@ __global__ void __launch_bounds__(256) oz_stack_output1_kernel(const int* __rest
         si[d] += vi[q];
       }
     }
-    const int sh = -12 - 7 * (NS - 1);
+    const int sh = -2 * OZ_TOP - OZ_BITS * (NS - 1);
     const double re = scale_pow2(diag_combine(sr, NS), ea[m] + eb[n] + sh);
     const double im = scale_pow2(diag_combine(si, NS), ea[m] + eb[N + n] + sh);
     cplx* p = o.C + m * o.scm + n * o.scn;
@@ -602,6 +603,7 @@ void launch_stack_output(int ns, bool one_split, bool warp, int grid, cudaStream
                          const OzStack& st, long long M, long long Np, const int* ea, const int* eb, const OzOut& o) {
   if (one_split) {
     switch (ns) {
+      case 4: oz_stack_output1_kernel<4, I><<<grid, 256, 0, s>>>(slabs, st, M, Np, ea, eb, o); return;
       case 5: oz_stack_output1_kernel<5, I><<<grid, 256, 0, s>>>(slabs, st, M, Np, ea, eb, o); return;
       case 6: oz_stack_output1_kernel<6, I><<<grid, 256, 0, s>>>(slabs, st, M, Np, ea, eb, o); return;
       case 7: oz_stack_output1_kernel<7, I><<<grid, 256, 0, s>>>(slabs, st, M, Np, ea, eb, o); return;
@@ -645,27 +647,36 @@ void oz_run(const SlicedRows& A, const SlicedRows& B, long long M, long long Np,
   const int ns = A.ns;
   const double slab_bytes = oz_slab_bytes();
   const long long kp = A.kp, ld = (long long)ns * kp;
-  const int max_splits = tc_exact_splits(M, Np, (long long)ns * kp);
-  const __nv_bfloat16* As = reinterpret_cast<const __nv_bfloat16*>(A.slices.p);
-  const __nv_bfloat16* Bs = reinterpret_cast<const __nv_bfloat16*>(B.slices.p);
-  if (4.0 * ns * max_splits * (double)M * (double)Np <= slab_bytes) {
+  const __half* As = reinterpret_cast<const __half*>(A.slices.p);
+  const __half* Bs = reinterpret_cast<const __half*>(B.slices.p);
+  // the diagonals' products, longest first: diagonal d is A slices 0..d against B slices d..0, concatenated along K
+  TcExactGroup eg[OZ_SLICES_MAX];
+  long long Ns[OZ_SLICES_MAX], ks[OZ_SLICES_MAX], off = 0;
+  for (int q = 0; q < ns; ++q) {
+    Ns[q] = Np;
+    ks[q] = (long long)(ns - q) * kp;
+  }
+  const int nk_split = tc_exact_nk_split(M, Ns, ks, ns);
+  OzDiags dg;
+  dg.nd = ns;
+  for (int q = 0; q < ns; ++q) {
+    const int d = ns - 1 - q;
+    eg[q].kA = 0;
+    eg[q].kB = (long long)q * kp;
+    eg[q].k_pad = ks[q];
+    eg[q].N = Np; eg[q].ldp = Np; eg[q].split_stride = M * Np;
+    eg[q].nk_split = nk_split;
+    dg.zs[d] = eg[q].zs();
+    dg.off[d] = off;
+    off = (off + (long long)dg.zs[d] * M * Np + 3) / 4 * 4;   // 16-byte aligned blocks (vector epilogue stores)
+  }
+  if (4.0 * (double)off <= slab_bytes) {
     // every diagonal's split sums side by side, then one pass that sums them into the output: the
     // output is touched once instead of once per diagonal
-    w.islabs.alloc((size_t)ns * max_splits * M * Np + 4 * ns);
+    w.islabs.alloc((size_t)off);
     if (w.err.n == 0) { w.err.alloc(1); w.err.zero(s); }
-    OzDiags dg;
-    dg.nd = ns;
-    long long off = 0;
-    for (int d = 0; d < ns; ++d) {
-      const long long kd = (long long)(d + 1) * kp;
-      const int zs = std::min(tc_exact_splits(M, Np, kd), max_splits);
-      TcOperand a(As, M, kd, ld);
-      TcOperand b(Bs + (long long)(ns - 1 - d) * kp, Np, kd, ld);
-      dg.off[d] = off;
-      dg.zs[d] = tc_gemm_exact(a, b, w.islabs.p + off, Np, M, Np, zs, M * Np, w.err.p, s, PROF_TC_SLICE);
-      dg.scale[d] = ldexp(1.0, -7 * d);
-      off = (off + (long long)zs * M * Np + 3) / 4 * 4;   // 16-byte aligned blocks (vector epilogue stores)
-    }
+    for (int q = 0; q < ns; ++q) eg[q].P = w.islabs.p + dg.off[ns - 1 - q];
+    tc_gemm_exact(TcOperand(As, M, ld, ld), TcOperand(Bs, Np, ld, ld), M, eg, ns, w.err.p, s, PROF_TC_SLICE);
     int splits = 0;
     for (int d = 0; d < ns; ++d) splits += dg.zs[d];
     const long long elements = o.complex_out ? M * (Np / 2) : M * Np;
@@ -695,6 +706,7 @@ void oz_run(const SlicedRows& A, const SlicedRows& B, long long M, long long Np,
   }
   // bytes of int32 split sums at a time (half the bound above)
   const long long slab_budget = (long long)std::max(1.0, std::min(2.0 * (1LL << 30), 0.5 * slab_bytes));
+  const int max_splits = dg.zs[ns - 1];   // of the longest diagonal
   long long nc = std::max<long long>(1, slab_budget / (4LL * M * max_splits));
   nc = std::min<long long>(Np, std::max<long long>(256, nc / 256 * 256));
   if (o.complex_out) nc = Np;
@@ -706,13 +718,12 @@ void oz_run(const SlicedRows& A, const SlicedRows& B, long long M, long long Np,
     OzOut oc = o;
     if (!o.complex_out) oc.out = o.out + n0;
     for (int d = 0; d < ns; ++d) {
-      // diagonal d: A slices 0..d against B slices d..0, concatenated along K
-      const long long kd = (long long)(d + 1) * kp;
-      const int zs = std::min(tc_exact_splits(M, nn, kd), max_splits);
-      TcOperand a(As, M, kd, ld);
-      TcOperand b(Bs + n0 * ld + (long long)(ns - 1 - d) * kp, nn, kd, ld);
-      const int zeff = tc_gemm_exact(a, b, w.islabs.p, nn, M, nn, zs, M * nn, w.err.p, s, PROF_TC_SLICE);
-      const double scale = ldexp(1.0, -7 * d);
+      TcExactGroup g = eg[ns - 1 - d];
+      g.N = nn; g.ldp = nn; g.split_stride = M * nn;
+      g.P = w.islabs.p;
+      tc_gemm_exact(TcOperand(As, M, ld, ld), TcOperand(Bs + n0 * ld, nn, ld, ld), M, &g, 1, w.err.p, s, PROF_TC_SLICE);
+      const int zeff = g.zs();
+      const double scale = ldexp(1.0, -OZ_BITS * d);
       const int first = d == 0 ? 1 : 0;
       const int mode = d < ns - 1 ? 0 : (o.complex_out ? 2 : 1);
       const long long elements = mode == 2 ? M * (nn / 2) : M * nn;
@@ -740,23 +751,41 @@ void oz_run(const SlicedRows& A, const SlicedRows& B, long long M, long long Np,
   }
 }
 
-// Split counts of the stacked form (one GEMM per A slice against B slices 0..ns-1-i) and the bytes of
-// their int32 partials.
-void stack_splits(long long M, long long Np, long long kp, int ns, int (&zs)[OZ_SLICES_MAX], double& bytes) {
-  bytes = 0.0;
+// The products of the stacked form (A slice i against B slices 0..ns-1-i, longest first) and the bytes of their
+// int32 partials.
+void stack_groups(long long M, long long Np, long long kp, int ns, TcExactGroup (&eg)[OZ_SLICES_MAX], OzStack& st,
+                  double& bytes) {
+  long long Ns[OZ_SLICES_MAX], ks[OZ_SLICES_MAX], off = 0;
   for (int i = 0; i < ns; ++i) {
-    zs[i] = tc_exact_splits(M, (ns - i) * Np, kp);
-    bytes += 4.0 * zs[i] * (double)M * (double)((ns - i) * Np) + 16.0;   // + alignment of each block
+    Ns[i] = (ns - i) * Np;
+    ks[i] = kp;
   }
+  const int nk_split = tc_exact_nk_split(M, Ns, ks, ns);
+  st.ns = ns;
+  for (int i = 0; i < ns; ++i) {
+    eg[i].kA = (long long)i * kp;
+    eg[i].kB = 0;
+    eg[i].k_pad = kp;
+    eg[i].N = Ns[i]; eg[i].ldp = Ns[i]; eg[i].split_stride = M * Ns[i];
+    eg[i].nk_split = nk_split;
+    st.off[i] = off;
+    st.ncol[i] = Ns[i];
+    st.zs[i] = eg[i].zs();
+    // the GEMM epilogue stores rows of four int32 at once where ncol is a multiple of 4: every block
+    // of partials starts on 16 bytes
+    off = (off + (long long)st.zs[i] * M * Ns[i] + 3) / 4 * 4;
+  }
+  bytes = 4.0 * (double)off;
 }
-// The stacked form pays when the A rows saved from re-reading, ns(ns-1)/2 kp bf16 per row, outweigh the
+// The stacked form pays when the A rows saved from re-reading, ns(ns-1)/2 kp f16 per row, outweigh the
 // extra partial sums it writes and reads back, about the same count times Np int32 per split, and its
 // partials fit in 4 GB.
 bool use_stacked(long long M, long long Np, long long kp, int ns) {
-  int zs[OZ_SLICES_MAX];
+  TcExactGroup eg[OZ_SLICES_MAX];
+  OzStack st;
   double bytes;
-  stack_splits(M, Np, kp, ns, zs, bytes);
-  return kp >= 4LL * Np * zs[0] && bytes <= oz_slab_bytes();
+  stack_groups(M, Np, kp, ns, eg, st, bytes);
+  return kp >= 4LL * Np * st.zs[0] && bytes <= oz_slab_bytes();
 }
 // Exact complex product in the stacked form: A sliced row-major (normal order), Bsm sliced slot-major
 // (normal order) with Np = 2N rows per slot.
@@ -764,32 +793,22 @@ void oz_run_stacked(const SlicedRows& A, const SlicedRows& Bsm, long long M, lon
                     OzWork& w, cudaStream_t s) {
   const int ns = A.ns;
   const long long kp = A.kp, ld = (long long)ns * kp;
-  int zs[OZ_SLICES_MAX];
+  TcExactGroup eg[OZ_SLICES_MAX];
+  OzStack st;
   double bytes;
-  stack_splits(M, Np, kp, ns, zs, bytes);
+  stack_groups(M, Np, kp, ns, eg, st, bytes);
   w.islabs.alloc((size_t)(bytes / 4.0));
   if (w.err.n == 0) { w.err.alloc(1); w.err.zero(s); }
-  const __nv_bfloat16* As = reinterpret_cast<const __nv_bfloat16*>(A.slices.p);
-  const __nv_bfloat16* Bs = reinterpret_cast<const __nv_bfloat16*>(Bsm.slices.p);
-  OzStack st;
-  st.ns = ns;
-  long long off = 0;
   bool one_split = true;
   int splits = 0;
   for (int i = 0; i < ns; ++i) {
-    const long long nc = (ns - i) * Np;
-    TcOperand a(As + (long long)i * kp, M, kp, ld);
-    TcOperand b(Bs, nc, kp, kp);
-    st.off[i] = off;
-    st.ncol[i] = nc;
-    st.zs[i] = tc_gemm_exact(a, b, w.islabs.p + off, nc, M, nc, zs[i], M * nc, w.err.p, s, PROF_TC_SLICE);
-    st.scale[i] = ldexp(1.0, -7 * i);
-    // the GEMM epilogue stores rows of four int32 at once where ncol is a multiple of 4: every block
-    // of partials starts on 16 bytes
-    off = (off + (long long)zs[i] * M * nc + 3) / 4 * 4;
+    eg[i].P = w.islabs.p + st.off[i];
     one_split = one_split && st.zs[i] == 1;
     splits += st.zs[i];
   }
+  tc_gemm_exact(TcOperand(reinterpret_cast<const __half*>(A.slices.p), M, ld, ld),
+                TcOperand(reinterpret_cast<const __half*>(Bsm.slices.p), ns * Np, kp, kp), M, eg, ns, w.err.p, s,
+                PROF_TC_SLICE);
   const long long elements = M * (Np / 2);
   const bool warp = !one_split && elements < 152LL * 256 && splits > 8 * ns;
   const int grid = warp ? (int)std::min<long long>(std::max<long long>((elements * 32 + 255) / 256, 1), 152LL * 32)
@@ -852,7 +871,7 @@ void zgemm_work_free(gfcc_ctx* c) {
 void zgemm_oz(const ZGemmDesc& g, int ns, cudaStream_t s) {
   const long long M = g.M, N = g.N, K = g.K;
   GFCC_CHECK(g.batch == 1, GFCC_ERR_ARG, "zgemm_oz: no batches");
-  GFCC_CHECK(ns >= 2 && ns <= OZ_SLICES_MAX, GFCC_ERR_ARG, "zgemm_oz: 2..8 slices");
+  GFCC_CHECK(ns >= 2 && ns <= OZ_SLICES_MAX, GFCC_ERR_ARG, "zgemm_oz: 2..7 slices");
   if (M <= 0 || N <= 0) return;
   ProfScope prof(PROF_OZ_ZGEMM, 8.0 * (double)M * (double)N * (double)K, s);
   ZWork local;
@@ -866,10 +885,10 @@ void zgemm_oz(const ZGemmDesc& g, int ns, cudaStream_t s) {
   const bool stacked = use_stacked(M, 2 * N, sa.kp, ns);
   sb.rows = 2 * N; sb.kp = sa.kp; sb.ns = ns; sb.reversed = !stacked;
   if (!reuse) {
-    sa.slices.alloc(sizeof(__nv_bfloat16) * M * ns * sa.kp);
+    sa.slices.alloc(sizeof(__half) * M * ns * sa.kp);
     sa.expo.alloc(M);
   }
-  sb.slices.alloc(sizeof(__nv_bfloat16) * 2 * N * ns * sb.kp);
+  sb.slices.alloc(sizeof(__half) * 2 * N * ns * sb.kp);
   sb.expo.alloc(2 * N);
   {
     // bytes: each complex operand read once and its slices written once (A only when not cached)
@@ -897,7 +916,7 @@ void zgemm_oz(const ZGemmDesc& g, int ns, cudaStream_t s) {
       with_ns(ns, [&](auto NSc) {
         zslice_kernel<decltype(NSc)::value><<<dim3((unsigned)kt, (unsigned)((M + ZT_R - 1) / ZT_R)), 256, 0, s>>>(
             g.A, g.sam, g.sak, g.conjA ? 1 : 0, M, K, 0, mxa.p, sa.kp, 0,
-            reinterpret_cast<__nv_bfloat16*>(sa.slices.p), sa.expo.p);
+            reinterpret_cast<__half*>(sa.slices.p), sa.expo.p);
       });
       GFCC_LAUNCH_CHECK();
       if (cache) {
@@ -909,7 +928,7 @@ void zgemm_oz(const ZGemmDesc& g, int ns, cudaStream_t s) {
     with_ns(ns, [&](auto NSc) {
       zslice_kernel<decltype(NSc)::value><<<dim3((unsigned)kt, (unsigned)((N + ZT_R - 1) / ZT_R)), 256, 0, s>>>(
           g.B, g.sbn, g.sbk, g.conjB ? 1 : 0, N, K, 1, mxb.p, sb.kp, stacked ? 0 : 1,
-          reinterpret_cast<__nv_bfloat16*>(sb.slices.p), sb.expo.p, stacked ? 1 : 0);
+          reinterpret_cast<__half*>(sb.slices.p), sb.expo.p, stacked ? 1 : 0);
     });
     GFCC_LAUNCH_CHECK();
   }
@@ -947,7 +966,7 @@ void oz_slice_into(const double* X, long long ldx, long long nrows, long long K,
   if (nrows == 0) return;
   // bytes: the FP64 rows read once, their slices written once
   ProfScope prof(PROF_OZ_SLICE, 8.0 * (double)nrows * (double)K + 2.0 * (double)nrows * out.ns * (double)out.kp, s);
-  __nv_bfloat16* o = reinterpret_cast<__nv_bfloat16*>(out.slices.p) + row0 * out.ns * out.kp;
+  __half* o = reinterpret_cast<__half*>(out.slices.p) + row0 * out.ns * out.kp;
   if (out.kp <= 2048) {   // short rows: a warp per row
     with_ns(out.ns, [&](auto NSc) {
       slice_rows_warp_kernel<decltype(NSc)::value><<<(unsigned)((nrows * 32 + 255) / 256), 256, 0, s>>>(
@@ -980,12 +999,12 @@ void oz_slice_into(const double* X, long long ldx, long long nrows, long long K,
 
 void oz_slice(const double* X, long long ldx, long long rows, long long K, bool reversed, SlicedRows& out,
               cudaStream_t s, int ns) {
-  GFCC_CHECK(ns >= 2 && ns <= OZ_SLICES_MAX, GFCC_ERR_ARG, "oz_slice: 2..8 slices");
+  GFCC_CHECK(ns >= 2 && ns <= OZ_SLICES_MAX, GFCC_ERR_ARG, "oz_slice: 2..7 slices");
   out.rows = rows;
   out.kp = tc_pad_k(TcKind::BF16, K);
   out.ns = ns;
   out.reversed = reversed;
-  out.slices.alloc(sizeof(__nv_bfloat16) * std::max<long long>(rows, 1) * ns * out.kp);
+  out.slices.alloc(sizeof(__half) * std::max<long long>(rows, 1) * ns * out.kp);
   out.expo.alloc(std::max<long long>(rows, 1));
   oz_slice_into(X, ldx, rows, K, out, 0, s);
 }

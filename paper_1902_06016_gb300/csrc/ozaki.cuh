@@ -1,28 +1,33 @@
-// FP64-accurate GEMM on the bf16 tensor cores by exact integer slicing (internal).
+// FP64-accurate GEMM on the f16 tensor cores by exact integer slicing (internal).
 //
 // Each row r of an FP64 operand is scaled by a power of two and written as
-//   x = 2^(e_r - 6) * sum_{i<S} a_i 2^(-7 i),   a_i integers with |a_i| <= 64,
-// so every a_i is exact in bf16 and every product a_i b_j is an integer of magnitude <= 2^12.
-// A K-chunk of at most 2048 such products sums to an integer below 2^23, which the FP32 tensor-core
-// accumulator holds exactly. The slice pairs with i + j = d ("diagonal" d) are one GEMM with the
+//   x = 2^(e_r - 8) * sum_{i<S} a_i 2^(-9 i),   a_i integers with |a_i| <= 256,
+// so every a_i is exact in f16 and every product a_i b_j is an integer of magnitude <= 2^16.
+// A K-chunk of at most 256 such products sums to an integer of at most 2^24, which the FP32 tensor-core
+// accumulator holds exactly. The slice pairs with i + j = d ("diagonal" d) are one product with the
 // slices concatenated along K (A slices in order 0..d, B slices in order d..0); its K-chunks are
 // accumulated exactly inside the GEMM kernel in int32 (each chunk's FP32 sum is an exact integer),
-// the per-split int32 sums are added in 64-bit integers and weighted by 2^(-7d) in FP64, and the total
-// is scaled by 2^(e_A + e_B - 12). With S = 6 slices the representation keeps 41 bits of each row (relative to its
-// largest element) and the dropped pairs (i + j >= S) weigh at most 2^-42 of the leading term: the
-// result is accurate to about 2^-40 of sum_k |a_mk||b_nk|, far below what FP32 or TF32 give.
+// the per-split int32 sums are added in 64-bit integers and weighted by 2^(-9d) in FP64, and the total
+// is scaled by 2^(e_A + e_B - 16). With S = 5 slices the representation keeps 44 bits of each row (relative to its
+// largest element) and the dropped pairs (i + j >= S) weigh at most 2^-45 of the leading term: the
+// result is accurate to about 2^-43 of sum_k |a_mk||b_nk|, far below what FP32 or TF32 give.
 // (Ozaki, Ogita, Oishi and Rump, "Error-free transformations of matrix multiplication by using fast
 // routines of matrix multiplication and its applications", Numer. Algorithms 59 (2012).)
+//
+// Why 9-bit digits in f16: the work is S(S+1)/2 tensor products and S bytes-pairs per element, so the fewest
+// slices win as long as the accumulator stays exact over chunks long enough to hide its draining (256
+// products here; 10-bit digits would leave 64). 7-bit digits in bf16 (chunks of 2048) need a slice more for
+// the same bits: 6 instead of 5 for the residual sigma (21 tensor products instead of 15).
 #pragma once
 #include "gfcc_internal.cuh"
 
 namespace gfcc {
 
-constexpr int OZ_SLICES = 6;       // residual sigma: 41 bits per row
-constexpr int OZ_SLICES_MAX = 8;   // 55 bits per row: as accurate as an FP64 GEMM
+constexpr int OZ_SLICES = 5;       // residual sigma: 44 bits per row
+constexpr int OZ_SLICES_MAX = 7;   // 62 bits per row: as accurate as an FP64 GEMM
 
 struct SlicedRows {
-  DBuf<uint8_t> slices;   // bf16 [rows][ns][kp] (order 0..ns-1, or reversed)
+  DBuf<uint8_t> slices;   // f16 [rows][ns][kp] (order 0..ns-1, or reversed)
   DBuf<int> expo;         // [rows]
   long long rows = 0;
   long long kp = 0;       // padded K (multiple of 64)

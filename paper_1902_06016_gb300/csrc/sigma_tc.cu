@@ -311,7 +311,7 @@ static LpState* lp_state(gfcc_ctx* c, bool transpose = false) {
   return reinterpret_cast<LpState*>(transpose ? c->lp.implT : c->lp.impl);
 }
 
-// FP64-accurate sigma from exact bf16 slices (residuals of the iterative refinement)
+// FP64-accurate sigma from exact f16 slices (residuals of the iterative refinement)
 struct EmuState {
   SlicedRows Wr, Woo, Aup, Adn;
   DBuf<double> stage, CT, C2, up;
@@ -391,7 +391,13 @@ void sigma_emulated(gfcc_ctx* c, const cplx* X, cplx* Y, int nb, const cplx* shi
   const double* A11 = op_view(c, transpose).A11;
   const int o = c->o, v = c->v, P = c->P;
   const long long ov = (long long)o * v, Pv = (long long)P * v, D = c->D;
-  const int chunk = 64;
+  // columns at a time: as many as keep the int32 split sums of the ring product within 2 GB, at least 64, in
+  // equal chunks. Small operators run all columns at once: at o = 14, v = 42 a 64-column chunk leaves most
+  // SMs without a tile (560 columns: 9 chunks of 24 launches of 15 us).
+  const long long fit = (2LL << 30) / (4LL * (OZ_SLICES + 2) * ov * 2LL * o);
+  const int most = (int)std::min<long long>(nb, std::max<long long>(64, fit));
+  const int nchunks = (nb + most - 1) / most;
+  const int chunk = (nb + nchunks - 1) / nchunks;
   for (int c0 = 0; c0 < nb; c0 += chunk) {
     const int nbc = std::min(chunk, nb - c0);
     const long long nring = 2LL * o * nbc, noo = 2LL * v * nbc, nsm = 2LL * nbc;

@@ -7,6 +7,7 @@
 #include <cuda.h>
 
 #include <algorithm>
+#include <cmath>
 #include <cstdlib>
 #include <map>
 #include <mutex>
@@ -67,17 +68,17 @@ __device__ __forceinline__ uint64_t sdesc(uint32_t addr) {
   return d;
 }
 
-// instruction descriptor: FP32 accumulate, A/B format (bf16 = 1 for kind::f16, tf32 = 2 for
+// instruction descriptor: FP32 accumulate, A/B format (f16 = 0 and bf16 = 1 for kind::f16, tf32 = 2 for
 // kind::tf32), both K-major, N = 256, M = 128
 template <TcKind K>
 __host__ __device__ constexpr uint32_t idesc() {
-  return (1u << 4) | ((K == TcKind::BF16 ? 1u : 2u) << 7) | ((K == TcKind::BF16 ? 1u : 2u) << 10) |
-         ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
+  constexpr uint32_t fmt = K == TcKind::F16 ? 0u : K == TcKind::BF16 ? 1u : 2u;
+  return (1u << 4) | (fmt << 7) | (fmt << 10) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
 }
 
 template <TcKind K>
 __device__ __forceinline__ void mma(uint32_t tmem, uint64_t a, uint64_t b, uint32_t acc) {
-  if constexpr (K == TcKind::BF16) {
+  if constexpr (K != TcKind::TF32) {
     asm volatile(
         "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(
             tmem),
@@ -94,7 +95,7 @@ __device__ __forceinline__ void mma(uint32_t tmem, uint64_t a, uint64_t b, uint3
 __device__ __forceinline__ void mma_commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
+__device__ __forceinline__ void tmem_ld32_issue(uint32_t taddr, uint32_t (&r)[32]) {
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
       "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
@@ -103,31 +104,88 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
         "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
         "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
       : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void tmem_ld16_issue(uint32_t taddr, uint32_t (&r)[16]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, "
+      "[%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr));
+}
+__device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+// after the wait: no use of the loaded registers may be scheduled before this point (volatile asm keeps its order)
+template <int N>
+__device__ __forceinline__ void tmem_ld_pin(uint32_t (&r)[N]) {
+#pragma unroll
+  for (int j = 0; j < N; ++j) asm volatile("" : "+r"(r[j]));
+}
+__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
+  tmem_ld32_issue(taddr, r);
+  tmem_ld_wait();
+  tmem_ld_pin(r);
+}
+
+// acc += v (modulo 2^32, up to EXACT_ADD_BIAS per call) for an integer |v| <= 2^24 by FP32 additions: v + 1.5 2^32
+// holds v rounded to multiples of 512 in its low mantissa bits, the exact rest (at most 256) is read the
+// same way from rest + 1.5 2^23. Five instructions on the FMA and ALU pipes; a float-to-integer conversion
+// is one, on a pipe of 16 lanes per clock. The epilogue converts every other column each way, so that the
+// pipes share the 2000 clocks that an accumulation's MMAs take.
+constexpr unsigned EXACT_ADD_BIAS = 512u * 0x4FC00000u + 0x4B400000u;
+__device__ __forceinline__ void exact_add(int& acc, float v) {
+  const float x = __fadd_rn(v, 6442450944.0f);                            // 1.5 2^32 + (v rounded to 512)
+  const float y = __fsub_rn(v, __fsub_rn(x, 6442450944.0f + 12582912.0f));   // 1.5 2^23 + (v - rounded)
+  acc = (int)((unsigned)acc + 512u * __float_as_uint(x) + __float_as_uint(y));
 }
 
 __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 
-// work unit u -> (split z, M tile, N tile). Within a split the M tiles are taken in groups of gm:
+// One launch covers up to TC_MAX_GROUPS products ("groups"): products that do not depend on each other, or the
+// diagonals of an exact product, share one persistent grid, so that a short product neither leaves SMs idle
+// nor pays a launch and a last partial wave of its own. Units are numbered group after group.
+struct TcGroup {
+  int map;                        // operand maps: A = maps[2 map], B = maps[2 map + 1]
+  int kA0, kB0;                   // first k-block of the operands' rows
+  int nk, nk_split, zs;           // k-blocks, k-blocks per split, splits
+  int tiles_m, tiles_n, gm, unit0;
+  int beta;
+  long long M, N, ldc, split_stride;
+  void* C;
+};
+struct TcGroups {
+  int n, total;
+  TcGroup g[TC_MAX_GROUPS];
+};
+struct TcMaps {
+  CUtensorMap m[2 * TC_MAX_MAPS];
+};
+
+// work unit u -> (group, split z, M tile, N tile). Within a split the M tiles are taken in groups of gm:
 // a group runs through all N tiles with its gm M tiles fastest, so that the CTAs working at the same
 // time share gm A tiles (kept in L2) and about (grid / gm) B tiles, each read from DRAM about once
 // per group instead of once per wave.
 struct Unit {
-  int z, mt, nt;
+  int g, z, mt, nt;
+  int kb0, nk;   // k-blocks [kb0, kb0 + nk) of the group's range
 };
-__device__ __forceinline__ Unit decode_unit(int u, int tiles_m, int tiles_n, int gm) {
-  const int per_z = tiles_m * tiles_n;
+__device__ __forceinline__ Unit decode_unit(int u, const TcGroups& gs) {
   Unit r;
-  r.z = u / per_z;
-  const int t = u - r.z * per_z;
-  const int g = t / (gm * tiles_n);
-  const int m0 = g * gm;
-  const int gsz = min(gm, tiles_m - m0);
-  const int w = t - m0 * tiles_n;
+  r.g = 0;
+  while (r.g + 1 < gs.n && u >= gs.g[r.g + 1].unit0) ++r.g;
+  const TcGroup& G = gs.g[r.g];
+  const int v = u - G.unit0, per_z = G.tiles_m * G.tiles_n;
+  r.z = v / per_z;
+  const int t = v - r.z * per_z;
+  const int g = t / (G.gm * G.tiles_n);
+  const int m0 = g * G.gm;
+  const int gsz = min(G.gm, G.tiles_m - m0);
+  const int w = t - m0 * G.tiles_n;
   r.nt = w / gsz;
   r.mt = m0 + (w - r.nt * gsz);
+  r.kb0 = r.z * G.nk_split;
+  r.nk = max(0, min(G.nk, r.kb0 + G.nk_split) - r.kb0);
   return r;
 }
 
@@ -138,19 +196,19 @@ __device__ __forceinline__ Unit decode_unit(int u, int tiles_m, int tiles_n, int
 // one accumulation, the MMAs of the next run into the other buffer.
 //
 // EXACT = false: one accumulation per unit; the epilogue writes FP32 C (beta = 1 adds to C).
-// EXACT = true (bf16 operands holding small integers, see ozaki.cuh): the unit's K range is cut into
-// accumulations of at most CH k-blocks (2048 products, whose FP32 sum is exact), and the epilogue
-// adds each one, converted to int32, into per-thread integer registers; the unit writes int32 sums to
-// C (as int) + z * split_stride. The caller bounds a unit to 255 accumulations, so |sum| < 2^31.
+// EXACT = true (f16 operands holding integers of magnitude <= 256, see ozaki.cuh): the unit's K range is cut
+// into accumulations of at most CH k-blocks (256 products, whose FP32 sum is exact: every partial sum is an
+// integer of magnitude <= 2^24), and the epilogue adds each one, converted to int32, into per-thread integer
+// registers; the unit writes int32 sums to C (as int) + z * split_stride. The caller bounds a unit to
+// TC_EXACT_MAX_KB k-blocks, so |sum| < 2^31. An accumulation of 256 products keeps the MMA pipe busy for
+// about 2000 clocks; draining it takes the eight epilogue warps about 1300 in its shadow.
 template <TcKind KIND, bool EXACT>
 __global__ void __launch_bounds__(EXACT ? 320 : 192, 1)
-    tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, void* Cv,
-                   long long ldc, long long M, long long N, int tiles_m, int tiles_n, int gm, int zs,
-                   int nk_total, int nk_split, long long split_stride, int beta, int* err) {
-  constexpr int KB_ELEMS = KIND == TcKind::BF16 ? 64 : 32;
-  constexpr int MMA_K_BYTES = 32;                            // K = 16 bf16 or 8 tf32 per instruction
+    tc_gemm_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcGroups gs, int* err) {
+  constexpr int KB_ELEMS = KIND == TcKind::TF32 ? 32 : 64;
+  constexpr int MMA_K_BYTES = 32;                            // K = 16 16-bit or 8 tf32 elements per instruction
   constexpr int NEPI = EXACT ? 8 : 4;                        // epilogue warps
-  constexpr int CH = 32;                                     // k-blocks per exact accumulation
+  constexpr int CH = TC_EXACT_CHUNK_KB;                      // k-blocks per exact accumulation
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* sA = smem;
@@ -162,7 +220,7 @@ __global__ void __launch_bounds__(EXACT ? 320 : 192, 1)
   __shared__ volatile int s_fail;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int total = zs * tiles_m * tiles_n;
+  const int total = gs.total;
   const uint32_t full0 = smem_u32(bars), empty0 = smem_u32(bars + STAGES);
   const uint32_t accf0 = smem_u32(bars + 2 * STAGES), acce0 = smem_u32(bars + 2 * STAGES + 2);
   const uint32_t drain = smem_u32(bars + 2 * STAGES + 4);
@@ -195,16 +253,17 @@ __global__ void __launch_bounds__(EXACT ? 320 : 192, 1)
     if (lane == 0) {   // TMA producer
       long long g = 0;  // k-blocks issued by this CTA
       for (int u = blockIdx.x; u < total && !s_fail; u += gridDim.x) {
-        const Unit w = decode_unit(u, tiles_m, tiles_n, gm);
-        const int kb0 = w.z * nk_split;
-        const int nk = max(0, min(nk_total, kb0 + nk_split) - kb0);
-        for (int kb = 0; kb < nk; ++kb, ++g) {
+        const Unit w = decode_unit(u, gs);
+        const TcGroup& G = gs.g[w.g];
+        const CUtensorMap *tmA = &maps.m[2 * G.map], *tmB = tmA + 1;
+        const int ka = (G.kA0 + w.kb0) * KB_ELEMS, kbx = (G.kB0 + w.kb0) * KB_ELEMS;
+        for (int kb = 0; kb < w.nk; ++kb, ++g) {
           const int st = (int)(g % STAGES);
           const uint32_t ph = (uint32_t)((g / STAGES) & 1);
           if (!mbar_wait(empty0 + 8 * st, ph ^ 1)) { s_fail = 1; break; }
           mbar_expect_tx(full0 + 8 * st, STAGE_BYTES);
-          tma_load_2d(smem_u32(sA + st * A_BYTES), &tmA, (kb0 + kb) * KB_ELEMS, w.mt * BM, full0 + 8 * st);
-          tma_load_2d(smem_u32(sB + st * B_BYTES), &tmB, (kb0 + kb) * KB_ELEMS, w.nt * BN, full0 + 8 * st);
+          tma_load_2d(smem_u32(sA + st * A_BYTES), tmA, ka + kb * KB_ELEMS, w.mt * BM, full0 + 8 * st);
+          tma_load_2d(smem_u32(sB + st * B_BYTES), tmB, kbx + kb * KB_ELEMS, w.nt * BN, full0 + 8 * st);
         }
       }
       // no copy may still be in flight when the CTA exits: wait (bounded) for the last stages issued
@@ -217,9 +276,7 @@ __global__ void __launch_bounds__(EXACT ? 320 : 192, 1)
       int seg = 0;      // accumulations started (TMEM buffer = seg & 1)
       bool ok = true;
       for (int u = blockIdx.x; u < total && ok && !s_fail; u += gridDim.x) {
-        const Unit w = decode_unit(u, tiles_m, tiles_n, gm);
-        const int kb0 = w.z * nk_split;
-        const int nk = max(0, min(nk_total, kb0 + nk_split) - kb0);
+        const int nk = decode_unit(u, gs).nk;
         const int nseg = nk == 0 ? 1 : (EXACT ? (nk + CH - 1) / CH : 1);
         for (int sgi = 0; sgi < nseg && ok; ++sgi, ++seg) {
           const int buf = seg & 1;
@@ -259,13 +316,15 @@ __global__ void __launch_bounds__(EXACT ? 320 : 192, 1)
     int seg = 0;
     bool ok = true;
     for (int u = blockIdx.x; u < total && ok; u += gridDim.x) {
-      const Unit w = decode_unit(u, tiles_m, tiles_n, gm);
-      const int kb0 = w.z * nk_split;
-      const int nk = max(0, min(nk_total, kb0 + nk_split) - kb0);
+      const Unit w = decode_unit(u, gs);
+      const TcGroup& G = gs.g[w.g];
+      const long long M = G.M, N = G.N, ldc = G.ldc;
+      const int nk = w.nk, beta = G.beta;
       const int nseg = nk == 0 ? 1 : (EXACT ? (nk + CH - 1) / CH : 1);
       const long long grow = (long long)w.mt * BM + q * 32 + lane;
       const long long gcol0 = (long long)w.nt * BN + half * NCOL;
       int iacc[EXACT ? NCOL : 1];
+      unsigned nadd = 0;   // accumulations added to iacc
       if constexpr (EXACT) {
 #pragma unroll
         for (int j = 0; j < NCOL; ++j) iacc[j] = 0;
@@ -277,19 +336,26 @@ __global__ void __launch_bounds__(EXACT ? 320 : 192, 1)
         tc_fence_after();
         const uint32_t trow = taddr + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * BN + half * NCOL);
         if constexpr (EXACT) {
+          // the load of one 16-column part runs while the one before is converted (wider parts would spill: a
+          // scheduler with three warps has 168 registers for each)
+          uint32_t r[2][16];
+          tmem_ld16_issue(trow, r[0]);
 #pragma unroll
-          for (int ch = 0; ch < NCOL / 32; ++ch) {
-            uint32_t r[32];
-            tmem_ld32(trow + (uint32_t)(ch * 32), r);
+          for (int ch = 0; ch < NCOL / 16; ++ch) {
+            tmem_ld_wait();
+            tmem_ld_pin(r[ch & 1]);
+            if (ch + 1 < NCOL / 16) tmem_ld16_issue(trow + (uint32_t)(ch * 16 + 16), r[(ch + 1) & 1]);
+            if (nk > 0) {
 #pragma unroll
-            for (int j = 0; j < 32; ++j) {
-              // exact integer |v| < 2^23: add 1.5 * 2^23 and read the low mantissa bits
-              const float v = nk == 0 ? 0.f : __uint_as_float(r[j]);
-              iacc[ch * 32 + j] += __float_as_int(v + 12582912.0f) - 0x4B400000;
+              for (int j = 0; j < 16; j += 2) {
+                iacc[ch * 16 + j] += __float2int_rn(__uint_as_float(r[ch & 1][j]));
+                exact_add(iacc[ch * 16 + j + 1], __uint_as_float(r[ch & 1][j + 1]));
+              }
             }
           }
+          nadd += nk > 0;
         } else {
-          float* Cz = reinterpret_cast<float*>(Cv) + (long long)w.z * split_stride;
+          float* Cz = reinterpret_cast<float*>(G.C) + (long long)w.z * G.split_stride;
           const bool vec = (ldc % 4 == 0);
 #pragma unroll 1
           for (int ch = 0; ch < NCOL / 32; ++ch) {
@@ -329,8 +395,10 @@ __global__ void __launch_bounds__(EXACT ? 320 : 192, 1)
         if (lane == 0) mbar_arrive(acce0 + 8 * buf);
       }
       if constexpr (EXACT) {
+#pragma unroll
+        for (int j = 1; j < NCOL; j += 2) iacc[j] = (int)((unsigned)iacc[j] - nadd * EXACT_ADD_BIAS);
         if (ok && grow < M) {
-          int* Pz = reinterpret_cast<int*>(Cv) + (long long)w.z * split_stride + grow * ldc;
+          int* Pz = reinterpret_cast<int*>(G.C) + (long long)w.z * G.split_stride + grow * ldc;
           if (ldc % 4 == 0 && gcol0 + NCOL <= N) {
 #pragma unroll
             for (int j = 0; j < NCOL; j += 4)
@@ -373,7 +441,7 @@ EncodeTiledFn encode_fn() {
 
 CUtensorMap make_map(TcKind kind, const TcOperand& op, int box_rows) {
   CUtensorMap m;
-  const int esize = kind == TcKind::BF16 ? 2 : 4;
+  const int esize = kind == TcKind::TF32 ? 4 : 2;
   GFCC_CHECK(op.k_pad % (KB_BYTES / esize) == 0, GFCC_ERR_ARG, "tc_gemm: K not padded to the k-block");
   GFCC_CHECK((reinterpret_cast<uintptr_t>(op.ptr) & 15) == 0, GFCC_ERR_ARG, "tc_gemm: operand not 16-byte aligned");
   GFCC_CHECK(op.ld >= op.k_pad && op.ld % (KB_BYTES / esize) == 0, GFCC_ERR_ARG, "tc_gemm: bad row stride");
@@ -381,7 +449,10 @@ CUtensorMap make_map(TcKind kind, const TcOperand& op, int box_rows) {
   cuuint64_t strides[1] = {(cuuint64_t)op.ld * esize};
   cuuint32_t box[2] = {(cuuint32_t)(KB_BYTES / esize), (cuuint32_t)box_rows};
   cuuint32_t estr[2] = {1, 1};
-  CUresult r = encode_fn()(&m, kind == TcKind::BF16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32,
+  const CUtensorMapDataType type = kind == TcKind::BF16  ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16
+                                   : kind == TcKind::F16 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16
+                                                         : CU_TENSOR_MAP_DATA_TYPE_FLOAT32;
+  CUresult r = encode_fn()(&m, type,
                            2, const_cast<void*>(op.ptr), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                            CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
@@ -406,14 +477,15 @@ int sm_count() {
 // is timed twice with CUDA events on the launching stream, and the fastest is kept for the process.
 // GFCC_AUTOTUNE=0 keeps the default (40 MB) everywhere.
 struct TuneKey {
-  int kind, exact, tiles_m, tn_log2, nk_split, zs;
+  int kind, exact, tiles_m, tn_log2, nk_split, zs, groups;
   bool operator<(const TuneKey& o) const {
-    return std::tie(kind, exact, tiles_m, tn_log2, nk_split, zs) <
-           std::tie(o.kind, o.exact, o.tiles_m, o.tn_log2, o.nk_split, o.zs);
+    return std::tie(kind, exact, tiles_m, tn_log2, nk_split, zs, groups) <
+           std::tie(o.kind, o.exact, o.tiles_m, o.tn_log2, o.nk_split, o.zs, o.groups);
   }
 };
 struct TuneResult {
-  int gm = 1, gm_default = 1;
+  int gm = 1, gm_default = 1;   // of the first group
+  long long budget_mb = 40;
   float ms_best = 0.f, ms_default = 0.f;
 };
 std::mutex g_tune_mu;
@@ -433,10 +505,19 @@ int gm_for_budget(long long budget_mb, long long a_tile_bytes, int tiles_m) {
   return (int)std::max<long long>(1, std::min<long long>(tiles_m, (budget_mb << 20) / std::max(a_tile_bytes, 1LL)));
 }
 
+// M-tile groups of a budget: the A tiles of one group (128 rows x the split's K) fit in it
+void set_gm(TcGroups& gs, long long budget_mb) {
+  for (int i = 0; i < gs.n; ++i)
+    gs.g[i].gm = gm_for_budget(budget_mb, (long long)BM * gs.g[i].nk_split * KB_BYTES, gs.g[i].tiles_m);
+}
+bool same_gm(const TcGroups& a, const TcGroups& b) {
+  for (int i = 0; i < a.n; ++i)
+    if (a.g[i].gm != b.g[i].gm) return false;
+  return true;
+}
+
 template <TcKind K, bool EXACT>
-void launch(const CUtensorMap& ma, const CUtensorMap& mb, void* C, long long ldc, long long M, long long N,
-            int tiles_m, int tiles_n, int zs, int nk_total, int nk_split, long long split_stride, int beta, int* err,
-            cudaStream_t s) {
+void launch(const TcMaps& maps, TcGroups gs, int* err, cudaStream_t s) {
   static bool attr[64] = {};   // function attributes belong to each device's context: set once per device
   int dev = 0;
   GFCC_CUDA(cudaGetDevice(&dev));
@@ -445,33 +526,41 @@ void launch(const CUtensorMap& ma, const CUtensorMap& mb, void* C, long long ldc
     GFCC_CUDA(cudaFuncSetAttribute(tc_gemm_kernel<K, EXACT>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES));
     attr[dev] = true;
   }
-  const long long units = (long long)zs * tiles_m * tiles_n;
+  bool overwrites = true;
+  long long units = 0;
+  for (int i = 0; i < gs.n; ++i) {
+    gs.g[i].unit0 = (int)units;
+    units += (long long)gs.g[i].zs * gs.g[i].tiles_m * gs.g[i].tiles_n;
+    overwrites = overwrites && gs.g[i].beta == 0;
+    GFCC_CHECK(units < (1LL << 31), GFCC_ERR_ARG, "tc_gemm: too many tiles");
+  }
+  gs.total = (int)units;
   const int grid = (int)std::min<long long>(units, sm_count());
-  auto run = [&](int gm) {
-    tc_gemm_kernel<K, EXACT><<<grid, EXACT ? 320 : 192, SMEM_BYTES, s>>>(ma, mb, C, ldc, M, N, tiles_m, tiles_n, gm,
-                                                                         zs, nk_total, nk_split, split_stride, beta,
-                                                                         err);
+  auto run = [&](const TcGroups& q) {
+    tc_gemm_kernel<K, EXACT><<<grid, EXACT ? 320 : 192, SMEM_BYTES, s>>>(maps, q, err);
     GFCC_LAUNCH_CHECK();
   };
-  // M-tile group: by default the A tiles of one group (128 rows x the split's K) fit in about 40 MB of L2
-  const long long a_tile_bytes = (long long)BM * nk_split * KB_BYTES;
-  const int gm_default = gm_for_budget(kGmDefaultMB, a_tile_bytes, tiles_m);
-  int gm = gm_default;
-  std::vector<int> cand;
+  set_gm(gs, kGmDefaultMB);
+  const TcGroups gs_default = gs;
+  std::vector<TcGroups> cand;
   for (long long mb : kGmBudgetMB) {
-    const int g = gm_for_budget(mb, a_tile_bytes, tiles_m);
-    if (std::find(cand.begin(), cand.end(), g) == cand.end()) cand.push_back(g);
+    TcGroups q = gs;
+    set_gm(q, mb);
+    bool known = false;
+    for (const TcGroups& c : cand) known = known || same_gm(c, q);
+    if (!known) cand.push_back(q);
   }
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  if (beta == 0 && cand.size() > 1 && autotune_enabled() && cudaStreamIsCapturing(s, &cap) == cudaSuccess &&
+  if (overwrites && cand.size() > 1 && autotune_enabled() && cudaStreamIsCapturing(s, &cap) == cudaSuccess &&
       cap == cudaStreamCaptureStatusNone) {
+    const TcGroup& f = gs.g[0];   // the launch's shape bucket is that of its first (longest) group
     int tl = 0;
-    while ((1 << tl) < tiles_n) ++tl;
-    const TuneKey key{K == TcKind::BF16 ? 0 : 1, EXACT ? 1 : 0, tiles_m, tl, nk_split, zs};
+    while ((1 << tl) < f.tiles_n) ++tl;
+    const TuneKey key{K == TcKind::TF32 ? 1 : 0, EXACT ? 1 : 0, f.tiles_m, tl, f.nk_split, f.zs, gs.n};
     std::lock_guard<std::mutex> lk(g_tune_mu);
     auto it = g_tune.find(key);
     if (it != g_tune.end()) {
-      gm = it->second.gm;
+      set_gm(gs, it->second.budget_mb);
     } else {
       std::vector<cudaEvent_t> ev(2 * cand.size());
       for (auto& e : ev) GFCC_CUDA(cudaEventCreate(&e));
@@ -495,77 +584,124 @@ void launch(const CUtensorMap& ma, const CUtensorMap& mb, void* C, long long ldc
       for (size_t i = 1; i < cand.size(); ++i)
         if (best[i] < best[ib]) ib = i;
       TuneResult r;
-      r.gm = cand[ib];
-      r.gm_default = gm_default;
+      r.gm = cand[ib].g[0].gm;
+      r.gm_default = gs_default.g[0].gm;
       r.ms_best = best[ib];
+      for (long long mb : kGmBudgetMB) {
+        TcGroups q = gs;
+        set_gm(q, mb);
+        if (same_gm(q, cand[ib])) { r.budget_mb = mb; break; }
+      }
       for (size_t i = 0; i < cand.size(); ++i)
-        if (cand[i] == gm_default) r.ms_default = best[i];
+        if (same_gm(cand[i], gs_default)) r.ms_default = best[i];
       g_tune[key] = r;
       g_tune_order.push_back(key);
       return;   // the output already holds the product (every candidate computes the same)
     }
   }
-  run(gm);
+  run(gs);
 }
 
 }  // namespace
 
+void tc_gemm_group(TcKind kind, const TcProduct* pr, int n, int* err_dev, cudaStream_t s, int prof_class) {
+  GFCC_CHECK(n >= 1 && n <= TC_MAX_MAPS && kind != TcKind::F16, GFCC_ERR_ARG, "tc_gemm: product count or kind");
+  TcMaps maps;
+  TcGroups gs;
+  gs.n = 0;
+  gs.total = 0;
+  double flops = 0.0;
+  for (int i = 0; i < n; ++i) {
+    const TcProduct& p = pr[i];
+    if (p.M <= 0 || p.N <= 0) continue;
+    GFCC_CHECK(p.A.k_pad == p.B.k_pad, GFCC_ERR_ARG, "tc_gemm: K mismatch");
+    GFCC_CHECK(p.A.rows >= p.M && p.B.rows >= p.N, GFCC_ERR_ARG, "tc_gemm: operand rows");
+    GFCC_CHECK(p.ksplit >= 1 && (p.ksplit == 1 || p.beta == 0), GFCC_ERR_ARG, "tc_gemm: split-K needs beta = 0");
+    GFCC_CHECK(p.A.rows < (1LL << 31) && p.B.rows < (1LL << 31), GFCC_ERR_ARG, "tc_gemm: too many rows");
+    const int kb_elems = tc_kblock(kind);
+    GFCC_CHECK(p.A.k_pad / kb_elems < (1LL << 30), GFCC_ERR_ARG, "tc_gemm: K too large");
+    TcGroup& G = gs.g[gs.n];
+    G.map = gs.n;
+    G.kA0 = G.kB0 = 0;
+    G.nk = (int)(p.A.k_pad / kb_elems);
+    G.nk_split = (G.nk + p.ksplit - 1) / p.ksplit;
+    G.zs = G.nk_split > 0 ? std::max(1, (G.nk + G.nk_split - 1) / G.nk_split) : 1;
+    const long long tm = (p.M + BM - 1) / BM, tn = (p.N + BN - 1) / BN;
+    GFCC_CHECK(tm * tn * G.zs < (1LL << 31), GFCC_ERR_ARG, "tc_gemm: too many tiles");
+    G.tiles_m = (int)tm;
+    G.tiles_n = (int)tn;
+    G.M = p.M; G.N = p.N; G.ldc = p.ldc; G.split_stride = p.split_stride;
+    G.beta = p.beta;
+    G.C = p.C;
+    maps.m[2 * gs.n] = make_map(kind, p.A, BM);
+    maps.m[2 * gs.n + 1] = make_map(kind, p.B, BN);
+    flops += 2.0 * (double)p.M * (double)p.N * (double)(p.k_alg > 0 ? p.k_alg : p.A.k_pad);
+    ++gs.n;
+  }
+  if (gs.n == 0) return;
+  ProfScope prof(prof_class, flops, s);
+  if (kind == TcKind::BF16) launch<TcKind::BF16, false>(maps, gs, err_dev, s);
+  else launch<TcKind::TF32, false>(maps, gs, err_dev, s);
+}
+
 void tc_gemm(TcKind kind, const TcOperand& A, const TcOperand& B, float* C, long long ldc, long long M, long long N,
              int beta, int ksplit, long long split_stride, int* err_dev, cudaStream_t s, int prof_class,
              long long k_alg) {
-  if (M <= 0 || N <= 0) return;
-  GFCC_CHECK(A.k_pad == B.k_pad, GFCC_ERR_ARG, "tc_gemm: K mismatch");
-  GFCC_CHECK(A.rows >= M && B.rows >= N, GFCC_ERR_ARG, "tc_gemm: operand rows");
-  GFCC_CHECK(ksplit >= 1 && (ksplit == 1 || beta == 0), GFCC_ERR_ARG, "tc_gemm: split-K needs beta = 0");
-  GFCC_CHECK(A.rows < (1LL << 31) && B.rows < (1LL << 31), GFCC_ERR_ARG, "tc_gemm: too many rows");
-  const int kb_elems = tc_kblock(kind);
-  GFCC_CHECK(A.k_pad / kb_elems < (1LL << 30), GFCC_ERR_ARG, "tc_gemm: K too large");
-  const int nk_total = (int)(A.k_pad / kb_elems);
-  const int nk_split = (nk_total + ksplit - 1) / ksplit;
-  const int zs = std::max(1, (nk_total + nk_split - 1) / nk_split);
-  const long long tiles_m = (M + BM - 1) / BM, tiles_n = (N + BN - 1) / BN;
-  GFCC_CHECK(tiles_m * tiles_n * zs < (1LL << 31), GFCC_ERR_ARG, "tc_gemm: too many tiles");
-  CUtensorMap ma = make_map(kind, A, BM);
-  CUtensorMap mb = make_map(kind, B, BN);
-  ProfScope prof(prof_class, 2.0 * (double)M * (double)N * (double)(k_alg > 0 ? k_alg : A.k_pad), s);
-  if (kind == TcKind::BF16)
-    launch<TcKind::BF16, false>(ma, mb, C, ldc, M, N, (int)tiles_m, (int)tiles_n, zs, nk_total, nk_split,
-                                split_stride, beta, err_dev, s);
-  else
-    launch<TcKind::TF32, false>(ma, mb, C, ldc, M, N, (int)tiles_m, (int)tiles_n, zs, nk_total, nk_split,
-                                split_stride, beta, err_dev, s);
+  TcProduct p;
+  p.A = A; p.B = B; p.C = C; p.ldc = ldc; p.M = M; p.N = N;
+  p.beta = beta; p.ksplit = ksplit; p.split_stride = split_stride; p.k_alg = k_alg;
+  tc_gemm_group(kind, &p, 1, err_dev, s, prof_class);
 }
 
-int tc_gemm_exact(const TcOperand& A, const TcOperand& B, int* P, long long ldp, long long M, long long N, int zs,
-                  long long split_stride, int* err_dev, cudaStream_t s, int prof_class) {
-  if (M <= 0 || N <= 0) return 0;
-  GFCC_CHECK(zs >= 1, GFCC_ERR_ARG, "tc_gemm_exact: zs < 1");
-  GFCC_CHECK(A.k_pad == B.k_pad, GFCC_ERR_ARG, "tc_gemm_exact: K mismatch");
-  GFCC_CHECK(A.rows >= M && B.rows >= N, GFCC_ERR_ARG, "tc_gemm_exact: operand rows");
-  GFCC_CHECK(A.rows < (1LL << 31) && B.rows < (1LL << 31), GFCC_ERR_ARG, "tc_gemm_exact: too many rows");
-  GFCC_CHECK(A.k_pad / 64 < (1LL << 30), GFCC_ERR_ARG, "tc_gemm_exact: K too large");
-  const int nk_total = (int)(A.k_pad / 64);
-  const int nk_split = std::max(1, (nk_total + zs - 1) / std::max(zs, 1));
-  GFCC_CHECK(nk_split <= TC_EXACT_MAX_KB, GFCC_ERR_ARG, "tc_gemm_exact: split too long for exact int32 sums");
-  const int z_eff = std::max(1, (nk_total + nk_split - 1) / nk_split);
-  const long long tiles_m = (M + BM - 1) / BM, tiles_n = (N + BN - 1) / BN;
-  GFCC_CHECK(tiles_m * tiles_n * z_eff < (1LL << 31), GFCC_ERR_ARG, "tc_gemm_exact: too many tiles");
-  CUtensorMap ma = make_map(TcKind::BF16, A, BM);
-  CUtensorMap mb = make_map(TcKind::BF16, B, BN);
-  ProfScope prof(prof_class, 2.0 * (double)M * (double)N * (double)A.k_pad, s);
-  GFCC_CHECK(z_eff <= zs, GFCC_ERR_ARG, "tc_gemm_exact: split count");
-  launch<TcKind::BF16, true>(ma, mb, P, ldp, M, N, (int)tiles_m, (int)tiles_n, z_eff, nk_total, nk_split,
-                             split_stride, 0, err_dev, s);
-  return z_eff;
+void tc_gemm_exact(const TcOperand& A, const TcOperand& B, long long M, const TcExactGroup* eg, int n, int* err_dev,
+                   cudaStream_t s, int prof_class) {
+  if (M <= 0 || n <= 0) return;
+  GFCC_CHECK(n <= TC_MAX_GROUPS, GFCC_ERR_ARG, "tc_gemm_exact: too many groups");
+  GFCC_CHECK(A.rows >= M && A.rows < (1LL << 31) && B.rows < (1LL << 31), GFCC_ERR_ARG, "tc_gemm_exact: operand rows");
+  TcMaps maps;
+  TcGroups gs;
+  gs.n = 0;
+  gs.total = 0;
+  double flops = 0.0;
+  for (int i = 0; i < n; ++i) {
+    const TcExactGroup& e = eg[i];
+    if (e.N <= 0) continue;
+    GFCC_CHECK(e.kA % 64 == 0 && e.kB % 64 == 0 && e.k_pad % 64 == 0 && e.kA + e.k_pad <= A.k_pad &&
+                   e.kB + e.k_pad <= B.k_pad && B.rows >= e.N && e.k_pad / 64 < (1LL << 30),
+               GFCC_ERR_ARG, "tc_gemm_exact: K range or rows");
+    GFCC_CHECK(e.nk_split >= 1 && e.nk_split <= TC_EXACT_MAX_KB, GFCC_ERR_ARG,
+               "tc_gemm_exact: split too long for exact int32 sums");
+    TcGroup& G = gs.g[gs.n++];
+    G.map = 0;
+    G.kA0 = (int)(e.kA / 64);
+    G.kB0 = (int)(e.kB / 64);
+    G.nk = (int)(e.k_pad / 64);
+    G.nk_split = e.nk_split;
+    G.zs = e.zs();
+    const long long tm = (M + BM - 1) / BM, tn = (e.N + BN - 1) / BN;
+    GFCC_CHECK(tm * tn * G.zs < (1LL << 31), GFCC_ERR_ARG, "tc_gemm_exact: too many tiles");
+    G.tiles_m = (int)tm;
+    G.tiles_n = (int)tn;
+    G.M = M; G.N = e.N; G.ldc = e.ldp; G.split_stride = e.split_stride;
+    G.beta = 0;
+    G.C = e.P;
+    flops += 2.0 * (double)M * (double)e.N * (double)e.k_pad;
+  }
+  if (gs.n == 0) return;
+  maps.m[0] = make_map(TcKind::F16, A, BM);
+  maps.m[1] = make_map(TcKind::F16, B, BN);
+  ProfScope prof(prof_class, flops, s);
+  launch<TcKind::F16, true>(maps, gs, err_dev, s);
 }
 
-int tc_exact_splits(long long M, long long N, long long k_pad) {
-  const long long nk = k_pad / 64;
-  const long long tiles = ((M + BM - 1) / BM) * ((N + BN - 1) / BN);
-  long long zs = std::max<long long>(1, (sm_count() + tiles - 1) / tiles);   // about one wave of units
-  zs = std::min<long long>(zs, std::max<long long>(1, nk / 32));              // at least 32 k-blocks per split
-  zs = std::max<long long>(zs, (nk + TC_EXACT_MAX_KB - 1) / TC_EXACT_MAX_KB);
-  return (int)zs;
+int tc_exact_nk_split(long long M, const long long* N, const long long* k_pad, int n) {
+  double work = 0.0;   // tile x k-block
+  for (int i = 0; i < n; ++i)
+    work += (double)(((M + BM - 1) / BM) * ((N[i] + BN - 1) / BN)) * (double)(k_pad[i] / 64);
+  // equal units, about two waves of them (so that the last, partial wave is short), not below 16 k-blocks
+  // (1024 products: the pipeline's fill is amortised) nor above the int32 bound
+  const double nk = work / (2.0 * sm_count());
+  return (int)std::max(16.0, std::min((double)TC_EXACT_MAX_KB, std::ceil(nk)));
 }
 
 }  // namespace gfcc

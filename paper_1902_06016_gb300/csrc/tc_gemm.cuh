@@ -10,9 +10,11 @@
 #pragma once
 #include "gfcc_internal.cuh"
 
+#include <algorithm>
+
 namespace gfcc {
 
-enum class TcKind { BF16 = 0, TF32 = 1 };
+enum class TcKind { BF16 = 0, TF32 = 1, F16 = 2 };   // F16: exact-slice digits only
 
 struct TcOperand {
   const void* ptr = nullptr;   // device, row-major
@@ -32,20 +34,37 @@ void tc_gemm(TcKind kind, const TcOperand& A, const TcOperand& B, float* C, long
              long long N, int beta, int ksplit, long long split_stride, int* err_dev, cudaStream_t s,
              int prof_class = 0, long long k_alg = 0);
 
-// Exact integer GEMM for the Ozaki slices: A and B bf16 holding integers of magnitude <= 64, so
-// that 2048 products sum exactly in FP32. P[z][m][n] (int32, row stride ldp, split z at
-// P + z * split_stride) = sum over the k-blocks of split z of A[m][k] B[n][k]; the K range is cut
-// into at most zs equal splits of at most TC_EXACT_MAX_KB k-blocks (255 exact FP32 accumulations of
-// 32 k-blocks, |sum| < 255 * 2^23 < 2^31). Rows >= M and columns >= N are not written. Returns the
-// number of splits written (<= zs; P must hold zs splits).
-constexpr int TC_EXACT_MAX_KB = 255 * 32;
-int tc_gemm_exact(const TcOperand& A, const TcOperand& B, int* P, long long ldp, long long M, long long N, int zs,
-                   long long split_stride, int* err_dev, cudaStream_t s, int prof_class = 0);
-// number of K splits for tc_gemm_exact: about one wave of work units, within the int32 bound
-int tc_exact_splits(long long M, long long N, long long k_pad);
+// Independent products of one launch (see TcGroup in tc_gemm.cu): the arguments of tc_gemm for each.
+constexpr int TC_MAX_GROUPS = 8, TC_MAX_MAPS = 3;
+struct TcProduct {
+  TcOperand A, B;
+  float* C = nullptr;
+  long long ldc = 0, M = 0, N = 0;
+  int beta = 0, ksplit = 1;
+  long long split_stride = 0, k_alg = 0;
+};
+void tc_gemm_group(TcKind kind, const TcProduct* pr, int n, int* err_dev, cudaStream_t s, int prof_class = 0);
 
-// k-block (elements) of a kind: 64 bf16 or 32 tf32 = 128 bytes
-inline int tc_kblock(TcKind k) { return k == TcKind::BF16 ? 64 : 32; }
+// Exact integer GEMMs for the slices of ozaki.cuh: A and B f16 holding integers of magnitude <= 256, so
+// that 256 products (TC_EXACT_CHUNK_KB k-blocks) sum exactly in FP32. For every group,
+// P[z][m][n] (int32, row stride ldp, split z at P + z * split_stride) = sum over the k-blocks of split z of
+// A[m][kA + k] B[n][kB + k], k < k_pad, in splits of nk_split <= TC_EXACT_MAX_KB k-blocks (|sum| < 2^31); rows
+// >= M and columns >= N are not written. All groups run in one launch; longest first balances them best.
+constexpr int TC_EXACT_CHUNK_KB = 4, TC_EXACT_MAX_KB = 508;
+struct TcExactGroup {
+  long long kA = 0, kB = 0, k_pad = 0;   // elements, multiples of 64
+  long long N = 0, ldp = 0, split_stride = 0;
+  int* P = nullptr;
+  int nk_split = 1;
+  int zs() const { return (int)std::max<long long>(1, (k_pad / 64 + nk_split - 1) / nk_split); }
+};
+void tc_gemm_exact(const TcOperand& A, const TcOperand& B, long long M, const TcExactGroup* eg, int n, int* err_dev,
+                   cudaStream_t s, int prof_class = 0);
+// k-blocks per split for n groups of M x N[i] x k_pad[i] in one launch
+int tc_exact_nk_split(long long M, const long long* N, const long long* k_pad, int n);
+
+// k-block (elements) of a kind: 64 16-bit or 32 tf32 = 128 bytes
+inline int tc_kblock(TcKind k) { return k == TcKind::TF32 ? 32 : 64; }
 inline int tc_pad_k(TcKind k, long long K) { int b = tc_kblock(k); return (int)((K + b - 1) / b * b); }
 
 }  // namespace gfcc

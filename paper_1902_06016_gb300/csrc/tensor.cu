@@ -140,7 +140,7 @@ void contract(double alpha, const TV& A, const TV& B, double beta, const TV& C, 
   double min_macs = 5e8;
   if (const char* env = getenv("GFCC_OZ_MIN_MACS")) min_macs = atof(env);
   if ((double)M * (double)N * (double)K >= min_macs && M >= 16 && N >= 16) {
-    // FP64-accurate GEMM from exact bf16 slices on the tensor cores (8 slices: FP64-level accuracy)
+    // FP64-accurate GEMM from exact f16 slices on the tensor cores (7 slices: FP64-level accuracy)
     const double* Aop2 = A.p;
     std::vector<int> pa2 = perm_of(la, Ml + Kl);
     if (!identity(pa2)) {
