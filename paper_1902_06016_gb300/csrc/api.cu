@@ -129,7 +129,7 @@ std::vector<int> q_positions(const std::vector<int>& porb, const std::vector<int
 // into caller-provided device buffers when non-null, and G [ncols][nq] when Gdev is non-null.
 void solve_pairs(gfcc_ctx* c, const std::vector<double>& wcol, const std::vector<int>& pcol, double eta,
                  const std::vector<int>& qorb, cplx* Gdev, cplx* Xall, cplx* Rall, gfcc_stats* st_out,
-                 const cplx* X0all = nullptr) {
+                 const cplx* X0all = nullptr, bool polish = false) {
   cudaStream_t s = c->stream;
   const long long D = c->D;
   const int nq = (int)qorb.size();
@@ -159,7 +159,7 @@ void solve_pairs(gfcc_ctx* c, const std::vector<double>& wcol, const std::vector
                                   cudaMemcpyDeviceToDevice, s));
     }
     gfcc::SolveStatus st;
-    gfcc::gmres_batched(c, B.p, X.p, R.p, sh.p, nb, st, false, X0all ? X0.p : nullptr);
+    gfcc::gmres_batched(c, B.p, X.p, R.p, sh.p, nb, st, false, X0all ? X0.p : nullptr, polish);
     for (int k = 0; k < nb; ++k) {
       maxres = std::max(maxres, st.relres[k]);
       if (!st.converged[k]) ++notconv;
@@ -190,7 +190,7 @@ void solve_pairs(gfcc_ctx* c, const std::vector<double>& wcol, const std::vector
 // Solve all (w, p) columns, column w * np + p (see solve_pairs).
 void solve_columns(gfcc_ctx* c, const std::vector<double>& ws, double eta, const std::vector<int>& porb,
                    const std::vector<int>& qorb, cplx* Gdev, cplx* Xall, cplx* Rall, gfcc_stats* st_out,
-                   const cplx* X0all = nullptr) {
+                   const cplx* X0all = nullptr, bool polish = false) {
   const size_t np = porb.size();
   std::vector<double> wcol(ws.size() * np);
   std::vector<int> pcol(ws.size() * np);
@@ -198,7 +198,7 @@ void solve_columns(gfcc_ctx* c, const std::vector<double>& ws, double eta, const
     wcol[k] = ws[k / np];
     pcol[k] = porb[k % np];
   }
-  solve_pairs(c, wcol, pcol, eta, qorb, Gdev, Xall, Rall, st_out, X0all);
+  solve_pairs(c, wcol, pcol, eta, qorb, Gdev, Xall, Rall, st_out, X0all, polish);
 }
 
 // Adjoint solves (w - i eta + M)^T y = c_q for every (w, q): columns (w, q) of Yall [D][nw*nq].
@@ -738,7 +738,8 @@ int gfcc_solve_full(gfcc_t c, const double* omegas, int nw, double eta, const in
   if (needG) Gd.alloc(ncols * nq);
   if (X) Xd.alloc(D * ncols);
   gfcc_stats st{};
-  solve_columns(c, ws, eta, porb, qv, needG ? Gd.p : nullptr, X ? Xd.p : nullptr, nullptr, &st);
+  const bool lowp = c->opts.precision == GFCC_PREC_TF32 || c->opts.precision == GFCC_PREC_BF16;
+  solve_columns(c, ws, eta, porb, qv, needG ? Gd.p : nullptr, X ? Xd.p : nullptr, nullptr, &st, nullptr, X && lowp);
   if (A) {
     std::vector<int> qi = q_positions(porb, qv);
     dq.alloc(np);
@@ -1410,6 +1411,8 @@ void gfcc_free(gfcc_t c) {
 gfcc_ctx::~gfcc_ctx() {
   gfcc::free_low_precision(this);
   gfcc::zgemm_work_free(this);
+  if (pin) cudaFreeHost(pin);
+  if (pin_event) cudaEventDestroy(pin_event);
 }
 
 extern "C" {

@@ -182,6 +182,7 @@ struct Operator {
   DBuf<double> T2p;    // [(pair(ij),a)][e]  Pv x v : t_ij^ae     (three-body, second half)
   DBuf<double> diag;   // [D] Fock-diagonal part: -F_ii (1h), F_aa - F_ii - F_jj (2h1p)
   DBuf<double> mdiag;  // [D] full diagonal of M (Jacobi preconditioner)
+  DBuf<float4> rowf;   // mdiag as pairs of FP32 numbers, and diag in FP32 (built with the first FP32-basis solve)
   // transposed-action copies are built lazily (adjoint systems)
   bool have_T = false;
   DBuf<double> WrT, WooT, A12T, A21T, VtT, T2pT;
@@ -289,6 +290,8 @@ struct gfcc_ctx {
   gfcc::DBuf<double> t1, t2; // kept for derivative work
   // kept for the T2 gradient: <mn||ef>, <mn||ie>, <ma||ef>, lambda2, F_me (row-major as the inputs)
   gfcc::DBuf<double> k_oovv, k_ooov, k_ovvv, k_l2, k_Fme;
+  int* pin = nullptr;              // page-locked word and event of the solver's column count (first solve)
+  cudaEvent_t pin_event = nullptr;
   void* zwork = nullptr;     // grow-only workspace of the exact-slice complex GEMMs (ozaki.cu)
   ~gfcc_ctx();
 };
@@ -389,9 +392,18 @@ void release_sigma_batch_buffers(gfcc_ctx* c);
 void release_scratch(gfcc_ctx* c);
 void sigma_lowprec(gfcc_ctx* c, const cplx* X, cplx* Y, int nb, const cplx* shift, cudaStream_t s,
                    bool transpose = false);
-// the same with FP32 complex vectors (the FP32 Krylov basis of the mixed-precision solver)
-void sigma_lowprec_f32(gfcc_ctx* c, const cuFloatComplex* X, cuFloatComplex* Y, int nb, const cplx* shift,
-                       cudaStream_t s, bool transpose = false);
+// the preconditioned action on the FP32 Krylov basis of the mixed-precision solver, in two parts, with z = P v:
+// prepare: v = w inv (the new basis vector, written to V) and the GEMM operands of z; apply: Y = (shift + M) z of
+// the vector prepared last
+void sigma_lp_prepare(gfcc_ctx* c, const cplx* W, const float* inv, cuFloatComplex* V, int nb, const float4* shift,
+                      cudaStream_t s, bool transpose);
+void sigma_lp_prepare(gfcc_ctx* c, const cuFloatComplex* W, const float* inv, cuFloatComplex* V, int nb,
+                      const float4* shift, cudaStream_t s, bool transpose);
+void sigma_lp_apply(gfcc_ctx* c, const cuFloatComplex* V, cuFloatComplex* Y, int nb, const float4* shift, cudaStream_t s,
+                    bool transpose);
+// the FP32 forms of shifts (one per column) and of the operator's diagonals (op.rowf, once) used there
+void split_shifts(const cplx* shift, int nb, float4* out, cudaStream_t s);
+void ensure_row_split(gfcc_ctx* c);
 int low_precision_error(gfcc_ctx* c);   // 1 if a tensor-core pipeline wait timed out
 int emulated_error(gfcc_ctx* c);
 void build_emulated(gfcc_ctx* c);
@@ -406,9 +418,11 @@ struct SolveStatus {
   std::vector<int> converged;   // per column
 };
 // Solve (shift_c + M) x_c = b_c for nb columns (batch-minor layout, ld = nb), starting from X0 (same
-// layout) when it is non-null, else from zero.
+// layout) when it is non-null, else from zero. polish: the solutions themselves are the result (not a functional of
+// them), and a low-precision inner action is in use: columns that only just meet the tolerance get one more cycle, so
+// that resonant columns, whose error is the residual times up to 1/eta, are not left at the tolerance itself.
 void gmres_batched(gfcc_ctx* c, const cplx* B, cplx* X, cplx* R, const cplx* shifts, int nb,
-                   SolveStatus& st, bool transpose, const cplx* X0 = nullptr);
+                   SolveStatus& st, bool transpose, const cplx* X0 = nullptr, bool polish = false);
 
 // ---- kernels shared between units ------------------------------------------------------------
 void gather_rows_real_to_cplx(const double* src, int ld_src, const int* rows, int nrows, int D,

@@ -9,6 +9,7 @@
 // cycles. The paper used a complex DIIS solver (convergence study after Table 1); any convergent
 // solver reaches the same solution of Eq. xplin.
 #include "gfcc_internal.cuh"
+#include "precond.cuh"
 
 #include <type_traits>
 
@@ -119,8 +120,7 @@ template <int NV> struct SwGroups {
 };
 template <int NV, int CW> constexpr size_t sweep_smem_bytes() {
   return sizeof(float2) * (size_t)SW_STAGES * (SwGroups<NV>::NPG + 1) * SW_THREADS   // load ring
-         + sizeof(float2) * 2 * SW_THREADS                                           // shares
-         + sizeof(cplx) * SW_THREADS;                                                // reductions
+         + sizeof(float2) * 2 * SW_THREADS;                                          // shares
 }
 
 __device__ __forceinline__ void cp_async8(void* smem, const void* gmem, bool pred) {
@@ -142,7 +142,6 @@ __global__ void __launch_bounds__(SW_THREADS, 2) sweep_kernel(const float2* __re
   extern __shared__ __align__(16) unsigned char sw_raw[];
   float2* ring = reinterpret_cast<float2*>(sw_raw);                       // [SW_STAGES][SLOTS][SW_THREADS]
   float2* share = ring + (size_t)SW_STAGES * SLOTS * SW_THREADS;          // [2][TY][CW]
-  cplx* red = reinterpret_cast<cplx*>(share + 2 * SW_THREADS);            // [TY][CW]
   const int tid = threadIdx.x, x = tid % CW, y = tid / CW;
   const int g = y / RPG, yr = y % RPG;
   const int c = blockIdx.x * CW + x;
@@ -223,25 +222,40 @@ __global__ void __launch_bounds__(SW_THREADS, 2) sweep_kernel(const float2* __re
     }
   }
   cp_async_wait<0>();
+  // sums over the thread rows, in FP64. All of them go to shared memory at once (the load ring is free now) and the
+  // whole block adds them, one output per thread: 2 RPG FP64 additions deep. (One basis vector at a time left the
+  // additions to one warp, NPG times: 5 us of a 20 us sweep at 264 columns of 4,785 rows.)
+  __syncthreads();
   if constexpr (MODE == 2) {
-    red[tid] = make_cuDoubleComplex(g == 0 ? (double)nrm : 0.0, 0.0);
+    double* part = reinterpret_cast<double*>(sw_raw);   // [TY][CW]
+    if (g == 0) part[tid] = (double)nrm;                 // g == 0: the first RPG thread rows
     __syncthreads();
-    if (y == 0 && c < nb) {
-      double t2 = 0.0;
-      for (int k = 0; k < RPG; ++k) t2 += red[k * CW + x].x;
-      partial[(long long)blockIdx.y * nb + c] = make_cuDoubleComplex(t2, 0.0);
-    }
+    // four threads per column
+    double t2 = 0.0;
+    if (tid < 4 * CW)
+      for (int k = tid / CW; k < RPG; k += 4) t2 += part[k * CW + tid % CW];
+    __syncthreads();
+    if (tid < 4 * CW) part[tid] = t2;
+    __syncthreads();
+    if (tid < CW && c < nb)
+      partial[(long long)blockIdx.y * nb + c] =
+          make_cuDoubleComplex((part[tid] + part[CW + tid]) + (part[2 * CW + tid] + part[3 * CW + tid]), 0.0);
   } else {
+    float2* part = reinterpret_cast<float2*>(sw_raw);   // [NPG][TY][CW]
 #pragma unroll
-    for (int li = 0; li < NPG; ++li) {
-      __syncthreads();
-      red[tid] = make_cuDoubleComplex((double)ax[li], (double)ay[li]);
-      __syncthreads();
-      const int i = i0 + li;
-      if (yr == 0 && c < nb && i < nv) {
-        cplx sum = red[tid];
-        for (int k = 1; k < RPG; ++k) { sum.x += red[tid + k * CW].x; sum.y += red[tid + k * CW].y; }
-        partial[((long long)blockIdx.y * nv + i) * nb + c] = sum;
+    for (int li = 0; li < NPG; ++li) part[li * SW_THREADS + tid] = make_float2(ax[li], ay[li]);
+    __syncthreads();
+    for (int q = tid; q < NV * CW; q += SW_THREADS) {   // output: vector i = q / CW of group i / NPG, column q % CW
+      const int i = q / CW, xx = q % CW, gg = i / NPG, li = i % NPG;
+      const int cc = blockIdx.x * CW + xx;
+      if (i < nv && cc < nb) {
+        cplx sum = make_cuDoubleComplex(0.0, 0.0);
+        for (int k = 0; k < RPG; ++k) {
+          const float2 v = part[li * SW_THREADS + (gg * RPG + k) * CW + xx];
+          sum.x += (double)v.x;
+          sum.y += (double)v.y;
+        }
+        partial[((long long)blockIdx.y * nv + i) * nb + cc] = sum;
       }
     }
   }
@@ -298,31 +312,46 @@ long long cgs_rows(long long D, int nb) {
   return std::max<long long>(64, (D + nchunk - 1) / nchunk);
 }
 
-// h[c*hld + hoff + i] (+)= sum_chunk partial[chunk][i][c]
-__global__ void reduce_partial_kernel(const cplx* __restrict__ partial, int nchunk, int nv, int nb,
-                                      cplx* __restrict__ h, int hld, int hoff, int accumulate) {
-  int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= nv * nb) return;
-  int i = t / nb, c = t % nb;
+// h[c*hld + hoff + i] = sum_chunk partial[chunk][i][c], also set in or added to the Hessenberg column Hc (entry
+// (hoff + i, c) at (hoff + i) nb + c). A block takes one i and 32 columns, its eight warps sharing the chunks
+// (one thread per sum walked them one after the other: 10 us for a few hundred chunks, now 2).
+__global__ void __launch_bounds__(256) reduce_partial_kernel(const cplx* __restrict__ partial, int nchunk, int nv, int nb,
+                                                             cplx* __restrict__ h, int hld, int hoff,
+                                                             cplx* __restrict__ Hc, int accumulate) {
+  __shared__ cplx red[8][32];
+  const int x = threadIdx.x, y = threadIdx.y, c = blockIdx.x * 32 + x, i = blockIdx.y;
   cplx s = make_cuDoubleComplex(0.0, 0.0);
-  for (int k = 0; k < nchunk; ++k) {
-    cplx p = partial[((long long)k * nv + i) * nb + c];
-    s.x += p.x; s.y += p.y;
+  if (c < nb) {
+#pragma unroll 4
+    for (int k = y; k < nchunk; k += 8) {
+      const cplx p = partial[((long long)k * nv + i) * nb + c];
+      s.x += p.x; s.y += p.y;
+    }
   }
-  cplx* dst = h + (long long)c * hld + hoff + i;
-  if (accumulate) { dst->x += s.x; dst->y += s.y; } else { *dst = s; }
+  red[y][x] = s;
+  __syncthreads();
+  if (y == 0 && c < nb) {
+    for (int k = 1; k < 8; ++k) { s.x += red[k][x].x; s.y += red[k][x].y; }
+    h[(long long)c * hld + hoff + i] = s;
+    if (Hc) {
+      cplx* d = Hc + (long long)(hoff + i) * nb + c;
+      if (accumulate) { s.x += d->x; s.y += d->y; }
+      *d = s;
+    }
+  }
 }
 
-// W[nu][c] += sign * sum_{i<nv} V_i[nu][c] h[c*hld + hoff + i]
+// W[nu][c] -= sum_{i<nv} V_i[nu][c] h[c*hld + i] (blocks as in el_grid)
 template <typename VT>
-__global__ void update_kernel(const VT* __restrict__ V, long long vstride, int nv, VT* __restrict__ W,
-                              long long D, int nb, const cplx* __restrict__ h, int hld, int hoff, double sign) {
+__global__ void __launch_bounds__(256) update_kernel(const VT* __restrict__ V, long long vstride, int nv,
+                                                     VT* __restrict__ W, long long D, int nb,
+                                                     const cplx* __restrict__ h, int hld) {
   using R = typename RealOf<VT>::type;
-  long long total = D * nb;
-  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total;
-       t += (long long)gridDim.x * blockDim.x) {
-    int c = (int)(t % nb);
-    const cplx* hc = h + (long long)c * hld + hoff;
+  const int c = blockIdx.x * blockDim.x + threadIdx.x;
+  if (c >= nb) return;
+  const cplx* hc = h + (long long)c * hld;
+  for (long long nu = blockIdx.y * (long long)blockDim.y + threadIdx.y; nu < D; nu += (long long)gridDim.y * blockDim.y) {
+    const long long t = nu * nb + c;
     // four independent partial sums keep several loads in flight
     R sx[4] = {R(0), R(0), R(0), R(0)}, sy[4] = {R(0), R(0), R(0), R(0)};
     int i = 0;
@@ -341,162 +370,272 @@ __global__ void update_kernel(const VT* __restrict__ V, long long vstride, int n
       sx[0] += vv.x * hx - vv.y * hy;
       sy[0] += vv.x * hy + vv.y * hx;
     }
-    W[t].x += (R)sign * ((sx[0] + sx[1]) + (sx[2] + sx[3]));
-    W[t].y += (R)sign * ((sy[0] + sy[1]) + (sy[2] + sy[3]));
+    W[t].x -= (sx[0] + sx[1]) + (sx[2] + sx[3]);
+    W[t].y -= (sy[0] + sy[1]) + (sy[2] + sy[3]);
   }
 }
 
-// H[c*hld + i] (+)= hb[c*hbld + i], i < n
-__global__ void add_h_kernel(const cplx* __restrict__ hb, int hbld, cplx* __restrict__ H, int hld, int n, int nb,
-                             int accumulate) {
-  int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= n * nb) return;
-  int c = t / n, i = t % n;
-  cplx v = hb[(long long)c * hbld + i];
-  cplx* d = H + (long long)c * hld + i;
-  if (accumulate) { d->x += v.x; d->y += v.y; } else { *d = v; }
-}
-
-// column 2-norms: partial over chunks then reduce (reuses multidot with V = W)
-__global__ void finalize_norm_kernel(const cplx* __restrict__ dots, int nb, double* __restrict__ out) {
-  int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c < nb) out[c] = sqrt(fmax(dots[c].x, 0.0));
-}
-
-// Z[nu][c] = V[nu][c] / (shift_c + mdiag[nu])
-template <typename VT>
-__global__ void precond_kernel(const VT* __restrict__ V, VT* __restrict__ Z, const double* __restrict__ md,
-                               const cplx* __restrict__ shift, long long D, int nb) {
-  using R = typename RealOf<VT>::type;
-  long long total = D * nb;
-  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total;
-       t += (long long)gridDim.x * blockDim.x) {
-    int c = (int)(t % nb);
-    long long nu = t / nb;
-    const R dr = (R)(shift[c].x + md[nu]), di = (R)shift[c].y;
-    const R inv = R(1) / (dr * dr + di * di);
-    const VT v = V[t];
-    Z[t].x = (v.x * dr + v.y * di) * inv;
-    Z[t].y = (v.y * dr - v.x * di) * inv;
+// out[c] = sqrt(sum_chunk partial[chunk][c].x) (32 columns a block, eight warps sharing the chunks)
+__global__ void __launch_bounds__(256) reduce_norm_kernel(const cplx* __restrict__ partial, int nchunk, int nb,
+                                                          double* __restrict__ out) {
+  __shared__ double red[8][32];
+  const int x = threadIdx.x, y = threadIdx.y, c = blockIdx.x * 32 + x;
+  double s = 0.0;
+  if (c < nb)
+    for (int k = y; k < nchunk; k += 8) s += partial[(long long)k * nb + c].x;
+  red[y][x] = s;
+  __syncthreads();
+  if (y == 0 && c < nb) {
+    for (int k = 1; k < 8; ++k) s += red[k][x];
+    out[c] = sqrt(fmax(s, 0.0));
   }
 }
 
-// V[nu][c] = W[nu][c] * scale[c]  (scale = 1/norm, 0 for broken-down columns), with conversion
-template <typename VI, typename VO>
-__global__ void scale_cols_kernel(const VI* __restrict__ W, VO* __restrict__ V, const double* __restrict__ nrm,
-                                  long long D, int nb) {
-  long long total = D * nb;
-  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total;
-       t += (long long)gridDim.x * blockDim.x) {
-    using R = typename RealOf<VO>::type;
-    int c = (int)(t % nb);
-    double n = nrm[c];
-    const R s = (n > 0.0 && isfinite(n)) ? (R)(1.0 / n) : R(0);
-    V[t].x = (R)W[t].x * s;
-    V[t].y = (R)W[t].y * s;
-  }
+// Elementwise kernels over a batch-minor block: blocks of CW columns (CW = sweep_cw(nb)) and EL_T / CW thread
+// rows, so that a thread keeps its column and what belongs to it (no division per element).
+constexpr int EL_T = 256;
+struct ElGrid {
+  dim3 grid, block;
+};
+ElGrid el_grid(long long D, int nb) {
+  const int cw = nb >= 32 ? 32 : nb > 8 ? 16 : nb > 4 ? 8 : 4;
+  const long long gx = (nb + cw - 1) / cw, rows = EL_T / cw;
+  const long long gy = std::max<long long>(1, std::min<long long>((D + rows - 1) / rows, std::max<long long>(1, 152LL * 24 / gx)));
+  return {dim3((unsigned)gx, (unsigned)std::min<long long>(gy, 65535)), dim3((unsigned)cw, (unsigned)(EL_T / cw))};
 }
 
-// R = B - Y
-__global__ void residual_kernel(const cplx* __restrict__ B, const cplx* __restrict__ Y, cplx* __restrict__ R,
-                                long long n) {
-  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n;
-       t += (long long)gridDim.x * blockDim.x)
-    R[t] = make_cuDoubleComplex(B[t].x - Y[t].x, B[t].y - Y[t].y);
-}
-
-// Per-column Givens step j on H[c] (column-major (k+1) x k), cs/sn/g; writes the residual
-// estimate |g_{j+1}| / bnorm and counts columns still above tol*0.5 that are active in this cycle.
-__global__ void givens_kernel(cplx* __restrict__ H, cplx* __restrict__ cs, cplx* __restrict__ sn,
-                              cplx* __restrict__ g, const double* __restrict__ hnext,
-                              const double* __restrict__ bnorm, int* __restrict__ kc, int* __restrict__ live,
-                              int nb, int k, int j, const double* __restrict__ thr, int* __restrict__ n_live) {
-  int c = blockIdx.x * blockDim.x + threadIdx.x;
+// V[nu][c] = W[nu][c] / nrm[c] (0 for broken-down columns), Z[nu][c] = V[nu][c] / (shift_c + mdiag[nu]) (FP64 basis)
+__global__ void __launch_bounds__(EL_T) scale_precond_kernel(const cplx* __restrict__ W, const double* __restrict__ nrm,
+                                                             cplx* __restrict__ V, cplx* __restrict__ Z,
+                                                             const double* __restrict__ md,
+                                                             const cplx* __restrict__ shift, long long D, int nb) {
+  const int c = blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= nb) return;
-  if (!live[c]) return;
-  cplx* Hc = H + (long long)c * (k + 1) * k;
-  cplx* col = Hc + (long long)j * (k + 1);
-  col[j + 1] = make_cuDoubleComplex(hnext[c], 0.0);
-  cplx* csc = cs + (long long)c * k;
-  cplx* snc = sn + (long long)c * k;
-  cplx* gc = g + (long long)c * (k + 1);
-  for (int i = 0; i < j; ++i) {
-    cplx a = col[i], b = col[i + 1];
-    cplx t = cuCadd(cuCmul(csc[i], a), cuCmul(snc[i], b));
-    cplx u = cuCadd(cuCmul(make_cuDoubleComplex(-snc[i].x, snc[i].y), a), cuCmul(cuConj(csc[i]), b));
-    col[i] = t;
-    col[i + 1] = u;
+  const double n = nrm[c], s = (n > 0.0 && isfinite(n)) ? 1.0 / n : 0.0;
+  const cplx sh = shift[c];
+  for (long long nu = blockIdx.y * (long long)blockDim.y + threadIdx.y; nu < D; nu += (long long)gridDim.y * blockDim.y) {
+    const long long t = nu * nb + c;
+    cplx v = W[t];
+    v.x *= s;
+    v.y *= s;
+    V[t] = v;
+    const double dr = sh.x + md[nu], di = sh.y, inv = 1.0 / (dr * dr + di * di);
+    Z[t] = make_cuDoubleComplex((v.x * dr + v.y * di) * inv, (v.y * dr - v.x * di) * inv);
   }
-  cplx a = col[j], b = col[j + 1];
-  double den = sqrt(a.x * a.x + a.y * a.y + b.x * b.x + b.y * b.y);
-  cplx cj, sj;
-  if (den > 0.0) {
-    cj = make_cuDoubleComplex(a.x / den, -a.y / den);
-    sj = make_cuDoubleComplex(b.x / den, -b.y / den);
+}
+// inv[c] = 1 / nrm[c] in FP32 (0 for broken-down columns)
+__global__ void inv_norm_kernel(const double* __restrict__ nrm, int nb, float* __restrict__ inv) {
+  const int c = blockIdx.x * blockDim.x + threadIdx.x;
+  if (c >= nb) return;
+  const double n = nrm[c];
+  inv[c] = (n > 0.0 && isfinite(n)) ? (float)(1.0 / n) : 0.f;
+}
+
+// R = B - Y and partial[chunk][c].x = sum_{nu in chunk} |R[nu][c]|^2 (chunk = blockIdx.y)
+__global__ void __launch_bounds__(EL_T) residual_kernel(const cplx* __restrict__ B, const cplx* __restrict__ Y,
+                                                        cplx* __restrict__ R, long long D, int nb,
+                                                        cplx* __restrict__ partial) {
+  __shared__ double red[EL_T];
+  const int c = blockIdx.x * blockDim.x + threadIdx.x, tid = threadIdx.y * blockDim.x + threadIdx.x;
+  double s = 0.0;
+  if (c < nb)
+    for (long long nu = blockIdx.y * (long long)blockDim.y + threadIdx.y; nu < D; nu += (long long)gridDim.y * blockDim.y) {
+      const long long t = nu * nb + c;
+      const cplx b = B[t], y = Y[t];
+      const cplx r = make_cuDoubleComplex(b.x - y.x, b.y - y.y);
+      R[t] = r;
+      s = fma(r.x, r.x, fma(r.y, r.y, s));
+    }
+  red[tid] = s;
+  __syncthreads();
+  if (threadIdx.y == 0 && c < nb) {
+    for (int k = 1; k < blockDim.y; ++k) s += red[k * blockDim.x + threadIdx.x];
+    partial[(long long)blockIdx.y * nb + c] = make_cuDoubleComplex(s, 0.0);
+  }
+}
+
+// End of Arnoldi step j: the norm of the new vector from its chunk sums (or, with nchunk = 0, already in nrm), its
+// reciprocal for the next step, the j earlier Givens rotations on the new Hessenberg column, the new rotation, the
+// residual estimate |g_{j+1}| / bnorm and the count of columns still above their threshold.
+// H[(jj (k+1) + i) nb + c], cs, sn, g [i nb + c]. Rotations have a real cosine: t = c a + s b, u = c b - conj(s) a.
+// Four lanes per column, one for each real component of (t, u): an FP64 instruction holds its scheduler for 75
+// clocks whatever the lanes in use, and a thread per column issued 16 of them per rotation (21 us at 15
+// rotations; four lanes issue 3).
+constexpr int GV_T = 512;   // sixteen warps share the chunk sums of 32 columns; the first four rotate
+__global__ void __launch_bounds__(GV_T) arnoldi_finish_kernel(const cplx* __restrict__ partial, int nchunk,
+                                                              double* __restrict__ nrm, float* __restrict__ invf,
+                                                              cplx* __restrict__ H, double* __restrict__ cs,
+                                                              cplx* __restrict__ sn, cplx* __restrict__ g,
+                                                              const double* __restrict__ bnorm, int* __restrict__ kc,
+                                                              int* __restrict__ live, int nb, int k, int j,
+                                                              const double* __restrict__ thr, int* __restrict__ n_live) {
+  __shared__ double red[GV_T / 32][32];
+  const int c0 = blockIdx.x * 32;
+  if (nchunk > 0) {
+    const int x = threadIdx.x & 31, y = threadIdx.x >> 5;
+    double s = 0.0;
+    if (c0 + x < nb) {
+#pragma unroll 8
+      for (int q = y; q < nchunk; q += GV_T / 32) s += partial[(long long)q * nb + c0 + x].x;
+    }
+    red[y][x] = s;
+    __syncthreads();
+    if (y == 0) {
+      for (int q = 1; q < GV_T / 32; ++q) s += red[q][x];
+      s = sqrt(fmax(s, 0.0));
+      red[0][x] = s;
+      if (c0 + x < nb) nrm[c0 + x] = s;
+    }
+    __syncthreads();
+  }
+  if (threadIdx.x >= 128) return;
+  const int x = threadIdx.x >> 2, q = threadIdx.x & 3, c = c0 + x;
+  const bool in = c < nb, on = in && live[c];
+  const double hn = in ? (nchunk > 0 ? red[0][x] : nrm[c]) : 0.0;
+  if (in && q == 0) invf[c] = (hn > 0.0 && isfinite(hn)) ? (float)(1.0 / hn) : 0.f;
+  if (!__any_sync(0xffffffffu, on)) return;
+  cplx* col = H + (long long)j * (k + 1) * nb + c;
+  // lanes: 0 t.re, 1 t.im, 2 u.re, 3 u.im of  ca a + cb b  with complex coefficients split into components
+  const bool isu = q >= 2, im = q & 1;
+  cplx a = on ? col[0] : make_cuDoubleComplex(0.0, 0.0);
+  constexpr int PF = 4;   // rotations loaded ahead of the serial chain
+  for (int i0 = 0; i0 < j; i0 += PF) {
+    cplx b[PF], s[PF];
+    double cc[PF];
+#pragma unroll
+    for (int r = 0; r < PF; ++r) {
+      const bool ok = on && i0 + r < j;
+      b[r] = ok ? col[(long long)(i0 + r + 1) * nb] : make_cuDoubleComplex(0.0, 0.0);
+      s[r] = ok ? sn[(long long)(i0 + r) * nb + c] : make_cuDoubleComplex(0.0, 0.0);
+      cc[r] = ok ? cs[(long long)(i0 + r) * nb + c] : 1.0;
+    }
+#pragma unroll
+    for (int r = 0; r < PF; ++r) {
+      if (i0 + r >= j) break;   // uniform
+      // t = cc a + s b: (cc a.re + s.re b.re - s.im b.im, cc a.im + s.re b.im + s.im b.re)
+      // u = cc b - conj(s) a: (cc b.re - s.re a.re - s.im a.im, cc b.im - s.re a.im + s.im a.re)
+      const cplx p = isu ? b[r] : a, o = isu ? a : b[r];   // multiplied by cc, by s
+      const double sr = isu ? -s[r].x : s[r].x;
+      const double si = im ? s[r].y : -s[r].y;
+      const double v = fma(cc[r], im ? p.y : p.x, fma(sr, im ? o.y : o.x, si * (im ? o.x : o.y)));
+      if (on && !isu) reinterpret_cast<double*>(col + (long long)(i0 + r) * nb)[im] = v;
+      a.x = __shfl_sync(0xffffffffu, v, 2, 4);
+      a.y = __shfl_sync(0xffffffffu, v, 3, 4);
+    }
+  }
+  if (!on || q != 0) return;
+  // new rotation of (a, hn), hn real: with den^2 = |a|^2 + hn^2, cosine |a| / den, sine (a / |a|) hn / den, new
+  // diagonal (a / |a|) den, all from one reciprocal root of |a|^2 den^2
+  const double a2 = a.x * a.x + a.y * a.y, d2 = a2 + hn * hn, ad = a2 * d2;
+  double cj, den;
+  cplx sj, tj;
+  if (ad > 1e-280 && ad < 1e280) {
+    const double r = rsqrt(ad);   // 1 / (|a| den)
+    cj = a2 * r;
+    sj = make_cuDoubleComplex(a.x * hn * r, a.y * hn * r);
+    tj = make_cuDoubleComplex(a.x * (d2 * r), a.y * (d2 * r));
+    den = 1.0;   // not zero
   } else {
-    cj = make_cuDoubleComplex(1.0, 0.0);
-    sj = make_cuDoubleComplex(0.0, 0.0);
+    const double aa = hypot(a.x, a.y);
+    den = hypot(aa, hn);
+    const cplx ph = aa > 0.0 ? make_cuDoubleComplex(a.x / aa, a.y / aa) : make_cuDoubleComplex(1.0, 0.0);
+    cj = den > 0.0 ? aa / den : 1.0;
+    const double hd = den > 0.0 ? hn / den : 0.0;
+    sj = make_cuDoubleComplex(ph.x * hd, ph.y * hd);
+    tj = make_cuDoubleComplex(ph.x * den, ph.y * den);
   }
-  csc[j] = cj;
-  snc[j] = sj;
-  col[j] = make_cuDoubleComplex(den, 0.0);
-  col[j + 1] = make_cuDoubleComplex(0.0, 0.0);
-  cplx gj = gc[j];
-  gc[j + 1] = cuCmul(make_cuDoubleComplex(-sj.x, sj.y), gj);
-  gc[j] = cuCmul(cj, gj);
+  cs[(long long)j * nb + c] = cj;
+  sn[(long long)j * nb + c] = sj;
+  col[(long long)j * nb] = tj;
+  col[(long long)(j + 1) * nb] = make_cuDoubleComplex(0.0, 0.0);
+  const cplx gj = g[(long long)j * nb + c];
+  const cplx gn = make_cuDoubleComplex(-(sj.x * gj.x + sj.y * gj.y), -(sj.x * gj.y - sj.y * gj.x));
+  g[(long long)(j + 1) * nb + c] = gn;
+  g[(long long)j * nb + c] = make_cuDoubleComplex(cj * gj.x, cj * gj.y);
   kc[c] = j + 1;
-  double est = cuCabs(gc[j + 1]) / bnorm[c];
-  if (!(est > thr[c]) || den == 0.0 || !isfinite(est)) {
+  // estimate |g_{j+1}| / bnorm against the threshold, squared
+  const double est2 = gn.x * gn.x + gn.y * gn.y, lim = thr[c] * bnorm[c];
+  if (!(est2 > lim * lim) || den == 0.0 || !isfinite(est2)) {
     live[c] = 0;   // converged (or broken down) within this cycle: stop extending its basis use
   } else {
     atomicAdd(n_live, 1);
   }
 }
 
-// y = H[:kc,:kc]^{-1} g (upper triangular), stored in g
-__global__ void backsolve_kernel(const cplx* __restrict__ H, cplx* __restrict__ g, const int* __restrict__ kc,
-                                 int nb, int k) {
-  int c = blockIdx.x * blockDim.x + threadIdx.x;
+// y = H[:kc,:kc]^{-1} g (upper triangular), stored in g; also in the basis precision in y. One warp per column,
+// column-oriented: row i of every remaining entry is updated by the lanes at once (at most 256 rows).
+template <typename VT>
+__global__ void __launch_bounds__(128) backsolve_kernel(const cplx* __restrict__ H, cplx* __restrict__ g,
+                                                        const int* __restrict__ kc, int nb, int k, VT* __restrict__ y) {
+  const int c = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (c >= nb) return;
-  const cplx* Hc = H + (long long)c * (k + 1) * k;
-  cplx* gc = g + (long long)c * (k + 1);
-  int n = kc[c];
-  for (int i = n - 1; i >= 0; --i) {
-    cplx s = gc[i];
-    for (int jj = i + 1; jj < n; ++jj) s = cuCsub(s, cuCmul(Hc[(long long)jj * (k + 1) + i], gc[jj]));
-    cplx d = Hc[(long long)i * (k + 1) + i];
-    gc[i] = (d.x == 0.0 && d.y == 0.0) ? make_cuDoubleComplex(0.0, 0.0) : cuCdiv(s, d);
+  const int n = kc[c];
+  for (int jj = n - 1; jj >= 0; --jj) {
+    const cplx d = H[((long long)jj * (k + 1) + jj) * nb + c];
+    const cplx v = g[(long long)jj * nb + c];
+    const cplx yj = (d.x == 0.0 && d.y == 0.0) ? make_cuDoubleComplex(0.0, 0.0) : cuCdiv(v, d);
+    __syncwarp();   // every lane has read g_jj before it is replaced
+    if (lane == 0) g[(long long)jj * nb + c] = yj;
+    for (int i = lane; i < jj; i += 32)
+      g[(long long)i * nb + c] = cuCsub(g[(long long)i * nb + c], cuCmul(H[((long long)jj * (k + 1) + i) * nb + c], yj));
+    __syncwarp();
   }
-  for (int i = n; i <= k; ++i) gc[i] = make_cuDoubleComplex(0.0, 0.0);
+  for (int i = lane; i < k; i += 32) {
+    const cplx v = i < n ? g[(long long)i * nb + c] : make_cuDoubleComplex(0.0, 0.0);
+    VT r;
+    r.x = v.x;
+    r.y = v.y;
+    y[(long long)i * nb + c] = r;
+  }
 }
 
-// X[nu][c] += P_c[nu] * sum_i V_i[nu][c] y_i[c]   (FP64 accumulation)
+// X[nu][c] += P_c[nu] * sum_{i < nv} V_i[nu][c] y_i[c]: the correction is formed in the basis precision, only its
+// addition to x is FP64 (y [i nb + c], zero beyond a column's own steps)
 template <typename VT>
-__global__ void correct_kernel(const VT* __restrict__ V, long long vstride, int nv, const cplx* __restrict__ y,
-                               int yld, cplx* __restrict__ X, const double* __restrict__ md,
-                               const cplx* __restrict__ shift, long long D, int nb) {
-  long long total = D * nb;
-  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total;
-       t += (long long)gridDim.x * blockDim.x) {
-    // the correction is formed in the basis precision; only its addition to x is FP64
-    using R = typename RealOf<VT>::type;
-    int c = (int)(t % nb);
-    long long nu = t / nb;
-    R sr = R(0), si = R(0);
-    const cplx* yc = y + (long long)c * yld;
-    for (int i = 0; i < nv; ++i) {
-      const cplx yi = yc[i];
-      if (yi.x != 0.0 || yi.y != 0.0) {
-        const VT vv = V[i * vstride + t];
-        const R yr = (R)yi.x, yim = (R)yi.y;
-        sr += vv.x * yr - vv.y * yim;
-        si += vv.x * yim + vv.y * yr;
+__global__ void __launch_bounds__(EL_T) correct_kernel(const VT* __restrict__ V, long long vstride, int nv,
+                                                       const VT* __restrict__ y, cplx* __restrict__ X,
+                                                       const double* __restrict__ md, const RowF* __restrict__ mdf,
+                                                       const cplx* __restrict__ shift,
+                                                       const ShiftF* __restrict__ shiftf, long long D, int nb) {
+  using R = typename RealOf<VT>::type;
+  const int c = blockIdx.x * blockDim.x + threadIdx.x;
+  if (c >= nb) return;
+  cplx sh = make_cuDoubleComplex(0.0, 0.0);
+  ShiftF shf = make_float4(0.f, 0.f, 0.f, 0.f);
+  if constexpr (sizeof(R) == 4) shf = shiftf[c];
+  else sh = shift[c];
+  for (long long nu = blockIdx.y * (long long)blockDim.y + threadIdx.y; nu < D; nu += (long long)gridDim.y * blockDim.y) {
+    const long long t = nu * nb + c;
+    R sr[4] = {R(0), R(0), R(0), R(0)}, si[4] = {R(0), R(0), R(0), R(0)};
+    int i = 0;
+    for (; i + 4 <= nv; i += 4) {
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const VT vv = V[(long long)(i + u) * vstride + t], yy = y[(long long)(i + u) * nb + c];
+        sr[u] += vv.x * yy.x - vv.y * yy.y;
+        si[u] += vv.x * yy.y + vv.y * yy.x;
       }
     }
-    const R dr = (R)(shift[c].x + md[nu]), di = (R)shift[c].y;
-    const R inv = R(1) / (dr * dr + di * di);
-    X[t].x += (double)((sr * dr + si * di) * inv);
-    X[t].y += (double)((si * dr - sr * di) * inv);
+    for (; i < nv; ++i) {
+      const VT vv = V[(long long)i * vstride + t], yy = y[(long long)i * nb + c];
+      sr[0] += vv.x * yy.x - vv.y * yy.y;
+      si[0] += vv.x * yy.y + vv.y * yy.x;
+    }
+    VT s;
+    s.x = (sr[0] + sr[1]) + (sr[2] + sr[3]);
+    s.y = (si[0] + si[1]) + (si[2] + si[3]);
+    if constexpr (sizeof(R) == 4) {
+      const float2 z = precond_f32(make_float2(s.x, s.y), mdf[nu], shf);
+      s.x = z.x;
+      s.y = z.y;
+    } else {
+      const double dr = sh.x + md[nu], di = sh.y, inv = 1.0 / (dr * dr + di * di);
+      s = make_cuDoubleComplex((s.x * dr + s.y * di) * inv, (s.y * dr - s.x * di) * inv);
+    }
+    cplx x = X[t];
+    x.x += (double)s.x;
+    x.y += (double)s.y;
+    X[t] = x;
   }
 }
 
@@ -534,25 +673,21 @@ __global__ void nonfinite_cplx_kernel(const cplx* x, long long n, int* flag) {
 // ------------------------------------------------------------------------------------------------
 // column norms of a batch-minor block: out[c] = ||W_c||  (device array)
 template <typename VT>
-static void col_norms(const VT* W, long long D, int nb, double* out, DBuf<cplx>& partial, DBuf<cplx>& tmp,
-                      cudaStream_t s) {
+static void col_norms(const VT* W, long long D, int nb, double* out, DBuf<cplx>& partial, cudaStream_t s) {
   const long long rows = std::max<long long>(256, (D + 511) / 512);
   const int nchunk = (int)((D + rows - 1) / rows);
   partial.alloc((long long)nchunk * nb);
-  tmp.alloc(nb);
   dim3 grid((nb + MD_TX - 1) / MD_TX, nchunk);
   multidot_kernel<VT, 4><<<grid, dim3(MD_TX, MD_TY), 0, s>>>(W, 0, 1, W, D, nb, rows, partial.p);
   GFCC_LAUNCH_CHECK();
-  reduce_partial_kernel<<<(nb + 255) / 256, 256, 0, s>>>(partial.p, nchunk, 1, nb, tmp.p, 1, 0, 0);
-  GFCC_LAUNCH_CHECK();
-  finalize_norm_kernel<<<(nb + 255) / 256, 256, 0, s>>>(tmp.p, nb, out);
+  reduce_norm_kernel<<<(nb + 31) / 32, dim3(32, 8), 0, s>>>(partial.p, nchunk, nb, out);
   GFCC_LAUNCH_CHECK();
 }
 
-// h[c][hoff + i] (+)= V_i^H W_c for i < nv, with chunked partial sums
+// h[c][i] = V_i^H W_c for i < nv, with chunked partial sums; set in or added to the Hessenberg column Hc
 template <typename VT>
 static void multidot(const VT* V, long long vstride, int nv, const VT* W, long long D, int nb, cplx* h, int hld,
-                     int hoff, bool accumulate, DBuf<cplx>& partial, cudaStream_t s) {
+                     cplx* Hc, bool accumulate, DBuf<cplx>& partial, cudaStream_t s) {
   for (int i0 = 0; i0 < nv; i0 += MD_MAXV) {
     int n = std::min(MD_MAXV, nv - i0);
     const long long rows = cgs_rows(D, nb);
@@ -564,20 +699,10 @@ static void multidot(const VT* V, long long vstride, int nv, const VT* W, long l
                                                                                   nb, rows, partial.p);
     });
     GFCC_LAUNCH_CHECK();
-    reduce_partial_kernel<<<(n * nb + 255) / 256, 256, 0, s>>>(partial.p, nchunk, n, nb, h, hld, hoff + i0,
-                                                               accumulate ? 1 : 0);
+    reduce_partial_kernel<<<dim3((nb + 31) / 32, n), dim3(32, 8), 0, s>>>(partial.p, nchunk, n, nb, h, hld, i0, Hc,
+                                                                          accumulate ? 1 : 0);
     GFCC_LAUNCH_CHECK();
   }
-}
-
-// inner action W = (shift + M) Z in the basis precision
-static void inner_sigma(gfcc_ctx* c, const cplx* Z, cplx* W, int nb, const cplx* sh, int prec, bool tr, cudaStream_t s) {
-  sigma_batch(c, Z, W, nb, nb, sh, prec, tr, s);
-}
-static void inner_sigma(gfcc_ctx* c, const cuFloatComplex* Z, cuFloatComplex* W, int nb, const cplx* sh, int prec,
-                        bool tr, cudaStream_t s) {
-  (void)prec;
-  sigma_lowprec_f32(c, Z, W, nb, sh, s, tr);
 }
 
 // Restarted GMRES with iterative refinement; VT is the precision of the Krylov basis (FP64 for the
@@ -586,7 +711,7 @@ static void inner_sigma(gfcc_ctx* c, const cuFloatComplex* Z, cuFloatComplex* W,
 // precision only bounds the progress of one cycle, not the final accuracy).
 template <typename VT>
 static void gmres_impl(gfcc_ctx* c, const cplx* Bin, cplx* Xout, cplx* Rout, const cplx* shifts_dev, int nb0,
-                       SolveStatus& st, bool transpose, const cplx* X0) {
+                       SolveStatus& st, bool transpose, const cplx* X0, bool polish) {
   cudaStream_t s = c->stream;
   const long long D = c->D;
   const int k = std::max(1, std::min(c->opts.restart, 256));
@@ -605,19 +730,27 @@ static void gmres_impl(gfcc_ctx* c, const cplx* Bin, cplx* Xout, cplx* Rout, con
   std::vector<cplx> hshift(nb0);
   GFCC_CUDA(cudaMemcpyAsync(hshift.data(), shifts_dev, sizeof(cplx) * nb0, cudaMemcpyDeviceToHost, s));
 
-  DBuf<cplx> Bw, Xw, Rw, Yw, Ztmp, H, cs, sn, g, partial, tmpc, shw, hb;
-  DBuf<VT> V, Zw, Ww;
-  DBuf<double> nrm, bnorm, thr;
+  constexpr bool F32 = sizeof(VT) == sizeof(cuFloatComplex);
+  DBuf<cplx> Bw, Xw, Rw, Yw, Ztmp, H, sn, g, partial, shw, hb;
+  DBuf<VT> V, Zw, Ww, yv;
+  DBuf<double> nrm, bnorm, thr, cs;
+  DBuf<float> invf;
   DBuf<int> kc, live, nlive, cols, flag;
+  DBuf<float4> shf;
+  if (F32) { ensure_row_split(c); shf.alloc(nb0); }
+  if (!c->pin) GFCC_CUDA(cudaMallocHost(reinterpret_cast<void**>(&c->pin), sizeof(int)));
+  if (!c->pin_event) GFCC_CUDA(cudaEventCreateWithFlags(&c->pin_event, cudaEventDisableTiming));
   Bw.alloc(D * nb0); Xw.alloc(D * nb0); Rw.alloc(D * nb0); Yw.alloc(D * nb0); Ztmp.alloc(D * nb0);
-  Zw.alloc(D * nb0); Ww.alloc(D * nb0);
+  if (!F32) Zw.alloc(D * nb0);   // the FP32 path forms z = P v where it is used
+  Ww.alloc(D * nb0);
   V.alloc((long long)(k + 1) * D * nb0);
   V.zero(s);
   H.alloc((long long)nb0 * (k + 1) * k);
   cs.alloc((long long)nb0 * k); sn.alloc((long long)nb0 * k); g.alloc((long long)nb0 * (k + 1));
   hb.alloc((long long)nb0 * (k + 1));
-  tmpc.alloc(nb0);
-  nrm.alloc(nb0); bnorm.alloc(nb0); thr.alloc(nb0); kc.alloc(nb0); live.alloc(nb0); nlive.alloc(1); cols.alloc(nb0);
+  yv.alloc((long long)nb0 * k);
+  invf.alloc(nb0);
+  nrm.alloc(nb0); bnorm.alloc(nb0); thr.alloc(nb0); kc.alloc(nb0); live.alloc(nb0); nlive.alloc(k); cols.alloc(nb0);
   shw.alloc(nb0);
   flag.alloc(1);
   {  // chunk partial sums of the Gram-Schmidt sweeps and norms, at their largest (no regrowth per step)
@@ -626,6 +759,7 @@ static void gmres_impl(gfcc_ctx* c, const cplx* Bin, cplx* Xout, cplx* Rout, con
     for (int b = 1; b <= nb0; ++b) {
       md = std::max(md, (D + cgs_rows(D, b) - 1) / cgs_rows(D, b) * b);
       md = std::max(md, (D + sweep_rows(D, b) - 1) / sweep_rows(D, b) * b);
+      md = std::max(md, (long long)el_grid(D, b).grid.y * b);
     }
     partial.alloc(std::max(md * (k + 1), (D + rows_cn - 1) / rows_cn * nb0));
   }
@@ -644,7 +778,7 @@ static void gmres_impl(gfcc_ctx* c, const cplx* Bin, cplx* Xout, cplx* Rout, con
     GFCC_CUDA(cudaStreamSynchronize(s));
     GFCC_CHECK(hf == 0, GFCC_ERR_NONFINITE, "solve: non-finite right-hand side or frequency");
   }
-  col_norms<cplx>(Bw.p, D, nb0, bnorm.p, partial, tmpc, s);
+  col_norms<cplx>(Bw.p, D, nb0, bnorm.p, partial, s);
   std::vector<double> hbn(nb0);
   GFCC_CUDA(cudaMemcpyAsync(hbn.data(), bnorm.p, sizeof(double) * nb0, cudaMemcpyDeviceToHost, s));
   GFCC_CUDA(cudaStreamSynchronize(s));
@@ -653,14 +787,20 @@ static void gmres_impl(gfcc_ctx* c, const cplx* Bin, cplx* Xout, cplx* Rout, con
   for (int i = 0; i < nb0; ++i) map[i] = i;
   int nb = nb0;
   std::vector<double> hres(nb0);
+  std::vector<char> polished(nb0, 0);
+  const double target = polish ? 0.1 : 0.5;   // of the tolerance, for the estimate that ends a cycle
   const int max_cycles = std::max(1, c->opts.max_restarts);
 
   for (int cycle = 0; cycle <= max_cycles && nb > 0; ++cycle) {
     // FP64-accurate residual R = B - (shift X + M X)
     sigma_batch(c, Xw.p, Yw.p, nb, nb, shw.p, resid_prec, transpose, s);
-    residual_kernel<<<grid_for(D * nb), 256, 0, s>>>(Bw.p, Yw.p, Rw.p, D * nb);
-    GFCC_LAUNCH_CHECK();
-    col_norms<cplx>(Rw.p, D, nb, nrm.p, partial, tmpc, s);
+    {
+      const ElGrid eg = el_grid(D, nb);
+      residual_kernel<<<eg.grid, eg.block, 0, s>>>(Bw.p, Yw.p, Rw.p, D, nb, partial.p);
+      GFCC_LAUNCH_CHECK();
+      reduce_norm_kernel<<<(nb + 31) / 32, dim3(32, 8), 0, s>>>(partial.p, (int)eg.grid.y, nb, nrm.p);
+      GFCC_LAUNCH_CHECK();
+    }
     GFCC_CUDA(cudaMemcpyAsync(hres.data(), nrm.p, sizeof(double) * nb, cudaMemcpyDeviceToHost, s));
     GFCC_CUDA(cudaStreamSynchronize(s));
     c->stats.restarts++;
@@ -672,17 +812,30 @@ static void gmres_impl(gfcc_ctx* c, const cplx* Bin, cplx* Xout, cplx* Rout, con
     if ((inner_prec != GFCC_PREC_FP64 || resid_prec != GFCC_PREC_FP64) && low_precision_error(c))
       throw Error{GFCC_ERR_CUDA, "solve: a tensor-core pipeline wait timed out"};
 
-    // classify columns
+    // classify columns: done = written out, keep = iterated on. With polish, a column that first meets the tolerance
+    // by less than a factor of four is written out and given one more cycle, whose result replaces it if its
+    // residual is smaller.
     std::vector<int> done, keep;
     for (int w = 0; w < nb; ++w) {
       int orig = map[w];
       double bn = hbn[orig];
       double rel = bn > 0.0 ? hres[w] / bn : 0.0;
       GFCC_CHECK(std::isfinite(rel), GFCC_ERR_NONFINITE, "solve: non-finite residual (singular shift?)");
+      if (polished[orig]) {
+        if (rel < st.relres[orig]) {
+          st.relres[orig] = rel;
+          done.push_back(w);
+        }
+        continue;
+      }
       st.relres[orig] = rel;
       if (rel <= tol || cycle == max_cycles) {
         done.push_back(w);
         st.converged[orig] = rel <= tol ? 1 : 0;
+        if (polish && rel > 0.25 * tol && cycle < max_cycles) {
+          polished[orig] = 1;
+          keep.push_back(w);
+        }
       } else {
         keep.push_back(w);
       }
@@ -735,40 +888,54 @@ static void gmres_impl(gfcc_ctx* c, const cplx* Bin, cplx* Xout, cplx* Rout, con
       std::vector<double> wb(nb), th(nb);
       for (int q = 0; q < nb; ++q) {
         wb[q] = hbn[map[q]];
-        th[q] = std::max(0.5 * tol, inner_rtol * hres[q] / wb[q]);
+        th[q] = std::max(target * tol, inner_rtol * hres[q] / wb[q]);
       }
       GFCC_CUDA(cudaMemcpyAsync(bnorm.p, wb.data(), sizeof(double) * nb, cudaMemcpyHostToDevice, s));
       GFCC_CUDA(cudaMemcpyAsync(thr.p, th.data(), sizeof(double) * nb, cudaMemcpyHostToDevice, s));
     }
     // GMRES(k) on the correction: V0 = R / ||R||, g = (||R||, 0, ...)
-    scale_cols_kernel<cplx, VT><<<grid_for(D * nb), 256, 0, s>>>(Rw.p, V.p, nrm.p, D, nb);
-    GFCC_LAUNCH_CHECK();
     {
       std::vector<cplx> g0((size_t)nb * (k + 1), make_cuDoubleComplex(0.0, 0.0));
-      for (int q = 0; q < nb; ++q) g0[(size_t)q * (k + 1)] = make_cuDoubleComplex(hres[q], 0.0);
+      for (int q = 0; q < nb; ++q) g0[q] = make_cuDoubleComplex(hres[q], 0.0);
       GFCC_CUDA(cudaMemcpyAsync(g.p, g0.data(), sizeof(cplx) * g0.size(), cudaMemcpyHostToDevice, s));
       std::vector<int> ones(nb, 1);
       GFCC_CUDA(cudaMemcpyAsync(live.p, ones.data(), sizeof(int) * nb, cudaMemcpyHostToDevice, s));
       GFCC_CUDA(cudaMemsetAsync(kc.p, 0, sizeof(int) * nb, s));
+      GFCC_CUDA(cudaMemsetAsync(nlive.p, 0, sizeof(int) * k, s));
       GFCC_CUDA(cudaMemsetAsync(H.p, 0, sizeof(cplx) * (size_t)nb * (k + 1) * k, s));
     }
     const long long vstride = D * nb;
-    for (int j = 0; j < k; ++j) {
-      VT* Vj = V.p + j * vstride;
-      VT* Vn = V.p + (j + 1) * vstride;
-      {
-        ProfScope pk(PROF_KRYLOV, 0.0, s);
-        precond_kernel<VT><<<grid_for(D * nb), 256, 0, s>>>(Vj, Zw.p, c->op.mdiag.p, shw.p, D, nb);
+    const ElGrid eg = el_grid(D, nb);
+    // v_j = w / ||w|| and what the inner action needs of z = P v_j: its operands (FP32 basis) or z itself
+    auto start_step = [&](const auto* w, int j) {
+      ProfScope pk(PROF_KRYLOV, 0.0, s);
+      if constexpr (F32) {
+        sigma_lp_prepare(c, w, invf.p, V.p + j * vstride, nb, shf.p, s, transpose);
+      } else {
+        scale_precond_kernel<<<eg.grid, eg.block, 0, s>>>(w, nrm.p, V.p + j * vstride, Zw.p, c->op.mdiag.p, shw.p, D, nb);
         GFCC_LAUNCH_CHECK();
       }
-      inner_sigma(c, Zw.p, Ww.p, nb, shw.p, inner_prec, transpose, s);
+    };
+    if (F32) {
+      split_shifts(shw.p, nb, shf.p, s);
+      inv_norm_kernel<<<(nb + 127) / 128, 128, 0, s>>>(nrm.p, nb, invf.p);
+      GFCC_LAUNCH_CHECK();
+    }
+    start_step(Rw.p, 0);
+    int steps = 0;
+    for (int j = 0; j < k; ++j) {
+      VT* Vj = V.p + j * vstride;
+      if constexpr (F32) sigma_lp_apply(c, Vj, Ww.p, nb, shf.p, s, transpose);
+      else sigma_batch(c, Zw.p, Ww.p, nb, nb, shw.p, inner_prec, transpose, s);
       ProfScope pk2(PROF_KRYLOV, 0.0, s);
       // CGS with one re-orthogonalisation: h1 = V^H w, w -= V h1, h2 = V^H w, w -= V h2; H[:, j] = h1 + h2.
       // With an FP32 basis of at most MD_MAXV vectors this takes three sweeps: h1; the first update with
       // h2 fused; the second update with ||w||^2 fused.
       const int nv = j + 1;
+      cplx* Hc = H.p + (long long)j * (k + 1) * nb;
+      int norm_chunks = 0;   // chunk sums of ||w||^2 left in partial
       bool fused = false;
-      if constexpr (sizeof(VT) == sizeof(cuFloatComplex)) {
+      if constexpr (F32) {
         if (nv <= MD_MAXV) {
           fused = true;
           // algorithmic HBM bytes of the three sweeps: V read three times, w read three times and
@@ -780,72 +947,64 @@ static void gmres_impl(gfcc_ctx* c, const cplx* Bin, cplx* Xout, cplx* Rout, con
           const int small = nb < MD_TX ? 1 : 0;
           const float2* Vf = reinterpret_cast<const float2*>(V.p);
           float2* Wf = reinterpret_cast<float2*>(Ww.p);
+          const dim3 rgrid((nb + 31) / 32, nv), rblock(32, 8);
           {
             ProfScope pk(small ? PROF_CGS_SMALL_NB : PROF_CGS_MULTIDOT, (nv + 1.0) * vbytes, s);
             launch_sweep<0>(Vf, vstride, nv, Wf, D, nb, nullptr, 0, partial.p, s);
           }
-          reduce_partial_kernel<<<(nv * nb + 255) / 256, 256, 0, s>>>(partial.p, nchunk, nv, nb, hb.p, k + 1, 0, 0);
-          GFCC_LAUNCH_CHECK();
-          add_h_kernel<<<(nb * nv + 255) / 256, 256, 0, s>>>(hb.p, k + 1, H.p + (long long)j * (k + 1), (k + 1) * k, nv,
-                                                             nb, 0);
+          reduce_partial_kernel<<<rgrid, rblock, 0, s>>>(partial.p, nchunk, nv, nb, hb.p, k + 1, 0, Hc, 0);
           GFCC_LAUNCH_CHECK();
           {
             ProfScope pk(small ? PROF_CGS_SMALL_NB : PROF_CGS_UPDATE_DOT, (nv + 2.0) * vbytes, s);
             launch_sweep<1>(Vf, vstride, nv, Wf, D, nb, hb.p, k + 1, partial.p, s);
           }
-          reduce_partial_kernel<<<(nv * nb + 255) / 256, 256, 0, s>>>(partial.p, nchunk, nv, nb, hb.p, k + 1, 0, 0);
-          GFCC_LAUNCH_CHECK();
-          add_h_kernel<<<(nb * nv + 255) / 256, 256, 0, s>>>(hb.p, k + 1, H.p + (long long)j * (k + 1), (k + 1) * k, nv,
-                                                             nb, 1);
+          reduce_partial_kernel<<<rgrid, rblock, 0, s>>>(partial.p, nchunk, nv, nb, hb.p, k + 1, 0, Hc, 1);
           GFCC_LAUNCH_CHECK();
           {
             ProfScope pk(small ? PROF_CGS_SMALL_NB : PROF_CGS_UPDATE_NORM, (nv + 2.0) * vbytes, s);
             launch_sweep<2>(Vf, vstride, nv, Wf, D, nb, hb.p, k + 1, partial.p, s);
           }
-          reduce_partial_kernel<<<(nb + 255) / 256, 256, 0, s>>>(partial.p, nchunk, 1, nb, tmpc.p, 1, 0, 0);
-          GFCC_LAUNCH_CHECK();
-          finalize_norm_kernel<<<(nb + 255) / 256, 256, 0, s>>>(tmpc.p, nb, nrm.p);
-          GFCC_LAUNCH_CHECK();
+          norm_chunks = nchunk;
         }
       }
       if (!fused) {
         for (int pass = 0; pass < 2; ++pass) {
-          multidot<VT>(V.p, vstride, nv, Ww.p, D, nb, hb.p, k + 1, 0, false, partial, s);
-          update_kernel<VT><<<grid_for(D * nb), 256, 0, s>>>(V.p, vstride, nv, Ww.p, D, nb, hb.p, k + 1, 0, -1.0);
-          GFCC_LAUNCH_CHECK();
-          add_h_kernel<<<(nb * nv + 255) / 256, 256, 0, s>>>(hb.p, k + 1, H.p + (long long)j * (k + 1), (k + 1) * k,
-                                                             nv, nb, pass == 0 ? 0 : 1);
+          multidot<VT>(V.p, vstride, nv, Ww.p, D, nb, hb.p, k + 1, Hc, pass == 1, partial, s);
+          update_kernel<VT><<<eg.grid, eg.block, 0, s>>>(V.p, vstride, nv, Ww.p, D, nb, hb.p, k + 1);
           GFCC_LAUNCH_CHECK();
         }
-        col_norms<VT>(Ww.p, D, nb, nrm.p, partial, tmpc, s);
+        col_norms<VT>(Ww.p, D, nb, nrm.p, partial, s);
       }
-      scale_cols_kernel<VT, VT><<<grid_for(D * nb), 256, 0, s>>>(Ww.p, Vn, nrm.p, D, nb);
+      arnoldi_finish_kernel<<<(nb + 31) / 32, GV_T, 0, s>>>(partial.p, norm_chunks, nrm.p, invf.p, H.p, cs.p, sn.p, g.p,
+                                                            bnorm.p, kc.p, live.p, nb, k, j, thr.p, nlive.p + j);
       GFCC_LAUNCH_CHECK();
-      GFCC_CUDA(cudaMemsetAsync(nlive.p, 0, sizeof(int), s));
-      givens_kernel<<<(nb + 127) / 128, 128, 0, s>>>(H.p, cs.p, sn.p, g.p, nrm.p, bnorm.p, kc.p, live.p, nb, k, j,
-                                                     thr.p, nlive.p);
-      GFCC_LAUNCH_CHECK();
-      int hl = 0;
-      GFCC_CUDA(cudaMemcpyAsync(&hl, nlive.p, sizeof(int), cudaMemcpyDeviceToHost, s));
-      GFCC_CUDA(cudaStreamSynchronize(s));
+      GFCC_CUDA(cudaMemcpyAsync(c->pin, nlive.p + j, sizeof(int), cudaMemcpyDeviceToHost, s));
+      GFCC_CUDA(cudaEventRecord(c->pin_event, s));
+      // the next step's first kernels run while the host waits for the count (if no column is left, they wrote
+      // one more basis vector that nothing uses)
+      if (j + 1 < k) start_step(Ww.p, j + 1);
+      GFCC_CUDA(cudaEventSynchronize(c->pin_event));
+      const int hl = *c->pin;
+      steps = j + 1;
       c->stats.gmres_iters++;
       for (int q = 0; q < nb; ++q) st.iters[map[q]]++;
       if (hl == 0) break;
     }
-    backsolve_kernel<<<(nb + 127) / 128, 128, 0, s>>>(H.p, g.p, kc.p, nb, k);
+    backsolve_kernel<VT><<<(nb + 3) / 4, 128, 0, s>>>(H.p, g.p, kc.p, nb, k, yv.p);
     GFCC_LAUNCH_CHECK();
     // X += P V y (only the first kc basis vectors carry weight; later y entries are zero)
-    correct_kernel<VT><<<grid_for(D * nb), 256, 0, s>>>(V.p, vstride, k, g.p, k + 1, Xw.p, c->op.mdiag.p, shw.p, D, nb);
+    correct_kernel<VT><<<eg.grid, eg.block, 0, s>>>(V.p, vstride, steps, yv.p, Xw.p, c->op.mdiag.p, c->op.rowf.p,
+                                                    shw.p, shf.p, D, nb);
     GFCC_LAUNCH_CHECK();
   }
   GFCC_CUDA(cudaStreamSynchronize(s));
 }
 
 void gmres_batched(gfcc_ctx* c, const cplx* Bin, cplx* Xout, cplx* Rout, const cplx* shifts_dev, int nb0,
-                   SolveStatus& st, bool transpose, const cplx* X0) {
+                   SolveStatus& st, bool transpose, const cplx* X0, bool polish) {
   const bool f32 = c->opts.precision == GFCC_PREC_TF32 || c->opts.precision == GFCC_PREC_BF16;
-  if (f32) gmres_impl<cuFloatComplex>(c, Bin, Xout, Rout, shifts_dev, nb0, st, transpose, X0);
-  else gmres_impl<cplx>(c, Bin, Xout, Rout, shifts_dev, nb0, st, transpose, X0);
+  if (f32) gmres_impl<cuFloatComplex>(c, Bin, Xout, Rout, shifts_dev, nb0, st, transpose, X0, polish);
+  else gmres_impl<cplx>(c, Bin, Xout, Rout, shifts_dev, nb0, st, transpose, X0, polish);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -908,7 +1067,7 @@ __global__ void green_partial_kernel(const double* __restrict__ cq, long long D,
                                      int ldb, int ncols, long long rows, cplx* __restrict__ part) {
   const long long r0 = blockIdx.x * rows, r1 = min(D, r0 + rows);
   const int npair = nq * ncols;
-  for (int t = threadIdx.x; t < npair; t += blockDim.x) {
+  for (int t = blockIdx.y * blockDim.x + threadIdx.x; t < npair; t += gridDim.y * blockDim.x) {
     const int q = t / ncols, c = t % ncols;
     const double* cr = cq + (long long)q * D;
     double sr = 0.0, si = 0.0;
@@ -947,7 +1106,9 @@ void green_from_batch(const double* cvec, int D, const int* qrows_host, int nq, 
   const long long rows = std::max<long long>(64, (D + 2 * 152 * 4 - 1) / (2 * 152 * 4));
   const int nchunk = (int)((D + rows - 1) / rows);
   part.alloc((long long)nchunk * nq * ncols);
-  green_partial_kernel<<<nchunk, 256, 0, s>>>(Cq.p, D, nq, X, ldb, ncols, rows, part.p);
+  // few chunks (small D): the pairs are spread over blocks too
+  const int gy = (int)std::max<long long>(1, std::min<long long>(((long long)nq * ncols + 255) / 256, 1216 / nchunk));
+  green_partial_kernel<<<dim3(nchunk, gy), 256, 0, s>>>(Cq.p, D, nq, X, ldb, ncols, rows, part.p);
   GFCC_LAUNCH_CHECK();
   green_reduce_kernel<<<(nq * ncols + 255) / 256, 256, 0, s>>>(part.p, nchunk, nq, ncols, G);
   GFCC_LAUNCH_CHECK();

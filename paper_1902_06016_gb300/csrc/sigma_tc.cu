@@ -9,6 +9,7 @@
 //   ring: CT[(a,i)][(j,c,r)]       = Wr (ov x ov) . U,  U[(j,c,r)][(m,e)] = r_mj^e
 #include "gfcc_internal.cuh"
 #include "ozaki.cuh"
+#include "precond.cuh"
 #include "tc_gemm.cuh"
 
 #include <nvtx3/nvToolsExt.h>
@@ -167,6 +168,217 @@ void prep_operand(const VT* X, int o, int v, int nb, typename E::T* out, int kpa
   }
 }
 
+// ---- operand preparation of the FP32 Krylov basis -------------------------------------------------
+// One pass over w: the basis vector v = w inv is written, z = P v formed, and every 2h1p element goes to the
+// three places the up and ring operands have for it, all of them along k = pair v + e of a tile of 32 k x 32 c:
+//   up:   B[c*2 + r][k];   ring: U[(j*nb + c)*2 + r][m v + e] = z, U[(m*nb + c)*2 + r][j v + e] = -z  (m < j)
+// The oooo operand runs along the pair index and is made from v by a second kernel. Before, scaling,
+// preconditioning and the three operands were five kernels, each reading a vector block. The blocks m = j of U
+// and the K padding stay zero: the buffers are zeroed when they are allocated, the blocks m = j (whose rows
+// depend on the batch width) also when the width has changed.
+template <typename E, typename WT>
+__global__ void __launch_bounds__(256) prep_fused_kernel(const WT* __restrict__ W, const float* __restrict__ inv,
+                                                         float2* __restrict__ V, const RowF* __restrict__ md,
+                                                         const ShiftF* __restrict__ shift, int o, int v, int nb,
+                                                         long long Pv, typename E::T* __restrict__ Bup, int kup,
+                                                         typename E::T* __restrict__ U, int kr,
+                                                         float2* __restrict__ z1) {
+  __shared__ float2 tile[PT][PT + 1];
+  const int c0 = blockIdx.y * PT, c = c0 + threadIdx.x;
+  const float s = c < nb ? inv[c] : 0.f;
+  const ShiftF sh = c < nb ? shift[c] : make_float4(0.f, 0.f, 0.f, 0.f);
+  if ((long long)blockIdx.x * PT >= Pv) {   // the last blocks: v and z of the o 1h rows
+    const int nu = (int)(blockIdx.x - (Pv + PT - 1) / PT) * PT;
+    for (int kk = threadIdx.y; kk < PT; kk += blockDim.y)
+      if (nu + kk < o && c < nb) {
+        const long long t = (long long)(nu + kk) * nb + c;
+        const WT w = W[t];
+        const float2 x = make_float2((float)w.x * s, (float)w.y * s);
+        V[t] = x;
+        z1[t] = precond_f32(x, md[nu + kk], sh);
+      }
+    return;
+  }
+  const long long k0 = (long long)blockIdx.x * PT;
+#pragma unroll
+  for (int kk = threadIdx.y; kk < PT; kk += 8) {
+    const long long k = k0 + kk;
+    float2 z = make_float2(0.f, 0.f);
+    if (k < Pv && c < nb) {
+      const long long t = (o + k) * nb + c;
+      const WT w = W[t];
+      const float2 x = make_float2((float)w.x * s, (float)w.y * s);
+      V[t] = x;
+      z = precond_f32(x, md[o + k], sh);
+    }
+    tile[kk][threadIdx.x] = z;
+  }
+  __syncthreads();
+  const long long k = k0 + threadIdx.x;
+  if (k >= Pv) return;
+  const int p = (int)(k / v), e = (int)(k - (long long)p * v);
+  int m, j;
+  unpair(p, m, j);
+#pragma unroll
+  for (int rr = threadIdx.y; rr < 2 * PT; rr += 8) {
+    const int cc = c0 + (rr >> 1), r = rr & 1;
+    if (cc < nb) {
+      const float2 z = tile[threadIdx.x][rr >> 1];
+      const float x = r ? z.y : z.x;
+      Bup[((long long)cc * 2 + r) * kup + k] = E::cvt(x);
+      U[(((long long)j * nb + cc) * 2 + r) * kr + m * v + e] = E::cvt(x);
+      U[(((long long)m * nb + cc) * 2 + r) * kr + j * v + e] = E::cvt(-x);
+    }
+  }
+}
+// oooo: B[(a*nb + c)*2 + r][p] = z_p^a of column c (component r)
+template <typename E>
+__global__ void __launch_bounds__(256) prep_oooo_kernel(const float2* __restrict__ V, const RowF* __restrict__ md,
+                                                        const ShiftF* __restrict__ shift, int o, int v, int nb, int P,
+                                                        typename E::T* __restrict__ B, int kp) {
+  __shared__ float2 tile[PT][PT + 1];
+  const int a = blockIdx.z, p0 = blockIdx.x * PT, c0 = blockIdx.y * PT, c = c0 + threadIdx.x;
+  const ShiftF sh = c < nb ? shift[c] : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+  for (int kk = threadIdx.y; kk < PT; kk += 8) {
+    float2 z = make_float2(0.f, 0.f);
+    if (p0 + kk < P && c < nb) {
+      const long long nu = o + (long long)(p0 + kk) * v + a;
+      z = precond_f32(V[nu * nb + c], md[nu], sh);
+    }
+    tile[kk][threadIdx.x] = z;
+  }
+  __syncthreads();
+  const int p = p0 + threadIdx.x;
+  if (p >= P) return;
+#pragma unroll
+  for (int rr = threadIdx.y; rr < 2 * PT; rr += 8) {
+    const int cc = c0 + (rr >> 1), r = rr & 1;
+    if (cc < nb) {
+      const float2 z = tile[threadIdx.x][rr >> 1];
+      B[(((long long)a * nb + cc) * 2 + r) * kp + p] = E::cvt(r ? z.y : z.x);
+    }
+  }
+}
+// U[(j*nb + c)*2 + r][j v + e] = 0
+template <typename E>
+__global__ void zero_ring_diag_kernel(typename E::T* __restrict__ U, int v, int nb, int kr) {
+  const int j = blockIdx.y;
+  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < 2LL * nb * v; t += (long long)gridDim.x * blockDim.x)
+    U[((long long)j * nb * 2 + t / v) * kr + (long long)j * v + t % v] = E::cvt(0.f);
+}
+__global__ void split_rows_kernel(const double* __restrict__ md, const double* __restrict__ diag, long long D,
+                                  RowF* __restrict__ out) {
+  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < D; t += (long long)gridDim.x * blockDim.x) {
+    const float h = (float)md[t];
+    out[t] = make_float4(h, (float)(md[t] - (double)h), (float)diag[t], 0.f);
+  }
+}
+__global__ void split_shifts_kernel(const cplx* __restrict__ shift, int nb, ShiftF* __restrict__ out) {
+  const int c = blockIdx.x * blockDim.x + threadIdx.x;
+  if (c >= nb) return;
+  const float h = (float)shift[c].x;
+  out[c] = make_float4(h, (float)(shift[c].x - (double)h), (float)shift[c].y, 0.f);
+}
+// down operand from the prepared vector: B[c*2 + r][e] = Xe[e][c*2 + r] (e < v), B[c*2 + r][v + m] = z_m. Threads run
+// along the up product's columns (coalesced); its K splits are summed here, in order; the o 1h rows that the
+// combine pass reads are kept in up, with A11 z added.
+template <typename E>
+__global__ void __launch_bounds__(128) prep_down_f32_kernel(const float* __restrict__ part, int zs, long long stride,
+                                                            long long ldu, float* __restrict__ up,
+                                                            const float* __restrict__ z1,
+                                                            const double* __restrict__ A11, int o, int v, int nb,
+                                                            typename E::T* __restrict__ B, int kpad) {
+  const int n = blockIdx.x * blockDim.x + threadIdx.x;
+  if (n >= 2 * nb) return;
+  const int k = blockIdx.y;
+  float x = 0.f;
+#pragma unroll 8
+  for (int z = 0; z < zs; ++z) x += part[z * stride + (long long)k * ldu + n];
+  if (k < v) {
+    B[(long long)n * kpad + k] = E::cvt(x);
+  } else {
+    const int i = k - v;
+    float y = 0.f;
+#pragma unroll 4
+    for (int m = 0; m < o; ++m) y += (float)A11[(long long)i * o + m] * z1[(long long)m * 2 * nb + n];
+    up[(long long)k * ldu + n] = x + y;
+  }
+  if (k < o) B[(long long)n * kpad + v + k] = E::cvt(z1[(long long)k * 2 * nb + n]);
+}
+// y = (diag + shift) z + up / C2 + ring terms for the FP32 basis, z = P v. Blocks of 2 CW columns x 256 / CW rows: a
+// thread takes columns c and c + CW of two rows at a time, so that the index arithmetic of a row (a division and
+// the pair it belongs to) is shared by two elements and the ten loads of the four elements are in flight
+// together. HBM-bound: five vector blocks read or written.
+__global__ void __launch_bounds__(256) combine_f32_kernel(const float2* __restrict__ V, float2* __restrict__ Y,
+                                                          const float2* __restrict__ up, const float2* __restrict__ C2,
+                                                          const float2* __restrict__ CT, const float2* __restrict__ z1,
+                                                          const RowF* __restrict__ md,
+                                                          const ShiftF* __restrict__ shift, int o, int v, int Pv, int nb) {
+  constexpr int RW = 2;
+  const int cw = blockDim.x, c0 = blockIdx.x * 2 * cw + threadIdx.x;
+  const bool on[2] = {c0 < nb, c0 + cw < nb};
+  if (!on[0]) return;
+  ShiftF sh[2];
+  sh[0] = shift[c0];
+  sh[1] = on[1] ? shift[c0 + cw] : sh[0];
+  const long long ldct = (long long)o * nb;
+  const int ry = blockIdx.y * blockDim.y + threadIdx.y, step = gridDim.y * blockDim.y;
+  auto shifted = [&](float d, const ShiftF& s, float2 z) {
+    const float dre = d + s.x, dim = s.z;
+    return make_float2(dre * z.x - dim * z.y, dre * z.y + dim * z.x);
+  };
+  for (int nu = ry; nu < o; nu += step)
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+      if (on[h]) {
+        const long long t = (long long)nu * nb + c0 + h * cw;
+        const float2 y = shifted(md[nu].z, sh[h], z1[t]), u = up[t + (long long)v * nb];
+        Y[t] = make_float2(y.x + u.x, y.y + u.y);
+      }
+  for (long long row0 = ry; row0 < Pv; row0 += (long long)RW * step) {
+    float2 x[RW][2], q[RW][2], c1[RW][2], c2[RW][2];
+    RowF m[RW];
+#pragma unroll
+    for (int r = 0; r < RW; ++r) {
+      const long long row = row0 + (long long)r * step;
+      if (row < Pv) {
+        const int p = (int)row / v, a = (int)row - p * v;
+        int i, j;
+        unpair(p, i, j);
+        m[r] = md[o + row];
+        const float2* px = V + (o + row) * nb + c0;
+        const float2* pq = C2 + row * nb + c0;
+        const float2* p1 = CT + ((long long)a * o + i) * ldct + (long long)j * nb + c0;
+        const float2* p2 = CT + ((long long)a * o + j) * ldct + (long long)i * nb + c0;
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+          if (on[h]) {
+            x[r][h] = px[h * cw];
+            q[r][h] = pq[h * cw];
+            c1[r][h] = p1[h * cw];
+            c2[r][h] = p2[h * cw];
+          }
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < RW; ++r) {
+      const long long row = row0 + (long long)r * step;
+      if (row < Pv) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+          if (on[h]) {
+            float2 y = shifted(m[r].z, sh[h], precond_f32(x[r][h], m[r], sh[h]));
+            y.x += q[r][h].x;
+            y.y += q[r][h].y;
+            y.x += c1[r][h].x - c2[r][h].x;
+            y.y += c1[r][h].y - c2[r][h].y;
+            Y[(o + row) * nb + c0 + h * cw] = y;
+          }
+      }
+    }
+  }
+}
 
 // ring: U[(j*nb + c)*2 + r][m*v + e] = r_mj^e (component r), K padded
 // oooo: B[(a*nb + c)*2 + r][pmn] = X2[(pmn*v + a)][c].r
@@ -303,8 +515,10 @@ struct LpState {
   DBuf<uint8_t> Wr, Woo, Aup, Adn;            // operands (bf16 or fp32 elements)
   DBuf<uint8_t> Bring, Boo, Bup, Bdn;         // per-batch operands
   DBuf<float> CT, C2, up_part, up;            // outputs
+  DBuf<float> z1;                             // z of the 1h rows [o][nb] (FP32 basis)
   DBuf<int> err;
-  int nb_cap = 0, ksplit = 1;
+  int nb_cap = 0;
+  int nb_prep = 0;   // batch width for which the ring operand's blocks m = j are zero (0: unknown)
 };
 
 static LpState* lp_state(gfcc_ctx* c, bool transpose = false) {
@@ -341,8 +555,9 @@ void release_sigma_batch_buffers(gfcc_ctx* c) {
   for (bool tr : {false, true}) {
     if (LpState* st = lp_state(c, tr)) {
       for (DBuf<uint8_t>* b : {&st->Bring, &st->Boo, &st->Bup, &st->Bdn}) b->release();
-      for (DBuf<float>* b : {&st->CT, &st->C2, &st->up_part, &st->up}) b->release();
+      for (DBuf<float>* b : {&st->CT, &st->C2, &st->up_part, &st->up, &st->z1}) b->release();
       st->nb_cap = 0;
+      st->nb_prep = 0;
     }
     if (EmuState* st = emu_state(c, tr)) {
       for (DBuf<double>* b : {&st->stage, &st->CT, &st->C2, &st->up}) b->release();
@@ -523,27 +738,51 @@ int low_precision_error(gfcc_ctx* c) {
   return 0;
 }
 
-template <TcKind K, typename VT>
-static void sigma_lp_impl(gfcc_ctx* c, LpState& st, const VT* X, VT* Y, int nb, const cplx* shift, cudaStream_t s,
+// batch buffers for nb columns; zeroed when allocated (the K padding of the operands is never written)
+template <TcKind K>
+static void lp_batch_buffers(gfcc_ctx* c, LpState& st, int nb, cudaStream_t s) {
+  using T = typename Elem<K>::T;
+  if (nb <= st.nb_cap) return;
+  const int o = c->o, v = c->v;
+  const long long ov = (long long)o * v, Pv = (long long)c->P * v;
+  const long long nring = 2LL * o * nb, noo = 2LL * v * nb, nsm = 2LL * nb;
+  st.Bring.alloc(sizeof(T) * nring * st.Kr);
+  st.Boo.alloc(sizeof(T) * noo * st.Kp);
+  st.Bup.alloc(sizeof(T) * nsm * st.Kpv);
+  st.Bdn.alloc(sizeof(T) * nsm * st.Kvo);
+  for (DBuf<uint8_t>* b : {&st.Bring, &st.Boo, &st.Bup, &st.Bdn}) b->zero(s);
+  st.CT.alloc(ov * nring);
+  st.C2.alloc(Pv * nsm);
+  st.up.alloc((long long)(v + o) * nsm);
+  st.z1.alloc((long long)o * nsm);
+  st.nb_cap = nb;
+  st.nb_prep = 0;
+}
+// K splits of the short-and-wide up product and the splits it writes
+template <TcKind K>
+static int lp_up_splits(const LpState& st, int rows, long long nsm, int* written) {
+  // about two waves of CTAs
+  const int mt = (rows + 127) / 128;
+  const int nk_up = st.Kpv / tc_kblock(K);
+  const int ksplit = std::max(1, std::min(nk_up, (2 * 152) / std::max(1, mt * (int)((nsm + 255) / 256))));
+  const int nk_split = (nk_up + ksplit - 1) / ksplit;
+  *written = (nk_up + nk_split - 1) / nk_split;
+  return ksplit;
+}
+
+// FP64 vectors (gfcc_sigma in TF32 or BF16)
+template <TcKind K>
+static void sigma_lp_impl(gfcc_ctx* c, LpState& st, const cplx* X, cplx* Y, int nb, const cplx* shift, cudaStream_t s,
                           const double* A11) {
+  using VT = cplx;
   using T = typename Elem<K>::T;
   const int o = c->o, v = c->v, P = c->P;
   const long long ov = (long long)o * v, Pv = (long long)P * v, D = c->D;
   const long long nring = 2LL * o * nb, noo = 2LL * v * nb, nsm = 2LL * nb;
-  if (nb > st.nb_cap) {
-    st.Bring.alloc(sizeof(T) * nring * st.Kr);
-    st.Boo.alloc(sizeof(T) * noo * st.Kp);
-    st.Bup.alloc(sizeof(T) * nsm * st.Kpv);
-    st.Bdn.alloc(sizeof(T) * nsm * st.Kvo);
-    st.CT.alloc(ov * nring);
-    st.C2.alloc(Pv * nsm);
-    st.up.alloc((long long)(v + o) * nsm);
-    st.nb_cap = nb;
-  }
-  // split-K for the short-and-wide "up" GEMM: about two waves of CTAs
-  const int mt = (v + o + 127) / 128;
-  const int nk_up = st.Kpv / tc_kblock(K);
-  int ksplit = std::max(1, std::min(nk_up, (2 * 152) / std::max(1, mt * (int)((nsm + 255) / 256))));
+  lp_batch_buffers<K>(c, st, nb, s);
+  st.nb_prep = 0;   // the ring operand's zero blocks are rewritten here
+  int zs = 1;
+  const int ksplit = lp_up_splits<K>(st, v + o, nsm, &zs);
   const long long part_stride = (long long)(v + o) * nsm;
   st.up_part.alloc(part_stride * ksplit);
 
@@ -570,8 +809,6 @@ static void sigma_lp_impl(gfcc_ctx* c, LpState& st, const VT* X, VT* Y, int nb, 
   }
   {
     ProfScope pc(PROF_LP_COMBINE, 0.0, s);
-    const int nk_split = (nk_up + ksplit - 1) / ksplit;
-    const int zs = (nk_up + nk_split - 1) / nk_split;
     reduce_splits_kernel<<<grid_for(part_stride), 256, 0, s>>>(st.up_part.p, zs, part_stride, part_stride, st.up.p);
     GFCC_LAUNCH_CHECK();
   }
@@ -602,26 +839,163 @@ static void sigma_lp_impl(gfcc_ctx* c, LpState& st, const VT* X, VT* Y, int nb, 
   GFCC_LAUNCH_CHECK();
 }
 
-void sigma_lowprec(gfcc_ctx* c, const cplx* X, cplx* Y, int nb, const cplx* shift, cudaStream_t s, bool transpose) {
-  LpState* st = transpose ? lp_state_transposed(c) : lp_state(c);
-  GFCC_CHECK(st != nullptr, GFCC_ERR_STATE, "low-precision operator not built");
-  const double* A11 = op_view(c, transpose).A11;
-  if (st->kind == TcKind::BF16) sigma_lp_impl<TcKind::BF16, cplx>(c, *st, X, Y, nb, shift, s, A11);
-  else sigma_lp_impl<TcKind::TF32, cplx>(c, *st, X, Y, nb, shift, s, A11);
-  c->stats.sigma_calls++;
-  c->stats.sigma_cols += nb;
+// ---- the FP32 basis: prepare (v, operands of z = P v) and apply -----------------------------------
+template <TcKind K, typename WT>
+static void lp_prepare_impl(gfcc_ctx* c, LpState& st, const WT* W, const float* inv, cuFloatComplex* V, int nb,
+                            const float4* shift, cudaStream_t s) {
+  using T = typename Elem<K>::T;
+  const int o = c->o, v = c->v, P = c->P;
+  const long long Pv = (long long)P * v;
+  lp_batch_buffers<K>(c, st, nb, s);
+  T* U = reinterpret_cast<T*>(st.Bring.p);
+  ProfScope pp(PROF_LP_PREP, 0.0, s);
+  if (st.nb_prep != nb) {
+    zero_ring_diag_kernel<Elem<K>><<<dim3((unsigned)std::min<long long>((2LL * nb * v + 255) / 256, 1024), o), 256, 0, s>>>(
+        U, v, nb, st.Kr);
+    GFCC_LAUNCH_CHECK();
+    st.nb_prep = nb;
+  }
+  float2* Vf = reinterpret_cast<float2*>(V);
+  const unsigned ct = (unsigned)((nb + PT - 1) / PT);
+  GFCC_CHECK((Pv + PT - 1) / PT + (o + PT - 1) / PT < (1LL << 31) && ct <= 65535 && v <= 65535, GFCC_ERR_ARG,
+             "sigma: batch or virtual count too large");
+  prep_fused_kernel<Elem<K>, WT><<<dim3((unsigned)((Pv + PT - 1) / PT + (o + PT - 1) / PT), ct), dim3(PT, 8), 0, s>>>(
+      W, inv, Vf, c->op.rowf.p, shift, o, v, nb, Pv, reinterpret_cast<T*>(st.Bup.p), st.Kpv, U, st.Kr,
+      reinterpret_cast<float2*>(st.z1.p));
+  GFCC_LAUNCH_CHECK();
+  prep_oooo_kernel<Elem<K>><<<dim3((unsigned)((P + PT - 1) / PT), ct, (unsigned)v), dim3(PT, 8), 0, s>>>(
+      Vf, c->op.rowf.p, shift, o, v, nb, P, reinterpret_cast<T*>(st.Boo.p), st.Kp);
+  GFCC_LAUNCH_CHECK();
 }
 
-void sigma_lowprec_f32(gfcc_ctx* c, const cuFloatComplex* X, cuFloatComplex* Y, int nb, const cplx* shift,
+template <TcKind K>
+static void lp_apply_impl(gfcc_ctx* c, LpState& st, const cuFloatComplex* V, cuFloatComplex* Y, int nb,
+                          const float4* shift, cudaStream_t s, const double* A11) {
+  using T = typename Elem<K>::T;
+  const int o = c->o, v = c->v, P = c->P;
+  const long long ov = (long long)o * v, Pv = (long long)P * v;
+  const long long nring = 2LL * o * nb, noo = 2LL * v * nb, nsm = 2LL * nb;
+  const double es = sizeof(T);
+  const float2* Vf = reinterpret_cast<const float2*>(V);
+  // the three products that do not depend on each other
+  TcProduct pr[3];
+  pr[0].A = TcOperand{st.Wr.p, ov, st.Kr};      // ring
+  pr[0].B = TcOperand{st.Bring.p, nring, st.Kr};
+  pr[0].C = st.CT.p; pr[0].ldc = nring; pr[0].M = ov; pr[0].N = nring; pr[0].k_alg = ov;
+  pr[1].A = TcOperand{st.Woo.p, P, st.Kp};      // oooo into C2
+  pr[1].B = TcOperand{st.Boo.p, noo, st.Kp};
+  pr[1].C = st.C2.p; pr[1].ldc = noo; pr[1].M = P; pr[1].N = noo;
+  pr[2].A = TcOperand{st.Aup.p, v + o, st.Kpv}; // up, split along K
+  pr[2].B = TcOperand{st.Bup.p, nsm, st.Kpv};
+  pr[2].ldc = nsm; pr[2].M = v + o; pr[2].N = nsm; pr[2].split_stride = (long long)(v + o) * nsm;
+  // One launch when the ring product alone does not keep the persistent grid busy for long (fewer than six
+  // waves of tiles): its last wave, the short oooo tiles and the K splits of up then fill each other's gaps, and up
+  // needs only as many splits as leave its units as long as the others' (each split is one more partial sum to
+  // read). Above that the tails are a few per cent and the ring is launched alone, as a class of its own.
+  // o = 9, v = 33 attachment half, 264 columns: 3 launches of 15.8 us -> one of 26.
+  const int kb = tc_kblock(K);
+  const long long t_ring = ((ov + 127) / 128) * ((nring + 255) / 256), t_oo = ((P + 127) / 128) * ((noo + 255) / 256);
+  const long long t_up = ((v + o + 127) / 128) * ((nsm + 255) / 256);
+  const bool grouped = t_ring < 6 * 152;
+  int zs = 1;
+  if (grouped) {
+    const int nk = st.Kpv / kb, longest = std::max({16, st.Kr / kb, st.Kp / kb});
+    const long long fill = std::max<long long>(1, (2 * 152 - t_ring - t_oo) / t_up);
+    pr[2].ksplit = (int)std::min<long long>(nk, std::max<long long>((nk + longest - 1) / longest, fill));
+    const int nk_split = (nk + pr[2].ksplit - 1) / pr[2].ksplit;
+    zs = (nk + nk_split - 1) / nk_split;
+  } else {
+    pr[2].ksplit = lp_up_splits<K>(st, v + o, nsm, &zs);
+  }
+  st.up_part.alloc(pr[2].split_stride * pr[2].ksplit);
+  pr[2].C = st.up_part.p;
+  if (grouped) {
+    nvtxRangePushA("gfcc_ring_gemm");
+    tc_gemm_group(K, pr, 3, st.err.p, s, PROF_TC_RING);
+    nvtxRangePop();
+  } else {
+    {
+      ProfScope pb(PROF_LP_SMALL_GEMMS, es * (double)(v + o + nsm) * (double)Pv + 4.0 * (double)(v + o) * nsm, s);
+      tc_gemm_group(K, pr + 2, 1, st.err.p, s);
+    }
+    {
+      ProfScope pb(PROF_LP_SMALL_GEMMS, es * (double)(P + noo) * (double)P + 4.0 * (double)P * noo, s);
+      tc_gemm_group(K, pr + 1, 1, st.err.p, s);
+    }
+    // ring (its own profiling class and NVTX range, so that its launches can be timed and profiled alone)
+    nvtxRangePushA("gfcc_ring_gemm");
+    tc_gemm_group(K, pr, 1, st.err.p, s, PROF_TC_RING);
+    nvtxRangePop();
+  }
+  {
+    ProfScope pp(PROF_LP_PREP, 0.0, s);
+    prep_down_f32_kernel<Elem<K>><<<dim3((unsigned)((nsm + 127) / 128), (unsigned)(v + o)), 128, 0, s>>>(
+        st.up_part.p, zs, pr[2].split_stride, nsm, st.up.p, st.z1.p, A11, o, v, nb, reinterpret_cast<T*>(st.Bdn.p), st.Kvo);
+    GFCC_LAUNCH_CHECK();
+  }
+  {
+    ProfScope pb(PROF_LP_SMALL_GEMMS, es * (double)(Pv + nsm) * (double)(v + o) + 8.0 * (double)Pv * nsm, s);
+    tc_gemm(K, TcOperand{st.Adn.p, Pv, st.Kvo}, TcOperand{st.Bdn.p, nsm, st.Kvo}, st.C2.p, nsm, Pv, nsm, 1, 1, 0, st.err.p,
+            s);
+  }
+  ProfScope pc(PROF_LP_COMBINE, 0.0, s);
+  const int cw = nb > 32 ? 32 : nb > 16 ? 16 : nb > 8 ? 8 : 4;
+  const long long gx = (nb + 2 * cw - 1) / (2 * cw);
+  const long long gy = std::max<long long>(1, std::min<long long>({(Pv + 512 / cw - 1) / (512 / cw), 152LL * 16 / gx, 65535}));
+  combine_f32_kernel<<<dim3((unsigned)gx, (unsigned)gy), dim3(cw, 256 / cw), 0, s>>>(
+      Vf, reinterpret_cast<float2*>(Y), reinterpret_cast<const float2*>(st.up.p), reinterpret_cast<const float2*>(st.C2.p),
+      reinterpret_cast<const float2*>(st.CT.p), reinterpret_cast<const float2*>(st.z1.p), c->op.rowf.p,
+      shift, o, v, (int)Pv, nb);
+  GFCC_LAUNCH_CHECK();
+}
+
+void ensure_row_split(gfcc_ctx* c) {
+  if (c->op.rowf.p) return;
+  c->op.rowf.alloc(c->D);
+  split_rows_kernel<<<grid_for(c->D), 256, 0, c->stream>>>(c->op.mdiag.p, c->op.diag.p, c->D, c->op.rowf.p);
+  GFCC_LAUNCH_CHECK();
+}
+void split_shifts(const cplx* shift, int nb, float4* out, cudaStream_t s) {
+  split_shifts_kernel<<<(nb + 127) / 128, 128, 0, s>>>(shift, nb, out);
+  GFCC_LAUNCH_CHECK();
+}
+
+template <typename WT>
+static void lp_prepare(gfcc_ctx* c, const WT* W, const float* inv, cuFloatComplex* V, int nb, const float4* shift,
                        cudaStream_t s, bool transpose) {
   LpState* st = transpose ? lp_state_transposed(c) : lp_state(c);
   GFCC_CHECK(st != nullptr, GFCC_ERR_STATE, "low-precision operator not built");
+  if (st->kind == TcKind::BF16) lp_prepare_impl<TcKind::BF16>(c, *st, W, inv, V, nb, shift, s);
+  else lp_prepare_impl<TcKind::TF32>(c, *st, W, inv, V, nb, shift, s);
+}
+void sigma_lp_prepare(gfcc_ctx* c, const cplx* W, const float* inv, cuFloatComplex* V, int nb, const float4* shift,
+                      cudaStream_t s, bool transpose) {
+  lp_prepare(c, W, inv, V, nb, shift, s, transpose);
+}
+void sigma_lp_prepare(gfcc_ctx* c, const cuFloatComplex* W, const float* inv, cuFloatComplex* V, int nb,
+                      const float4* shift, cudaStream_t s, bool transpose) {
+  lp_prepare(c, W, inv, V, nb, shift, s, transpose);
+}
+void sigma_lp_apply(gfcc_ctx* c, const cuFloatComplex* V, cuFloatComplex* Y, int nb, const float4* shift, cudaStream_t s,
+                    bool transpose) {
+  LpState* st = transpose ? lp_state_transposed(c) : lp_state(c);
+  GFCC_CHECK(st != nullptr && st->nb_prep == nb, GFCC_ERR_STATE, "sigma: no prepared vectors");
   const double fo = c->o, fv = c->v, fP = c->P;   // algorithmic flops, as in sigma_batch
   ProfScope prof(PROF_SIGMA_LP,
                  2.0 * nb * (2.0 * fo * fv * fo * fv * fo + 2.0 * fP * fP * fv + 4.0 * fP * fv * fv + 4.0 * fo * fP * fv), s);
   const double* A11 = op_view(c, transpose).A11;
-  if (st->kind == TcKind::BF16) sigma_lp_impl<TcKind::BF16, cuFloatComplex>(c, *st, X, Y, nb, shift, s, A11);
-  else sigma_lp_impl<TcKind::TF32, cuFloatComplex>(c, *st, X, Y, nb, shift, s, A11);
+  if (st->kind == TcKind::BF16) lp_apply_impl<TcKind::BF16>(c, *st, V, Y, nb, shift, s, A11);
+  else lp_apply_impl<TcKind::TF32>(c, *st, V, Y, nb, shift, s, A11);
+  c->stats.sigma_calls++;
+  c->stats.sigma_cols += nb;
+}
+
+void sigma_lowprec(gfcc_ctx* c, const cplx* X, cplx* Y, int nb, const cplx* shift, cudaStream_t s, bool transpose) {
+  LpState* st = transpose ? lp_state_transposed(c) : lp_state(c);
+  GFCC_CHECK(st != nullptr, GFCC_ERR_STATE, "low-precision operator not built");
+  const double* A11 = op_view(c, transpose).A11;
+  if (st->kind == TcKind::BF16) sigma_lp_impl<TcKind::BF16>(c, *st, X, Y, nb, shift, s, A11);
+  else sigma_lp_impl<TcKind::TF32>(c, *st, X, Y, nb, shift, s, A11);
   c->stats.sigma_calls++;
   c->stats.sigma_cols += nb;
 }
