@@ -262,7 +262,7 @@ __global__ void __launch_bounds__(256) zslice_kernel(const cplx* __restrict__ Z,
   }
 }
 
-// Output of an exact-slice product: real, out[m ldo + n] = beta out + P[m][n]; or complex (the real
+// Output of an exact-slice product: real, out[m ldo + n] = alpha P[m][n] + beta out (alpha real); or complex (the real
 // columns n and N + n of P hold the real and imaginary parts), C(m, n) = alpha P(m, n) + beta C(m, n).
 struct OzOut {
   bool complex_out = false;
@@ -319,8 +319,9 @@ __device__ __forceinline__ cplx out_value(const OzOut& o, double re, double im, 
   }
   return r;
 }
-// real output value: v + beta out
+// real output value: alpha v + beta out
 __device__ __forceinline__ double out_value_real(const OzOut& o, double v, const double* p) {
+  if (o.alpha_kind != 1) v = o.alpha_kind == 2 ? -v : o.alpha.x * v;
   return o.beta_kind == 0 ? v : o.beta_kind == 1 ? v + *p : o.beta * (*p) + v;
 }
 
@@ -832,7 +833,8 @@ double oz_slab_bytes() {
 }
 
 double oz_min_macs() {
-  double v = 1e9;
+  // a complex multiply-add is four FP64 ones: 1.6e7 of them keep the FP64 pipe busy for 0.13 ms at best
+  double v = 1.6e7;
   if (const char* env = getenv("GFCC_OZ_MIN_MACS")) v = atof(env);
   return v;
 }
@@ -1010,7 +1012,7 @@ void oz_slice(const double* X, long long ldx, long long rows, long long K, bool 
 }
 
 void oz_gemm(const SlicedRows& A, const SlicedRows& B, long long M, long long N, double* out, long long ldo,
-             double beta, OzWork& w, cudaStream_t s) {
+             double beta, OzWork& w, cudaStream_t s, double alpha) {
   if (M <= 0 || N <= 0) return;
   GFCC_CHECK(!A.reversed && B.reversed && A.kp == B.kp && A.ns == B.ns, GFCC_ERR_ARG,
              "oz_gemm: operand slicing mismatch");
@@ -1019,6 +1021,7 @@ void oz_gemm(const SlicedRows& A, const SlicedRows& B, long long M, long long N,
   o.out = out;
   o.ldo = ldo;
   o.beta = beta;
+  o.alpha = make_cuDoubleComplex(alpha, 0.0);
   o.set_kinds();
   oz_run(A, B, M, N, o, w, s);
 }

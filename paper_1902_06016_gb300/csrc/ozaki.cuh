@@ -43,7 +43,7 @@ void oz_slice(const double* X, long long ldx, long long rows, long long K, bool 
 void oz_slice_into(const double* X, long long ldx, long long nrows, long long K, SlicedRows& out, long long row0,
                    cudaStream_t s);
 
-// out[m][n] = beta * out[m][n] + sum_k A[m][k] B[n][k] for m < M, n < N (out row stride ldo), with
+// out[m][n] = beta * out[m][n] + alpha * sum_k A[m][k] B[n][k] for m < M, n < N (out row stride ldo), with
 // A = sliced rows (normal order) and B = sliced rows (reversed order), same kp.
 struct OzWork {
   DBuf<int> islabs;   // int32 split sums of one diagonal of a column chunk
@@ -51,12 +51,12 @@ struct OzWork {
   DBuf<int> err;
 };
 void oz_gemm(const SlicedRows& A, const SlicedRows& B, long long M, long long N, double* out, long long ldo,
-             double beta, OzWork& w, cudaStream_t s);
+             double beta, OzWork& w, cudaStream_t s, double alpha = 1.0);
 
 // Complex GEMM C = alpha op(A) op(B) + beta C (strided, see ZGemmDesc) evaluated as one real
 // exact-slice GEMM: K interleaves (re, im) and the N axis stacks the real and imaginary parts.
 void zgemm_oz(const ZGemmDesc& g, int ns, cudaStream_t s);
-// multiply-adds above which zgemm() uses zgemm_oz (GFCC_OZ_MIN_MACS overrides)
+// complex multiply-adds above which zgemm() uses zgemm_oz (GFCC_OZ_MIN_MACS overrides)
 double oz_min_macs();
 // bytes of int32 split sums up to which all diagonals of an exact product are kept side by side and
 // summed into the output in one pass (default 4 GiB; GFCC_OZ_SLAB_BYTES overrides, so that tests can

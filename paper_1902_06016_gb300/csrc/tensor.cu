@@ -19,19 +19,73 @@ struct PermArgs {
   double alpha, beta;
 };
 
+__device__ __forceinline__ void perm_store(double* d, double v, double alpha, double beta) {
+  v *= alpha;
+  *d = (beta == 0.0) ? v : v + beta * *d;
+}
+// source offset of the leading n axes at linear index t (row-major over them), 32-bit arithmetic when it fits
+template <typename I>
+__device__ __forceinline__ long long perm_offset(const PermArgs& a, int n, long long t) {
+  I rem = (I)t;
+  long long off = 0;
+#pragma unroll
+  for (int k = 5; k >= 0; --k) {
+    if (k >= n) continue;
+    const I d = (I)a.dst_dims[k], q = rem / d;
+    off += (long long)(rem - q * d) * a.src_stride[k];
+    rem = q;
+  }
+  return off;
+}
+template <typename I>
 __global__ void permute_kernel(const double* __restrict__ src, double* __restrict__ dst, PermArgs a) {
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < a.total;
-       t += (long long)gridDim.x * blockDim.x) {
-    long long rem = t, off = 0;
-#pragma unroll
-    for (int k = 5; k >= 0; --k) {
-      if (k >= a.nd) continue;
-      long long c = rem % a.dst_dims[k];
-      rem /= a.dst_dims[k];
-      off += c * a.src_stride[k];
+       t += (long long)gridDim.x * blockDim.x)
+    perm_store(dst + t, src[perm_offset<I>(a, a.nd, t)], a.alpha, a.beta);
+}
+// The last axis is contiguous in both: a warp per row, the index arithmetic once per row instead of per element.
+__global__ void __launch_bounds__(256) permute_rows_kernel(const double* __restrict__ src, double* __restrict__ dst,
+                                                           PermArgs a) {
+  const int n = (int)a.dst_dims[a.nd - 1], lane = threadIdx.x & 31;
+  const long long rows = a.total / n;
+  for (long long r = (blockIdx.x * 256LL + threadIdx.x) >> 5; r < rows; r += gridDim.x * 8LL) {
+    const double* s = src + perm_offset<long long>(a, a.nd - 1, r);
+    double* d = dst + r * n;
+#pragma unroll 4
+    for (int k = lane; k < n; k += 32) perm_store(d + k, s[k], a.alpha, a.beta);
+  }
+}
+// The source's contiguous axis is dst axis q, not the last: 32 x 32 tiles of (q, last) through shared memory, so
+// that both sides move along their contiguous axis; the other axes are the batch (blocks walk the tiles).
+__global__ void __launch_bounds__(256) permute_tiles_kernel(const double* __restrict__ src, double* __restrict__ dst,
+                                                            PermArgs a, int q, long long tiles, int tq, int tn) {
+  __shared__ double tile[32][33];
+  const int nq = (int)a.dst_dims[q], n = (int)a.dst_dims[a.nd - 1];
+  const long long sn = a.src_stride[a.nd - 1];
+  long long dq = 1;   // dst stride of axis q
+  for (int k = q + 1; k < a.nd; ++k) dq *= a.dst_dims[k];
+  const int x = threadIdx.x & 31, y = threadIdx.x >> 5;
+  for (long long t = blockIdx.x; t < tiles; t += gridDim.x) {
+    long long rem = t / ((long long)tq * tn);
+    const int w = (int)(t - rem * tq * tn), q0 = w / tn * 32, n0 = w % tn * 32;
+    long long so = 0, doff = 0, dstr = n;
+    for (int k = a.nd - 2; k >= 0; --k) {   // the batch axes
+      if (k != q) {
+        const long long d = a.dst_dims[k], i = rem % d;
+        rem /= d;
+        so += i * a.src_stride[k];
+        doff += i * dstr;
+      }
+      dstr *= a.dst_dims[k];
     }
-    double v = a.alpha * src[off];
-    dst[t] = (a.beta == 0.0) ? v : v + a.beta * dst[t];
+#pragma unroll
+    for (int h = 0; h < 4; ++h)
+      if (const int r = y + 8 * h; q0 + x < nq && n0 + r < n) tile[r][x] = src[so + (q0 + x) + (long long)(n0 + r) * sn];
+    __syncthreads();
+#pragma unroll
+    for (int h = 0; h < 4; ++h)
+      if (const int r = y + 8 * h; q0 + r < nq && n0 + x < n) perm_store(dst + doff + (q0 + r) * dq + n0 + x, tile[x][r], a.alpha, a.beta);
+    __syncthreads();
   }
 }
 
@@ -66,7 +120,47 @@ void permute(const double* src, const int* dims, int nd, const int* perm, double
   a.alpha = alpha;
   a.beta = beta;
   if (a.total == 0) return;
-  permute_kernel<<<grid_for(a.total), 256, 0, s>>>(src, dst, a);
+  // axes that stay neighbours are one axis
+  for (int k = 0; k + 1 < a.nd;) {
+    if (a.dst_dims[k + 1] == 1 || a.dst_dims[k] == 1 || a.src_stride[k] == a.dst_dims[k + 1] * a.src_stride[k + 1]) {
+      const bool keep = a.dst_dims[k + 1] == 1;   // a unit axis disappears, whichever side it is on
+      const long long st = keep ? a.src_stride[k] : a.src_stride[k + 1];
+      a.dst_dims[k] *= a.dst_dims[k + 1];
+      a.src_stride[k] = st;
+      for (int j = k + 1; j + 1 < a.nd; ++j) {
+        a.dst_dims[j] = a.dst_dims[j + 1];
+        a.src_stride[j] = a.src_stride[j + 1];
+      }
+      --a.nd;
+    } else {
+      ++k;
+    }
+  }
+  // Rows and tiles read and write whole lines with an index computation per row or tile; the element-wise kernel
+  // computes one per element (61 M elements of a 4-index tensor: 283 us; they are 150 us of HBM time).
+  const int last = a.nd - 1;
+  int q = -1;
+  for (int k = 0; k < a.nd; ++k)
+    if (a.src_stride[k] == 1 && a.dst_dims[k] > 1) q = k;
+  constexpr long long kInt = 0x7fffffffLL;
+  if (a.nd == 1 && a.src_stride[0] == 1) {   // a copy
+    axpby(a.total, alpha, src, beta, dst, s);
+    return;
+  }
+  if (q == last && a.dst_dims[last] >= 32 && a.dst_dims[last] <= kInt && a.total / a.dst_dims[last] >= 2048) {
+    const long long rows = a.total / a.dst_dims[last];
+    permute_rows_kernel<<<(unsigned)std::min<long long>((rows + 7) / 8, 152LL * 32), 256, 0, s>>>(src, dst, a);
+  } else if (q >= 0 && q < last && a.dst_dims[q] >= 8 && a.dst_dims[last] >= 8 && a.dst_dims[q] <= kInt &&
+             a.dst_dims[last] <= kInt) {
+    const long long tq = (a.dst_dims[q] + 31) / 32, tn = (a.dst_dims[last] + 31) / 32;
+    const long long tiles = a.total / (a.dst_dims[q] * a.dst_dims[last]) * tq * tn;
+    permute_tiles_kernel<<<(unsigned)std::min<long long>(tiles, 152LL * 16), 256, 0, s>>>(src, dst, a, q, tiles, (int)tq,
+                                                                                         (int)tn);
+  } else if (a.total < (1LL << 32)) {
+    permute_kernel<unsigned><<<grid_for(a.total), 256, 0, s>>>(src, dst, a);
+  } else {
+    permute_kernel<unsigned long long><<<grid_for(a.total), 256, 0, s>>>(src, dst, a);
+  }
   GFCC_LAUNCH_CHECK();
 }
 
@@ -136,8 +230,10 @@ void contract(double alpha, const TV& A, const TV& B, double beta, const TV& C, 
   std::string lt0 = Ml + Nl;
   std::vector<int> pc0 = perm_of(lt0, lc);
   // contractions above this many multiply-adds use the tensor cores (GFCC_OZ_MIN_MACS overrides it,
-  // which the tests use to exercise this path at small sizes)
-  double min_macs = 5e8;
+  // which the tests use to exercise this path at small sizes). The FP64 pipe does 5e11 of them a second at best and
+  // about half that in 64 x 64 tiles, so 3e7 take it 0.1 ms, about what the eight launches of the exact form
+  // take; its 62 bits per row leave less error than FP64 sums.
+  double min_macs = 3e7;
   if (const char* env = getenv("GFCC_OZ_MIN_MACS")) min_macs = atof(env);
   if ((double)M * (double)N * (double)K >= min_macs && M >= 16 && N >= 16) {
     // FP64-accurate GEMM from exact f16 slices on the tensor cores (7 slices: FP64-level accuracy)
@@ -160,12 +256,16 @@ void contract(double alpha, const TV& A, const TV& B, double beta, const TV& C, 
     oz_slice(Bop2, K, N, K, true, sb, s, OZ_SLICES_MAX);
     Ap.release();
     Bp.release();
-    Cp.alloc(M * N);
     OzWork w;
-    oz_gemm(sa, sb, M, N, Cp.p, N, 0.0, w, s);
-    std::vector<int> dt;
-    for (char ch : lt0) dt.push_back(size[ch]);
-    permute(Cp.p, dt.data(), (int)dt.size(), pc0.data(), C.p, alpha, beta, s);
+    if (identity(pc0)) {   // straight into C
+      oz_gemm(sa, sb, M, N, C.p, N, beta, w, s, alpha);
+    } else {
+      Cp.alloc(M * N);
+      oz_gemm(sa, sb, M, N, Cp.p, N, 0.0, w, s);
+      std::vector<int> dt;
+      for (char ch : lt0) dt.push_back(size[ch]);
+      permute(Cp.p, dt.data(), (int)dt.size(), pc0.data(), C.p, alpha, beta, s);
+    }
     int herr = 0;
     GFCC_CUDA(cudaMemcpyAsync(&herr, w.err.p, sizeof(int), cudaMemcpyDeviceToHost, s));
     GFCC_CUDA(cudaStreamSynchronize(s));
