@@ -646,6 +646,14 @@ int gfcc_sigma(gfcc_t c, const double* X, double* Y, int nvec, int ld, int preci
   const long long D = c->D;
   if ((precision == GFCC_PREC_TF32 || precision == GFCC_PREC_BF16) && c->lp.kind != precision)
     gfcc::build_low_precision(c, precision);
+  const double *x1 = X + 2LL * nvec * ld, *y1 = Y + 2LL * nvec * ld;
+  if (gfcc::sigma_is_dense(c, precision) && (x1 <= Y || y1 <= X) && is_device_ptr(X) && is_device_ptr(Y)) {
+    // one launch on the caller's buffers (which must not overlap: elsewhere they are copied first)
+    gfcc::sigma_dense(c, reinterpret_cast<const cplx*>(X), reinterpret_cast<cplx*>(Y), nvec, 1, ld, nullptr,
+                      transpose != 0, s);
+    GFCC_CUDA(cudaStreamSynchronize(s));
+    return GFCC_OK;
+  }
   const int nbmax = std::max(1, std::min(nvec, c->opts.max_batch > 0 ? c->opts.max_batch : 256));
   DBuf<cplx> stage, Xb, Yb;
   stage.alloc((long long)nbmax * ld);

@@ -183,6 +183,7 @@ struct Operator {
   DBuf<double> diag;   // [D] Fock-diagonal part: -F_ii (1h), F_aa - F_ii - F_jj (2h1p)
   DBuf<double> mdiag;  // [D] full diagonal of M (Jacobi preconditioner)
   DBuf<float4> rowf;   // mdiag as pairs of FP32 numbers, and diag in FP32 (built with the first FP32-basis solve)
+  DBuf<double> Mdense; // [D][D] M itself, for small operators (built with the first FP64 sigma)
   // transposed-action copies are built lazily (adjoint systems)
   bool have_T = false;
   DBuf<double> WrT, WooT, A12T, A21T, VtT, T2pT;
@@ -378,6 +379,10 @@ void build_operator_ea(gfcc_ctx* c, const HostInputs& in);
 // leading dimension ldb (complex elements per row). shift may be null.
 void sigma_batch(gfcc_ctx* c, const cplx* X, cplx* Y, int nb, int ldb, const cplx* shift,
                  int precision, bool transpose, cudaStream_t s);
+// small operators: the FP64 sigma as one dense product, element (nu, c) of X and Y at nu sk + c sc
+bool sigma_is_dense(const gfcc_ctx* c, int precision);
+void sigma_dense(gfcc_ctx* c, const cplx* X, cplx* Y, int nb, long long sk, long long sc, const cplx* shift,
+                 bool transpose, cudaStream_t s);
 void ensure_workspace(gfcc_ctx* c, int nb);
 void build_transpose_operator(gfcc_ctx* c);
 

@@ -309,7 +309,9 @@ long long cgs_rows(long long D, int nb) {
   const long long gx = (nb + MD_TX - 1) / MD_TX, slots = 152LL * 2;
   long long nchunk = std::max<long long>(256, 2 * slots / gx);
   nchunk = std::max<long long>(1, (nchunk * gx + slots - 1) / slots * slots / gx);
-  return std::max<long long>(64, (D + nchunk - 1) / nchunk);
+  // short vectors: chunks of 16 rows rather than leave SMs without a block (D = 52, 1024 columns: one chunk of 64
+  // rows was 32 blocks)
+  return std::max<long long>(D < 4096 ? 16 : 64, (D + nchunk - 1) / nchunk);
 }
 
 // h[c*hld + hoff + i] = sum_chunk partial[chunk][i][c], also set in or added to the Hessenberg column Hc (entry

@@ -85,7 +85,93 @@ __global__ void combine_kernel(const cplx* __restrict__ X, cplx* __restrict__ Y,
   }
 }
 
+// ---- small operators: M as a dense matrix ----------------------------------------------------------
+// dst[nu D + k] = Re Y[nu][k] of the identity's image
+__global__ void dense_take_kernel(const cplx* __restrict__ Y, long long n, double* __restrict__ dst) {
+  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n; t += (long long)gridDim.x * blockDim.x)
+    dst[t] = Y[t].x;
+}
+__global__ void identity_kernel(cplx* __restrict__ X, int D) {
+  const long long n = (long long)D * D;
+  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n; t += (long long)gridDim.x * blockDim.x)
+    X[t] = make_cuDoubleComplex(t / D == t % D ? 1.0 : 0.0, 0.0);
+}
+// Y(nu, c) = sum_k M(nu, k) X(k, c) + shift[c] X(nu, c), X(k, c) at X[k sk + c sc] and Y alike; M(nu, k) at
+// M[nu mn + k mk]. KS neighbouring lanes share an output (k strided over them). No tiling: an FP64 instruction
+// holds a scheduler for 75 clocks, in which the loads of the next elements come from L1.
+template <int KS>
+__global__ void __launch_bounds__(128) dense_sigma_kernel(const double* __restrict__ M, int mn, int mk,
+                                                          const cplx* __restrict__ X, cplx* __restrict__ Y,
+                                                          long long sk, long long sc, const cplx* __restrict__ shift,
+                                                          int D, int nb) {
+  const long long t = (blockIdx.x * 128LL + threadIdx.x) / KS;
+  const int ks = threadIdx.x % KS;
+  const bool on = t < (long long)D * nb;
+  const int nu = on ? (int)(t / nb) : 0, c = on ? (int)(t - (long long)nu * nb) : 0;
+  const double* m = M + (long long)nu * mn;
+  const cplx* x = X + (long long)c * sc;
+  double re = 0.0, im = 0.0;
+  if (on) {
+#pragma unroll 4
+    for (int k = ks; k < D; k += KS) {
+      const double a = m[(long long)k * mk];
+      const cplx v = x[k * sk];
+      re = fma(a, v.x, re);
+      im = fma(a, v.y, im);
+    }
+  }
+#pragma unroll
+  for (int w = KS / 2; w > 0; w >>= 1) {
+    re += __shfl_down_sync(0xffffffffu, re, w, KS);
+    im += __shfl_down_sync(0xffffffffu, im, w, KS);
+  }
+  if (!on || ks != 0) return;
+  if (shift) {
+    const cplx s = shift[c], v = x[nu * sk];
+    re += s.x * v.x - s.y * v.y;
+    im += s.x * v.y + s.y * v.x;
+  }
+  Y[nu * sk + c * sc] = make_cuDoubleComplex(re, im);
+}
+
 }  // namespace
+
+// Up to this dimension the FP64 sigma runs on M as a dense matrix: 2 D^2 FP64 multiply-adds a column, about what the
+// structured products take there (D = 52: 5,400 against 11,000; D = 216: 93,000 against 110,000), in one launch
+// instead of twelve whose 64 x 64 tiles are mostly empty (D = 52, 1024 columns: 250 us -> 17).
+constexpr int DENSE_MAX_D = 256;
+bool sigma_is_dense(const gfcc_ctx* c, int precision) { return precision == GFCC_PREC_FP64 && c->D <= DENSE_MAX_D; }
+
+static void sigma_structured(gfcc_ctx* c, const cplx* X, cplx* Y, int nb, const cplx* shift, bool transpose,
+                             cudaStream_t s);
+
+void sigma_dense(gfcc_ctx* c, const cplx* X, cplx* Y, int nb, long long sk, long long sc, const cplx* shift,
+                 bool transpose, cudaStream_t s) {
+  const int D = c->D;
+  if (!c->op.Mdense.p) {   // the images of the unit vectors, once per context
+    const long long n = (long long)D * D;
+    DBuf<cplx> X1, Y1;
+    DBuf<double> M;
+    X1.alloc(n);
+    Y1.alloc(n);
+    M.alloc(n);
+    identity_kernel<<<grid_for(n), 256, 0, s>>>(X1.p, D);
+    GFCC_LAUNCH_CHECK();
+    sigma_structured(c, X1.p, Y1.p, D, nullptr, false, s);
+    dense_take_kernel<<<grid_for(n), 256, 0, s>>>(Y1.p, n, M.p);
+    GFCC_LAUNCH_CHECK();
+    c->op.Mdense = std::move(M);
+  }
+  const double* M = c->op.Mdense.p;
+  const int mn = transpose ? 1 : D, mk = transpose ? D : 1;
+  const long long n = (long long)D * nb;
+  // eight lanes per output when the outputs alone would leave schedulers without a warp
+  if (n >= 152LL * 4 * 32) dense_sigma_kernel<1><<<(unsigned)((n + 127) / 128), 128, 0, s>>>(M, mn, mk, X, Y, sk, sc, shift, D, nb);
+  else dense_sigma_kernel<8><<<(unsigned)((n * 8 + 127) / 128), 128, 0, s>>>(M, mn, mk, X, Y, sk, sc, shift, D, nb);
+  GFCC_LAUNCH_CHECK();
+  c->stats.sigma_calls++;
+  c->stats.sigma_cols += nb;
+}
 
 void ensure_workspace(gfcc_ctx* c, int nb) {
   if ((size_t)nb <= c->ws.nb_cap) return;
@@ -128,6 +214,17 @@ void sigma_batch(gfcc_ctx* c, const cplx* X, cplx* Y, int nb, int ldb, const cpl
     sigma_lowprec(c, X, Y, nb, shift, s, transpose);
     return;
   }
+  if (sigma_is_dense(c, precision)) {
+    sigma_dense(c, X, Y, nb, nb, 1, shift, transpose, s);
+    return;
+  }
+  sigma_structured(c, X, Y, nb, shift, transpose, s);
+  c->stats.sigma_calls++;
+  c->stats.sigma_cols += nb;
+}
+
+static void sigma_structured(gfcc_ctx* c, const cplx* X, cplx* Y, int nb, const cplx* shift, bool transpose,
+                             cudaStream_t s) {
   const int o = c->o, v = c->v, P = c->P;
   const long long D = c->D, Pv = (long long)P * v, ov = (long long)o * v;
   Operator& op = c->op;
@@ -187,8 +284,6 @@ void sigma_batch(gfcc_ctx* c, const cplx* X, cplx* Y, int nb, int ldb, const cpl
   }
   combine_kernel<<<grid_for(D * nb), 256, 0, s>>>(X, Y, CT, op.diag.p, shift, o, v, D, nb);
   GFCC_LAUNCH_CHECK();
-  c->stats.sigma_calls++;
-  c->stats.sigma_cols += nb;
 }
 
 // M^T: 1h-1h A11^T (read transposed), 1h<-2h1p = A21^T, 2h1p<-1h = A12^T, oooo Woo^T,
