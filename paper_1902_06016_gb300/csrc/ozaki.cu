@@ -287,22 +287,41 @@ __device__ __forceinline__ double scale_pow2(double x, int k) {
   if (k >= -1022 && k <= 1023) return x * __longlong_as_double((long long)(k + 1023) << 52);
   return ldexp(x, k);
 }
-// sum_d S_d 2^(9 (nd - 1 - d)) for nd <= 7 per-diagonal integer sums |S_d| < 2^43: up to three diagonals at a
-// time are combined exactly in a 64-bit integer (below 2^62) and the two or three integers joined by fused
-// multiply-adds, instead of an FP64 conversion and multiply-add per diagonal (FP64 is the scarce pipe on this
-// GPU: the output passes were bound by it). The caller scales by 2^(-9 (nd - 1)).
-__device__ __forceinline__ double pow2(int k) { return __longlong_as_double((long long)(k + 1023) << 52); }
-__device__ __forceinline__ double diag_combine(const long long* S, int nd) {
-  const int H = nd < 3 ? nd : 3, L = nd < 6 ? nd : 6;   // diagonals [0, H), [H, L), [L, nd)
+// 2^e sum_d S_d 2^(9 (NS - 1 - d)) for NS <= 7 per-diagonal integer sums |S_d| < 2^43, rounded once to nearest: the sum
+// is formed exactly (three diagonals at a time in 64 bits, joined in 128) and the double assembled from its bits.
+// Integer instructions throughout: the FP64 form (two conversions, a fused multiply-add, a scaling) held each
+// scheduler for 300 clocks per warp and bound the output passes.
+template <int NS>
+__device__ __forceinline__ double diag_value(const long long (&S)[NS], int e) {
+  constexpr int H = NS < 3 ? NS : 3, L = NS < 6 ? NS : 6;   // diagonals [0, H), [H, L), [L, NS)
   long long hi = 0, mid = 0, lo = 0;
 #pragma unroll
-  for (int d = 0; d < OZ_SLICES_MAX; ++d) {
+  for (int d = 0; d < NS; ++d) {
     if (d < H) hi += S[d] * (1LL << (OZ_BITS * (H - 1 - d)));
     else if (d < L) mid += S[d] * (1LL << (OZ_BITS * (L - 1 - d)));
-    else if (d < nd) lo += S[d];
+    else lo += S[d];
   }
-  if (nd <= 6) return fma((double)hi, pow2(OZ_BITS * (nd - H)), (double)mid);
-  return fma((double)hi, pow2(OZ_BITS * (nd - H)), fma((double)mid, pow2(OZ_BITS * (nd - L)), (double)lo));
+  const __int128 T = (__int128)hi * ((__int128)1 << (OZ_BITS * (NS - H))) + (__int128)mid * ((__int128)1 << (OZ_BITS * (NS - L))) + lo;
+  if (T == 0) return 0.0;
+  const bool neg = T < 0;
+  const unsigned __int128 A = neg ? -(unsigned __int128)T : (unsigned __int128)T;
+  const unsigned long long ah = (unsigned long long)(A >> 64), al = (unsigned long long)A;
+  const int n = ah ? 128 - __clzll((long long)ah) : 64 - __clzll((long long)al);   // bits
+  // the top 64 bits, left-aligned, and whether anything is left below them
+  const int sh = 128 - n;
+  const unsigned __int128 B = A << sh;
+  const unsigned long long top = (unsigned long long)(B >> 64);
+  const bool rest = (unsigned long long)B != 0;
+  unsigned long long m = top >> 11;                       // 53 bits
+  const unsigned long long low = top & 0x7FFULL;          // and 11 more
+  if (low > 0x400ULL || (low == 0x400ULL && (rest || (m & 1)))) ++m;   // to nearest, ties to even
+  const int E = n - 1 + e + 1023 + (int)(m >> 53);        // a carry out of the mantissa leaves m = 2^53
+  if (E < 1 || E > 2046) {                                // subnormal or overflowing: by the library
+    const double v = ldexp((double)m, n - 53 + e);
+    return neg ? -v : v;
+  }
+  const unsigned long long bits = ((unsigned long long)E << 52) | (m & 0xFFFFFFFFFFFFFULL);
+  return __longlong_as_double((long long)(neg ? bits | 0x8000000000000000ULL : bits));
 }
 // complex output value: alpha (re + i im) + beta C
 __device__ __forceinline__ cplx out_value(const OzOut& o, double re, double im, const cplx* p) {
@@ -406,214 +425,135 @@ __global__ void __launch_bounds__(256) oz_accumulate_kernel(const int* __restric
     }
   }
 }
-// All diagonals at once (their split sums held side by side: diagonal d at slabs + off[d], zs[d]
-// splits of stride M Np each), summed and written to the output in one pass (MODE 1 real, 2 complex).
-struct OzDiags {
-  long long off[OZ_SLICES_MAX];
-  int zs[OZ_SLICES_MAX];
-  int nd;
-};
-// sum_d 2^(-9d) (split sums of diagonal d), times 2^(9 (nd - 1)) (see diag_combine)
-template <bool WARP>
-__device__ __forceinline__ double diag_total(const int* __restrict__ slabs, const OzDiags& dg, long long stride,
-                                             long long t, int lane) {
-  long long S[OZ_SLICES_MAX];
-#pragma unroll
-  for (int d = 0; d < OZ_SLICES_MAX; ++d)
-    S[d] = d < dg.nd ? split_sum<WARP>(slabs + dg.off[d] + t, dg.zs[d], stride, lane) : 0;
-  return diag_combine(S, dg.nd);
-}
-template <bool WARP, int MODE, typename I>
-__global__ void __launch_bounds__(256) oz_output_kernel(const int* __restrict__ slabs, OzDiags dg, long long M,
-                                                        long long Np, const int* __restrict__ ea,
-                                                        const int* __restrict__ eb, OzOut o) {
-  const long long stride = M * Np;
-  const long long total = MODE == 2 ? M * (Np / 2) : stride;
-  const int lane = threadIdx.x & 31;
-  const bool writer = !WARP || lane == 0;
-  const long long gid = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  const long long nthreads = (long long)gridDim.x * blockDim.x;
-  const long long start = WARP ? gid >> 5 : gid, step = WARP ? nthreads >> 5 : nthreads;
-  for (long long t = start; t < total; t += step) {
-    if constexpr (MODE == 1) {
-      long long m, n;
-      divmod<I>(t, Np, m, n);
-      const double v = scale_pow2(diag_total<WARP>(slabs, dg, stride, t, lane), ea[m] + eb[n] - 2 * OZ_TOP - OZ_BITS * (dg.nd - 1));
-      if (writer) {
-        double* p = o.out + m * o.ldo + n;
-        *p = out_value_real(o, v, p);
-      }
-    } else {
-      const long long N = Np / 2;
-      long long m, n;
-      divmod<I>(t, N, m, n);
-      const long long tr = m * Np + n;
-      const int sh = -2 * OZ_TOP - OZ_BITS * (dg.nd - 1);
-      const double re = scale_pow2(diag_total<WARP>(slabs, dg, stride, tr, lane), ea[m] + eb[n] + sh);
-      const double im = scale_pow2(diag_total<WARP>(slabs, dg, stride, tr + N, lane), ea[m] + eb[N + n] + sh);
-      if (writer) {
-        cplx* p = o.C + m * o.scm + n * o.scn;
-        *p = out_value(o, re, im, p);
-      }
-    }
-  }
-}
-// The common case of one split per diagonal (a short K): the NS loads of an element are issued
-// together, so that each thread keeps NS (complex: 2 NS) independent loads in flight.
-template <int NS, int MODE, typename I>
-__global__ void __launch_bounds__(256) oz_output1_kernel(const int* __restrict__ slabs, OzDiags dg, long long M,
-                                                         long long Np, const int* __restrict__ ea,
-                                                         const int* __restrict__ eb, OzOut o) {
-  const long long stride = M * Np;
-  const long long total = MODE == 2 ? M * (Np / 2) : stride;
-  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total;
-       t += (long long)gridDim.x * blockDim.x) {
-    if constexpr (MODE == 1) {
-      long long v[OZ_SLICES_MAX] = {};
-#pragma unroll
-      for (int d = 0; d < NS; ++d) v[d] = slabs[dg.off[d] + t];
-      long long m, n;
-      divmod<I>(t, Np, m, n);
-      const double r = scale_pow2(diag_combine(v, NS), ea[m] + eb[n] - 2 * OZ_TOP - OZ_BITS * (NS - 1));
-      double* p = o.out + m * o.ldo + n;
-      *p = out_value_real(o, r, p);
-    } else {
-      const long long N = Np / 2;
-      long long m, n;
-      divmod<I>(t, N, m, n);
-      const long long tr = m * Np + n, ti = tr + N;
-      long long vr[OZ_SLICES_MAX] = {}, vi[OZ_SLICES_MAX] = {};
-#pragma unroll
-      for (int d = 0; d < NS; ++d) {
-        vr[d] = slabs[dg.off[d] + tr];
-        vi[d] = slabs[dg.off[d] + ti];
-      }
-      const int sh = -2 * OZ_TOP - OZ_BITS * (NS - 1);
-      const double re = scale_pow2(diag_combine(vr, NS), ea[m] + eb[n] + sh);
-      const double im = scale_pow2(diag_combine(vi, NS), ea[m] + eb[N + n] + sh);
-      cplx* p = o.C + m * o.scm + n * o.scn;
-      *p = out_value(o, re, im, p);
-    }
-  }
-}
-template <int MODE, typename I>
-void launch_output1(int ns, int grid, cudaStream_t s, const int* slabs, const OzDiags& dg, long long M, long long Np,
-                    const int* ea, const int* eb, const OzOut& o) {
-  switch (ns) {
-    case 2: oz_output1_kernel<2, MODE, I><<<grid, 256, 0, s>>>(slabs, dg, M, Np, ea, eb, o); break;
-    case 3: oz_output1_kernel<3, MODE, I><<<grid, 256, 0, s>>>(slabs, dg, M, Np, ea, eb, o); break;
-    case 4: oz_output1_kernel<4, MODE, I><<<grid, 256, 0, s>>>(slabs, dg, M, Np, ea, eb, o); break;
-    case 5: oz_output1_kernel<5, MODE, I><<<grid, 256, 0, s>>>(slabs, dg, M, Np, ea, eb, o); break;
-    case 6: oz_output1_kernel<6, MODE, I><<<grid, 256, 0, s>>>(slabs, dg, M, Np, ea, eb, o); break;
-    default: oz_output1_kernel<7, MODE, I><<<grid, 256, 0, s>>>(slabs, dg, M, Np, ea, eb, o); break;
-  }
-}
-
-template <bool WARP, int MODE>
-void launch_output(bool small, int grid, cudaStream_t s, const int* slabs, const OzDiags& dg, long long M,
-                   long long Np, const int* ea, const int* eb, const OzOut& o) {
-  if (small) oz_output_kernel<WARP, MODE, unsigned><<<grid, 256, 0, s>>>(slabs, dg, M, Np, ea, eb, o);
-  else oz_output_kernel<WARP, MODE, unsigned long long><<<grid, 256, 0, s>>>(slabs, dg, M, Np, ea, eb, o);
-}
-
-// ---- stacked form for a narrow right operand --------------------------------------------------------
-// When B has few rows and A is large, one GEMM per A slice i multiplies it by B slices 0..ns-1-i
-// stacked as rows (B sliced slot-major), so that A is read ns times instead of ns(ns+1)/2 times and the
-// narrow B fills more of each tile. Partials of slice i: slabs + off[i], [zs[i]][M][ncol[i]] with
-// ncol[i] = (ns - i) Np, B slice j in columns [j Np, (j + 1) Np). Diagonal d = i + j is summed exactly
-// in 64-bit integers before the FP64 weighting, so the result equals the diagonal-by-diagonal one.
-struct OzStack {
+// All diagonals at once: their split sums held side by side, summed and written to the output in one pass.
+// The partial sums of a real column col of row m, diagonal d, are those of the pieces i (one per diagonal in the plain
+// form: i = d; in the stacked form, below, the products i = 0..d): piece i starts at off[i], has rows of ncol[i], zs[i]
+// splits, and holds the value at column (STACK ? (d - i) Np : 0) + col.
+struct OzParts {
   long long off[OZ_SLICES_MAX];
   long long ncol[OZ_SLICES_MAX];
   int zs[OZ_SLICES_MAX];
-  int ns;
 };
-template <bool WARP>
-__device__ __forceinline__ double stack_total(const int* __restrict__ slabs, const OzStack& st, long long M,
-                                              long long Np, long long m, long long col, int lane) {
-  long long S[OZ_SLICES_MAX];
+template <int NS, bool STACK>
+__device__ __forceinline__ void diag_sums(const int* __restrict__ slabs, const OzParts& q, long long M, long long Np,
+                                          long long m, long long col, int z0, int zstep, long long (&S)[NS]) {
 #pragma unroll
-  for (int d = 0; d < OZ_SLICES_MAX; ++d) {
-    S[d] = 0;
-    if (d < st.ns)
-      for (int i = 0; i <= d; ++i)
-        S[d] += split_sum<WARP>(slabs + st.off[i] + m * st.ncol[i] + (d - i) * Np + col, st.zs[i], M * st.ncol[i], lane);
+  for (int d = 0; d < NS; ++d) S[d] = 0;
+  if (z0 == 0) {   // the first split of every piece, all loads in flight together
+#pragma unroll
+    for (int d = 0; d < NS; ++d) {
+#pragma unroll
+      for (int i = STACK ? 0 : d; i <= d; ++i) S[d] += slabs[q.off[i] + m * q.ncol[i] + (STACK ? (d - i) * Np : 0) + col];
+    }
   }
-  return diag_combine(S, st.ns);   // times 2^(9 (ns - 1))
-}
-// complex output C(m, n) = alpha (re + i im) + beta C (real columns n and N + n of the Np = 2N)
-template <bool WARP, typename I>
-__global__ void __launch_bounds__(256) oz_stack_output_kernel(const int* __restrict__ slabs, OzStack st, long long M,
-                                                              long long Np, const int* __restrict__ ea,
-                                                              const int* __restrict__ eb, OzOut o) {
-  const long long N = Np / 2, total = M * N;
-  const int lane = threadIdx.x & 31;
-  const long long gid = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  const long long nthreads = (long long)gridDim.x * blockDim.x;
-  const long long start = WARP ? gid >> 5 : gid, step = WARP ? nthreads >> 5 : nthreads;
-  for (long long t = start; t < total; t += step) {
-    long long m, n;
-    divmod<I>(t, N, m, n);
-    const int sh = -2 * OZ_TOP - OZ_BITS * (st.ns - 1);
-    const double re = scale_pow2(stack_total<WARP>(slabs, st, M, Np, m, n, lane), ea[m] + eb[n] + sh);
-    const double im = scale_pow2(stack_total<WARP>(slabs, st, M, Np, m, N + n, lane), ea[m] + eb[N + n] + sh);
-    if (!WARP || lane == 0) {
-      cplx* p = o.C + m * o.scm + n * o.scn;
-      *p = out_value(o, re, im, p);
+#pragma unroll
+  for (int d = 0; d < NS; ++d) {
+#pragma unroll
+    for (int i = STACK ? 0 : d; i <= d; ++i) {
+      const long long stride = M * q.ncol[i];
+      const int* p = slabs + q.off[i] + m * q.ncol[i] + (STACK ? (d - i) * Np : 0) + col;
+#pragma unroll 4
+      for (int z = z0 == 0 ? zstep : z0; z < q.zs[i]; z += zstep) S[d] += p[z * stride];
     }
   }
 }
-// one split per slice product: all NS (NS + 1) / 2 loads of each part issued together
-template <int NS, typename I>
-__global__ void __launch_bounds__(256) oz_stack_output1_kernel(const int* __restrict__ slabs, OzStack st, long long M,
-                                                               long long Np, const int* __restrict__ ea,
-                                                               const int* __restrict__ eb, OzOut o) {
-  constexpr int NQ = NS * (NS + 1) / 2;
-  const long long N = Np / 2, total = M * N;
+// One thread per output element (complex: both parts).
+template <int NS, bool STACK, bool CPLX, typename I>
+__global__ void __launch_bounds__(256) oz_output_kernel(const int* __restrict__ slabs, OzParts q, long long M,
+                                                        long long Np, const int* __restrict__ ea,
+                                                        const int* __restrict__ eb, OzOut o) {
+  const long long N = CPLX ? Np / 2 : Np, total = M * N;
+  constexpr int sh = -2 * OZ_TOP - OZ_BITS * (NS - 1);
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total;
        t += (long long)gridDim.x * blockDim.x) {
     long long m, n;
     divmod<I>(t, N, m, n);
-    int vr[NQ], vi[NQ];
-#pragma unroll
-    for (int d = 0, q = 0; d < NS; ++d)
-#pragma unroll
-      for (int i = 0; i <= d; ++i, ++q) {
-        const int* p = slabs + st.off[i] + m * st.ncol[i] + (d - i) * Np + n;
-        vr[q] = p[0];
-        vi[q] = p[N];
-      }
-    long long sr[OZ_SLICES_MAX] = {}, si[OZ_SLICES_MAX] = {};
-#pragma unroll
-    for (int d = 0, q = 0; d < NS; ++d) {
-#pragma unroll
-      for (int i = 0; i <= d; ++i, ++q) {
-        sr[d] += vr[q];
-        si[d] += vi[q];
-      }
-    }
-    const int sh = -2 * OZ_TOP - OZ_BITS * (NS - 1);
-    const double re = scale_pow2(diag_combine(sr, NS), ea[m] + eb[n] + sh);
-    const double im = scale_pow2(diag_combine(si, NS), ea[m] + eb[N + n] + sh);
-    cplx* p = o.C + m * o.scm + n * o.scn;
-    *p = out_value(o, re, im, p);
-  }
-}
-template <typename I>
-void launch_stack_output(int ns, bool one_split, bool warp, int grid, cudaStream_t s, const int* slabs,
-                         const OzStack& st, long long M, long long Np, const int* ea, const int* eb, const OzOut& o) {
-  if (one_split) {
-    switch (ns) {
-      case 4: oz_stack_output1_kernel<4, I><<<grid, 256, 0, s>>>(slabs, st, M, Np, ea, eb, o); return;
-      case 5: oz_stack_output1_kernel<5, I><<<grid, 256, 0, s>>>(slabs, st, M, Np, ea, eb, o); return;
-      case 6: oz_stack_output1_kernel<6, I><<<grid, 256, 0, s>>>(slabs, st, M, Np, ea, eb, o); return;
-      case 7: oz_stack_output1_kernel<7, I><<<grid, 256, 0, s>>>(slabs, st, M, Np, ea, eb, o); return;
-      default: break;
+    long long S[NS];
+    diag_sums<NS, STACK>(slabs, q, M, Np, m, n, 0, 1, S);
+    const double re = diag_value<NS>(S, ea[m] + eb[n] + sh);
+    if constexpr (CPLX) {
+      diag_sums<NS, STACK>(slabs, q, M, Np, m, N + n, 0, 1, S);
+      const double im = diag_value<NS>(S, ea[m] + eb[N + n] + sh);
+      cplx* p = o.C + m * o.scm + n * o.scn;
+      *p = out_value(o, re, im, p);
+    } else {
+      double* p = o.out + m * o.ldo + n;
+      *p = out_value_real(o, re, p);
     }
   }
-  if (warp) oz_stack_output_kernel<true, I><<<grid, 256, 0, s>>>(slabs, st, M, Np, ea, eb, o);
-  else oz_stack_output_kernel<false, I><<<grid, 256, 0, s>>>(slabs, st, M, Np, ea, eb, o);
 }
+// Outputs too small to occupy the GPU that have many K splits: 32 elements per block (coalesced along the row), whose
+// splits the eight warps share (a warp per element read one 4-byte sum per 32-byte sector: 87 us for a 270 x 32 product
+// with 100 splits).
+template <int NS, bool STACK, bool CPLX>
+__global__ void __launch_bounds__(256) oz_output_split_kernel(const int* __restrict__ slabs, OzParts q, long long M,
+                                                              long long Np, const int* __restrict__ ea,
+                                                              const int* __restrict__ eb, OzOut o) {
+  __shared__ long long red[8][NS][32];
+  __shared__ double val[2][32];
+  const long long N = CPLX ? Np / 2 : Np, total = M * N;
+  constexpr int sh = -2 * OZ_TOP - OZ_BITS * (NS - 1);
+  const int x = threadIdx.x & 31, y = threadIdx.x >> 5;
+  for (long long t0 = blockIdx.x * 32LL; t0 < total; t0 += gridDim.x * 32LL) {
+    const long long t = t0 + x, m = t / N, n = t - m * N;
+    const bool on = t < total;
+#pragma unroll
+    for (int part = 0; part < (CPLX ? 2 : 1); ++part) {
+      const long long col = part ? N + n : n;
+      long long S[NS];
+      if (on) diag_sums<NS, STACK>(slabs, q, M, Np, m, col, y, 8, S);
+#pragma unroll
+      for (int d = 0; d < NS; ++d) red[y][d][x] = on ? S[d] : 0;
+      __syncthreads();
+      if (y < NS) {
+        long long s = 0;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) s += red[k][y][x];
+        red[0][y][x] = s;   // read and written by this thread alone
+      }
+      __syncthreads();
+      if (y == 0 && on) {
+#pragma unroll
+        for (int d = 0; d < NS; ++d) S[d] = red[0][d][x];
+        val[part][x] = diag_value<NS>(S, ea[m] + eb[col] + sh);
+      }
+      __syncthreads();
+    }
+    if (y == 0 && on) {
+      if constexpr (CPLX) {
+        cplx* p = o.C + m * o.scm + n * o.scn;
+        *p = out_value(o, val[0][x], val[1][x], p);
+      } else {
+        double* p = o.out + m * o.ldo + n;
+        *p = out_value_real(o, val[0][x], p);
+      }
+    }
+  }
+}
+template <bool STACK, bool CPLX>
+void launch_output(int ns, int splits, cudaStream_t s, const int* slabs, const OzParts& q, long long M, long long Np,
+                   const int* ea, const int* eb, const OzOut& o) {
+  const long long elements = M * (CPLX ? Np / 2 : Np);
+  const bool split = elements < 152LL * 256 && splits > 4 * ns;
+  const bool small = M * Np < (1LL << 32);
+  with_ns(ns, [&](auto NSc) {
+    constexpr int NS = decltype(NSc)::value;
+    if (split)
+      oz_output_split_kernel<NS, STACK, CPLX><<<(unsigned)((elements + 31) / 32), 256, 0, s>>>(slabs, q, M, Np, ea, eb, o);
+    else if (small)
+      oz_output_kernel<NS, STACK, CPLX, unsigned><<<grid_for(elements), 256, 0, s>>>(slabs, q, M, Np, ea, eb, o);
+    else
+      oz_output_kernel<NS, STACK, CPLX, unsigned long long><<<grid_for(elements), 256, 0, s>>>(slabs, q, M, Np, ea, eb, o);
+  });
+  GFCC_LAUNCH_CHECK();
+}
+
+// ---- stacked form for a narrow right operand --------------------------------------------------------
+// When B has few rows and A is large, one product per A slice i multiplies it by B slices 0..ns-1-i
+// stacked as rows (B sliced slot-major), so that A is read ns times instead of ns(ns+1)/2 times and the
+// narrow B fills more of each tile. Partials of slice i: slabs + off[i], [zs[i]][M][ncol[i]] with
+// ncol[i] = (ns - i) Np rounded up to a multiple of four, B slice j in columns [j Np, (j + 1) Np). Diagonal d = i + j is summed exactly
+// in 64-bit integers, so the result equals the diagonal-by-diagonal one.
 
 template <bool WARP, int MODE>
 void launch_accumulate(bool small, int grid, cudaStream_t s, const int* part, int zs, long long M, long long Np,
@@ -658,18 +598,21 @@ void oz_run(const SlicedRows& A, const SlicedRows& B, long long M, long long Np,
     ks[q] = (long long)(ns - q) * kp;
   }
   const int nk_split = tc_exact_nk_split(M, Ns, ks, ns);
-  OzDiags dg;
-  dg.nd = ns;
+  OzParts dg;
+  int splits = 0;
+  const long long Np4 = (Np + 3) / 4 * 4;   // rows of split sums start on 16 bytes (vector epilogue stores)
   for (int q = 0; q < ns; ++q) {
     const int d = ns - 1 - q;
     eg[q].kA = 0;
     eg[q].kB = (long long)q * kp;
     eg[q].k_pad = ks[q];
-    eg[q].N = Np; eg[q].ldp = Np; eg[q].split_stride = M * Np;
+    eg[q].N = Np; eg[q].ldp = Np4; eg[q].split_stride = M * Np4;
     eg[q].nk_split = nk_split;
     dg.zs[d] = eg[q].zs();
     dg.off[d] = off;
-    off = (off + (long long)dg.zs[d] * M * Np + 3) / 4 * 4;   // 16-byte aligned blocks (vector epilogue stores)
+    dg.ncol[d] = Np4;
+    splits += dg.zs[d];
+    off += (long long)dg.zs[d] * M * Np4;
   }
   if (4.0 * (double)off <= slab_bytes) {
     // every diagonal's split sums side by side, then one pass that sums them into the output: the
@@ -678,31 +621,10 @@ void oz_run(const SlicedRows& A, const SlicedRows& B, long long M, long long Np,
     if (w.err.n == 0) { w.err.alloc(1); w.err.zero(s); }
     for (int q = 0; q < ns; ++q) eg[q].P = w.islabs.p + dg.off[ns - 1 - q];
     tc_gemm_exact(TcOperand(As, M, ld, ld), TcOperand(Bs, Np, ld, ld), M, eg, ns, w.err.p, s, PROF_TC_SLICE);
-    int splits = 0;
-    for (int d = 0; d < ns; ++d) splits += dg.zs[d];
-    const long long elements = o.complex_out ? M * (Np / 2) : M * Np;
-    const bool warp = elements < 152LL * 256 && splits > 8 * ns;
-    const int grid = warp ? (int)std::min<long long>(std::max<long long>((elements * 32 + 255) / 256, 1), 152LL * 32)
-                          : grid_for(elements);
-    const bool small = M * Np < (1LL << 32);
     // bytes: every int32 split sum read once, the output written once
     ProfScope pa(PROF_OZ_ACCUM, 4.0 * splits * (double)M * (double)Np + out_bytes(o, M, Np), s);
-    if (splits == ns) {   // one split per diagonal
-      if (o.complex_out) {
-        if (small) launch_output1<2, unsigned>(ns, grid, s, w.islabs.p, dg, M, Np, A.expo.p, B.expo.p, o);
-        else launch_output1<2, unsigned long long>(ns, grid, s, w.islabs.p, dg, M, Np, A.expo.p, B.expo.p, o);
-      } else {
-        if (small) launch_output1<1, unsigned>(ns, grid, s, w.islabs.p, dg, M, Np, A.expo.p, B.expo.p, o);
-        else launch_output1<1, unsigned long long>(ns, grid, s, w.islabs.p, dg, M, Np, A.expo.p, B.expo.p, o);
-      }
-    } else if (o.complex_out) {
-      if (warp) launch_output<true, 2>(small, grid, s, w.islabs.p, dg, M, Np, A.expo.p, B.expo.p, o);
-      else launch_output<false, 2>(small, grid, s, w.islabs.p, dg, M, Np, A.expo.p, B.expo.p, o);
-    } else {
-      if (warp) launch_output<true, 1>(small, grid, s, w.islabs.p, dg, M, Np, A.expo.p, B.expo.p, o);
-      else launch_output<false, 1>(small, grid, s, w.islabs.p, dg, M, Np, A.expo.p, B.expo.p, o);
-    }
-    GFCC_LAUNCH_CHECK();
+    if (o.complex_out) launch_output<false, true>(ns, splits, s, w.islabs.p, dg, M, Np, A.expo.p, B.expo.p, o);
+    else launch_output<false, false>(ns, splits, s, w.islabs.p, dg, M, Np, A.expo.p, B.expo.p, o);
     return;
   }
   // bytes of int32 split sums at a time (half the bound above)
@@ -720,7 +642,7 @@ void oz_run(const SlicedRows& A, const SlicedRows& B, long long M, long long Np,
     if (!o.complex_out) oc.out = o.out + n0;
     for (int d = 0; d < ns; ++d) {
       TcExactGroup g = eg[ns - 1 - d];
-      g.N = nn; g.ldp = nn; g.split_stride = M * nn;
+      g.N = nn; g.ldp = nn; g.split_stride = M * nn;   // oz_accumulate_kernel's layout
       g.P = w.islabs.p;
       tc_gemm_exact(TcOperand(As, M, ld, ld), TcOperand(Bs + n0 * ld, nn, ld, ld), M, &g, 1, w.err.p, s, PROF_TC_SLICE);
       const int zeff = g.zs();
@@ -754,7 +676,7 @@ void oz_run(const SlicedRows& A, const SlicedRows& B, long long M, long long Np,
 
 // The products of the stacked form (A slice i against B slices 0..ns-1-i, longest first) and the bytes of their
 // int32 partials.
-void stack_groups(long long M, long long Np, long long kp, int ns, TcExactGroup (&eg)[OZ_SLICES_MAX], OzStack& st,
+void stack_groups(long long M, long long Np, long long kp, int ns, TcExactGroup (&eg)[OZ_SLICES_MAX], OzParts& st,
                   double& bytes) {
   long long Ns[OZ_SLICES_MAX], ks[OZ_SLICES_MAX], off = 0;
   for (int i = 0; i < ns; ++i) {
@@ -762,19 +684,17 @@ void stack_groups(long long M, long long Np, long long kp, int ns, TcExactGroup 
     ks[i] = kp;
   }
   const int nk_split = tc_exact_nk_split(M, Ns, ks, ns);
-  st.ns = ns;
   for (int i = 0; i < ns; ++i) {
     eg[i].kA = (long long)i * kp;
     eg[i].kB = 0;
     eg[i].k_pad = kp;
-    eg[i].N = Ns[i]; eg[i].ldp = Ns[i]; eg[i].split_stride = M * Ns[i];
+    const long long ld4 = (Ns[i] + 3) / 4 * 4;   // rows of partials start on 16 bytes (vector epilogue stores)
+    eg[i].N = Ns[i]; eg[i].ldp = ld4; eg[i].split_stride = M * ld4;
     eg[i].nk_split = nk_split;
     st.off[i] = off;
-    st.ncol[i] = Ns[i];
+    st.ncol[i] = ld4;
     st.zs[i] = eg[i].zs();
-    // the GEMM epilogue stores rows of four int32 at once where ncol is a multiple of 4: every block
-    // of partials starts on 16 bytes
-    off = (off + (long long)st.zs[i] * M * Ns[i] + 3) / 4 * 4;
+    off += (long long)st.zs[i] * M * ld4;
   }
   bytes = 4.0 * (double)off;
 }
@@ -783,7 +703,7 @@ void stack_groups(long long M, long long Np, long long kp, int ns, TcExactGroup 
 // partials fit in 4 GB.
 bool use_stacked(long long M, long long Np, long long kp, int ns) {
   TcExactGroup eg[OZ_SLICES_MAX];
-  OzStack st;
+  OzParts st;
   double bytes;
   stack_groups(M, Np, kp, ns, eg, st, bytes);
   return kp >= 4LL * Np * st.zs[0] && bytes <= oz_slab_bytes();
@@ -795,34 +715,23 @@ void oz_run_stacked(const SlicedRows& A, const SlicedRows& Bsm, long long M, lon
   const int ns = A.ns;
   const long long kp = A.kp, ld = (long long)ns * kp;
   TcExactGroup eg[OZ_SLICES_MAX];
-  OzStack st;
+  OzParts st;
   double bytes;
   stack_groups(M, Np, kp, ns, eg, st, bytes);
   w.islabs.alloc((size_t)(bytes / 4.0));
   if (w.err.n == 0) { w.err.alloc(1); w.err.zero(s); }
-  bool one_split = true;
   int splits = 0;
+  double part_bytes = 0.0;
   for (int i = 0; i < ns; ++i) {
     eg[i].P = w.islabs.p + st.off[i];
-    one_split = one_split && st.zs[i] == 1;
     splits += st.zs[i];
+    part_bytes += 4.0 * st.zs[i] * (double)M * (double)st.ncol[i];
   }
   tc_gemm_exact(TcOperand(reinterpret_cast<const __half*>(A.slices.p), M, ld, ld),
                 TcOperand(reinterpret_cast<const __half*>(Bsm.slices.p), ns * Np, kp, kp), M, eg, ns, w.err.p, s,
                 PROF_TC_SLICE);
-  const long long elements = M * (Np / 2);
-  const bool warp = !one_split && elements < 152LL * 256 && splits > 8 * ns;
-  const int grid = warp ? (int)std::min<long long>(std::max<long long>((elements * 32 + 255) / 256, 1), 152LL * 32)
-                        : grid_for(elements);
-  double part_bytes = 0.0;
-  for (int i = 0; i < ns; ++i) part_bytes += 4.0 * st.zs[i] * (double)M * (double)st.ncol[i];
   ProfScope pa(PROF_OZ_ACCUM, part_bytes + out_bytes(o, M, Np), s);
-  if (M * Np < (1LL << 32))
-    launch_stack_output<unsigned>(ns, one_split, warp, grid, s, w.islabs.p, st, M, Np, A.expo.p, Bsm.expo.p, o);
-  else
-    launch_stack_output<unsigned long long>(ns, one_split, warp, grid, s, w.islabs.p, st, M, Np, A.expo.p,
-                                            Bsm.expo.p, o);
-  GFCC_LAUNCH_CHECK();
+  launch_output<true, true>(ns, splits, s, w.islabs.p, st, M, Np, A.expo.p, Bsm.expo.p, o);
 }
 }  // namespace
 

@@ -171,7 +171,10 @@ void prep_operand(const VT* X, int o, int v, int nb, typename E::T* out, int kpa
 // ---- operand preparation of the FP32 Krylov basis -------------------------------------------------
 // One pass over w: the basis vector v = w inv is written, z = P v formed, and every 2h1p element goes to the
 // three places the up and ring operands have for it, all of them along k = pair v + e of a tile of 32 k x 32 c:
-//   up:   B[c*2 + r][k];   ring: U[(j*nb + c)*2 + r][m v + e] = z, U[(m*nb + c)*2 + r][j v + e] = -z  (m < j)
+//   up:   B[c*2 + r][k];   ring: U[(j*nbp + c)*2 + r][m v + e] = z, U[(m*nbp + c)*2 + r][j v + e] = -z  (m < j)
+// nbp is the batch width rounded up to even: the products' output rows then start on 16 bytes and their epilogue
+// stores four words at a time (o = 23, v = 77, 207 columns: the short products of 64 MB took 166 us with the odd
+// width, 45 with the even one). What the extra column holds is finite and not read.
 // The oooo operand runs along the pair index and is made from v by a second kernel. Before, scaling,
 // preconditioning and the three operands were five kernels, each reading a vector block. The blocks m = j of U
 // and the K padding stay zero: the buffers are zeroed when they are allocated, the blocks m = j (whose rows
@@ -180,7 +183,7 @@ template <typename E, typename WT>
 __global__ void __launch_bounds__(256) prep_fused_kernel(const WT* __restrict__ W, const float* __restrict__ inv,
                                                          float2* __restrict__ V, const RowF* __restrict__ md,
                                                          const ShiftF* __restrict__ shift, int o, int v, int nb,
-                                                         long long Pv, typename E::T* __restrict__ Bup, int kup,
+                                                         int nbp, long long Pv, typename E::T* __restrict__ Bup, int kup,
                                                          typename E::T* __restrict__ U, int kr,
                                                          float2* __restrict__ z1) {
   __shared__ float2 tile[PT][PT + 1];
@@ -226,15 +229,15 @@ __global__ void __launch_bounds__(256) prep_fused_kernel(const WT* __restrict__ 
       const float2 z = tile[threadIdx.x][rr >> 1];
       const float x = r ? z.y : z.x;
       Bup[((long long)cc * 2 + r) * kup + k] = E::cvt(x);
-      U[(((long long)j * nb + cc) * 2 + r) * kr + m * v + e] = E::cvt(x);
-      U[(((long long)m * nb + cc) * 2 + r) * kr + j * v + e] = E::cvt(-x);
+      U[(((long long)j * nbp + cc) * 2 + r) * kr + m * v + e] = E::cvt(x);
+      U[(((long long)m * nbp + cc) * 2 + r) * kr + j * v + e] = E::cvt(-x);
     }
   }
 }
-// oooo: B[(a*nb + c)*2 + r][p] = z_p^a of column c (component r)
+// oooo: B[(a*nbp + c)*2 + r][p] = z_p^a of column c (component r)
 template <typename E>
 __global__ void __launch_bounds__(256) prep_oooo_kernel(const float2* __restrict__ V, const RowF* __restrict__ md,
-                                                        const ShiftF* __restrict__ shift, int o, int v, int nb, int P,
+                                                        const ShiftF* __restrict__ shift, int o, int v, int nb, int nbp, int P,
                                                         typename E::T* __restrict__ B, int kp) {
   __shared__ float2 tile[PT][PT + 1];
   const int a = blockIdx.z, p0 = blockIdx.x * PT, c0 = blockIdx.y * PT, c = c0 + threadIdx.x;
@@ -256,11 +259,11 @@ __global__ void __launch_bounds__(256) prep_oooo_kernel(const float2* __restrict
     const int cc = c0 + (rr >> 1), r = rr & 1;
     if (cc < nb) {
       const float2 z = tile[threadIdx.x][rr >> 1];
-      B[(((long long)a * nb + cc) * 2 + r) * kp + p] = E::cvt(r ? z.y : z.x);
+      B[(((long long)a * nbp + cc) * 2 + r) * kp + p] = E::cvt(r ? z.y : z.x);
     }
   }
 }
-// U[(j*nb + c)*2 + r][j v + e] = 0
+// U[(j*nb + c)*2 + r][j v + e] = 0 (nb: the even width)
 template <typename E>
 __global__ void zero_ring_diag_kernel(typename E::T* __restrict__ U, int v, int nb, int kr) {
   const int j = blockIdx.y;
@@ -314,7 +317,8 @@ __global__ void __launch_bounds__(256) combine_f32_kernel(const float2* __restri
                                                           const float2* __restrict__ up, const float2* __restrict__ C2,
                                                           const float2* __restrict__ CT, const float2* __restrict__ z1,
                                                           const RowF* __restrict__ md,
-                                                          const ShiftF* __restrict__ shift, int o, int v, int Pv, int nb) {
+                                                          const ShiftF* __restrict__ shift, int o, int v, int Pv, int nb,
+                                                          int nbp) {
   constexpr int RW = 2;
   const int cw = blockDim.x, c0 = blockIdx.x * 2 * cw + threadIdx.x;
   const bool on[2] = {c0 < nb, c0 + cw < nb};
@@ -322,7 +326,7 @@ __global__ void __launch_bounds__(256) combine_f32_kernel(const float2* __restri
   ShiftF sh[2];
   sh[0] = shift[c0];
   sh[1] = on[1] ? shift[c0 + cw] : sh[0];
-  const long long ldct = (long long)o * nb;
+  const long long ldct = (long long)o * nbp;
   const int ry = blockIdx.y * blockDim.y + threadIdx.y, step = gridDim.y * blockDim.y;
   auto shifted = [&](float d, const ShiftF& s, float2 z) {
     const float dre = d + s.x, dim = s.z;
@@ -333,7 +337,7 @@ __global__ void __launch_bounds__(256) combine_f32_kernel(const float2* __restri
     for (int h = 0; h < 2; ++h)
       if (on[h]) {
         const long long t = (long long)nu * nb + c0 + h * cw;
-        const float2 y = shifted(md[nu].z, sh[h], z1[t]), u = up[t + (long long)v * nb];
+        const float2 y = shifted(md[nu].z, sh[h], z1[t]), u = up[(long long)(v + nu) * nbp + c0 + h * cw];
         Y[t] = make_float2(y.x + u.x, y.y + u.y);
       }
   for (long long row0 = ry; row0 < Pv; row0 += (long long)RW * step) {
@@ -348,9 +352,9 @@ __global__ void __launch_bounds__(256) combine_f32_kernel(const float2* __restri
         unpair(p, i, j);
         m[r] = md[o + row];
         const float2* px = V + (o + row) * nb + c0;
-        const float2* pq = C2 + row * nb + c0;
-        const float2* p1 = CT + ((long long)a * o + i) * ldct + (long long)j * nb + c0;
-        const float2* p2 = CT + ((long long)a * o + j) * ldct + (long long)i * nb + c0;
+        const float2* pq = C2 + row * nbp + c0;
+        const float2* p1 = CT + ((long long)a * o + i) * ldct + (long long)j * nbp + c0;
+        const float2* p2 = CT + ((long long)a * o + j) * ldct + (long long)i * nbp + c0;
 #pragma unroll
         for (int h = 0; h < 2; ++h)
           if (on[h]) {
@@ -742,6 +746,7 @@ int low_precision_error(gfcc_ctx* c) {
 template <TcKind K>
 static void lp_batch_buffers(gfcc_ctx* c, LpState& st, int nb, cudaStream_t s) {
   using T = typename Elem<K>::T;
+  nb = (nb + 1) / 2 * 2;   // the FP32 path's even width
   if (nb <= st.nb_cap) return;
   const int o = c->o, v = c->v;
   const long long ov = (long long)o * v, Pv = (long long)c->P * v;
@@ -846,12 +851,13 @@ static void lp_prepare_impl(gfcc_ctx* c, LpState& st, const WT* W, const float* 
   using T = typename Elem<K>::T;
   const int o = c->o, v = c->v, P = c->P;
   const long long Pv = (long long)P * v;
+  const int nbp = (nb + 1) / 2 * 2;
   lp_batch_buffers<K>(c, st, nb, s);
   T* U = reinterpret_cast<T*>(st.Bring.p);
   ProfScope pp(PROF_LP_PREP, 0.0, s);
   if (st.nb_prep != nb) {
-    zero_ring_diag_kernel<Elem<K>><<<dim3((unsigned)std::min<long long>((2LL * nb * v + 255) / 256, 1024), o), 256, 0, s>>>(
-        U, v, nb, st.Kr);
+    zero_ring_diag_kernel<Elem<K>><<<dim3((unsigned)std::min<long long>((2LL * nbp * v + 255) / 256, 1024), o), 256, 0, s>>>(
+        U, v, nbp, st.Kr);
     GFCC_LAUNCH_CHECK();
     st.nb_prep = nb;
   }
@@ -860,11 +866,11 @@ static void lp_prepare_impl(gfcc_ctx* c, LpState& st, const WT* W, const float* 
   GFCC_CHECK((Pv + PT - 1) / PT + (o + PT - 1) / PT < (1LL << 31) && ct <= 65535 && v <= 65535, GFCC_ERR_ARG,
              "sigma: batch or virtual count too large");
   prep_fused_kernel<Elem<K>, WT><<<dim3((unsigned)((Pv + PT - 1) / PT + (o + PT - 1) / PT), ct), dim3(PT, 8), 0, s>>>(
-      W, inv, Vf, c->op.rowf.p, shift, o, v, nb, Pv, reinterpret_cast<T*>(st.Bup.p), st.Kpv, U, st.Kr,
+      W, inv, Vf, c->op.rowf.p, shift, o, v, nb, nbp, Pv, reinterpret_cast<T*>(st.Bup.p), st.Kpv, U, st.Kr,
       reinterpret_cast<float2*>(st.z1.p));
   GFCC_LAUNCH_CHECK();
   prep_oooo_kernel<Elem<K>><<<dim3((unsigned)((P + PT - 1) / PT), ct, (unsigned)v), dim3(PT, 8), 0, s>>>(
-      Vf, c->op.rowf.p, shift, o, v, nb, P, reinterpret_cast<T*>(st.Boo.p), st.Kp);
+      Vf, c->op.rowf.p, shift, o, v, nb, nbp, P, reinterpret_cast<T*>(st.Boo.p), st.Kp);
   GFCC_LAUNCH_CHECK();
 }
 
@@ -874,7 +880,8 @@ static void lp_apply_impl(gfcc_ctx* c, LpState& st, const cuFloatComplex* V, cuF
   using T = typename Elem<K>::T;
   const int o = c->o, v = c->v, P = c->P;
   const long long ov = (long long)o * v, Pv = (long long)P * v;
-  const long long nring = 2LL * o * nb, noo = 2LL * v * nb, nsm = 2LL * nb;
+  const int nbp = (nb + 1) / 2 * 2;
+  const long long nring = 2LL * o * nbp, noo = 2LL * v * nbp, nsm = 2LL * nbp;
   const double es = sizeof(T);
   const float2* Vf = reinterpret_cast<const float2*>(V);
   // the three products that do not depend on each other
@@ -945,7 +952,7 @@ static void lp_apply_impl(gfcc_ctx* c, LpState& st, const cuFloatComplex* V, cuF
   combine_f32_kernel<<<dim3((unsigned)gx, (unsigned)gy), dim3(cw, 256 / cw), 0, s>>>(
       Vf, reinterpret_cast<float2*>(Y), reinterpret_cast<const float2*>(st.up.p), reinterpret_cast<const float2*>(st.C2.p),
       reinterpret_cast<const float2*>(st.CT.p), reinterpret_cast<const float2*>(st.z1.p), c->op.rowf.p,
-      shift, o, v, (int)Pv, nb);
+      shift, o, v, (int)Pv, nb, nbp);
   GFCC_LAUNCH_CHECK();
 }
 
