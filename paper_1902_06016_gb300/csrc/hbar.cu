@@ -248,6 +248,68 @@ int grid_for(long long n) {
   return (int)std::min<long long>(std::max<long long>(g, 1), 152LL * 32);
 }
 
+// ---- packed antisymmetric index pairs ------------------------------------------------------------
+// The integrals <pq||rs> and the amplitudes are antisymmetric in p, q and in r, s (the input contract), so that a sum
+// over two contracted indices of the same kind is twice the sum over e < f, and a result antisymmetric in i, j needs
+// only i < j. Packed index of a < b out of n: a n - a (a + 1) / 2 + b - a - 1 (contiguous in b).
+__device__ __forceinline__ long long tri(int a, int b, int n) { return (long long)a * n - (long long)a * (a + 1) / 2 + b - a - 1; }
+// dst[r][tri(e, f)] = src[r][e][f], e < f: a warp per (r, e)
+__global__ void __launch_bounds__(256) pack_last_kernel(const double* __restrict__ src, long long rows, int v,
+                                                        double* __restrict__ dst) {
+  const int lane = threadIdx.x & 31;
+  const long long V = (long long)v * (v - 1) / 2;
+  for (long long q = (blockIdx.x * 256LL + threadIdx.x) >> 5; q < rows * v; q += gridDim.x * 8LL) {
+    const long long r = q / v;
+    const int e = (int)(q - r * v);
+    const double* s = src + q * v;
+    double* d = dst + r * V + tri(e, e + 1, v);
+    for (int f = e + 1 + lane; f < v; f += 32) d[f - e - 1] = s[f];
+  }
+}
+// dst[tri(i, j)][k] = src[i][j][k], i < j
+__global__ void __launch_bounds__(256) take_pairs_kernel(const double* __restrict__ src, int o, long long n,
+                                                         double* __restrict__ dst) {
+  const int i = blockIdx.y / o, j = blockIdx.y % o;
+  if (i >= j) return;
+  const double* s = src + ((long long)i * o + j) * n;
+  double* d = dst + tri(i, j, o) * n;
+  for (long long k = blockIdx.x * 256LL + threadIdx.x; k < n; k += gridDim.x * 256LL) d[k] = s[k];
+}
+// W[r][i][j] += R[r][tri(i, j)] for i < j and W[r][j][i] -= the same
+__global__ void add_pairs_kernel(const double* __restrict__ R, long long rows, int o, double* __restrict__ W) {
+  const long long n = (long long)o * o;
+  const long long np = (long long)o * (o - 1) / 2;
+  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < rows * n; t += (long long)gridDim.x * blockDim.x) {
+    const long long r = t / n;
+    const int k = (int)(t - r * n), i = k / o, j = k - i * o;
+    if (i < j) W[t] += R[r * np + tri(i, j, o)];
+    else if (i > j) W[t] -= R[r * np + tri(j, i, o)];
+  }
+}
+// W[m][n][i][j] += R[tri(m, n)][tri(i, j)], antisymmetric in both pairs
+__global__ void add_pair_pairs_kernel(const double* __restrict__ R, int o, double* __restrict__ W) {
+  const long long n = (long long)o * o, np = (long long)o * (o - 1) / 2;
+  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n * n; t += (long long)gridDim.x * blockDim.x) {
+    const int a = (int)(t / n), b = (int)(t - a * n);
+    int m = a / o, q = a % o, i = b / o, j = b % o;
+    if (m == q || i == j) continue;
+    double s = 1.0;
+    if (m > q) { const int x = m; m = q; q = x; s = -s; }
+    if (i > j) { const int x = i; i = j; j = x; s = -s; }
+    W[t] += s * R[tri(m, q, o) * np + tri(i, j, o)];
+  }
+}
+void pack_last(const Tensor& src, long long rows, int v, Tensor& dst, cudaStream_t s) {
+  pack_last_kernel<<<(unsigned)std::min<long long>((rows * v + 7) / 8, 152LL * 32), 256, 0, s>>>(src.p(), rows, v, dst.p());
+  GFCC_LAUNCH_CHECK();
+}
+void take_pairs(const Tensor& src, int o, long long n, Tensor& dst, cudaStream_t s) {
+  GFCC_CHECK((long long)o * o <= 65535, GFCC_ERR_ARG, "take_pairs: too many pairs");
+  take_pairs_kernel<<<dim3((unsigned)std::min<long long>((n + 255) / 256, 64), (unsigned)(o * o)), 256, 0, s>>>(src.p(), o, n,
+                                                                                                        dst.p());
+  GFCC_LAUNCH_CHECK();
+}
+
 __global__ void nonfinite_kernel(const double* x, long long n, int* flag) {
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n;
        t += (long long)gridDim.x * blockDim.x)
@@ -310,11 +372,23 @@ std::unique_ptr<HbarCommon> build_common(const HostInputs& in, int o, int v, cud
   // one-body elements
   contract(1.0, t1->as("nf"), v_oovv->as("mnef"), 0.0, Fme.as("me"), s);
   contract(1.0, t1->as("ne"), v_ooov->as("mnie"), 0.0, Fmi.as("mi"), s);
-  contract(0.5, tau.as("inef"), v_oovv->as("mnef"), 1.0, Fmi.as("mi"), s);
+  const int V = v * (v - 1) / 2, P = o * (o - 1) / 2;
+  if (V > 0) {   // 1/2 tau_in^ef <mn||ef> over e < f
+    h->tauP = std::make_unique<Tensor>("int", std::vector<int>{o, o, V});
+    h->oovvP = std::make_unique<Tensor>("mnt", std::vector<int>{o, o, V});
+    pack_last(tau, (long long)o * o, v, *h->tauP, s);
+    pack_last(*v_oovv, (long long)o * o, v, *h->oovvP, s);
+    contract(1.0, h->tauP->as("int"), h->oovvP->as("mnt"), 1.0, Fmi.as("mi"), s);
+  }
   add_diag_kernel<<<(o + 255) / 256, 256, 0, s>>>(Fmi.p(), o, h->eps->p(), 1.0);
   GFCC_LAUNCH_CHECK();
   contract(-1.0, t1->as("mf"), v_ovvv->as("maef"), 0.0, Fae.as("ae"), s);      // <am||ef> = -<ma||ef>
-  contract(-0.5, tau.as("mnaf"), v_oovv->as("mnef"), 1.0, Fae.as("ae"), s);
+  if (P > 0) {   // -1/2 tau_mn^af <mn||ef> over m < n
+    Tensor tp("paf", {P, v, v}), vp("pef", {P, v, v});
+    take_pairs(tau, o, (long long)v * v, tp, s);
+    take_pairs(*v_oovv, o, (long long)v * v, vp, s);
+    contract(-1.0, tp.as("paf"), vp.as("pef"), 1.0, Fae.as("ae"), s);
+  }
   add_diag_kernel<<<(v + 255) / 256, 256, 0, s>>>(Fae.p(), v, h->eps->p() + o, 1.0);
   GFCC_LAUNCH_CHECK();
 
@@ -348,9 +422,27 @@ void build_operator(gfcc_ctx* c, const HostInputs& in) {
   // W_mnij
   Tensor Wmnij("mnij", {o, o, o, o});
   perm(v_oooo->as("mnij"), 1.0, 0.0, Wmnij.as("mnij"), s);
-  contract(1.0, t1->as("je"), v_ooov->as("mnie"), 1.0, Wmnij.as("mnij"), s);
-  contract(-1.0, t1->as("ie"), v_ooov->as("mnje"), 1.0, Wmnij.as("mnij"), s);
-  contract(0.5, tau.as("ijef"), v_oovv->as("mnef"), 1.0, Wmnij.as("mnij"), s);
+  {  // P(ij) t_j^e <mn||ie>
+    Tensor Z("mnij", {o, o, o, o});
+    contract(1.0, t1->as("je"), v_ooov->as("mnie"), 0.0, Z.as("mnij"), s);
+    perm(Z.as("mnij"), 1.0, 1.0, Wmnij.as("mnij"), s);
+    perm(Z.as("mnji"), -1.0, 1.0, Wmnij.as("mnij"), s);
+  }
+  // 1/2 tau_ij^ef <mn||ef> over e < f, m < n, i < j: an eighth of the multiply-adds
+  const int V = v * (v - 1) / 2;
+  std::unique_ptr<Tensor> tauPP;
+  if (V > 0) {
+    tauPP = std::make_unique<Tensor>("pt", std::vector<int>{P, V});
+    Tensor vPP("qt", {P, V}), R("qp", {P, P});
+    take_pairs(*hc->tauP, o, V, *tauPP, s);
+    take_pairs(*hc->oovvP, o, V, vPP, s);
+    contract(1.0, vPP.as("qt"), tauPP->as("pt"), 0.0, R.as("qp"), s);
+    add_pair_pairs_kernel<<<grid_for((long long)o * o * o * o), 256, 0, s>>>(R.p(), o, Wmnij.p());
+    GFCC_LAUNCH_CHECK();
+    GFCC_CUDA(cudaStreamSynchronize(s));   // R is released here
+  }
+  hc->tauP.reset();
+  hc->oovvP.reset();
 
   // W_mnie
   Tensor Wmnie("mnie", {o, o, o, v});
@@ -362,15 +454,23 @@ void build_operator(gfcc_ctx* c, const HostInputs& in) {
   perm(v_ooov->as("ijmb"), 1.0, 0.0, Wmbij.as("mbij"), s);                      // <mb||ij> = <ij||mb>
   contract(-1.0, Fme.as("me"), t2->as("ijbe"), 1.0, Wmbij.as("mbij"), s);
   contract(-1.0, t1->as("nb"), Wmnij.as("mnij"), 1.0, Wmbij.as("mbij"), s);
-  contract(0.5, v_ovvv->as("mbef"), tau.as("ijef"), 1.0, Wmbij.as("mbij"), s);
-  contract(-1.0, v_ooov->as("mnje"), t2->as("inbe"), 1.0, Wmbij.as("mbij"), s);
-  contract(1.0, v_ooov->as("mnie"), t2->as("jnbe"), 1.0, Wmbij.as("mbij"), s);
-  {
-    Tensor X("mbej", {o, v, v, o});                                              // <mb||ej> - t_nj^bf <mn||ef>
+  if (V > 0) {   // 1/2 <mb||ef> tau_ij^ef over e < f, i < j: a quarter of the multiply-adds
+    Tensor vP("mbt", {o, v, V}), R("mbp", {o, v, P});
+    pack_last(*v_ovvv, (long long)o * v, v, vP, s);
+    contract(1.0, vP.as("mbt"), tauPP->as("pt"), 0.0, R.as("mbp"), s);
+    add_pairs_kernel<<<grid_for((long long)o * v * o * o), 256, 0, s>>>(R.p(), (long long)o * v, o, Wmbij.p());
+    GFCC_LAUNCH_CHECK();
+    GFCC_CUDA(cudaStreamSynchronize(s));
+  }
+  tauPP.reset();
+  {  // -P(ij) <mn||je> t_in^be + P(ij) t_i^e (<mb||ej> - t_nj^bf <mn||ef>): one product each, antisymmetrised after
+    Tensor Z("mbij", {o, v, o, o}), X("mbej", {o, v, v, o});
     perm(v_ovov->as("mbje"), -1.0, 0.0, X.as("mbej"), s);
     perm(Y.as("mbej"), -1.0, 1.0, X.as("mbej"), s);
-    contract(1.0, t1->as("ie"), X.as("mbej"), 1.0, Wmbij.as("mbij"), s);
-    contract(-1.0, t1->as("je"), X.as("mbei"), 1.0, Wmbij.as("mbij"), s);
+    contract(-1.0, v_ooov->as("mnje"), t2->as("inbe"), 0.0, Z.as("mbij"), s);
+    contract(1.0, t1->as("ie"), X.as("mbej"), 1.0, Z.as("mbij"), s);
+    perm(Z.as("mbij"), 1.0, 1.0, Wmbij.as("mbij"), s);
+    perm(Z.as("mbji"), -1.0, 1.0, Wmbij.as("mbij"), s);
   }
 
   // ---- scatter into the sigma operands -------------------------------------------------------
