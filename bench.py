@@ -330,8 +330,7 @@ def run_ours(args, rank, world):
     small_gemms = G.profile_read(31)   # up, oooo, down GEMMs of the low-precision sigma (bytes)
     sig_lp, sig_ex = G.profile_read(3), G.profile_read(4)      # whole sigmas (algorithmic flops)
     cgs_parts = {name: G.profile_read(k) for k, name in
-                 ((15, "multidot_kernel"), (16, "cgs_update_kernel<dot>"), (17, "cgs_update_kernel<norm>"),
-                  (18, "all three, batches < 32 columns"))}
+                 ((15, "sweep_kernel<dots>"), (16, "sweep_kernel<update>"), (18, "both, batches < 32 columns"))}
     G.profile(False)
     clk = clocks.stop()
     spectrum = spectrum_peaks(A_dev.cpu().numpy(), grid, sign=1.0 if ea else -1.0)
@@ -467,7 +466,7 @@ def run_ours(args, rank, world):
                    "parallelism": f"replicas x{world}"},
         "e2e": e2e, "gpu_launches": int(launches), "gpu_launches_per_step": int(launches // args.steps),
         "roofline": roof, "gemm_classes": kernels, "phases_ms": phases, "device_allocations_per_step": allocs,
-        "hbm_kernels": {"arnoldi_cgs_sweeps (multidot_kernel, cgs_update_kernel x2)": {
+        "hbm_kernels": {"arnoldi_cgs_sweeps (sweep_kernel dots and update)": {
             "bound": "hbm", "steps": cgs[0], "ms": cgs[1], "algorithmic_bytes": cgs[2],
             "achieved": cgs[2] / (cgs[1] / 1e3) / 1e9 if cgs[1] > 0 else None, "unit": "GB/s",
             "peak": peaks.get("hbm_gbs"), "frac": (cgs[2] / (cgs[1] / 1e3) / 1e9) / peaks["hbm_gbs"]
@@ -477,7 +476,7 @@ def run_ours(args, rank, world):
             **{name: {"bound": "hbm", "launches": n, "ms": ms, "algorithmic_bytes": b, "unit": "GB/s",
                       "achieved": b / (ms / 1e3) / 1e9 if ms > 0 else None, "peak": peaks.get("hbm_gbs"),
                       "frac": b / (ms / 1e3) / 1e9 / peaks["hbm_gbs"] if ms > 0 and peaks.get("hbm_gbs") else None}
-               for name, (n, ms, b) in (("exact_slicing (FP64 rows -> bf16 integer slices)", slicing),
+               for name, (n, ms, b) in (("exact_slicing (FP64 rows -> f16 integer slices)", slicing),
                                         ("exact_slice_accumulate (int32 split sums -> FP64 output)", accum),
                                         (f"tc_gemm_kernel<{args.precision}> up, oooo, down GEMMs of the inner sigma "
                                          "(short or thin shapes: operands read once, outputs written once)",
@@ -523,7 +522,7 @@ def rank_seed(base_seed: int, rank: int) -> int:
 
 
 def full_compare(args, ctx, grid, porb, eta, stream):
-    """Full-dimension FP64-accurate GMRES-IR solves (inner and residual sigma on exact bf16 slices) at every
+    """Full-dimension FP64-accurate GMRES-IR solves (inner and residual sigma on exact f16 slices) at every
     full_stride-th frequency of the output grid, at every frequency the reduced model sampled and at the
     middle of the window; returns their G points/s and the reduced model's A and G errors against them
     (normwise relative: max over the subset of |error| / max |full|)."""
@@ -555,7 +554,7 @@ def full_compare(args, ctx, grid, porb, eta, stream):
         return float(np.abs(a - b).max() / np.abs(b).max())
 
     return {"value": len(sub) * len(porb) / (ms / 1e3), "unit": UNIT, "ms": ms, "n_omega": int(len(sub)),
-            "n_p": len(porb), "solver": "GMRES-IR, FP64-accurate inner and residual sigma (exact bf16 slices)",
+            "n_p": len(porb), "solver": "GMRES-IR, FP64-accurate inner and residual sigma (exact f16 slices)",
             "converged": bool(r["converged"]), "max_rel_res": st.max_rel_res, "gmres_iters": st.gmres_iters,
             "mor_A_rel_err": err(mor["A"][:ng], Af[:ng]), "mor_G_rel_err": err(mor["G"][:ng], Gf[:ng]),
             "mor_A_rel_err_at_samples": err(mor["A"][ng:ng + ns], Af[ng:ng + ns]) if ns else None,

@@ -333,8 +333,8 @@ long long gfcc_launch_count(void);
  * inside new blocks; 10 extension of the residual basis; 11 the ring-term GEMM of the low-precision
  * sigma (counted here instead of class 0); 12 whole FP64-accurate complex GEMMs on exact slices;
  * 13 splitting of FP64 rows into exact slices; 14 the fused Gram-Schmidt sweeps of FP32-basis Arnoldi
- * steps; 15, 16, 17 the first, second and third of those sweeps alone for batches of at least 32
- * columns; 18 the three sweeps of batches of fewer than 32 columns (classes 14-18 count algorithmic
+ * steps; 15 and 16 the dot-product and the update sweep alone for batches of at least 32
+ * columns (17: none); 18 both sweeps of batches of fewer than 32 columns (classes 14-18 count algorithmic
  * HBM bytes in the "flops" field, as do classes 13 and 24; classes 3 and 4 count the sigma's algorithmic
  * flops, whatever arithmetic carries them out); 19 Householder reductions of Hhat to Hessenberg form; 20 the
  * per-frequency shifted Hessenberg solves; 21, 22 the coefficient products and updates of the block

@@ -56,12 +56,11 @@ enum ProfClass {
   PROF_MOR_BASIS = 10,   // extension of the orthonormal residual basis Q
   PROF_TC_RING = 11,     // the ring-term GEMM of the low-precision sigma (tf32/bf16 tcgen05)
   PROF_OZ_ZGEMM = 12,    // whole FP64-accurate complex GEMMs on exact slices (operand gathers to scatter)
-  PROF_OZ_SLICE = 13,    // splitting FP64 rows into exact bf16 slices (every use)
-  PROF_KRYLOV_CGS = 14,  // the three fused Gram-Schmidt sweeps of an FP32-basis Arnoldi step (bytes)
-  PROF_CGS_MULTIDOT = 15,     // first sweep alone (batches of >= 32 columns; bytes)
-  PROF_CGS_UPDATE_DOT = 16,   // second sweep alone (batches of >= 32 columns; bytes)
-  PROF_CGS_UPDATE_NORM = 17,  // third sweep alone (batches of >= 32 columns; bytes)
-  PROF_CGS_SMALL_NB = 18,     // the three sweeps of batches of fewer than 32 columns (bytes)
+  PROF_OZ_SLICE = 13,    // splitting FP64 rows into exact f16 slices (every use)
+  PROF_KRYLOV_CGS = 14,  // the two Gram-Schmidt sweeps of an FP32-basis Arnoldi step (bytes)
+  PROF_CGS_DOTS = 15,         // dot-product sweep alone (batches of >= 32 columns; bytes)
+  PROF_CGS_UPDATE = 16,       // update sweep alone (batches of >= 32 columns; bytes)
+  PROF_CGS_SMALL_NB = 18,     // both sweeps of batches of fewer than 32 columns (bytes)
   PROF_EVAL_HESS = 19,        // Householder reduction of Hhat to Hessenberg form (evaluation, guesses)
   PROF_EVAL_SOLVE = 20,       // per-frequency shifted Hessenberg solves
   PROF_ORTHO_GRAM = 21,       // block Gram-Schmidt coefficient products (basis^H block)

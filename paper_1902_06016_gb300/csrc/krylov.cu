@@ -3,8 +3,8 @@
 //
 // Each restart cycle is one refinement step: the residual r = b - (shift x + M x) is formed with
 // the FP64 sigma, then GMRES(k) on the correction runs with the sigma in the requested
-// precision (classical Gram-Schmidt with one re-orthogonalisation, FP64 basis, Givens least
-// squares), and x += P V y with the Jacobi right preconditioner P = (shift + diag M)^{-1}.
+// precision (classical Gram-Schmidt with one re-orthogonalisation, Givens least squares), and
+// x += P V y with the Jacobi right preconditioner P = (shift + diag M)^{-1}.
 // Columns whose FP64 residual meets the tolerance are written out and compacted away between
 // cycles. The paper used a complex DIIS solver (convergence study after Table 1); any convergent
 // solver reaches the same solution of Eq. xplin.
@@ -29,7 +29,7 @@ template <typename VT> struct RealOf;
 template <> struct RealOf<cplx> { using type = double; };
 template <> struct RealOf<cuFloatComplex> { using type = float; };
 
-constexpr int MD_TX = 32, MD_TY = 8, MD_MAXV = 32;
+constexpr int MD_TX = 32, MD_TY = 8, MD_MAXV = 32;   // blocks of the sweeps; basis vectors per sweep
 // The kernels below are instantiated for NV = 4, 8, 16, 32 basis vectors (nv <= NV used).
 template <typename F>
 void with_nv(int nv, F&& f) {
@@ -103,24 +103,33 @@ __global__ void __launch_bounds__(256, 2) multidot_kernel(const VT* __restrict__
 }
 
 // ---- pipelined Gram-Schmidt sweeps of the FP32 basis ---------------------------------------------
-// The three sweeps of a CGS2 Arnoldi step with an FP32 basis (MODE 0: partial sums of conj(V_i) w, the
-// layout of multidot_kernel's partials; 1: w -= V h, then partial sums
-// of conj(V_i) w; 2: w -= V h, then partial sums of |w|^2), with the loads decoupled from the
-// arithmetic: every thread streams its own elements (its NPG basis vectors and w at one row per step)
-// through a SW_STAGES-deep ring in shared memory by 8-byte asynchronous copies (cp.async, zero-filled
-// outside the batch), so that about three steps of loads are in flight per block without holding
+// Classical Gram-Schmidt with re-orthogonalisation, the second pass of a vector delayed by one step, so that it shares
+// its reads of the basis with the first pass of the next vector (the basis is read twice per step instead of three
+// times, the sweeps being HBM-bound). At step j, with V_0 .. V_{j-1} final, a the normalised vector that has had its
+// first pass and u the image of a:
+//   sweep DOTS:    g_i = V_i^H a, r_i = V_i^H u (i < j), a^H a, a^H u
+//   coefficients:  rho^2 = a^H a - |g|^2, s = (a^H u - g^H r) / rho; Hessenberg column (r_0 .. r_{j-1}, s)
+//   sweep UPDATE:  V_j = (a - V g) / rho,  u -= V r + V_j s (u has had its first pass), partial sums of |u|^2
+// u is the action on a, not on V_j: they differ by |g|, the FP32 rounding level (1e-7 times the cancellation of the
+// first pass), far below the rounding of the low-precision action itself; the residual of every cycle is recomputed.
+// (o = 30, v = 130, TF32 solves to 1e-10: kernels of the whole solve 276 -> 247 ms, all of it the sweeps; the numbers
+// of Arnoldi steps did not change by more than 2 in 440.)
+//
+// The loads are decoupled from the arithmetic: every thread streams its own elements (its NPG basis vectors, a and u
+// at one row per step) through a SW_STAGES-deep ring in shared memory by 8-byte asynchronous copies (cp.async,
+// zero-filled outside the batch), so that about three steps of loads are in flight per block without holding
 // registers. A block is CW columns wide (32, 16, 8 or 4: narrow batches keep every thread busy) and
-// SW_THREADS / CW thread rows high; the thread rows form MdGroups-like groups that each own NPG basis
-// vectors (IG groups), and the groups' shares of V h are added through shared memory as above. Each
-// thread reads only the ring slots it filled itself.
+// SW_THREADS / CW thread rows high; the thread rows form IG groups that each own NPG basis vectors, and the groups'
+// shares of V g and V r are added through shared memory. Each thread reads only the ring slots it filled itself.
+// Bases of more than MD_MAXV vectors take a pair of sweeps per MD_MAXV of them.
 constexpr int SW_THREADS = 256, SW_STAGES = 4;
 template <int NV> struct SwGroups {
   static constexpr int IG = NV >= 16 ? NV / 8 : 1;
   static constexpr int NPG = NV / IG;
 };
 template <int NV, int CW> constexpr size_t sweep_smem_bytes() {
-  return sizeof(float2) * (size_t)SW_STAGES * (SwGroups<NV>::NPG + 1) * SW_THREADS   // load ring
-         + sizeof(float2) * 2 * SW_THREADS;                                          // shares
+  return sizeof(float2) * (size_t)SW_STAGES * (SwGroups<NV>::NPG + 2) * SW_THREADS   // load ring
+         + sizeof(float4) * 2 * SW_THREADS;                                          // shares
 }
 
 __device__ __forceinline__ void cp_async8(void* smem, const void* gmem, bool pred) {
@@ -131,49 +140,64 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
-template <int NV, int MODE, int CW>
-__global__ void __launch_bounds__(SW_THREADS, 2) sweep_kernel(const float2* __restrict__ V, long long vstride, int nv,
-                                                              float2* __restrict__ W, long long D, int nb,
-                                                              long long rows_per_chunk, const cplx* __restrict__ h,
-                                                              int hld, cplx* __restrict__ partial) {
+struct SweepArgs {
+  const float2* V;        // the nv basis vectors of this sweep (stride vstride)
+  long long vstride;
+  int nv;
+  float2 *a, *u;          // read (DOTS), read and written (UPDATE)
+  long long D;
+  int nb;
+  long long rows_per_chunk;
+  // DOTS: partial[chunk][q][c], q < 2 nv (+ 2 when scalars): g_0 .. g_{nv-1}, r_0 .. r_{nv-1}, a^H a, a^H u
+  cplx* partial;
+  int scalars;
+  // UPDATE: coefficients [i nb + c]; last: finish V_j and u with (1 / rho, s) per column and sum |u|^2
+  const float2 *g, *r;
+  const float4* fin;      // (1 / rho, s.x, s.y, -)
+  int last;
+};
+template <int NV, bool UPDATE, int CW>
+__global__ void __launch_bounds__(SW_THREADS, 2) sweep_kernel(SweepArgs p) {
   constexpr int TY = SW_THREADS / CW, IG = SwGroups<NV>::IG, NPG = SwGroups<NV>::NPG, RPG = TY / IG;
-  constexpr int SLOTS = NPG + 1;
+  constexpr int SLOTS = NPG + 2;
   static_assert(TY % IG == 0, "thread rows per group");
   extern __shared__ __align__(16) unsigned char sw_raw[];
-  float2* ring = reinterpret_cast<float2*>(sw_raw);                       // [SW_STAGES][SLOTS][SW_THREADS]
-  float2* share = ring + (size_t)SW_STAGES * SLOTS * SW_THREADS;          // [2][TY][CW]
+  float2* ring = reinterpret_cast<float2*>(sw_raw);                                                    // [SW_STAGES][SLOTS][SW_THREADS]
+  float4* share = reinterpret_cast<float4*>(ring + (size_t)SW_STAGES * SLOTS * SW_THREADS);             // [2][TY][CW]
+  const int nv = p.nv, nb = p.nb;
   const int tid = threadIdx.x, x = tid % CW, y = tid / CW;
-  const int g = y / RPG, yr = y % RPG;
+  const int gi = y / RPG, yr = y % RPG;
   const int c = blockIdx.x * CW + x;
-  const int i0 = g * NPG, ng = nv - i0;
-  const long long r0 = blockIdx.y * rows_per_chunk;
-  const long long r1 = min(D, r0 + rows_per_chunk);
+  const int i0 = gi * NPG, ng = nv - i0;
+  const long long r0 = blockIdx.y * p.rows_per_chunk;
+  const long long r1 = min(p.D, r0 + p.rows_per_chunk);
   const long long nsteps = (r1 - r0 + RPG - 1) / RPG;   // the same for every thread (barriers inside)
-  const float2* Vg = V + (long long)i0 * vstride;
+  const float2* Vg = p.V + (long long)i0 * p.vstride;
   auto issue = [&](long long t) {
     float2* st = ring + (size_t)(t % SW_STAGES) * SLOTS * SW_THREADS + tid;
     const long long nu = r0 + t * RPG + yr;
     const bool ok = c < nb && nu < r1;
     const long long off = ok ? nu * nb + c : 0;
-    // predicated-off copies zero-fill and read nothing; they are given the valid base address V
+    // predicated-off copies zero-fill and read nothing; they are given a valid base address
 #pragma unroll
     for (int li = 0; li < NPG; ++li) {
       const bool on = ok && li < ng;
-      cp_async8(st + li * SW_THREADS, on ? Vg + li * vstride + off : V, on);
+      cp_async8(st + li * SW_THREADS, on ? Vg + li * p.vstride + off : p.a, on);
     }
-    cp_async8(st + NPG * SW_THREADS, W + off, ok);
+    cp_async8(st + NPG * SW_THREADS, p.a + off, ok);
+    cp_async8(st + (NPG + 1) * SW_THREADS, p.u + off, ok);
   };
-  float2 hv[NPG];
+  // UPDATE: coefficients of the thread's vectors; DOTS: accumulators
+  float2 cg[NPG], cr[NPG];
 #pragma unroll
   for (int li = 0; li < NPG; ++li) {
-    const bool on = MODE != 0 && c < nb && li < ng;
-    hv[li] = on ? make_float2((float)h[(long long)c * hld + i0 + li].x, (float)h[(long long)c * hld + i0 + li].y)
-                : make_float2(0.f, 0.f);
+    const bool on = UPDATE && c < nb && li < ng;
+    cg[li] = on ? p.g[(long long)(i0 + li) * nb + c] : make_float2(0.f, 0.f);
+    cr[li] = on ? p.r[(long long)(i0 + li) * nb + c] : make_float2(0.f, 0.f);
   }
-  float ax[NPG], ay[NPG];
-#pragma unroll
-  for (int li = 0; li < NPG; ++li) { ax[li] = 0.f; ay[li] = 0.f; }
-  float nrm = 0.f;
+  float4 fin = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (UPDATE && p.last && c < nb) fin = p.fin[c];
+  float aa = 0.f, aux = 0.f, auy = 0.f;   // DOTS: a^H a, a^H u; UPDATE: aa = |u|^2
 #pragma unroll
   for (int t = 0; t < SW_STAGES - 1; ++t) {
     if (t < nsteps) issue(t);
@@ -184,81 +208,155 @@ __global__ void __launch_bounds__(SW_THREADS, 2) sweep_kernel(const float2* __re
     cp_async_commit();
     cp_async_wait<SW_STAGES - 1>();   // this thread's copies of step t have landed
     const float2* st = ring + (size_t)(t % SW_STAGES) * SLOTS * SW_THREADS + tid;
-    float2 w = st[NPG * SW_THREADS];
-    float2 v[NPG];
-#pragma unroll
-    for (int li = 0; li < NPG; ++li) v[li] = st[li * SW_THREADS];
-    const long long nu = r0 + t * RPG + yr;
-    const bool ok = c < nb && nu < r1;
-    if constexpr (MODE != 0) {
-      float sx = 0.f, sy = 0.f;
+    float2 a = st[NPG * SW_THREADS], u = st[(NPG + 1) * SW_THREADS];
+    if constexpr (!UPDATE) {
 #pragma unroll
       for (int li = 0; li < NPG; ++li) {
-        sx += v[li].x * hv[li].x - v[li].y * hv[li].y;
-        sy += v[li].x * hv[li].y + v[li].y * hv[li].x;
+        const float2 v = st[li * SW_THREADS];
+        cg[li].x += v.x * a.x + v.y * a.y;
+        cg[li].y += v.x * a.y - v.y * a.x;
+        cr[li].x += v.x * u.x + v.y * u.y;
+        cr[li].y += v.x * u.y - v.y * u.x;
       }
-      if constexpr (IG == 1) {
-        w.x -= sx; w.y -= sy;
-      } else {
-        float2* sh = share + (size_t)(t & 1) * SW_THREADS;
-        sh[tid] = make_float2(sx, sy);
-        __syncthreads();
+      aa += a.x * a.x + a.y * a.y;
+      aux += a.x * u.x + a.y * u.y;
+      auy += a.x * u.y - a.y * u.x;
+    } else {
+      float4 s = make_float4(0.f, 0.f, 0.f, 0.f);   // V g, V r
 #pragma unroll
-        for (int gg = 0; gg < IG; ++gg) {
-          const float2 o = sh[(gg * RPG + yr) * CW + x];
-          w.x -= o.x; w.y -= o.y;
+      for (int li = 0; li < NPG; ++li) {
+        const float2 v = st[li * SW_THREADS];
+        s.x += v.x * cg[li].x - v.y * cg[li].y;
+        s.y += v.x * cg[li].y + v.y * cg[li].x;
+        s.z += v.x * cr[li].x - v.y * cr[li].y;
+        s.w += v.x * cr[li].y + v.y * cr[li].x;
+      }
+      if constexpr (IG > 1) {
+        float4* sh = share + (size_t)(t & 1) * SW_THREADS;
+        sh[tid] = s;
+        __syncthreads();
+        s = sh[yr * CW + x];
+#pragma unroll
+        for (int gg = 1; gg < IG; ++gg) {
+          const float4 o = sh[(gg * RPG + yr) * CW + x];
+          s.x += o.x; s.y += o.y; s.z += o.z; s.w += o.w;
         }
       }
-      if (g == 0 && ok) W[nu * nb + c] = w;
-    }
-    if constexpr (MODE == 0 || MODE == 1) {
-#pragma unroll
-      for (int li = 0; li < NPG; ++li) {
-        ax[li] += v[li].x * w.x + v[li].y * w.y;
-        ay[li] += v[li].x * w.y - v[li].y * w.x;
+      const long long nu = r0 + t * RPG + yr;
+      if (gi == 0 && c < nb && nu < r1) {
+        a.x -= s.x; a.y -= s.y;
+        u.x -= s.z; u.y -= s.w;
+        if (p.last) {
+          a.x *= fin.x; a.y *= fin.x;
+          u.x -= a.x * fin.y - a.y * fin.z;
+          u.y -= a.x * fin.z + a.y * fin.y;
+          aa += u.x * u.x + u.y * u.y;
+        }
+        p.a[nu * nb + c] = a;
+        p.u[nu * nb + c] = u;
       }
-    } else {
-      nrm += w.x * w.x + w.y * w.y;
     }
   }
   cp_async_wait<0>();
   // sums over the thread rows, in FP64. All of them go to shared memory at once (the load ring is free now) and the
-  // whole block adds them, one output per thread: 2 RPG FP64 additions deep. (One basis vector at a time left the
-  // additions to one warp, NPG times: 5 us of a 20 us sweep at 264 columns of 4,785 rows.)
+  // whole block adds them, one output per thread and step: 2 RPG FP64 additions deep. (One basis vector at a time left
+  // the additions to one warp: 5 us of a 20 us sweep at 264 columns of 4,785 rows.)
   __syncthreads();
-  if constexpr (MODE == 2) {
+  if constexpr (UPDATE) {
+    if (!p.last) return;   // uniform
     double* part = reinterpret_cast<double*>(sw_raw);   // [TY][CW]
-    if (g == 0) part[tid] = (double)nrm;                 // g == 0: the first RPG thread rows
+    if (gi == 0) part[tid] = (double)aa;                // the first RPG thread rows
     __syncthreads();
-    // four threads per column
-    double t2 = 0.0;
+    double t2 = 0.0;                                    // four threads per column
     if (tid < 4 * CW)
       for (int k = tid / CW; k < RPG; k += 4) t2 += part[k * CW + tid % CW];
     __syncthreads();
     if (tid < 4 * CW) part[tid] = t2;
     __syncthreads();
     if (tid < CW && c < nb)
-      partial[(long long)blockIdx.y * nb + c] =
+      p.partial[(long long)blockIdx.y * nb + c] =
           make_cuDoubleComplex((part[tid] + part[CW + tid]) + (part[2 * CW + tid] + part[3 * CW + tid]), 0.0);
   } else {
-    float2* part = reinterpret_cast<float2*>(sw_raw);   // [NPG][TY][CW]
+    float2* part = reinterpret_cast<float2*>(sw_raw);   // [2 NPG][TY][CW], then a^H a and a^H u [2][TY][CW]
+    static_assert((2 * NPG + 2) <= SW_STAGES * SLOTS, "sums fit in the load ring");
 #pragma unroll
-    for (int li = 0; li < NPG; ++li) part[li * SW_THREADS + tid] = make_float2(ax[li], ay[li]);
+    for (int li = 0; li < NPG; ++li) {
+      part[li * SW_THREADS + tid] = cg[li];
+      part[(NPG + li) * SW_THREADS + tid] = cr[li];
+    }
+    part[2 * NPG * SW_THREADS + tid] = make_float2(aa, 0.f);
+    part[(2 * NPG + 1) * SW_THREADS + tid] = make_float2(aux, auy);
     __syncthreads();
-    for (int q = tid; q < NV * CW; q += SW_THREADS) {   // output: vector i = q / CW of group i / NPG, column q % CW
-      const int i = q / CW, xx = q % CW, gg = i / NPG, li = i % NPG;
-      const int cc = blockIdx.x * CW + xx;
-      if (i < nv && cc < nb) {
-        cplx sum = make_cuDoubleComplex(0.0, 0.0);
-        for (int k = 0; k < RPG; ++k) {
-          const float2 v = part[li * SW_THREADS + (gg * RPG + k) * CW + xx];
-          sum.x += (double)v.x;
-          sum.y += (double)v.y;
-        }
-        partial[((long long)blockIdx.y * nv + i) * nb + cc] = sum;
+    const int nq = 2 * nv + (p.scalars ? 2 : 0);
+    for (int q = tid; q < (2 * NV + 2) * CW; q += SW_THREADS) {
+      // output k = q / CW of column q % CW: g_i, r_i (i < NV) or a scalar (k = 2 NV, 2 NV + 1: summed by group 0)
+      const int k = q / CW, xx = q % CW, cc = blockIdx.x * CW + xx;
+      const bool sc = k >= 2 * NV;
+      const int i = sc ? 0 : k % NV, kind = sc ? 0 : k / NV;
+      if (cc >= nb || (sc ? !p.scalars : i >= nv)) continue;
+      const int slot = sc ? k - 2 * NV + 2 * NPG : kind * NPG + i % NPG;
+      const int row0 = sc ? 0 : (i / NPG) * RPG;
+      cplx sum = make_cuDoubleComplex(0.0, 0.0);
+      for (int m = 0; m < RPG; ++m) {
+        const float2 v = part[slot * SW_THREADS + (row0 + m) * CW + xx];
+        sum.x += (double)v.x;
+        sum.y += (double)v.y;
       }
+      const int out = sc ? 2 * nv + (k - 2 * NV) : kind * nv + i;
+      p.partial[((long long)blockIdx.y * nq + out) * nb + cc] = sum;
     }
   }
+}
+
+// sums[q nb + c] = sum_chunk partial[chunk][q][c], also in FP32 (a block takes one q and 32 columns)
+__global__ void __launch_bounds__(256) reduce_dots_kernel(const cplx* __restrict__ partial, int nchunk, int nq, int nb,
+                                                          cplx* __restrict__ sums, float2* __restrict__ sums_f) {
+  __shared__ cplx red[8][32];
+  const int x = threadIdx.x, y = threadIdx.y, c = blockIdx.x * 32 + x, q = blockIdx.y;
+  cplx s = make_cuDoubleComplex(0.0, 0.0);
+  if (c < nb) {
+#pragma unroll 4
+    for (int k = y; k < nchunk; k += 8) {
+      const cplx p = partial[((long long)k * nq + q) * nb + c];
+      s.x += p.x; s.y += p.y;
+    }
+  }
+  red[y][x] = s;
+  __syncthreads();
+  if (y == 0 && c < nb) {
+    for (int k = 1; k < 8; ++k) { s.x += red[k][x].x; s.y += red[k][x].y; }
+    sums[(long long)q * nb + c] = s;
+    sums_f[(long long)q * nb + c] = make_float2((float)s.x, (float)s.y);
+  }
+}
+// The coefficients of a column from its sums (g_i at g[i nb + c], r_i, a^H a and a^H u at sc): Hessenberg column Hc
+// (entry (i, c) at i nb + c) and fin = (1 / rho, s). Eight lanes per column.
+__global__ void __launch_bounds__(128) delayed_coef_kernel(const cplx* __restrict__ g, const cplx* __restrict__ r, int nv,
+                                                           const cplx* __restrict__ sc, int nb, cplx* __restrict__ Hc,
+                                                           float4* __restrict__ fin) {
+  const int c = blockIdx.x * 16 + (threadIdx.x >> 3), q = threadIdx.x & 7;
+  const bool on = c < nb;
+  double gg = 0.0, gx = 0.0, gy = 0.0;
+  if (on)
+    for (int i = q; i < nv; i += 8) {
+      const cplx a = g[(long long)i * nb + c], b = r[(long long)i * nb + c];
+      gg += a.x * a.x + a.y * a.y;
+      gx += a.x * b.x + a.y * b.y;   // conj(g) r
+      gy += a.x * b.y - a.y * b.x;
+      Hc[(long long)i * nb + c] = b;
+    }
+#pragma unroll
+  for (int w = 4; w > 0; w >>= 1) {
+    gg += __shfl_down_sync(0xffffffffu, gg, w, 8);
+    gx += __shfl_down_sync(0xffffffffu, gx, w, 8);
+    gy += __shfl_down_sync(0xffffffffu, gy, w, 8);
+  }
+  if (!on || q != 0) return;
+  const double rho2 = sc[c].x - gg;
+  const double inv = rho2 > 0.0 && isfinite(rho2) ? rsqrt(rho2) : 0.0;   // a zero (broken-down) column stays zero
+  const cplx s = make_cuDoubleComplex((sc[nb + c].x - gx) * inv, (sc[nb + c].y - gy) * inv);
+  Hc[(long long)nv * nb + c] = s;
+  fin[c] = make_float4((float)inv, (float)s.x, (float)s.y, 0.f);
 }
 
 // column width of the sweep blocks for a batch of nb columns
@@ -272,32 +370,30 @@ long long sweep_rows(long long D, int nb) {
   return std::max<long long>(64, (D + nchunk - 1) / nchunk);
 }
 
-template <int NV, int MODE, int CW>
-void launch_sweep_cw(const float2* V, long long vstride, int nv, float2* W, long long D, int nb, const cplx* h, int hld,
-                     cplx* partial, cudaStream_t s) {
+template <int NV, bool UPDATE, int CW>
+void launch_sweep_cw(SweepArgs p, cudaStream_t s) {
   static bool attr[64] = {};   // dynamic shared memory above 48 KB: set once per device
   int dev = 0;
   GFCC_CUDA(cudaGetDevice(&dev));
   GFCC_CHECK(dev >= 0 && dev < 64, GFCC_ERR_ARG, "device ordinal above 63");
   constexpr size_t bytes = sweep_smem_bytes<NV, CW>();
   if (!attr[dev]) {
-    GFCC_CUDA(cudaFuncSetAttribute(sweep_kernel<NV, MODE, CW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+    GFCC_CUDA(cudaFuncSetAttribute(sweep_kernel<NV, UPDATE, CW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
     attr[dev] = true;
   }
-  const long long rows = sweep_rows(D, nb);
-  const dim3 grid((unsigned)((nb + CW - 1) / CW), (unsigned)((D + rows - 1) / rows));
-  sweep_kernel<NV, MODE, CW><<<grid, SW_THREADS, bytes, s>>>(V, vstride, nv, W, D, nb, rows, h, hld, partial);
+  p.rows_per_chunk = sweep_rows(p.D, p.nb);
+  const dim3 grid((unsigned)((p.nb + CW - 1) / CW), (unsigned)((p.D + p.rows_per_chunk - 1) / p.rows_per_chunk));
+  sweep_kernel<NV, UPDATE, CW><<<grid, SW_THREADS, bytes, s>>>(p);
 }
-template <int MODE>
-void launch_sweep(const float2* V, long long vstride, int nv, float2* W, long long D, int nb, const cplx* h, int hld,
-                  cplx* partial, cudaStream_t s) {
-  with_nv(nv, [&](auto NVc) {
+template <bool UPDATE>
+void launch_sweep(const SweepArgs& p, cudaStream_t s) {
+  with_nv(p.nv, [&](auto NVc) {
     constexpr int NV = decltype(NVc)::value;
-    switch (sweep_cw(nb)) {
-      case 32: launch_sweep_cw<NV, MODE, 32>(V, vstride, nv, W, D, nb, h, hld, partial, s); break;
-      case 16: launch_sweep_cw<NV, MODE, 16>(V, vstride, nv, W, D, nb, h, hld, partial, s); break;
-      case 8: launch_sweep_cw<NV, MODE, 8>(V, vstride, nv, W, D, nb, h, hld, partial, s); break;
-      default: launch_sweep_cw<NV, MODE, 4>(V, vstride, nv, W, D, nb, h, hld, partial, s); break;
+    switch (sweep_cw(p.nb)) {
+      case 32: launch_sweep_cw<NV, UPDATE, 32>(p, s); break;
+      case 16: launch_sweep_cw<NV, UPDATE, 16>(p, s); break;
+      case 8: launch_sweep_cw<NV, UPDATE, 8>(p, s); break;
+      default: launch_sweep_cw<NV, UPDATE, 4>(p, s); break;
     }
   });
   GFCC_LAUNCH_CHECK();
@@ -736,10 +832,20 @@ static void gmres_impl(gfcc_ctx* c, const cplx* Bin, cplx* Xout, cplx* Rout, con
   DBuf<cplx> Bw, Xw, Rw, Yw, Ztmp, H, sn, g, partial, shw, hb;
   DBuf<VT> V, Zw, Ww, yv;
   DBuf<double> nrm, bnorm, thr, cs;
+  DBuf<cplx> sums, gr;       // FP32 basis: the delayed pass's sums (and g, r of bases longer than one sweep)
+  DBuf<float2> sums_f;
+  DBuf<float4> fin;
   DBuf<float> invf;
   DBuf<int> kc, live, nlive, cols, flag;
   DBuf<float4> shf;
-  if (F32) { ensure_row_split(c); shf.alloc(nb0); }
+  if (F32) {
+    ensure_row_split(c);
+    shf.alloc(nb0);
+    sums.alloc((long long)nb0 * (2 * k + 2));
+    sums_f.alloc((long long)nb0 * (2 * k + 2));
+    fin.alloc(nb0);
+    if (k > MD_MAXV) gr.alloc((long long)nb0 * 2 * k);
+  }
   if (!c->pin) GFCC_CUDA(cudaMallocHost(reinterpret_cast<void**>(&c->pin), sizeof(int)));
   if (!c->pin_event) GFCC_CUDA(cudaEventCreateWithFlags(&c->pin_event, cudaEventDisableTiming));
   Bw.alloc(D * nb0); Xw.alloc(D * nb0); Rw.alloc(D * nb0); Yw.alloc(D * nb0); Ztmp.alloc(D * nb0);
@@ -763,7 +869,8 @@ static void gmres_impl(gfcc_ctx* c, const cplx* Bin, cplx* Xout, cplx* Rout, con
       md = std::max(md, (D + sweep_rows(D, b) - 1) / sweep_rows(D, b) * b);
       md = std::max(md, (long long)el_grid(D, b).grid.y * b);
     }
-    partial.alloc(std::max(md * (k + 1), (D + rows_cn - 1) / rows_cn * nb0));
+    const int nq = std::max(std::min(k + 1, MD_MAXV), 2 * std::min(k, MD_MAXV) + 2);   // sums per chunk
+    partial.alloc(std::max(md * nq, (D + rows_cn - 1) / rows_cn * nb0));
   }
   GFCC_CUDA(cudaMemcpyAsync(Bw.p, Bin, sizeof(cplx) * D * nb0, cudaMemcpyDeviceToDevice, s));
   GFCC_CUDA(cudaMemcpyAsync(shw.p, shifts_dev, sizeof(cplx) * nb0, cudaMemcpyDeviceToDevice, s));
@@ -930,46 +1037,69 @@ static void gmres_impl(gfcc_ctx* c, const cplx* Bin, cplx* Xout, cplx* Rout, con
       if constexpr (F32) sigma_lp_apply(c, Vj, Ww.p, nb, shf.p, s, transpose);
       else sigma_batch(c, Zw.p, Ww.p, nb, nb, shw.p, inner_prec, transpose, s);
       ProfScope pk2(PROF_KRYLOV, 0.0, s);
-      // CGS with one re-orthogonalisation: h1 = V^H w, w -= V h1, h2 = V^H w, w -= V h2; H[:, j] = h1 + h2.
-      // With an FP32 basis of at most MD_MAXV vectors this takes three sweeps: h1; the first update with
-      // h2 fused; the second update with ||w||^2 fused.
       const int nv = j + 1;
       cplx* Hc = H.p + (long long)j * (k + 1) * nb;
       int norm_chunks = 0;   // chunk sums of ||w||^2 left in partial
-      bool fused = false;
       if constexpr (F32) {
-        if (nv <= MD_MAXV) {
-          fused = true;
-          // algorithmic HBM bytes of the three sweeps: V read three times, w read three times and
-          // written twice
-          ProfScope pcgs(PROF_KRYLOV_CGS, (3.0 * nv + 5.0) * (double)D * nb * sizeof(VT), s);
-          const long long rows = sweep_rows(D, nb);
-          const int nchunk = (int)((D + rows - 1) / rows);
-          const double vbytes = (double)D * nb * sizeof(VT);   // one basis vector of the batch
-          const int small = nb < MD_TX ? 1 : 0;
-          const float2* Vf = reinterpret_cast<const float2*>(V.p);
-          float2* Wf = reinterpret_cast<float2*>(Ww.p);
-          const dim3 rgrid((nb + 31) / 32, nv), rblock(32, 8);
+        // CGS with delayed re-orthogonalisation (see the sweeps): final V_j, w through its first pass, ||w||^2
+        // algorithmic HBM bytes: V read twice; a and u read twice and written once
+        const double vbytes = (double)D * nb * sizeof(VT);   // one vector of the batch
+        ProfScope pcgs(PROF_KRYLOV_CGS, (2.0 * j + 6.0) * vbytes, s);
+        const long long rows = sweep_rows(D, nb);
+        const int nchunk = (int)((D + rows - 1) / rows), small = nb < MD_TX ? 1 : 0;
+        SweepArgs sa{};
+        sa.vstride = vstride;
+        sa.a = reinterpret_cast<float2*>(Vj);
+        sa.u = reinterpret_cast<float2*>(Ww.p);
+        sa.D = D; sa.nb = nb;
+        sa.partial = partial.p;
+        // sums [g (j) | r (j) | scalars (2)]: a part of i0 .. i0 + n of the basis writes its g and r next to each other,
+        // from 2 i0 on
+        for (int i0 = 0; i0 == 0 || i0 < j; i0 += MD_MAXV) {
+          const int n = std::min(MD_MAXV, j - i0);
+          const int nq = 2 * n + (i0 == 0 ? 2 : 0);
+          sa.V = reinterpret_cast<const float2*>(V.p) + i0 * vstride;
+          sa.nv = n;
+          sa.scalars = i0 == 0;
           {
-            ProfScope pk(small ? PROF_CGS_SMALL_NB : PROF_CGS_MULTIDOT, (nv + 1.0) * vbytes, s);
-            launch_sweep<0>(Vf, vstride, nv, Wf, D, nb, nullptr, 0, partial.p, s);
+            ProfScope pk(small ? PROF_CGS_SMALL_NB : PROF_CGS_DOTS, (n + 2.0) * vbytes, s);
+            launch_sweep<false>(sa, s);
           }
-          reduce_partial_kernel<<<rgrid, rblock, 0, s>>>(partial.p, nchunk, nv, nb, hb.p, k + 1, 0, Hc, 0);
+          // the first part's scalars follow its g and r; later parts start behind them
+          const long long o0 = (i0 == 0 ? 0 : 2LL * i0 + 2) * nb;
+          reduce_dots_kernel<<<dim3((nb + 31) / 32, nq), dim3(32, 8), 0, s>>>(partial.p, nchunk, nq, nb, sums.p + o0,
+                                                                             sums_f.p + o0);
           GFCC_LAUNCH_CHECK();
-          {
-            ProfScope pk(small ? PROF_CGS_SMALL_NB : PROF_CGS_UPDATE_DOT, (nv + 2.0) * vbytes, s);
-            launch_sweep<1>(Vf, vstride, nv, Wf, D, nb, hb.p, k + 1, partial.p, s);
-          }
-          reduce_partial_kernel<<<rgrid, rblock, 0, s>>>(partial.p, nchunk, nv, nb, hb.p, k + 1, 0, Hc, 1);
-          GFCC_LAUNCH_CHECK();
-          {
-            ProfScope pk(small ? PROF_CGS_SMALL_NB : PROF_CGS_UPDATE_NORM, (nv + 2.0) * vbytes, s);
-            launch_sweep<2>(Vf, vstride, nv, Wf, D, nb, hb.p, k + 1, partial.p, s);
-          }
-          norm_chunks = nchunk;
         }
-      }
-      if (!fused) {
+        const int n0 = std::min(MD_MAXV, j);
+        if (j > n0) {   // g and r of all parts in two rows of blocks
+          for (int i0 = 0; i0 < j; i0 += MD_MAXV) {
+            const int n = std::min(MD_MAXV, j - i0);
+            const cplx* src = sums.p + (i0 == 0 ? 0 : 2LL * i0 + 2) * nb;
+            GFCC_CUDA(cudaMemcpyAsync(gr.p + (long long)i0 * nb, src, sizeof(cplx) * n * nb, cudaMemcpyDeviceToDevice, s));
+            GFCC_CUDA(cudaMemcpyAsync(gr.p + (long long)(j + i0) * nb, src + (long long)n * nb, sizeof(cplx) * n * nb,
+                                      cudaMemcpyDeviceToDevice, s));
+          }
+        }
+        const cplx* gp = j > n0 ? gr.p : sums.p;
+        delayed_coef_kernel<<<(nb + 15) / 16, 128, 0, s>>>(gp, gp + (long long)j * nb, j, sums.p + 2LL * n0 * nb, nb, Hc,
+                                                           fin.p);
+        GFCC_LAUNCH_CHECK();
+        for (int i0 = 0; i0 == 0 || i0 < j; i0 += MD_MAXV) {
+          const int n = std::min(MD_MAXV, j - i0);
+          const long long o0 = (i0 == 0 ? 0 : 2LL * i0 + 2) * nb;
+          sa.V = reinterpret_cast<const float2*>(V.p) + i0 * vstride;
+          sa.nv = n;
+          sa.g = sums_f.p + o0;
+          sa.r = sums_f.p + o0 + (long long)n * nb;
+          sa.fin = fin.p;
+          sa.last = i0 + MD_MAXV >= j;
+          ProfScope pk(small ? PROF_CGS_SMALL_NB : PROF_CGS_UPDATE, (n + 4.0) * vbytes, s);
+          launch_sweep<true>(sa, s);
+        }
+        norm_chunks = nchunk;
+      } else {
+        // CGS with one re-orthogonalisation: h1 = V^H w, w -= V h1, h2 = V^H w, w -= V h2; H[:, j] = h1 + h2
         for (int pass = 0; pass < 2; ++pass) {
           multidot<VT>(V.p, vstride, nv, Ww.p, D, nb, hb.p, k + 1, Hc, pass == 1, partial, s);
           update_kernel<VT><<<eg.grid, eg.block, 0, s>>>(V.p, vstride, nv, Ww.p, D, nb, hb.p, k + 1);

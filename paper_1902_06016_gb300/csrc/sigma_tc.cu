@@ -36,11 +36,6 @@ __device__ __forceinline__ void unpair(int p, int& i, int& j) {
   i = p - jj * (jj - 1) / 2;
 }
 
-// real type of a complex vector element: the FP32 Krylov path keeps all its arithmetic in FP32
-template <typename VT> struct VReal;
-template <> struct VReal<cplx> { using type = double; };
-template <> struct VReal<cuFloatComplex> { using type = float; };
-
 // element conversion (round to nearest)
 template <TcKind K> struct Elem;
 template <> struct Elem<TcKind::BF16> {
@@ -102,7 +97,7 @@ constexpr int PT = 32;
 template <typename E, typename VT, int KIND>
 __global__ void __launch_bounds__(256) prep_tiled_kernel(const VT* __restrict__ X, int o, int v, int nb,
                                                          typename E::T* __restrict__ out, int kpad) {
-  using R = typename VReal<VT>::type;
+  using R = double;
   __shared__ VT tile[PT][PT + 1];
   const int g = blockIdx.z;
   const int k0 = blockIdx.x * PT, c0 = blockIdx.y * PT;
@@ -403,7 +398,7 @@ __global__ void prep_down_kernel(const U* __restrict__ up, long long ldu, const 
   const long long total = 2LL * nb * kpad;
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total;
        t += (long long)gridDim.x * blockDim.x) {
-    using R = typename VReal<VT>::type;
+    using R = double;
     int n = (int)(t / kpad);
     int k = (int)(t % kpad);
     R val = R(0);
@@ -426,7 +421,7 @@ __global__ void combine_lp_kernel(const VT* __restrict__ X, VT* __restrict__ Y, 
   const long long ldct = 2LL * o * nb;
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total;
        t += (long long)gridDim.x * blockDim.x) {
-    using R = typename VReal<VT>::type;
+    using R = double;
     const int c = (int)(t % nb);
     const long long nu = t / nb;
     const VT x = X[t];
