@@ -100,8 +100,8 @@ __global__ void bilinear_partial_kernel(const cplx* __restrict__ X, const cplx* 
     double sr = 0.0, si = 0.0;
     for (long long nu = r0; nu < r1; ++nu) {
       const cplx x = X[nu * ldx + w * np + p], y = Y[nu * ldy + w * nq + q];
-      sr += x.x * y.x - x.y * y.y;
-      si += x.x * y.y + x.y * y.x;
+      sr = fma(x.x, y.x, fma(-x.y, y.y, sr));
+      si = fma(x.x, y.y, fma(x.y, y.x, si));
     }
     part[(long long)blockIdx.x * ntrip + t] = make_cuDoubleComplex(sr, si);
   }

@@ -93,7 +93,7 @@ __global__ void cterm_kernel(const cplx* __restrict__ X, long long S, const cplx
   double acc = 0.0;
   for (long long sidx = 0; sidx < S; ++sidx) {
     const cplx g = Gbar[sidx * nq + q], x = X[(long long)k * S + sidx];
-    acc += g.x * x.x + g.y * x.y;   // Re(conj(g) x)
+    acc = fma(g.x, x.x, fma(g.y, x.y, acc));   // Re(conj(g) x)
   }
   atomicAdd(&cbar1[(long long)i * o + k], acc);
 }

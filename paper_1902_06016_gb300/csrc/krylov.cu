@@ -42,15 +42,19 @@ void with_nv(int nv, F&& f) {
 // partial[chunk][i][c] = sum_{nu in chunk} conj(V_i[nu][c]) W[nu][c], i < nv (V_i = V + i*stride);
 // per-thread sums in the vector's precision, partials written in FP64.
 // Block (MD_TX columns) x (MD_TY): the MD_TY thread rows form IG = NV/8 groups (at least 1); group g
-// owns the accumulators of basis vectors [g NPG, (g+1) NPG), NPG = NV / IG, and its threads stride the
+// owns the accumulators of basis vectors g, g + IG, ... (NPG = NV / IG at most), and its threads stride the
 // chunk's rows by MD_TY / IG. Fewer accumulators per thread keep the registers, and so the number of
-// resident warps, independent of the basis size.
+// resident warps, independent of the basis size; the groups' shares differ by one vector at most (with contiguous
+// shares of 8 the groups of one warp scheduler held 14 of 22 vectors, those of another 8). Bound by the FP64 pipe:
+// the products go into the sums by two multiply-adds per component (a sum of products added on would be a product, a
+// multiply-add and an addition). 560 columns of D = 3,836, 17 to 28 vectors: 675 -> 523 us; update_kernel 382 -> 246 us
+// (92 % of the FP64 rate); norms 75 us -> 15.
 template <int NV> struct MdGroups {
   static constexpr int IG = NV >= 16 ? NV / 8 : 1;
   static constexpr int NPG = NV / IG;
   static constexpr int RPG = MD_TY / IG;   // thread rows per group
 };
-// sum the per-thread values acc[li] of group g over its RPG thread rows; partial for i = g NPG + li
+// sum the per-thread values acc[li] of group g over its RPG thread rows; partial for i = li IG + g
 template <typename VT, int NV, typename R>
 __device__ __forceinline__ void md_reduce(const R (&ax)[MdGroups<NV>::NPG], const R (&ay)[MdGroups<NV>::NPG], int nv,
                                           int c, int nb, cplx* __restrict__ partial, cplx (*red)[MD_TX]) {
@@ -60,7 +64,7 @@ __device__ __forceinline__ void md_reduce(const R (&ax)[MdGroups<NV>::NPG], cons
   for (int li = 0; li < G::NPG; ++li) {
     red[threadIdx.y][threadIdx.x] = make_cuDoubleComplex((double)ax[li], (double)ay[li]);
     __syncthreads();
-    const int i = g * G::NPG + li;
+    const int i = li * G::IG + g;
     if (yr == 0 && c < nb && i < nv) {
       cplx s = red[threadIdx.y][threadIdx.x];
       for (int k = 1; k < G::RPG; ++k) { s.x += red[threadIdx.y + k][threadIdx.x].x; s.y += red[threadIdx.y + k][threadIdx.x].y; }
@@ -81,25 +85,58 @@ __global__ void __launch_bounds__(256, 2) multidot_kernel(const VT* __restrict__
   const int g = threadIdx.y / G::RPG, yr = threadIdx.y % G::RPG;
   const long long r0 = blockIdx.y * rows_per_chunk;
   const long long r1 = min(D, r0 + rows_per_chunk);
-  const VT* Vg = V + (long long)g * G::NPG * vstride;
-  const int ng = nv - g * G::NPG;   // vectors of this group present (may be <= 0)
+  const VT* Vg = V + (long long)g * vstride;
+  const int ng = (nv - g + G::IG - 1) / G::IG;   // vectors of this group present (may be <= 0)
   R ax[G::NPG], ay[G::NPG];
 #pragma unroll
   for (int i = 0; i < G::NPG; ++i) { ax[i] = R(0); ay[i] = R(0); }
   if (c < nb && ng > 0) {
     for (long long nu = r0 + yr; nu < r1; nu += G::RPG) {
       const VT w = W[nu * nb + c];
+      VT vv[G::NPG];   // all loads of a row before its arithmetic
+#pragma unroll
+      for (int i = 0; i < G::NPG; ++i) vv[i] = i < ng ? Vg[i * G::IG * vstride + nu * nb + c] : w;
 #pragma unroll
       for (int i = 0; i < G::NPG; ++i) {
         if (i < ng) {
-          const VT vv = Vg[i * vstride + nu * nb + c];
-          ax[i] += vv.x * w.x + vv.y * w.y;
-          ay[i] += vv.x * w.y - vv.y * w.x;
+          ax[i] = fma(vv[i].x, w.x, fma(vv[i].y, w.y, ax[i]));
+          ay[i] = fma(vv[i].x, w.y, fma(-vv[i].y, w.x, ay[i]));
         }
       }
     }
   }
   md_reduce<VT, NV, R>(ax, ay, nv, c, nb, partial, red);
+}
+
+// partial[chunk][c].x = sum_{nu in chunk} |W[nu][c]|^2 (block MD_TX columns x MD_TY rows, four rows of a thread in
+// flight)
+template <typename VT>
+__global__ void __launch_bounds__(256) norm_partial_kernel(const VT* __restrict__ W, long long D, int nb,
+                                                           long long rows_per_chunk, cplx* __restrict__ partial) {
+  using R = typename RealOf<VT>::type;
+  __shared__ double red[MD_TY][MD_TX];
+  const int c = blockIdx.x * MD_TX + threadIdx.x;
+  const long long r0 = blockIdx.y * rows_per_chunk, r1 = min(D, r0 + rows_per_chunk);
+  R a[4] = {R(0), R(0), R(0), R(0)};
+  if (c < nb)
+    for (long long nu = r0 + threadIdx.y; nu < r1; nu += 4 * MD_TY) {
+      VT w[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const bool in = nu + u * MD_TY < r1;
+        w[u] = W[(in ? nu + u * MD_TY : nu) * nb + c];
+        if (!in) w[u].x = w[u].y = R(0);
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) a[u] = fma(w[u].x, w[u].x, fma(w[u].y, w[u].y, a[u]));
+    }
+  red[threadIdx.y][threadIdx.x] = (double)((a[0] + a[1]) + (a[2] + a[3]));
+  __syncthreads();
+  if (threadIdx.y == 0 && c < nb) {
+    double s = red[0][threadIdx.x];
+    for (int k = 1; k < MD_TY; ++k) s += red[k][threadIdx.x];
+    partial[(long long)blockIdx.y * nb + c] = make_cuDoubleComplex(s, 0.0);
+  }
 }
 
 // ---- pipelined Gram-Schmidt sweeps of the FP32 basis ---------------------------------------------
@@ -213,23 +250,23 @@ __global__ void __launch_bounds__(SW_THREADS, 2) sweep_kernel(SweepArgs p) {
 #pragma unroll
       for (int li = 0; li < NPG; ++li) {
         const float2 v = st[li * SW_THREADS];
-        cg[li].x += v.x * a.x + v.y * a.y;
-        cg[li].y += v.x * a.y - v.y * a.x;
-        cr[li].x += v.x * u.x + v.y * u.y;
-        cr[li].y += v.x * u.y - v.y * u.x;
+        cg[li].x = fma(v.x, a.x, fma(v.y, a.y, cg[li].x));
+        cg[li].y = fma(v.x, a.y, fma(-v.y, a.x, cg[li].y));
+        cr[li].x = fma(v.x, u.x, fma(v.y, u.y, cr[li].x));
+        cr[li].y = fma(v.x, u.y, fma(-v.y, u.x, cr[li].y));
       }
-      aa += a.x * a.x + a.y * a.y;
-      aux += a.x * u.x + a.y * u.y;
-      auy += a.x * u.y - a.y * u.x;
+      aa = fma(a.x, a.x, fma(a.y, a.y, aa));
+      aux = fma(a.x, u.x, fma(a.y, u.y, aux));
+      auy = fma(a.x, u.y, fma(-a.y, u.x, auy));
     } else {
       float4 s = make_float4(0.f, 0.f, 0.f, 0.f);   // V g, V r
 #pragma unroll
       for (int li = 0; li < NPG; ++li) {
         const float2 v = st[li * SW_THREADS];
-        s.x += v.x * cg[li].x - v.y * cg[li].y;
-        s.y += v.x * cg[li].y + v.y * cg[li].x;
-        s.z += v.x * cr[li].x - v.y * cr[li].y;
-        s.w += v.x * cr[li].y + v.y * cr[li].x;
+        s.x = fma(v.x, cg[li].x, fma(-v.y, cg[li].y, s.x));
+        s.y = fma(v.x, cg[li].y, fma(v.y, cg[li].x, s.y));
+        s.z = fma(v.x, cr[li].x, fma(-v.y, cr[li].y, s.z));
+        s.w = fma(v.x, cr[li].y, fma(v.y, cr[li].x, s.w));
       }
       if constexpr (IG > 1) {
         float4* sh = share + (size_t)(t & 1) * SW_THREADS;
@@ -248,9 +285,9 @@ __global__ void __launch_bounds__(SW_THREADS, 2) sweep_kernel(SweepArgs p) {
         u.x -= s.z; u.y -= s.w;
         if (p.last) {
           a.x *= fin.x; a.y *= fin.x;
-          u.x -= a.x * fin.y - a.y * fin.z;
-          u.y -= a.x * fin.z + a.y * fin.y;
-          aa += u.x * u.x + u.y * u.y;
+          u.x = fma(-a.x, fin.y, fma(a.y, fin.z, u.x));
+          u.y = fma(-a.x, fin.z, fma(-a.y, fin.y, u.y));
+          aa = fma(u.x, u.x, fma(u.y, u.y, aa));
         }
         p.a[nu * nb + c] = a;
         p.u[nu * nb + c] = u;
@@ -340,9 +377,9 @@ __global__ void __launch_bounds__(128) delayed_coef_kernel(const cplx* __restric
   if (on)
     for (int i = q; i < nv; i += 8) {
       const cplx a = g[(long long)i * nb + c], b = r[(long long)i * nb + c];
-      gg += a.x * a.x + a.y * a.y;
-      gx += a.x * b.x + a.y * b.y;   // conj(g) r
-      gy += a.x * b.y - a.y * b.x;
+      gg = fma(a.x, a.x, fma(a.y, a.y, gg));
+      gx = fma(a.x, b.x, fma(a.y, b.y, gx));   // conj(g) r
+      gy = fma(a.x, b.y, fma(-a.y, b.x, gy));
       Hc[(long long)i * nb + c] = b;
     }
 #pragma unroll
@@ -399,15 +436,13 @@ void launch_sweep(const SweepArgs& p, cudaStream_t s) {
   GFCC_LAUNCH_CHECK();
 }
 
-// rows per chunk of the CGS sweeps: at least 256 chunks and two waves of blocks (two resident blocks
-// per SM), with the chunk count trimmed so that the blocks fill their last wave
+// rows per chunk of the dot products of the FP64 basis and of norms: two whole waves of blocks (two resident per SM), short vectors in
+// chunks of at least 16 rows (a third, partial wave cost 11 % at 560 columns of 3,836 rows; one chunk of 64 rows for
+// 1024 columns of 52 left most SMs without a block)
 long long cgs_rows(long long D, int nb) {
   const long long gx = (nb + MD_TX - 1) / MD_TX, slots = 152LL * 2;
-  long long nchunk = std::max<long long>(256, 2 * slots / gx);
-  nchunk = std::max<long long>(1, (nchunk * gx + slots - 1) / slots * slots / gx);
-  // short vectors: chunks of 16 rows rather than leave SMs without a block (D = 52, 1024 columns: one chunk of 64
-  // rows was 32 blocks)
-  return std::max<long long>(D < 4096 ? 16 : 64, (D + nchunk - 1) / nchunk);
+  const long long nchunk = std::max<long long>(1, 2 * slots / gx);
+  return std::max<long long>(16, (D + nchunk - 1) / nchunk);
 }
 
 // h[c*hld + hoff + i] = sum_chunk partial[chunk][i][c], also set in or added to the Hessenberg column Hc (entry
@@ -458,15 +493,15 @@ __global__ void __launch_bounds__(256) update_kernel(const VT* __restrict__ V, l
       for (int u = 0; u < 4; ++u) {
         const VT vv = V[(long long)(i + u) * vstride + t];
         const R hx = (R)hc[i + u].x, hy = (R)hc[i + u].y;
-        sx[u] += vv.x * hx - vv.y * hy;
-        sy[u] += vv.x * hy + vv.y * hx;
+        sx[u] = fma(vv.x, hx, fma(-vv.y, hy, sx[u]));
+        sy[u] = fma(vv.x, hy, fma(vv.y, hx, sy[u]));
       }
     }
     for (; i < nv; ++i) {
       const VT vv = V[(long long)i * vstride + t];
       const R hx = (R)hc[i].x, hy = (R)hc[i].y;
-      sx[0] += vv.x * hx - vv.y * hy;
-      sy[0] += vv.x * hy + vv.y * hx;
+      sx[0] = fma(vv.x, hx, fma(-vv.y, hy, sx[0]));
+      sy[0] = fma(vv.x, hy, fma(vv.y, hx, sy[0]));
     }
     W[t].x -= (sx[0] + sx[1]) + (sx[2] + sx[3]);
     W[t].y -= (sy[0] + sy[1]) + (sy[2] + sy[3]);
@@ -498,7 +533,10 @@ struct ElGrid {
 ElGrid el_grid(long long D, int nb) {
   const int cw = nb >= 32 ? 32 : nb > 8 ? 16 : nb > 4 ? 8 : 4;
   const long long gx = (nb + cw - 1) / cw, rows = EL_T / cw;
-  const long long gy = std::max<long long>(1, std::min<long long>((D + rows - 1) / rows, std::max<long long>(1, 152LL * 24 / gx)));
+  // the same number of row steps for every block (up to the last)
+  const long long most = std::max<long long>(1, 152LL * 24 / gx);
+  const long long steps = std::max<long long>(1, (D + rows * most - 1) / (rows * most));
+  const long long gy = std::max<long long>(1, (D + rows * steps - 1) / (rows * steps));
   return {dim3((unsigned)gx, (unsigned)std::min<long long>(gy, 65535)), dim3((unsigned)cw, (unsigned)(EL_T / cw))};
 }
 
@@ -710,14 +748,14 @@ __global__ void __launch_bounds__(EL_T) correct_kernel(const VT* __restrict__ V,
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
         const VT vv = V[(long long)(i + u) * vstride + t], yy = y[(long long)(i + u) * nb + c];
-        sr[u] += vv.x * yy.x - vv.y * yy.y;
-        si[u] += vv.x * yy.y + vv.y * yy.x;
+        sr[u] = fma(vv.x, yy.x, fma(-vv.y, yy.y, sr[u]));
+        si[u] = fma(vv.x, yy.y, fma(vv.y, yy.x, si[u]));
       }
     }
     for (; i < nv; ++i) {
       const VT vv = V[(long long)i * vstride + t], yy = y[(long long)i * nb + c];
-      sr[0] += vv.x * yy.x - vv.y * yy.y;
-      si[0] += vv.x * yy.y + vv.y * yy.x;
+      sr[0] = fma(vv.x, yy.x, fma(-vv.y, yy.y, sr[0]));
+      si[0] = fma(vv.x, yy.y, fma(vv.y, yy.x, si[0]));
     }
     VT s;
     s.x = (sr[0] + sr[1]) + (sr[2] + sr[3]);
@@ -772,11 +810,11 @@ __global__ void nonfinite_cplx_kernel(const cplx* x, long long n, int* flag) {
 // column norms of a batch-minor block: out[c] = ||W_c||  (device array)
 template <typename VT>
 static void col_norms(const VT* W, long long D, int nb, double* out, DBuf<cplx>& partial, cudaStream_t s) {
-  const long long rows = std::max<long long>(256, (D + 511) / 512);
+  const long long rows = cgs_rows(D, nb);
   const int nchunk = (int)((D + rows - 1) / rows);
   partial.alloc((long long)nchunk * nb);
   dim3 grid((nb + MD_TX - 1) / MD_TX, nchunk);
-  multidot_kernel<VT, 4><<<grid, dim3(MD_TX, MD_TY), 0, s>>>(W, 0, 1, W, D, nb, rows, partial.p);
+  norm_partial_kernel<VT><<<grid, dim3(MD_TX, MD_TY), 0, s>>>(W, D, nb, rows, partial.p);
   GFCC_LAUNCH_CHECK();
   reduce_norm_kernel<<<(nb + 31) / 32, dim3(32, 8), 0, s>>>(partial.p, nchunk, nb, out);
   GFCC_LAUNCH_CHECK();
@@ -862,15 +900,14 @@ static void gmres_impl(gfcc_ctx* c, const cplx* Bin, cplx* Xout, cplx* Rout, con
   shw.alloc(nb0);
   flag.alloc(1);
   {  // chunk partial sums of the Gram-Schmidt sweeps and norms, at their largest (no regrowth per step)
-    const long long rows_cn = std::max<long long>(256, (D + 511) / 512);
-    long long md = 0;   // the chunk count of the sweeps depends on the batch width
+    long long md = 0, el = 0;   // the chunk counts depend on the batch width
     for (int b = 1; b <= nb0; ++b) {
       md = std::max(md, (D + cgs_rows(D, b) - 1) / cgs_rows(D, b) * b);
       md = std::max(md, (D + sweep_rows(D, b) - 1) / sweep_rows(D, b) * b);
-      md = std::max(md, (long long)el_grid(D, b).grid.y * b);
+      el = std::max(el, (long long)el_grid(D, b).grid.y * b);   // one sum per chunk
     }
     const int nq = std::max(std::min(k + 1, MD_MAXV), 2 * std::min(k, MD_MAXV) + 2);   // sums per chunk
-    partial.alloc(std::max(md * nq, (D + rows_cn - 1) / rows_cn * nb0));
+    partial.alloc(std::max(md * nq, el));
   }
   GFCC_CUDA(cudaMemcpyAsync(Bw.p, Bin, sizeof(cplx) * D * nb0, cudaMemcpyDeviceToDevice, s));
   GFCC_CUDA(cudaMemcpyAsync(shw.p, shifts_dev, sizeof(cplx) * nb0, cudaMemcpyDeviceToDevice, s));

@@ -52,7 +52,7 @@ __global__ void append_cols_kernel(const cplx* __restrict__ src, int lds, const 
 __global__ void house_kernel(const cplx* __restrict__ x, int len, cplx* __restrict__ v, double* __restrict__ tau) {
   __shared__ double red[256];
   double s = 0.0;
-  for (int i = threadIdx.x; i < len; i += blockDim.x) s += x[i].x * x[i].x + x[i].y * x[i].y;
+  for (int i = threadIdx.x; i < len; i += blockDim.x) s = fma(x[i].x, x[i].x, fma(x[i].y, x[i].y, s));
   red[threadIdx.x] = s;
   __syncthreads();
   for (int w = 128; w > 0; w >>= 1) {
@@ -92,8 +92,8 @@ __global__ void house_left2_kernel(cplx* __restrict__ A, long long lda, int c0a,
   cplx sdot = cz();
   for (int i = threadIdx.x; i < len; i += blockDim.x) {
     const cplx vv = v[i], aa = a[i];
-    sdot.x += vv.x * aa.x + vv.y * aa.y;
-    sdot.y += vv.x * aa.y - vv.y * aa.x;
+    sdot.x = fma(vv.x, aa.x, fma(vv.y, aa.y, sdot.x));
+    sdot.y = fma(vv.x, aa.y, fma(-vv.y, aa.x, sdot.y));
   }
   red[threadIdx.x] = sdot;
   __syncthreads();
@@ -166,8 +166,8 @@ __global__ void house_rows_kernel(cplx* __restrict__ Y, long long ldy, long long
   cplx sdot = cz();
   for (int k = 0; k < len; ++k) {
     const cplx vv = v[k], yy = Y[(long long)(r0 + k) * ldy + n];
-    sdot.x += vv.x * yy.x + vv.y * yy.y;
-    sdot.y += vv.x * yy.y - vv.y * yy.x;
+    sdot.x = fma(vv.x, yy.x, fma(vv.y, yy.y, sdot.x));
+    sdot.y = fma(vv.x, yy.y, fma(-vv.y, yy.x, sdot.y));
   }
   const double t = *tau;
   for (int k = 0; k < len; ++k) {
@@ -648,7 +648,7 @@ __global__ void resnorm_kernel(const cplx* __restrict__ C, long long ldc, int qn
   double s = 0.0;
   for (int r = 0; r < qn; ++r) {
     const cplx d = cuCsub(C[(long long)r * ldc + n], RB[r + (long long)p * qn]);
-    s += d.x * d.x + d.y * d.y;
+    s = fma(d.x, d.x, fma(d.y, d.y, s));
   }
   res[n] = sqrt(s) / bn[p];
 }
@@ -718,7 +718,7 @@ __global__ void colnorms_partial_kernel(const cplx* __restrict__ Y, int nc, long
   if (c < nc)
     for (long long nu = r0 + threadIdx.y; nu < r1; nu += PTY) {
       const cplx a = Y[nu * nc + c];
-      acc += a.x * a.x + a.y * a.y;
+      acc = fma(a.x, a.x, fma(a.y, a.y, acc));
     }
   red[threadIdx.y][threadIdx.x] = acc;
   __syncthreads();
@@ -747,8 +747,8 @@ __global__ void pdot_kernel(const cplx* __restrict__ Y, int nc, long long D, int
 #pragma unroll 4
     for (long long nu = r0 + threadIdx.y; nu < r1; nu += PTY) {
       const cplx a = Y[nu * nc + c0 + i], b = Y[nu * nc + j];
-      acc.x += a.x * b.x + a.y * b.y;
-      acc.y += a.x * b.y - a.y * b.x;
+      acc.x = fma(a.x, b.x, fma(a.y, b.y, acc.x));
+      acc.y = fma(a.x, b.y, fma(-a.y, b.x, acc.y));
     }
   red[threadIdx.y][i] = acc;
   __syncthreads();
@@ -783,6 +783,29 @@ __global__ void preduce_kernel(const cplx* __restrict__ partial, int nchunk, int
 // sum |Y[nu][j]|^2. Lane i holds panel column c0 + i; each warp takes PU rows per step (independent
 // shuffle reductions in flight), block (32, PTY).
 constexpr int PU = 4;
+// Sums over the 32 lanes of the components of PU = 4 complex numbers s: the eight values are halved between lane pairs
+// while they are summed (9 additions instead of 40: FP64 additions are what bounds this kernel; D = 56,580, 32-column
+// panels: 73 -> 40 us a launch), after which lanes
+// with lane >> 2 == 2 u + component hold the total of component (0: re, 1: im) of s[u].
+__device__ __forceinline__ double warp_sum4(const cplx (&s)[PU], int lane) {
+  static_assert(PU == 4, "four rows");
+  const bool h16 = lane & 16, h8 = lane & 8, h4 = lane & 4;
+  cplx t0 = h16 ? s[2] : s[0], t1 = h16 ? s[3] : s[1];
+  const cplx o0 = h16 ? s[0] : s[2], o1 = h16 ? s[1] : s[3];
+  t0.x += __shfl_xor_sync(0xffffffffu, o0.x, 16);
+  t0.y += __shfl_xor_sync(0xffffffffu, o0.y, 16);
+  t1.x += __shfl_xor_sync(0xffffffffu, o1.x, 16);
+  t1.y += __shfl_xor_sync(0xffffffffu, o1.y, 16);
+  cplx t = h8 ? t1 : t0;
+  const cplx o = h8 ? t0 : t1;
+  t.x += __shfl_xor_sync(0xffffffffu, o.x, 8);
+  t.y += __shfl_xor_sync(0xffffffffu, o.y, 8);
+  double v = h4 ? t.y : t.x;
+  v += __shfl_xor_sync(0xffffffffu, h4 ? t.x : t.y, 4);
+  v += __shfl_xor_sync(0xffffffffu, v, 2);
+  v += __shfl_xor_sync(0xffffffffu, v, 1);
+  return v;
+}
 __global__ void pupdate_kernel(cplx* __restrict__ Y, cplx* __restrict__ MY, int nc, long long D, int c0, int n,
                                int j, long long rows, const cplx* __restrict__ h, int mode,
                                cplx* __restrict__ partial) {
@@ -792,28 +815,21 @@ __global__ void pupdate_kernel(cplx* __restrict__ Y, cplx* __restrict__ MY, int 
   const cplx hi = i < n ? h[i] : cz();
   cplx acc = cz();
   for (long long base = r0 + (long long)threadIdx.y * PU; base < r1; base += (long long)PTY * PU) {
-    cplx a[PU], y[PU];
-    double sx[PU], sy[PU];
+    cplx a[PU], y[PU], s[PU];
 #pragma unroll
     for (int u = 0; u < PU; ++u) {
       const long long nu = base + u;
       const bool in = nu < r1;
       a[u] = (in && i < n) ? Y[nu * nc + c0 + i] : cz();
-      y[u] = in ? Y[nu * nc + j] : cz();   // read by every lane before lane 0 writes it (the shuffles order them)
-      sx[u] = a[u].x * hi.x - a[u].y * hi.y;
-      sy[u] = a[u].x * hi.y + a[u].y * hi.x;
+      y[u] = in ? Y[nu * nc + j] : cz();   // read by every lane before lane 0 writes it
+      s[u] = make_cuDoubleComplex(a[u].x * hi.x - a[u].y * hi.y, a[u].x * hi.y + a[u].y * hi.x);
     }
-    for (int off = 16; off > 0; off >>= 1) {
-#pragma unroll
-      for (int u = 0; u < PU; ++u) {
-        sx[u] += __shfl_xor_sync(0xffffffffu, sx[u], off);
-        sy[u] += __shfl_xor_sync(0xffffffffu, sy[u], off);
-      }
-    }
+    double v = warp_sum4(s, i);
+    __syncwarp();
 #pragma unroll
     for (int u = 0; u < PU; ++u) {
-      y[u].x -= sx[u];
-      y[u].y -= sy[u];
+      y[u].x -= __shfl_sync(0xffffffffu, v, 8 * u);
+      y[u].y -= __shfl_sync(0xffffffffu, v, 8 * u + 4);
       if (i == 0 && base + u < r1) Y[(base + u) * nc + j] = y[u];
     }
     if (MY) {
@@ -821,29 +837,19 @@ __global__ void pupdate_kernel(cplx* __restrict__ Y, cplx* __restrict__ MY, int 
       for (int u = 0; u < PU; ++u) {
         const long long nu = base + u;
         const cplx b = (nu < r1 && i < n) ? MY[nu * nc + c0 + i] : cz();
-        sx[u] = b.x * hi.x - b.y * hi.y;
-        sy[u] = b.x * hi.y + b.y * hi.x;
+        s[u] = make_cuDoubleComplex(b.x * hi.x - b.y * hi.y, b.x * hi.y + b.y * hi.x);
       }
-      for (int off = 16; off > 0; off >>= 1) {
-#pragma unroll
-        for (int u = 0; u < PU; ++u) {
-          sx[u] += __shfl_xor_sync(0xffffffffu, sx[u], off);
-          sy[u] += __shfl_xor_sync(0xffffffffu, sy[u], off);
-        }
-      }
-      if (i == 0) {
-#pragma unroll
-        for (int u = 0; u < PU; ++u)
-          if (base + u < r1) { MY[(base + u) * nc + j].x -= sx[u]; MY[(base + u) * nc + j].y -= sy[u]; }
-      }
+      v = warp_sum4(s, i);
+      const long long nu = base + (i >> 3);   // lanes 0, 4, 8, ...: one component of a row each
+      if ((i & 3) == 0 && nu < r1) reinterpret_cast<double*>(MY + nu * nc + j)[(i >> 2) & 1] -= v;
     }
 #pragma unroll
     for (int u = 0; u < PU; ++u) {
       if (mode == 0) {
-        acc.x += a[u].x * y[u].x + a[u].y * y[u].y;
-        acc.y += a[u].x * y[u].y - a[u].y * y[u].x;
+        acc.x = fma(a[u].x, y[u].x, fma(a[u].y, y[u].y, acc.x));
+        acc.y = fma(a[u].x, y[u].y, fma(-a[u].y, y[u].x, acc.y));
       } else if (i == 0) {
-        acc.x += y[u].x * y[u].x + y[u].y * y[u].y;
+        acc.x = fma(y[u].x, y[u].x, fma(y[u].y, y[u].y, acc.x));
       }
     }
   }

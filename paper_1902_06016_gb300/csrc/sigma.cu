@@ -69,8 +69,8 @@ __global__ void combine_kernel(const cplx* __restrict__ X, cplx* __restrict__ Y,
     double dre = diag[nu], dim = 0.0;
     if (shift) { dre += shift[c].x; dim = shift[c].y; }
     cplx y = Y[t];
-    y.x += dre * x.x - dim * x.y;
-    y.y += dre * x.y + dim * x.x;
+    y.x = fma(dre, x.x, fma(-dim, x.y, y.x));
+    y.y = fma(dre, x.y, fma(dim, x.x, y.y));
     if (nu >= o && CT) {
       long long r = nu - o;
       int pij = (int)(r / v), a = (int)(r % v);
@@ -128,8 +128,8 @@ __global__ void __launch_bounds__(128) dense_sigma_kernel(const double* __restri
   if (!on || ks != 0) return;
   if (shift) {
     const cplx s = shift[c], v = x[nu * sk];
-    re += s.x * v.x - s.y * v.y;
-    im += s.x * v.y + s.y * v.x;
+    re = fma(s.x, v.x, fma(-s.y, v.y, re));
+    im = fma(s.x, v.y, fma(s.y, v.x, im));
   }
   Y[nu * sk + c * sc] = make_cuDoubleComplex(re, im);
 }
