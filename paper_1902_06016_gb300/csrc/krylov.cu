@@ -48,7 +48,7 @@ void with_nv(int nv, F&& f) {
 // shares of 8 the groups of one warp scheduler held 14 of 22 vectors, those of another 8). Bound by the FP64 pipe:
 // the products go into the sums by two multiply-adds per component (a sum of products added on would be a product, a
 // multiply-add and an addition). 560 columns of D = 3,836, 17 to 28 vectors: 675 -> 523 us; update_kernel 382 -> 246 us
-// (92 % of the FP64 rate); norms 75 us -> 15.
+// (92 % of the FP64 rate); norms 77 us -> 12.
 template <int NV> struct MdGroups {
   static constexpr int IG = NV >= 16 ? NV / 8 : 1;
   static constexpr int NPG = NV / IG;

@@ -691,16 +691,16 @@ void regrow_cm(DBuf<cplx>& b, int old_ld, int new_ld, int alloc_cols, int nrows,
 }
 
 // FP64 arithmetic runs on a narrow pipe on this GPU: every product of the orthonormalisation above a
-// small size goes to the exact-slice tensor-core GEMM (6 slices, 53 bits per row). Fewer bits are
+// small size goes to the exact-slice tensor-core GEMM (7 slices of 7 bits, 48 bits per row). Fewer bits are
 // not enough: the residual basis resolves the solver-residual directions of Z = M S, about 1e-8 of
 // the columns' norms, and 41-bit products perturb them enough to spoil the refinement estimates.
 // The coefficients of the first Gram-Schmidt pass are the exception (ns = 4, 35 bits): the reconstruction
 // y = Q (C1 + C2) + y'' holds for whatever C1 the first update subtracts, and the second pass, whose
-// coefficients and both updates keep 6 slices, removes what a less accurate C1 leaves along Q. The
+// coefficients and both updates keep the 48 bits, removes what a less accurate C1 leaves along Q. The
 // second-pass and panel Gram products need the full accuracy even for the residual basis: with 34 bits the
 // refinement no longer converged (the model grew to the size limit).
-void fp64_accurate_zgemm(const ZGemmDesc& g, cudaStream_t s, int ns = 6) {
-  if ((double)g.M * (double)g.N * (double)g.K >= (double)(1 << 22) && g.batch == 1) zgemm_oz(g, ns, s);
+void fp64_accurate_zgemm(const ZGemmDesc& g, cudaStream_t s, int ns = OZ_SLICES_MOR, int bits = OZ_BITS_MOR) {
+  if ((double)g.M * (double)g.N * (double)g.K >= (double)(1 << 22) && g.batch == 1) zgemm_oz(g, ns, s, bits);
   else zgemm(g, s);
 }
 
@@ -1088,7 +1088,8 @@ std::vector<int> ortho_block(gfcc_ctx* c, const cplx* Bs, int cap, int n_cur, cp
       g.work = zgemm_work(c);
       {
         ProfScope pg(PROF_ORTHO_GRAM, 0.0, s);
-        fp64_accurate_zgemm(g, s, pass == 0 ? 4 : 6);
+        if (pass == 0) fp64_accurate_zgemm(g, s, 4, OZ_BITS);
+        else fp64_accurate_zgemm(g, s);
       }
       ZGemmDesc u;
       u.M = (int)D; u.N = ncols; u.K = np_;

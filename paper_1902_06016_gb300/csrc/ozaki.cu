@@ -24,32 +24,31 @@ int grid_for(long long n) {
 __device__ __forceinline__ unsigned long long abs_bits(double x) {
   return (unsigned long long)__double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFULL;
 }
-constexpr int OZ_BITS = 9, OZ_TOP = 8;   // bits per digit; the leading digit's weight is 2^(e - OZ_TOP)
 constexpr int ZERO_ROW = -100000;   // row exponent marker of a zero (or subnormal-only) row
 __device__ __forceinline__ int row_exponent(unsigned long long maxbits) {
   const int ex = (int)(maxbits >> 52);
   return ex == 0 ? ZERO_ROW : ex - 1022;
 }
-// Balanced base-512 digits of x relative to 2^(e - 8):  x ~ 2^(e-8) sum_{i<ns} a_i 2^(-9i), |a_i| <= 256.
+// Balanced digits of B bits of x relative to 2^(e - B + 1), for B = 9:  x ~ 2^(e-8) sum_{i<ns} a_i 2^(-9i), |a_i| <= 256.
 // V = round(|x| 2^(8 - e + 9(ns-1))) is formed exactly from the mantissa (|V| <= 2^(8 + 9(ns-1)) <= 2^62);
 // digit i is V / 2^(9(ns-1-i)) rounded half up, V keeps the remainder (|remainder| <= 2^(shift-1)), and
 // the signs of all digits follow x (so -x gives exactly the negated digits). a[i] holds digit i. The slice
 // count NS is a template argument (no predicated iterations, constant shifts).
-template <int NS>
+template <int NS, int B = OZ_BITS>
 __device__ __forceinline__ void digits_t(double x, int e, int (&a)[NS]) {
   const long long bits = __double_as_longlong(x);
   const int ex = (int)((bits >> 52) & 0x7FF);
   long long V = 0;
   if (ex != 0 && e != ZERO_ROW) {
     const long long m = (bits & 0xFFFFFFFFFFFFFLL) | 0x10000000000000LL;
-    const int t = ex - 1075 + OZ_TOP - e + OZ_BITS * (NS - 1);
+    const int t = ex - 1075 + (B - 1) - e + B * (NS - 1);
     if (t >= 0) V = m << t;
     else if (t > -62) V = (m + (1LL << (-t - 1))) >> (-t);
   }
   const bool neg = bits < 0;
 #pragma unroll
   for (int i = 0; i < NS; ++i) {
-    const int shift = OZ_BITS * (NS - 1 - i);
+    const int shift = B * (NS - 1 - i);
     const long long d = (i < NS - 1) ? ((V + (1LL << (shift - 1))) >> shift) : V;
     V -= d << shift;
     a[i] = neg ? -(int)d : (int)d;
@@ -157,6 +156,13 @@ void with_ns(int ns, F&& f) {
   }
 }
 
+// and the digits' width: 9 bits, or 7 with 7 slices (see OZ_BITS_MOR)
+template <typename F>
+void with_digits(int ns, int bits, F&& f) {
+  if (bits == OZ_BITS) with_ns(ns, [&](auto NSc) { f(NSc, std::integral_constant<int, OZ_BITS>{}); });
+  else f(std::integral_constant<int, OZ_SLICES_MOR>{}, std::integral_constant<int, OZ_BITS_MOR>{});
+}
+
 // ---- complex operands of zgemm_oz, sliced straight from their strided storage ----------------------
 // Operand element (r, k) = Z[r * s_r + k * s_k] (complex), conjugated when conj. Real rows written:
 //   mode 0 (left operand):  row r      = (Re, Im) interleaved along k
@@ -209,7 +215,7 @@ __global__ void __launch_bounds__(256) zrowmax_kernel(const cplx* __restrict__ Z
 
 // Slices of row r at (r ns + slot) kp (row-major), or with slot_major at (slot rows_total + r) kp, where
 // rows_total = R (mode 0) or 2R (mode 1): then slots 0..j of all rows form one contiguous block of rows.
-template <int NS>
+template <int NS, int B>
 __global__ void __launch_bounds__(256) zslice_kernel(const cplx* __restrict__ Z, long long s_r, long long s_k,
                                                      int conj, long long R, long long K, int mode,
                                                      const unsigned long long* __restrict__ rowmax, long long kp,
@@ -241,8 +247,8 @@ __global__ void __launch_bounds__(256) zslice_kernel(const cplx* __restrict__ Z,
       if (2 * k >= kp) break;
       const cplx v = tile[tr][tk];
       int are[NS], aim[NS];
-      digits_t<NS>(v.x, e, are);
-      digits_t<NS>(v.y, e, aim);
+      digits_t<NS, B>(v.x, e, are);
+      digits_t<NS, B>(v.y, e, aim);
 #pragma unroll
       for (int i = 0; i < NS; ++i) {
         {
@@ -271,6 +277,7 @@ struct OzOut {
   double beta = 0.0;
   cplx* C = nullptr;
   long long scm = 0, scn = 0;
+  int bits = OZ_BITS;   // of the operands' digits
   cplx alpha = {1.0, 0.0}, cbeta = {0.0, 0.0};
   // the common cases, so that the output pass spends no FP64 multiplications on them (set by set_kinds):
   // alpha_kind 1: alpha = 1, 2: alpha = -1, 0: general; beta_kind 0: beta = 0, 1: beta = 1, 2: general
@@ -287,21 +294,21 @@ __device__ __forceinline__ double scale_pow2(double x, int k) {
   if (k >= -1022 && k <= 1023) return x * __longlong_as_double((long long)(k + 1023) << 52);
   return ldexp(x, k);
 }
-// 2^e sum_d S_d 2^(9 (NS - 1 - d)) for NS <= 7 per-diagonal integer sums |S_d| < 2^43, rounded once to nearest: the sum
+// 2^e sum_d S_d 2^(B (NS - 1 - d)) for NS <= 7, B <= 9 per-diagonal integer sums |S_d| < 2^43, rounded once to nearest: the sum
 // is formed exactly (three diagonals at a time in 64 bits, joined in 128) and the double assembled from its bits.
 // Integer instructions throughout: the FP64 form (two conversions, a fused multiply-add, a scaling) held each
 // scheduler for 300 clocks per warp and bound the output passes.
-template <int NS>
+template <int NS, int B>
 __device__ __forceinline__ double diag_value(const long long (&S)[NS], int e) {
   constexpr int H = NS < 3 ? NS : 3, L = NS < 6 ? NS : 6;   // diagonals [0, H), [H, L), [L, NS)
   long long hi = 0, mid = 0, lo = 0;
 #pragma unroll
   for (int d = 0; d < NS; ++d) {
-    if (d < H) hi += S[d] * (1LL << (OZ_BITS * (H - 1 - d)));
-    else if (d < L) mid += S[d] * (1LL << (OZ_BITS * (L - 1 - d)));
+    if (d < H) hi += S[d] * (1LL << (B * (H - 1 - d)));
+    else if (d < L) mid += S[d] * (1LL << (B * (L - 1 - d)));
     else lo += S[d];
   }
-  const __int128 T = (__int128)hi * ((__int128)1 << (OZ_BITS * (NS - H))) + (__int128)mid * ((__int128)1 << (OZ_BITS * (NS - L))) + lo;
+  const __int128 T = (__int128)hi * ((__int128)1 << (B * (NS - H))) + (__int128)mid * ((__int128)1 << (B * (NS - L))) + lo;
   if (T == 0) return 0.0;
   const bool neg = T < 0;
   const unsigned __int128 A = neg ? -(unsigned __int128)T : (unsigned __int128)T;
@@ -309,9 +316,9 @@ __device__ __forceinline__ double diag_value(const long long (&S)[NS], int e) {
   const int n = ah ? 128 - __clzll((long long)ah) : 64 - __clzll((long long)al);   // bits
   // the top 64 bits, left-aligned, and whether anything is left below them
   const int sh = 128 - n;
-  const unsigned __int128 B = A << sh;
-  const unsigned long long top = (unsigned long long)(B >> 64);
-  const bool rest = (unsigned long long)B != 0;
+  const unsigned __int128 Al = A << sh;
+  const unsigned long long top = (unsigned long long)(Al >> 64);
+  const bool rest = (unsigned long long)Al != 0;
   unsigned long long m = top >> 11;                       // 53 bits
   const unsigned long long low = top & 0x7FFULL;          // and 11 more
   if (low > 0x400ULL || (low == 0x400ULL && (rest || (m & 1)))) ++m;   // to nearest, ties to even
@@ -400,7 +407,7 @@ __global__ void __launch_bounds__(256) oz_accumulate_kernel(const int* __restric
       if (!first) a = acc[t] + a;
       long long m, n;
       divmod<I>(t, Np, m, n);
-      const double v = scale_pow2(a, ea[m] + eb[n] - 2 * OZ_TOP);
+      const double v = scale_pow2(a, ea[m] + eb[n] - 2 * (o.bits - 1));
       if (writer) {
         double* p = o.out + m * o.ldo + n;
         *p = out_value_real(o, v, p);
@@ -416,8 +423,8 @@ __global__ void __launch_bounds__(256) oz_accumulate_kernel(const int* __restric
         ar = acc[tr] + ar;
         ai = acc[ti] + ai;
       }
-      const double re = scale_pow2(ar, ea[m] + eb[n] - 2 * OZ_TOP),
-                   im = scale_pow2(ai, ea[m] + eb[N + n] - 2 * OZ_TOP);
+      const double re = scale_pow2(ar, ea[m] + eb[n] - 2 * (o.bits - 1)),
+                   im = scale_pow2(ai, ea[m] + eb[N + n] - 2 * (o.bits - 1));
       if (writer) {
         cplx* p = o.C + m * o.scm + n * o.scn;
         *p = out_value(o, re, im, p);
@@ -458,22 +465,22 @@ __device__ __forceinline__ void diag_sums(const int* __restrict__ slabs, const O
   }
 }
 // One thread per output element (complex: both parts).
-template <int NS, bool STACK, bool CPLX, typename I>
+template <int NS, int B, bool STACK, bool CPLX, typename I>
 __global__ void __launch_bounds__(256) oz_output_kernel(const int* __restrict__ slabs, OzParts q, long long M,
                                                         long long Np, const int* __restrict__ ea,
                                                         const int* __restrict__ eb, OzOut o) {
   const long long N = CPLX ? Np / 2 : Np, total = M * N;
-  constexpr int sh = -2 * OZ_TOP - OZ_BITS * (NS - 1);
+  constexpr int sh = -2 * (B - 1) - B * (NS - 1);
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total;
        t += (long long)gridDim.x * blockDim.x) {
     long long m, n;
     divmod<I>(t, N, m, n);
     long long S[NS];
     diag_sums<NS, STACK>(slabs, q, M, Np, m, n, 0, 1, S);
-    const double re = diag_value<NS>(S, ea[m] + eb[n] + sh);
+    const double re = diag_value<NS, B>(S, ea[m] + eb[n] + sh);
     if constexpr (CPLX) {
       diag_sums<NS, STACK>(slabs, q, M, Np, m, N + n, 0, 1, S);
-      const double im = diag_value<NS>(S, ea[m] + eb[N + n] + sh);
+      const double im = diag_value<NS, B>(S, ea[m] + eb[N + n] + sh);
       cplx* p = o.C + m * o.scm + n * o.scn;
       *p = out_value(o, re, im, p);
     } else {
@@ -485,14 +492,14 @@ __global__ void __launch_bounds__(256) oz_output_kernel(const int* __restrict__ 
 // Outputs too small to occupy the GPU that have many K splits: 32 elements per block (coalesced along the row), whose
 // splits the eight warps share (a warp per element read one 4-byte sum per 32-byte sector: 87 us for a 270 x 32 product
 // with 100 splits).
-template <int NS, bool STACK, bool CPLX>
+template <int NS, int B, bool STACK, bool CPLX>
 __global__ void __launch_bounds__(256) oz_output_split_kernel(const int* __restrict__ slabs, OzParts q, long long M,
                                                               long long Np, const int* __restrict__ ea,
                                                               const int* __restrict__ eb, OzOut o) {
   __shared__ long long red[8][NS][32];
   __shared__ double val[2][32];
   const long long N = CPLX ? Np / 2 : Np, total = M * N;
-  constexpr int sh = -2 * OZ_TOP - OZ_BITS * (NS - 1);
+  constexpr int sh = -2 * (B - 1) - B * (NS - 1);
   const int x = threadIdx.x & 31, y = threadIdx.x >> 5;
   for (long long t0 = blockIdx.x * 32LL; t0 < total; t0 += gridDim.x * 32LL) {
     const long long t = t0 + x, m = t / N, n = t - m * N;
@@ -515,7 +522,7 @@ __global__ void __launch_bounds__(256) oz_output_split_kernel(const int* __restr
       if (y == 0 && on) {
 #pragma unroll
         for (int d = 0; d < NS; ++d) S[d] = red[0][d][x];
-        val[part][x] = diag_value<NS>(S, ea[m] + eb[col] + sh);
+        val[part][x] = diag_value<NS, B>(S, ea[m] + eb[col] + sh);
       }
       __syncthreads();
     }
@@ -536,15 +543,19 @@ void launch_output(int ns, int splits, cudaStream_t s, const int* slabs, const O
   const long long elements = M * (CPLX ? Np / 2 : Np);
   const bool split = elements < 152LL * 256 && splits > 4 * ns;
   const bool small = M * Np < (1LL << 32);
-  with_ns(ns, [&](auto NSc) {
-    constexpr int NS = decltype(NSc)::value;
+  auto launch = [&](auto NSc, auto Bc) {
+    constexpr int NS = decltype(NSc)::value, B = decltype(Bc)::value;
     if (split)
-      oz_output_split_kernel<NS, STACK, CPLX><<<(unsigned)((elements + 31) / 32), 256, 0, s>>>(slabs, q, M, Np, ea, eb, o);
+      oz_output_split_kernel<NS, B, STACK, CPLX><<<(unsigned)((elements + 31) / 32), 256, 0, s>>>(slabs, q, M, Np, ea, eb,
+                                                                                                o);
     else if (small)
-      oz_output_kernel<NS, STACK, CPLX, unsigned><<<grid_for(elements), 256, 0, s>>>(slabs, q, M, Np, ea, eb, o);
+      oz_output_kernel<NS, B, STACK, CPLX, unsigned><<<grid_for(elements), 256, 0, s>>>(slabs, q, M, Np, ea, eb, o);
     else
-      oz_output_kernel<NS, STACK, CPLX, unsigned long long><<<grid_for(elements), 256, 0, s>>>(slabs, q, M, Np, ea, eb, o);
-  });
+      oz_output_kernel<NS, B, STACK, CPLX, unsigned long long><<<grid_for(elements), 256, 0, s>>>(slabs, q, M, Np, ea, eb,
+                                                                                                o);
+  };
+  if constexpr (CPLX) with_digits(ns, o.bits, launch);
+  else with_ns(ns, [&](auto NSc) { launch(NSc, std::integral_constant<int, OZ_BITS>{}); });
   GFCC_LAUNCH_CHECK();
 }
 
@@ -646,7 +657,7 @@ void oz_run(const SlicedRows& A, const SlicedRows& B, long long M, long long Np,
       g.P = w.islabs.p;
       tc_gemm_exact(TcOperand(As, M, ld, ld), TcOperand(Bs + n0 * ld, nn, ld, ld), M, &g, 1, w.err.p, s, PROF_TC_SLICE);
       const int zeff = g.zs();
-      const double scale = ldexp(1.0, -OZ_BITS * d);
+      const double scale = ldexp(1.0, -o.bits * d);
       const int first = d == 0 ? 1 : 0;
       const int mode = d < ns - 1 ? 0 : (o.complex_out ? 2 : 1);
       const long long elements = mode == 2 ? M * (nn / 2) : M * nn;
@@ -754,7 +765,7 @@ struct ZSliceCache {   // slices of a left operand kept for several products wit
   bool valid = false;
   const cplx* A = nullptr;   // the operand they were made from (checked on reuse)
   long long M = 0, K = 0, sam = 0, sak = 0;
-  int ns = 0;
+  int ns = 0, bits = 0;
   bool conjA = false;
 };
 struct ZWork {          // buffers of zgemm_oz, kept between calls (grow-only)
@@ -779,17 +790,19 @@ void zgemm_work_free(gfcc_ctx* c) {
   c->zwork = nullptr;
 }
 
-void zgemm_oz(const ZGemmDesc& g, int ns, cudaStream_t s) {
+void zgemm_oz(const ZGemmDesc& g, int ns, cudaStream_t s, int bits) {
   const long long M = g.M, N = g.N, K = g.K;
   GFCC_CHECK(g.batch == 1, GFCC_ERR_ARG, "zgemm_oz: no batches");
   GFCC_CHECK(ns >= 2 && ns <= OZ_SLICES_MAX, GFCC_ERR_ARG, "zgemm_oz: 2..7 slices");
+  GFCC_CHECK(bits == OZ_BITS || (bits == OZ_BITS_MOR && ns == OZ_SLICES_MOR), GFCC_ERR_ARG, "zgemm_oz: digits");
   if (M <= 0 || N <= 0) return;
   ProfScope prof(PROF_OZ_ZGEMM, 8.0 * (double)M * (double)N * (double)K, s);
   ZWork local;
   ZWork& z = g.work ? *static_cast<ZWork*>(g.work) : local;
   ZSliceCache* cache = static_cast<ZSliceCache*>(g.a_cache);
   const bool reuse = cache && cache->valid && cache->A == g.A && cache->M == M && cache->K == K &&
-                     cache->sam == g.sam && cache->sak == g.sak && cache->ns == ns && cache->conjA == g.conjA;
+                     cache->sam == g.sam && cache->sak == g.sak && cache->ns == ns && cache->bits == bits &&
+                     cache->conjA == g.conjA;
   SlicedRows& sa = cache ? cache->sa : z.sa;
   SlicedRows& sb = z.sb;
   sa.rows = M; sa.kp = tc_pad_k(TcKind::BF16, 2 * K); sa.ns = ns; sa.reversed = false;
@@ -824,8 +837,9 @@ void zgemm_oz(const ZGemmDesc& g, int ns, cudaStream_t s) {
     zrowmax_kernel<<<dim3((unsigned)kt_in, (unsigned)((N + ZT_R - 1) / ZT_R)), 256, 0, s>>>(g.B, g.sbn, g.sbk, N, K, mxb.p);
     GFCC_LAUNCH_CHECK();
     if (!reuse) {
-      with_ns(ns, [&](auto NSc) {
-        zslice_kernel<decltype(NSc)::value><<<dim3((unsigned)kt, (unsigned)((M + ZT_R - 1) / ZT_R)), 256, 0, s>>>(
+      with_digits(ns, bits, [&](auto NSc, auto Bc) {
+        const dim3 grid((unsigned)kt, (unsigned)((M + ZT_R - 1) / ZT_R));
+        zslice_kernel<decltype(NSc)::value, decltype(Bc)::value><<<grid, 256, 0, s>>>(
             g.A, g.sam, g.sak, g.conjA ? 1 : 0, M, K, 0, mxa.p, sa.kp, 0,
             reinterpret_cast<__half*>(sa.slices.p), sa.expo.p);
       });
@@ -833,11 +847,12 @@ void zgemm_oz(const ZGemmDesc& g, int ns, cudaStream_t s) {
       if (cache) {
         cache->valid = true;
         cache->A = g.A; cache->M = M; cache->K = K; cache->sam = g.sam; cache->sak = g.sak;
-        cache->ns = ns; cache->conjA = g.conjA;
+        cache->ns = ns; cache->bits = bits; cache->conjA = g.conjA;
       }
     }
-    with_ns(ns, [&](auto NSc) {
-      zslice_kernel<decltype(NSc)::value><<<dim3((unsigned)kt, (unsigned)((N + ZT_R - 1) / ZT_R)), 256, 0, s>>>(
+    with_digits(ns, bits, [&](auto NSc, auto Bc) {
+      const dim3 grid((unsigned)kt, (unsigned)((N + ZT_R - 1) / ZT_R));
+      zslice_kernel<decltype(NSc)::value, decltype(Bc)::value><<<grid, 256, 0, s>>>(
           g.B, g.sbn, g.sbk, g.conjB ? 1 : 0, N, K, 1, mxb.p, sb.kp, stacked ? 0 : 1,
           reinterpret_cast<__half*>(sb.slices.p), sb.expo.p, stacked ? 1 : 0);
     });
@@ -850,6 +865,7 @@ void zgemm_oz(const ZGemmDesc& g, int ns, cudaStream_t s) {
   o.scn = g.scn;
   o.alpha = g.alpha;
   o.cbeta = g.beta;
+  o.bits = bits;
   o.set_kinds();
   OzWork& w = z.w;
   if (stacked) oz_run_stacked(sa, sb, M, 2 * N, o, w, s);

@@ -23,8 +23,14 @@
 
 namespace gfcc {
 
+constexpr int OZ_BITS = 9;         // bits per digit (the leading one: a bit fewer)
 constexpr int OZ_SLICES = 5;       // residual sigma: 44 bits per row
 constexpr int OZ_SLICES_MAX = 7;   // 62 bits per row: as accurate as an FP64 GEMM
+
+// The orthonormalisation of a reduced model (Gram and update products) stays on 7 slices of 7 bits (48 bits, 28 products
+// where 6 slices of 9 bits take 21): what its rounding leaves between Z and M S moves weak elements of the model's G by
+// up to 6e-8 of their size (benzene size, order 336), and models keep repeating the spectra of the models built so far.
+constexpr int OZ_BITS_MOR = 7, OZ_SLICES_MOR = 7;
 
 struct SlicedRows {
   DBuf<uint8_t> slices;   // f16 [rows][ns][kp] (order 0..ns-1, or reversed)
@@ -55,7 +61,7 @@ void oz_gemm(const SlicedRows& A, const SlicedRows& B, long long M, long long N,
 
 // Complex GEMM C = alpha op(A) op(B) + beta C (strided, see ZGemmDesc) evaluated as one real
 // exact-slice GEMM: K interleaves (re, im) and the N axis stacks the real and imaginary parts.
-void zgemm_oz(const ZGemmDesc& g, int ns, cudaStream_t s);
+void zgemm_oz(const ZGemmDesc& g, int ns, cudaStream_t s, int bits = OZ_BITS);
 // complex multiply-adds above which zgemm() uses zgemm_oz (GFCC_OZ_MIN_MACS overrides)
 double oz_min_macs();
 // bytes of int32 split sums up to which all diagonals of an exact product are kept side by side and
