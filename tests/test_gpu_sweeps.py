@@ -1,6 +1,6 @@
-"""Arnoldi sweeps of the FP32 basis with delayed re-orthogonalisation: batches of every block width (4, 8, 16 and 32
-columns, full and ragged), bases beyond the 32 vectors of one sweep, spaces smaller than the restart length (the basis
-breaks down) and a restart length of one."""
+"""Arnoldi sweeps of the FP32 basis with delayed re-orthogonalisation, and the dot products, updates and norms of the
+FP64 basis: batches of every block width (4, 8, 16 and 32 columns, full and ragged), bases beyond the 32 vectors of
+one sweep, spaces smaller than the restart length (the basis breaks down) and a restart length of one."""
 import numpy as np
 import pytest
 
@@ -17,7 +17,7 @@ def torch():
     return need_gpu()
 
 
-@pytest.mark.parametrize("prec", ["bf16", "tf32"])
+@pytest.mark.parametrize("prec", ["bf16", "tf32", "fp64", "fp64_tc"])
 @pytest.mark.parametrize("o,v,np_,nw,restart,eta", [
     (2, 1, 1, 1, 30, 0.05), (2, 1, 2, 3, 40, 0.05),
     (4, 8, 1, 1, 40, 0.005), (4, 8, 3, 1, 70, 0.005), (4, 8, 1, 5, 33, 0.005), (4, 8, 3, 3, 32, 0.005),
