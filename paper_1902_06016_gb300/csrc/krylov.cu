@@ -634,6 +634,8 @@ __global__ void __launch_bounds__(GV_T) arnoldi_finish_kernel(const cplx* __rest
   // lanes: 0 t.re, 1 t.im, 2 u.re, 3 u.im of  ca a + cb b  with complex coefficients split into components
   const bool isu = q >= 2, im = q & 1;
   cplx a = on ? col[0] : make_cuDoubleComplex(0.0, 0.0);
+  __syncwarp();           // every lane has read its column's first entry before lanes 0 and 1 replace it below; an entry
+                          // further down is replaced only after a shuffle that follows every lane's read of it
   constexpr int PF = 4;   // rotations loaded ahead of the serial chain
   for (int i0 = 0; i0 < j; i0 += PF) {
     cplx b[PF], s[PF];
