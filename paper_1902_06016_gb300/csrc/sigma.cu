@@ -176,6 +176,7 @@ void sigma_dense(gfcc_ctx* c, const cplx* X, cplx* Y, int nb, long long sk, long
 void ensure_workspace(gfcc_ctx* c, int nb) {
   if ((size_t)nb <= c->ws.nb_cap) return;
   const long long ov = (long long)c->o * c->v;
+  c->ws.nb_cap = 0;   // a failed allocation leaves no width ready
   c->ws.ut.alloc(2 * ov * c->o * (long long)nb);
   c->ws.ct.alloc(2 * ov * c->o * (long long)nb);
   c->ws.xe.alloc(2LL * c->v * nb);

@@ -746,6 +746,9 @@ static void lp_batch_buffers(gfcc_ctx* c, LpState& st, int nb, cudaStream_t s) {
   const int o = c->o, v = c->v;
   const long long ov = (long long)o * v, Pv = (long long)c->P * v;
   const long long nring = 2LL * o * nb, noo = 2LL * v * nb, nsm = 2LL * nb;
+  // no width is ready until all of this has succeeded: an allocation that fails leaves buffers that are gone, or new and
+  // not zeroed, and the next call (with a narrower batch, say) has to start over
+  st.nb_cap = st.nb_prep = 0;
   st.Bring.alloc(sizeof(T) * nring * st.Kr);
   st.Boo.alloc(sizeof(T) * noo * st.Kp);
   st.Bup.alloc(sizeof(T) * nsm * st.Kpv);
@@ -756,7 +759,6 @@ static void lp_batch_buffers(gfcc_ctx* c, LpState& st, int nb, cudaStream_t s) {
   st.up.alloc((long long)(v + o) * nsm);
   st.z1.alloc((long long)o * nsm);
   st.nb_cap = nb;
-  st.nb_prep = 0;
 }
 // K splits of the short-and-wide up product and the splits it writes
 template <TcKind K>
