@@ -608,7 +608,16 @@ void sigma_emulated(gfcc_ctx* c, const cplx* X, cplx* Y, int nb, const cplx* shi
   // columns at a time: as many as keep the int32 split sums of the ring product within 2 GB, at least 64, in
   // equal chunks. Small operators run all columns at once: at o = 14, v = 42 a 64-column chunk leaves most
   // SMs without a tile (560 columns: 9 chunks of 24 launches of 15 us).
-  const long long fit = (2LL << 30) / (4LL * (OZ_SLICES + 2) * ov * 2LL * o);
+  // A chunk takes about 2.4 times its split sums in all (digits, operands, outputs): where that is above half a gigabyte,
+  // the split sums also stay within an eighth of the memory that is free or already theirs.
+  const long long col = 4LL * (OZ_SLICES + 2) * ov * 2LL * o;   // bytes of split sums per column
+  long long budget = 2LL << 30;
+  if (nb > 64 && col * nb > (256LL << 20)) {
+    size_t freeb = device_free_bytes();
+    if (freeb == 0) freeb = 8ull << 30;
+    budget = std::min<long long>(budget, (long long)((freeb + 10 * st.work.islabs.n) / 8));
+  }
+  const long long fit = budget / col;
   const int most = (int)std::min<long long>(nb, std::max<long long>(64, fit));
   const int nchunks = (nb + most - 1) / most;
   const int chunk = (nb + nchunks - 1) / nchunks;
