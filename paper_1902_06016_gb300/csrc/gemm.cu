@@ -317,10 +317,14 @@ void dgemm(const GemmDesc& d, cudaStream_t s) {
 void zgemm(const ZGemmDesc& d, cudaStream_t s) {
   // Complex products of some size (the subspace projections of the reduced model, its evaluation) go to the
   // exact-slice tensor-core GEMM: 6 slices (53 bits per row) for the large ones, 7 (62 bits) for those whose extra
-  // slice costs little. 270 x 30 x 56,580: 8.3 ms on the FP64 pipe.
+  // slice costs little. 270 x 30 x 56,580: 8.3 ms on the FP64 pipe. A product that would be slow there (a billion
+  // multiply-adds, 8 ms at best) takes the scratch it needs; a smaller or shorter one stays on the FP64 pipe, which needs
+  // none, when memory is short.
   const double macs = (double)d.M * (double)d.N * (double)d.K;
-  if (d.batch == 1 && macs >= oz_min_macs() && d.M >= 16 && d.N >= 1 && d.K >= 64) {
-    zgemm_oz(d, macs >= 1e9 ? 6 : 7, s);
+  const int ns = macs >= 1e9 ? 6 : 7;
+  if (d.batch == 1 && macs >= oz_min_macs() && d.M >= 16 && d.N >= 1 && d.K >= 64 &&
+      ((macs >= 1e9 && d.K >= 256) || zgemm_oz_fits(d, ns))) {
+    zgemm_oz(d, ns, s);
     return;
   }
   Args<cplx> a{d.M, d.N, d.K, d.A, d.sam, d.sak, d.bsa, d.conjA, d.B, d.sbk, d.sbn, d.bsb, d.conjB,

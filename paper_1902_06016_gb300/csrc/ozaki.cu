@@ -169,7 +169,8 @@ void with_digits(int ns, int bits, F&& f) {
 //   mode 1 (right operand): row r      = (Re, -Im)    and row R + r = (Im, Re)
 // so that sum over the 2K real columns of left row m times right row n (or R + n) gives the real
 // (imaginary) part of the complex product. Tiles of 32 rows x 64 complex k go through shared memory
-// so that both the strided reads and the row-contiguous slice writes are coalesced.
+// so that both the strided reads and the row-contiguous slice writes are coalesced; the blocks walk the row
+// tiles (any number of rows).
 constexpr int ZT_R = 32, ZT_K = 64;
 
 __device__ __forceinline__ void load_ztile(const cplx* __restrict__ Z, long long s_r, long long s_k, int conj,
@@ -201,15 +202,18 @@ __global__ void __launch_bounds__(256) zrowmax_kernel(const cplx* __restrict__ Z
                                                       long long R, long long K,
                                                       unsigned long long* __restrict__ rowmax) {
   __shared__ cplx tile[ZT_R][ZT_K + 1];
-  const long long r0 = (long long)blockIdx.y * ZT_R, k0 = (long long)blockIdx.x * ZT_K;
-  load_ztile(Z, s_r, s_k, 0, R, K, r0, k0, tile);
-  __syncthreads();
+  const long long k0 = (long long)blockIdx.x * ZT_K;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int tr = warp; tr < ZT_R; tr += blockDim.x >> 5) {
-    unsigned long long mx = 0;
-    for (int tk = lane; tk < ZT_K; tk += 32) mx = max(mx, max(abs_bits(tile[tr][tk].x), abs_bits(tile[tr][tk].y)));
-    for (int off = 16; off > 0; off >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, off));
-    if (lane == 0 && r0 + tr < R && mx > 0) atomicMax(rowmax + r0 + tr, mx);
+  for (long long r0 = (long long)blockIdx.y * ZT_R; r0 < R; r0 += (long long)gridDim.y * ZT_R) {
+    load_ztile(Z, s_r, s_k, 0, R, K, r0, k0, tile);
+    __syncthreads();
+    for (int tr = warp; tr < ZT_R; tr += blockDim.x >> 5) {
+      unsigned long long mx = 0;
+      for (int tk = lane; tk < ZT_K; tk += 32) mx = max(mx, max(abs_bits(tile[tr][tk].x), abs_bits(tile[tr][tk].y)));
+      for (int off = 16; off > 0; off >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, off));
+      if (lane == 0 && r0 + tr < R && mx > 0) atomicMax(rowmax + r0 + tr, mx);
+    }
+    __syncthreads();
   }
 }
 
@@ -223,48 +227,51 @@ __global__ void __launch_bounds__(256) zslice_kernel(const cplx* __restrict__ Z,
                                                      int* __restrict__ expo, int slot_major = 0) {
   constexpr int ns = NS;
   __shared__ cplx tile[ZT_R][ZT_K + 1];
-  const long long r0 = (long long)blockIdx.y * ZT_R, k0 = (long long)blockIdx.x * ZT_K;
-  load_ztile(Z, s_r, s_k, conj, R, K, r0, k0, tile);
-  __syncthreads();
+  const long long k0 = (long long)blockIdx.x * ZT_K;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int tr = warp; tr < ZT_R; tr += blockDim.x >> 5) {
-    const long long r = r0 + tr;
-    if (r >= R) break;
-    const int e = row_exponent(rowmax[r]);
-    if (k0 == 0 && lane == 0) {
-      expo[r] = e == ZERO_ROW ? 0 : e;
-      if (mode == 1) expo[R + r] = e == ZERO_ROW ? 0 : e;
-    }
-    const long long rows_total = mode == 1 ? 2 * R : R;
-    // element offset of slot 0 of a row and the distance between its slots
-    const long long b0 = slot_major ? r * kp : r * (long long)ns * kp;
-    const long long b1 = slot_major ? (R + r) * kp : (R + r) * (long long)ns * kp;
-    const long long sstep = slot_major ? rows_total * kp : kp;
-    __half* o0 = out + b0;
-    __half* o1 = out + b1;
-    for (int tk = lane; tk < ZT_K; tk += 32) {
-      const long long k = k0 + tk;
-      if (2 * k >= kp) break;
-      const cplx v = tile[tr][tk];
-      int are[NS], aim[NS];
-      digits_t<NS, B>(v.x, e, are);
-      digits_t<NS, B>(v.y, e, aim);
+  for (long long r0 = (long long)blockIdx.y * ZT_R; r0 < R; r0 += (long long)gridDim.y * ZT_R) {
+    load_ztile(Z, s_r, s_k, conj, R, K, r0, k0, tile);
+    __syncthreads();
+    for (int tr = warp; tr < ZT_R; tr += blockDim.x >> 5) {
+      const long long r = r0 + tr;
+      if (r >= R) break;
+      const int e = row_exponent(rowmax[r]);
+      if (k0 == 0 && lane == 0) {
+        expo[r] = e == ZERO_ROW ? 0 : e;
+        if (mode == 1) expo[R + r] = e == ZERO_ROW ? 0 : e;
+      }
+      const long long rows_total = mode == 1 ? 2 * R : R;
+      // element offset of slot 0 of a row and the distance between its slots
+      const long long b0 = slot_major ? r * kp : r * (long long)ns * kp;
+      const long long b1 = slot_major ? (R + r) * kp : (R + r) * (long long)ns * kp;
+      const long long sstep = slot_major ? rows_total * kp : kp;
+      __half* o0 = out + b0;
+      __half* o1 = out + b1;
+      for (int tk = lane; tk < ZT_K; tk += 32) {
+        const long long k = k0 + tk;
+        if (2 * k >= kp) break;
+        const cplx v = tile[tr][tk];
+        int are[NS], aim[NS];
+        digits_t<NS, B>(v.x, e, are);
+        digits_t<NS, B>(v.y, e, aim);
 #pragma unroll
-      for (int i = 0; i < NS; ++i) {
-        {
-          const long long off = (long long)(reversed ? ns - 1 - i : i) * sstep + 2 * k;
-          if (mode == 0) {
-            *reinterpret_cast<__half2*>(o0 + off) = __halves2half2(__int2half_rn(are[i]),
-                                                                               __int2half_rn(aim[i]));
-          } else {
-            *reinterpret_cast<__half2*>(o0 + off) = __halves2half2(__int2half_rn(are[i]),
-                                                                               __int2half_rn(-aim[i]));
-            *reinterpret_cast<__half2*>(o1 + off) = __halves2half2(__int2half_rn(aim[i]),
-                                                                               __int2half_rn(are[i]));
+        for (int i = 0; i < NS; ++i) {
+          {
+            const long long off = (long long)(reversed ? ns - 1 - i : i) * sstep + 2 * k;
+            if (mode == 0) {
+              *reinterpret_cast<__half2*>(o0 + off) = __halves2half2(__int2half_rn(are[i]),
+                                                                                 __int2half_rn(aim[i]));
+            } else {
+              *reinterpret_cast<__half2*>(o0 + off) = __halves2half2(__int2half_rn(are[i]),
+                                                                                 __int2half_rn(-aim[i]));
+              *reinterpret_cast<__half2*>(o1 + off) = __halves2half2(__int2half_rn(aim[i]),
+                                                                                 __int2half_rn(are[i]));
+            }
           }
         }
       }
     }
+    __syncthreads();
   }
 }
 
@@ -790,6 +797,19 @@ void zgemm_work_free(gfcc_ctx* c) {
   c->zwork = nullptr;
 }
 
+bool zgemm_oz_fits(const ZGemmDesc& g, int ns) {
+  const double kp = (double)tc_pad_k(TcKind::F16, 2LL * g.K), out = 2.0 * (double)g.M * (double)g.N;
+  const double sums = 4.0 * ns * out;   // one split of every diagonal; beyond the limit, of one diagonal and its FP64 sum
+  const double need = 2.0 * ns * kp * ((double)g.M + 2.0 * g.N) + (sums <= oz_slab_bytes() ? sums : 12.0 * out);
+  if (need <= (double)(1LL << 30)) return true;
+  double have = (double)device_free_bytes();
+  if (g.work) {
+    const ZWork& z = *static_cast<const ZWork*>(g.work);
+    have += (double)(z.sa.slices.n + z.sb.slices.n) + 4.0 * (double)z.w.islabs.n + 8.0 * (double)z.w.acc.n;
+  }
+  return need <= 0.25 * have;
+}
+
 void zgemm_oz(const ZGemmDesc& g, int ns, cudaStream_t s, int bits) {
   const long long M = g.M, N = g.N, K = g.K;
   GFCC_CHECK(g.batch == 1, GFCC_ERR_ARG, "zgemm_oz: no batches");
@@ -827,18 +847,19 @@ void zgemm_oz(const ZGemmDesc& g, int ns, cudaStream_t s, int bits) {
     GFCC_CUDA(cudaMemsetAsync(mxb.p, 0, sizeof(unsigned long long) * N, s));
     const long long kt = (sa.kp / 2 + ZT_K - 1) / ZT_K;   // k tiles covering the padded width
     const long long kt_in = (K + ZT_K - 1) / ZT_K;
-    GFCC_CHECK((M + ZT_R - 1) / ZT_R <= 65535 && (N + ZT_R - 1) / ZT_R <= 65535, GFCC_ERR_ARG, "zgemm_oz: too many rows");
+    // row tiles on grid.y, which ends at 65535 (2,097,120 rows): the blocks walk what is beyond
+    const unsigned rtA = (unsigned)std::min<long long>((M + ZT_R - 1) / ZT_R, 65535);
+    const unsigned rtB = (unsigned)std::min<long long>((N + ZT_R - 1) / ZT_R, 65535);
     // A(m, k) = A[m sam + k sak]; B rows n: B(k, n) = B[k sbk + n sbn] -> r = n, s_r = sbn, s_k = sbk
     if (!reuse) {
-      zrowmax_kernel<<<dim3((unsigned)kt_in, (unsigned)((M + ZT_R - 1) / ZT_R)), 256, 0, s>>>(g.A, g.sam, g.sak, M, K,
-                                                                                           mxa.p);
+      zrowmax_kernel<<<dim3((unsigned)kt_in, rtA), 256, 0, s>>>(g.A, g.sam, g.sak, M, K, mxa.p);
       GFCC_LAUNCH_CHECK();
     }
-    zrowmax_kernel<<<dim3((unsigned)kt_in, (unsigned)((N + ZT_R - 1) / ZT_R)), 256, 0, s>>>(g.B, g.sbn, g.sbk, N, K, mxb.p);
+    zrowmax_kernel<<<dim3((unsigned)kt_in, rtB), 256, 0, s>>>(g.B, g.sbn, g.sbk, N, K, mxb.p);
     GFCC_LAUNCH_CHECK();
     if (!reuse) {
       with_digits(ns, bits, [&](auto NSc, auto Bc) {
-        const dim3 grid((unsigned)kt, (unsigned)((M + ZT_R - 1) / ZT_R));
+        const dim3 grid((unsigned)kt, rtA);
         zslice_kernel<decltype(NSc)::value, decltype(Bc)::value><<<grid, 256, 0, s>>>(
             g.A, g.sam, g.sak, g.conjA ? 1 : 0, M, K, 0, mxa.p, sa.kp, 0,
             reinterpret_cast<__half*>(sa.slices.p), sa.expo.p);
@@ -851,7 +872,7 @@ void zgemm_oz(const ZGemmDesc& g, int ns, cudaStream_t s, int bits) {
       }
     }
     with_digits(ns, bits, [&](auto NSc, auto Bc) {
-      const dim3 grid((unsigned)kt, (unsigned)((N + ZT_R - 1) / ZT_R));
+      const dim3 grid((unsigned)kt, rtB);
       zslice_kernel<decltype(NSc)::value, decltype(Bc)::value><<<grid, 256, 0, s>>>(
           g.B, g.sbn, g.sbk, g.conjB ? 1 : 0, N, K, 1, mxb.p, sb.kp, stacked ? 0 : 1,
           reinterpret_cast<__half*>(sb.slices.p), sb.expo.p, stacked ? 1 : 0);

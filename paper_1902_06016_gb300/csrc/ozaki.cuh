@@ -62,6 +62,9 @@ void oz_gemm(const SlicedRows& A, const SlicedRows& B, long long M, long long N,
 // Complex GEMM C = alpha op(A) op(B) + beta C (strided, see ZGemmDesc) evaluated as one real
 // exact-slice GEMM: K interleaves (re, im) and the N axis stacks the real and imaginary parts.
 void zgemm_oz(const ZGemmDesc& g, int ns, cudaStream_t s, int bits = OZ_BITS);
+// whether the digits and split sums of zgemm_oz take at most 1 GB or a quarter of the memory that is free (with what
+// the workspace holds already)
+bool zgemm_oz_fits(const ZGemmDesc& g, int ns);
 // complex multiply-adds above which zgemm() uses zgemm_oz (GFCC_OZ_MIN_MACS overrides)
 double oz_min_macs();
 // bytes of int32 split sums up to which all diagonals of an exact product are kept side by side and
