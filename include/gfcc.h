@@ -52,7 +52,8 @@ typedef struct gfcc_ctx* gfcc_t;
 
 /* Antisymmetrised two-electron integral blocks <pq||rs>, real, row-major, occupied index range
  * first: oooo[i][j][k][l], ooov[i][j][k][a], oovv[i][j][a][b], ovov[i][a][j][b], ovvv[i][a][b][c].
- * Host or device pointers. (No vvvv block is needed by the IP space.) */
+ * The arrays have the antisymmetry of <pq||rs> in p, q and in r, s wherever both indices of a pair are of one
+ * kind (the build reads one element of each antisymmetric pair). Host or device pointers. (No vvvv block is needed by the IP space.) */
 typedef struct {
   const double* oooo;
   const double* ooov;

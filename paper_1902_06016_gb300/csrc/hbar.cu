@@ -249,11 +249,14 @@ int grid_for(long long n) {
 }
 
 // ---- packed antisymmetric index pairs ------------------------------------------------------------
-// The integrals <pq||rs> and the amplitudes are antisymmetric in p, q and in r, s (the input contract), so that a sum
-// over two contracted indices of the same kind is twice the sum over e < f, and a result antisymmetric in i, j needs
-// only i < j. Packed index of a < b out of n: a n - a (a + 1) / 2 + b - a - 1 (contiguous in b).
+// The integrals <pq||rs> are antisymmetric in p, q and in r, s (the input contract), so that a sum over two contracted
+// indices of the same kind is twice the sum over e < f, and a result antisymmetric in i, j needs only i < j. The
+// amplitudes are packed as (tau^ef - tau^fe) / 2 (or over m, n): beside antisymmetric integrals that is what the full
+// sum takes of them, whatever the array holds (a caller may have moved one element of it alone). Packed index of a < b
+// out of n: a n - a (a + 1) / 2 + b - a - 1 (contiguous in b).
 __device__ __forceinline__ long long tri(int a, int b, int n) { return (long long)a * n - (long long)a * (a + 1) / 2 + b - a - 1; }
-// dst[r][tri(e, f)] = src[r][e][f], e < f: a warp per (r, e)
+// dst[r][tri(e, f)] = src[r][e][f], or (src[r][e][f] - src[r][f][e]) / 2 with ANTI, e < f: a warp per (r, e)
+template <bool ANTI>
 __global__ void __launch_bounds__(256) pack_last_kernel(const double* __restrict__ src, long long rows, int v,
                                                         double* __restrict__ dst) {
   const int lane = threadIdx.x & 31;
@@ -262,18 +265,21 @@ __global__ void __launch_bounds__(256) pack_last_kernel(const double* __restrict
     const long long r = q / v;
     const int e = (int)(q - r * v);
     const double* s = src + q * v;
+    const double* st = src + r * v * v + e;   // column e of the same block
     double* d = dst + r * V + tri(e, e + 1, v);
-    for (int f = e + 1 + lane; f < v; f += 32) d[f - e - 1] = s[f];
+    for (int f = e + 1 + lane; f < v; f += 32) d[f - e - 1] = ANTI ? 0.5 * (s[f] - st[(long long)f * v]) : s[f];
   }
 }
-// dst[tri(i, j)][k] = src[i][j][k], i < j
+// dst[tri(i, j)][k] = src[i][j][k], or (src[i][j][k] - src[j][i][k]) / 2 with ANTI, i < j
+template <bool ANTI>
 __global__ void __launch_bounds__(256) take_pairs_kernel(const double* __restrict__ src, int o, long long n,
                                                          double* __restrict__ dst) {
   const int i = blockIdx.y / o, j = blockIdx.y % o;
   if (i >= j) return;
   const double* s = src + ((long long)i * o + j) * n;
+  const double* st = src + ((long long)j * o + i) * n;
   double* d = dst + tri(i, j, o) * n;
-  for (long long k = blockIdx.x * 256LL + threadIdx.x; k < n; k += gridDim.x * 256LL) d[k] = s[k];
+  for (long long k = blockIdx.x * 256LL + threadIdx.x; k < n; k += gridDim.x * 256LL) d[k] = ANTI ? 0.5 * (s[k] - st[k]) : s[k];
 }
 // W[r][i][j] += R[r][tri(i, j)] for i < j and W[r][j][i] -= the same
 __global__ void add_pairs_kernel(const double* __restrict__ R, long long rows, int o, double* __restrict__ W) {
@@ -299,14 +305,17 @@ __global__ void add_pair_pairs_kernel(const double* __restrict__ R, int o, doubl
     W[t] += s * R[tri(m, q, o) * np + tri(i, j, o)];
   }
 }
+template <bool ANTI = false>
 void pack_last(const Tensor& src, long long rows, int v, Tensor& dst, cudaStream_t s) {
-  pack_last_kernel<<<(unsigned)std::min<long long>((rows * v + 7) / 8, 152LL * 32), 256, 0, s>>>(src.p(), rows, v, dst.p());
+  pack_last_kernel<ANTI><<<(unsigned)std::min<long long>((rows * v + 7) / 8, 152LL * 32), 256, 0, s>>>(src.p(), rows, v,
+                                                                                                      dst.p());
   GFCC_LAUNCH_CHECK();
 }
+template <bool ANTI = false>
 void take_pairs(const Tensor& src, int o, long long n, Tensor& dst, cudaStream_t s) {
   GFCC_CHECK((long long)o * o <= 65535, GFCC_ERR_ARG, "take_pairs: too many pairs");
-  take_pairs_kernel<<<dim3((unsigned)std::min<long long>((n + 255) / 256, 64), (unsigned)(o * o)), 256, 0, s>>>(src.p(), o, n,
-                                                                                                        dst.p());
+  const dim3 grid((unsigned)std::min<long long>((n + 255) / 256, 64), (unsigned)(o * o));
+  take_pairs_kernel<ANTI><<<grid, 256, 0, s>>>(src.p(), o, n, dst.p());
   GFCC_LAUNCH_CHECK();
 }
 
@@ -376,7 +385,7 @@ std::unique_ptr<HbarCommon> build_common(const HostInputs& in, int o, int v, cud
   if (V > 0) {   // 1/2 tau_in^ef <mn||ef> over e < f
     h->tauP = std::make_unique<Tensor>("int", std::vector<int>{o, o, V});
     h->oovvP = std::make_unique<Tensor>("mnt", std::vector<int>{o, o, V});
-    pack_last(tau, (long long)o * o, v, *h->tauP, s);
+    pack_last<true>(tau, (long long)o * o, v, *h->tauP, s);
     pack_last(*v_oovv, (long long)o * o, v, *h->oovvP, s);
     contract(1.0, h->tauP->as("int"), h->oovvP->as("mnt"), 1.0, Fmi.as("mi"), s);
   }
@@ -385,7 +394,7 @@ std::unique_ptr<HbarCommon> build_common(const HostInputs& in, int o, int v, cud
   contract(-1.0, t1->as("mf"), v_ovvv->as("maef"), 0.0, Fae.as("ae"), s);      // <am||ef> = -<ma||ef>
   if (P > 0) {   // -1/2 tau_mn^af <mn||ef> over m < n
     Tensor tp("paf", {P, v, v}), vp("pef", {P, v, v});
-    take_pairs(tau, o, (long long)v * v, tp, s);
+    take_pairs<true>(tau, o, (long long)v * v, tp, s);
     take_pairs(*v_oovv, o, (long long)v * v, vp, s);
     contract(-1.0, tp.as("paf"), vp.as("pef"), 1.0, Fae.as("ae"), s);
   }
