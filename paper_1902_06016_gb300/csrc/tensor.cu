@@ -230,10 +230,11 @@ void contract(double alpha, const TV& A, const TV& B, double beta, const TV& C, 
   std::string lt0 = Ml + Nl;
   std::vector<int> pc0 = perm_of(lt0, lc);
   // contractions above this many multiply-adds use the tensor cores (GFCC_OZ_MIN_MACS overrides it,
-  // which the tests use to exercise this path at small sizes). The FP64 pipe does 5e11 of them a second at best and
-  // about half that in 64 x 64 tiles, so 3e7 take it 0.1 ms, about what the eight launches of the exact form
-  // take; its 62 bits per row leave less error than FP64 sums.
-  double min_macs = 3e7;
+  // which the tests use to exercise this path at small sizes). The digits keep 62 bits below a row's largest element:
+  // closer to 64 bits than FP64 sums where a row is of one magnitude, but an element more than 2^9 below its row's
+  // largest keeps fewer than its 53 bits, and small operators, whose contractions are all below this, stay free of that.
+  // (A line at 3e7 gains 10 ms of 375 in the whole method at o = 30, v = 130, and 0.3 of 75 in the build at o = 42, v = 186.)
+  double min_macs = 5e8;
   if (const char* env = getenv("GFCC_OZ_MIN_MACS")) min_macs = atof(env);
   if ((double)M * (double)N * (double)K >= min_macs && M >= 16 && N >= 16) {
     // FP64-accurate GEMM from exact f16 slices on the tensor cores (7 slices: FP64-level accuracy)
