@@ -273,35 +273,6 @@ __device__ __forceinline__ float4 dfc_split(cplx z) {
   const df2 r = df_split(z.x), i = df_split(z.y);
   return make_float4(r.h, r.l, i.h, i.l);
 }
-// a b (complex double-float)
-__device__ __forceinline__ float4 dfc_mul(float4 a, float4 b) {
-  const df2 z{0.f, 0.f}, ar{a.x, a.y}, ai{a.z, a.w}, nai{-a.z, -a.w}, br{b.x, b.y}, bi{b.z, b.w};
-  const df2 r = df_dot2(z, ar, br, nai, bi), i = df_dot2(z, ar, bi, ai, br);
-  return make_float4(r.h, r.l, i.h, i.l);
-}
-// (h, l) -= a b without renormalising: the leading product exactly (fma), its sum with h exactly (two-sum),
-// the rest added to l in FP32. The caller renormalises every few terms, which keeps l small enough that
-// its own rounding stays at the 2^-48 level.
-__device__ __forceinline__ void df_acc(float& h, float& l, float ah, float al, float bh, float bl) {
-  const float p = __fmul_rn(ah, bh);
-  const float e = __fmaf_rn(ah, bh, -p);
-  const df2 s = two_sum(h, -p);
-  h = s.h;
-  l = __fadd_rn(l, __fsub_rn(s.l, e));
-  l = __fmaf_rn(-ah, bl, l);
-  l = __fmaf_rn(-al, bh, l);
-}
-__device__ __forceinline__ void dfc_acc(float4& c, const float4& u, const float4& y) {   // c -= u y
-  df_acc(c.x, c.y, u.x, u.y, y.x, y.y);
-  df_acc(c.x, c.y, -u.z, -u.w, y.z, y.w);
-  df_acc(c.z, c.w, u.x, u.y, y.z, y.w);
-  df_acc(c.z, c.w, u.z, u.w, y.x, y.y);
-}
-__device__ __forceinline__ void dfc_renorm(float4& c) {
-  const df2 r = fast_two_sum(c.x, c.y), i = fast_two_sum(c.z, c.w);
-  c = make_float4(r.h, r.l, i.h, i.l);
-}
-
 __device__ __forceinline__ void cp_async16(void* smem, const void* gmem, bool on) {
   const uint32_t d = (uint32_t)__cvta_generic_to_shared(smem);
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(gmem), "r"(on ? 16 : 0) : "memory");
@@ -425,9 +396,13 @@ __global__ void __launch_bounds__(EF_T) eval_factor_kernel(EvalArgs a, int w0, c
 
 // Back substitution, one CTA per (frequency, group of P = 8 C right-hand sides), by blocks of 32 rows from
 // the bottom: acc = R_J - sum_{K > J} U_JK Y_K in double-float with 2 x C register tiles, then the 32 x 32
-// triangular solve by four lanes per right-hand side with one warp barrier per row. U and Y arrive by
-// cp.async in steps of 16 columns of U, double-buffered: per step a thread takes 2 + C shared loads for 2 C
-// complex multiply-adds of 48 FP32 operations, so the FP32 pipe is what bounds it; 34-43 KB of shared memory
+// triangular solve by four lanes per right-hand side with one warp barrier per row. Every row takes its terms one after
+// the other from the last column down, renormalised after each: the sums of a plain column-by-column substitution, bit
+// for bit. (Renormalising every eighth term and going up through the columns of a tile was 13 % faster and 1.7 to 2.9
+// times further from extended precision, orders 40 to 800.) The division by the diagonal is a product with its
+// reciprocal, both in FP64, shared by two lanes: a complex division is thirty instructions on the FP64 pipe, this five.
+// U and Y arrive by cp.async in steps of 16 columns of U, double-buffered: per step a thread takes 2 + C shared loads
+// for 2 C complex multiply-adds of 56 FP32 operations, so the FP32 pipe is what bounds it; 34-43 KB of shared memory
 // and 128 threads whatever P keep four CTAs (one warp each per scheduler) on an SM. Solved blocks are kept
 // in Y as double-float and converted to FP64 at the end.
 constexpr int EB_T = 128, EK = ET / 2;
@@ -437,7 +412,7 @@ __global__ void __launch_bounds__(EB_T, 4) eval_backsub_kernel(EvalArgs a, int w
   extern __shared__ float4 eb_sm[];
   float4* sU = eb_sm;                      // [2][ET][US]: a half tile each; both halves of the diagonal tile
   float4* sY = sU + 2 * ET * US;           // [2][EK][P]; the block's right-hand sides during its solve
-  float4* sD = sY + 2 * EK * P;            // [ET] reciprocal diagonal
+  cplx* sD = reinterpret_cast<cplx*>(sY + 2 * EK * P);   // [ET] reciprocal diagonal
   const int m = a.m, np = a.np, tid = threadIdx.x, f = blockIdx.x, w = w0 + f;
   const int p0 = blockIdx.y * P, pn = min(P, np - p0);
   const float4* U = a.U + (long long)f * eval_tiles(m) * (ET * ET);
@@ -462,8 +437,8 @@ __global__ void __launch_bounds__(EB_T, 4) eval_backsub_kernel(EvalArgs a, int w
   };
   for (int J = T - 1; J >= 0; --J) {
     if (J < T - 1) {
-      load_u(J, T - 1, 0);
-      load_y(T - 1, 0);
+      load_u(J, T - 1, 1);
+      load_y(T - 1, 1);
       cp_async_commit();
     }
     float4 acc[2][C];
@@ -476,34 +451,27 @@ __global__ void __launch_bounds__(EB_T, 4) eval_backsub_kernel(EvalArgs a, int w
       }
     for (int K = T - 1; K > J; --K) {
 #pragma unroll 1
-      for (int h = 0; h < 2; ++h) {
-        // the next half tile: the second half of this one, the first of the next; after the last the diagonal
+      for (int h = 1; h >= 0; --h) {
+        // the next half tile: the first half of this one, the second of the next; after the last the diagonal
         // tile is loaded below
-        if (h == 0 || K - 1 > J) {
-          load_u(J, h == 0 ? K : K - 1, h ^ 1);
-          load_y(h == 0 ? K : K - 1, h ^ 1);
+        if (h == 1 || K - 1 > J) {
+          load_u(J, h == 1 ? K : K - 1, h ^ 1);
+          load_y(h == 1 ? K : K - 1, h ^ 1);
         }
         cp_async_commit();
         cp_async_wait<1>();
         __syncthreads();
         const float4* u = sU + (h * ET + 2 * ty) * US;
         const float4* y = sY + h * EK * P + tx;
-#pragma unroll 1
-        for (int k0 = 0; k0 < EK; k0 += 8) {
 #pragma unroll 2
-          for (int k = k0; k < k0 + 8; ++k) {
-            const float4 u0 = u[k], u1 = u[US + k];
+        for (int k = EK - 1; k >= 0; --k) {
+          const float4 u0 = u[k], u1 = u[US + k];
 #pragma unroll
-            for (int i = 0; i < C; ++i) {
-              const float4 yy = y[k * P + 8 * i];
-              dfc_acc(acc[0][i], u0, yy);
-              dfc_acc(acc[1][i], u1, yy);
-            }
+          for (int i = 0; i < C; ++i) {
+            const float4 yy = y[k * P + 8 * i];
+            acc[0][i] = dfc_sub_mul(acc[0][i], u0, yy);
+            acc[1][i] = dfc_sub_mul(acc[1][i], u1, yy);
           }
-#pragma unroll
-          for (int r = 0; r < 2; ++r)
-#pragma unroll
-            for (int i = 0; i < C; ++i) dfc_renorm(acc[r][i]);
         }
         __syncthreads();
       }
@@ -518,8 +486,7 @@ __global__ void __launch_bounds__(EB_T, 4) eval_backsub_kernel(EvalArgs a, int w
       for (int i = 0; i < C; ++i) sR[(2 * ty + r) * P + tx + 8 * i] = acc[r][i];
     if (tid < ET && J * ET + tid < m) {
       const cplx d = dU[J * ET + tid];
-      sD[tid] = (d.x == 0.0 && d.y == 0.0) ? make_float4(0.f, 0.f, 0.f, 0.f)
-                                           : dfc_from(cuCdiv(make_cuDoubleComplex(1.0, 0.0), d));
+      sD[tid] = (d.x == 0.0 && d.y == 0.0) ? cz() : cuCdiv(make_cuDoubleComplex(1.0, 0.0), d);
     }
     cp_async_wait<0>();
     __syncthreads();
@@ -530,7 +497,14 @@ __global__ void __launch_bounds__(EB_T, 4) eval_backsub_kernel(EvalArgs a, int w
         const int p = c8 * 8 + (tid & 7);
         for (int j = min(ET, m - J * ET) - 1; j >= 0; --j) {
           const float4* u = sU + (j / EK) * ET * US + j % EK;
-          const float4 y = dfc_mul(sR[j * P + p], sD[j]);
+          // lanes with even g form the real part of sR_j sD_j, those with odd g the imaginary one
+          const float4 r = sR[j * P + p];
+          const cplx d = sD[j];
+          const bool im = g & 1;
+          const double mine = im ? df_to(r.z, r.w) : df_to(r.x, r.y), other = __shfl_xor_sync(0xffffffffu, mine, 8);
+          const df2 v = df_split(fma(mine, d.x, other * (im ? d.y : -d.y)));
+          const float oh = __shfl_xor_sync(0xffffffffu, v.h, 8), ol = __shfl_xor_sync(0xffffffffu, v.l, 8);
+          const float4 y = im ? make_float4(oh, ol, v.h, v.l) : make_float4(v.h, v.l, oh, ol);
           for (int i = g; i < j; i += 4) sR[i * P + p] = dfc_sub_mul(sR[i * P + p], u[i * US], y);
           __syncwarp();
           if (g == 0) sR[j * P + p] = y;
