@@ -274,7 +274,7 @@ __global__ void __launch_bounds__(256) pack_last_kernel(const double* __restrict
 template <bool ANTI>
 __global__ void __launch_bounds__(256) take_pairs_kernel(const double* __restrict__ src, int o, long long n,
                                                          double* __restrict__ dst) {
-  const int i = blockIdx.y / o, j = blockIdx.y % o;
+  const int i = blockIdx.y, j = blockIdx.z;
   if (i >= j) return;
   const double* s = src + ((long long)i * o + j) * n;
   const double* st = src + ((long long)j * o + i) * n;
@@ -313,8 +313,7 @@ void pack_last(const Tensor& src, long long rows, int v, Tensor& dst, cudaStream
 }
 template <bool ANTI = false>
 void take_pairs(const Tensor& src, int o, long long n, Tensor& dst, cudaStream_t s) {
-  GFCC_CHECK((long long)o * o <= 65535, GFCC_ERR_ARG, "take_pairs: too many pairs");
-  const dim3 grid((unsigned)std::min<long long>((n + 255) / 256, 64), (unsigned)(o * o));
+  const dim3 grid((unsigned)std::min<long long>((n + 255) / 256, 64), (unsigned)o, (unsigned)o);
   take_pairs_kernel<ANTI><<<grid, 256, 0, s>>>(src.p(), o, n, dst.p());
   GFCC_LAUNCH_CHECK();
 }
