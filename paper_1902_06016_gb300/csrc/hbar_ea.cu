@@ -305,6 +305,8 @@ void build_operator_ea(gfcc_ctx* c, const HostInputs& in) {
   GFCC_CHECK(in.vvvv != nullptr, GFCC_ERR_ARG, "gfcc_init_ea: vvvv is null");
   ProfScope prof(PROF_INIT, 0.0, s);
   std::unique_ptr<HbarCommon> hc = build_common(in, o, v, s);
+  hc->tauP.reset();   // packed pairs for the ionisation build only
+  hc->oovvP.reset();
   Tensor *t1 = hc->t1.get(), *t2 = hc->t2.get(), *l1 = hc->l1.get(), *l2 = hc->l2.get();
   Tensor *v_ooov = hc->v_ooov.get(), *v_oovv = hc->v_oovv.get(), *v_ovov = hc->v_ovov.get();
   Tensor *v_ovvv = hc->v_ovvv.get();

@@ -38,7 +38,7 @@ struct HbarCommon {
   int o, v;
   std::unique_ptr<Tensor> eps, v_oooo, v_ooov, v_oovv, v_ovov, v_ovvv, t1, t2, l1, l2;
   Tensor tau, Fme, Fmi, Fae, Y, Wmbej;
-  std::unique_ptr<Tensor> tauP, oovvP;   // tau and <mn||ef> with e < f packed (hbar.cu), for the build that follows
+  std::unique_ptr<Tensor> tauP, oovvP;   // tau and <mn||ef> with e < f packed (hbar.cu), for the ionisation build
   HbarCommon(int o_, int v_);
 };
 std::unique_ptr<HbarCommon> build_common(const HostInputs& in, int o, int v, cudaStream_t s);
