@@ -147,8 +147,14 @@ __global__ void __launch_bounds__(256) norm_partial_kernel(const VT* __restrict_
 //   sweep DOTS:    g_i = V_i^H a, r_i = V_i^H u (i < j), a^H a, a^H u
 //   coefficients:  rho^2 = a^H a - |g|^2, s = (a^H u - g^H r) / rho; Hessenberg column (r_0 .. r_{j-1}, s)
 //   sweep UPDATE:  V_j = (a - V g) / rho,  u -= V r + V_j s (u has had its first pass), partial sums of |u|^2
-// u is the action on a, not on V_j: they differ by |g|, the FP32 rounding level (1e-7 times the cancellation of the
-// first pass), far below the rounding of the low-precision action itself; the residual of every cycle is recomputed.
+// What this leaves out, with w the image whose first pass gave hn a: a = V g + rho V_j, so that column j - 1 would gain hn g
+// and its subdiagonal be hn rho. Both are at most |g| hn, and g is the rounding of the first pass, a few 2^-24 ||w|| / hn:
+// the Arnoldi relation of that column holds to a few 2^-24 ||w||, however much the pass cancelled. Column j has the
+// image u of a in the place of that of V_j, |g| ||A|| off: less than the rounding of the low-precision action itself (2^-11
+// in TF32) while the pass cancels less than a factor of some thousand, more beyond that. It costs steps, not accuracy: the
+// residual of every cycle is recomputed. A vector of which the second pass takes more than half (rho^2 <= a^H a / 2; the
+// criterion of Daniel, Gragg, Kaufman and Stewart, Math. Comp. 30 (1976)) is rounding noise: its column ends its cycle with
+// the vectors before it, so that 1 / rho is never above sqrt 2.
 // (o = 30, v = 130, TF32 solves to 1e-10: kernels of the whole solve 276 -> 247 ms, all of it the sweeps; the numbers
 // of Arnoldi steps did not change by more than 2 in 440.)
 //
@@ -367,7 +373,7 @@ __global__ void __launch_bounds__(256) reduce_dots_kernel(const cplx* __restrict
   }
 }
 // The coefficients of a column from its sums (g_i at g[i nb + c], r_i, a^H a and a^H u at sc): Hessenberg column Hc
-// (entry (i, c) at i nb + c) and fin = (1 / rho, s). Eight lanes per column.
+// (entry (i, c) at i nb + c) and fin = (1 / rho, s), zero where a lies in the span of the basis. Eight lanes per column.
 __global__ void __launch_bounds__(128) delayed_coef_kernel(const cplx* __restrict__ g, const cplx* __restrict__ r, int nv,
                                                            const cplx* __restrict__ sc, int nb, cplx* __restrict__ Hc,
                                                            float4* __restrict__ fin) {
@@ -390,7 +396,8 @@ __global__ void __launch_bounds__(128) delayed_coef_kernel(const cplx* __restric
   }
   if (!on || q != 0) return;
   const double rho2 = sc[c].x - gg;
-  const double inv = rho2 > 0.0 && isfinite(rho2) ? rsqrt(rho2) : 0.0;   // a zero (broken-down) column stays zero
+  // a zero column stays zero (rho^2 and a^H a are differences and sums of FP32 results: a difference far below them is noise)
+  const double inv = rho2 > 0.5 * sc[c].x && isfinite(rho2) ? rsqrt(rho2) : 0.0;
   const cplx s = make_cuDoubleComplex((sc[nb + c].x - gx) * inv, (sc[nb + c].y - gy) * inv);
   Hc[(long long)nv * nb + c] = s;
   fin[c] = make_float4((float)inv, (float)s.x, (float)s.y, 0.f);
@@ -604,7 +611,8 @@ __global__ void __launch_bounds__(GV_T) arnoldi_finish_kernel(const cplx* __rest
                                                               cplx* __restrict__ sn, cplx* __restrict__ g,
                                                               const double* __restrict__ bnorm, int* __restrict__ kc,
                                                               int* __restrict__ live, int nb, int k, int j,
-                                                              const double* __restrict__ thr, int* __restrict__ n_live) {
+                                                              const double* __restrict__ thr, int* __restrict__ n_live,
+                                                              const float4* __restrict__ fin) {
   __shared__ double red[GV_T / 32][32];
   const int c0 = blockIdx.x * 32;
   if (nchunk > 0) {
@@ -626,7 +634,10 @@ __global__ void __launch_bounds__(GV_T) arnoldi_finish_kernel(const cplx* __rest
   }
   if (threadIdx.x >= 128) return;
   const int x = threadIdx.x >> 2, q = threadIdx.x & 3, c = c0 + x;
-  const bool in = c < nb, on = in && live[c];
+  // fin (FP32 basis): a column whose vector j was found in the span of the basis keeps its j vectors and ends its cycle
+  const bool in = c < nb, was = in && live[c], broken = was && fin && fin[c].x == 0.f, on = was && !broken;
+  __syncwarp();
+  if (broken && q == 0) live[c] = 0;
   const double hn = in ? (nchunk > 0 ? red[0][x] : nrm[c]) : 0.0;
   if (in && q == 0) invf[c] = (hn > 0.0 && isfinite(hn)) ? (float)(1.0 / hn) : 0.f;
   if (!__any_sync(0xffffffffu, on)) return;
@@ -1147,7 +1158,8 @@ static void gmres_impl(gfcc_ctx* c, const cplx* Bin, cplx* Xout, cplx* Rout, con
         col_norms<VT>(Ww.p, D, nb, nrm.p, partial, s);
       }
       arnoldi_finish_kernel<<<(nb + 31) / 32, GV_T, 0, s>>>(partial.p, norm_chunks, nrm.p, invf.p, H.p, cs.p, sn.p, g.p,
-                                                            bnorm.p, kc.p, live.p, nb, k, j, thr.p, nlive.p + j);
+                                                            bnorm.p, kc.p, live.p, nb, k, j, thr.p, nlive.p + j,
+                                                            F32 ? fin.p : nullptr);
       GFCC_LAUNCH_CHECK();
       GFCC_CUDA(cudaMemcpyAsync(c->pin, nlive.p + j, sizeof(int), cudaMemcpyDeviceToHost, s));
       GFCC_CUDA(cudaEventRecord(c->pin_event, s));
