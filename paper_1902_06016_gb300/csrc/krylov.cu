@@ -739,7 +739,8 @@ __global__ void __launch_bounds__(128) backsolve_kernel(const cplx* __restrict__
 }
 
 // X[nu][c] += P_c[nu] * sum_{i < nv} V_i[nu][c] y_i[c]: the correction is formed in the basis precision, only its
-// addition to x is FP64 (y [i nb + c], zero beyond a column's own steps)
+// addition to x is FP64 (y [i nb + c], zero beyond a column's own steps). A vector whose coefficient is zero is not read:
+// what a finished column's later vectors hold, made because its batch went on, stays out of the sum whatever it is.
 template <typename VT>
 __global__ void __launch_bounds__(EL_T) correct_kernel(const VT* __restrict__ V, long long vstride, int nv,
                                                        const VT* __restrict__ y, cplx* __restrict__ X,
@@ -753,6 +754,12 @@ __global__ void __launch_bounds__(EL_T) correct_kernel(const VT* __restrict__ V,
   ShiftF shf = make_float4(0.f, 0.f, 0.f, 0.f);
   if constexpr (sizeof(R) == 4) shf = shiftf[c];
   else sh = shift[c];
+  auto vector = [&](int i, long long t, const VT& yy) {
+    VT vv;
+    vv.x = vv.y = R(0);
+    if (yy.x != R(0) || yy.y != R(0)) vv = V[(long long)i * vstride + t];
+    return vv;
+  };
   for (long long nu = blockIdx.y * (long long)blockDim.y + threadIdx.y; nu < D; nu += (long long)gridDim.y * blockDim.y) {
     const long long t = nu * nb + c;
     R sr[4] = {R(0), R(0), R(0), R(0)}, si[4] = {R(0), R(0), R(0), R(0)};
@@ -760,13 +767,13 @@ __global__ void __launch_bounds__(EL_T) correct_kernel(const VT* __restrict__ V,
     for (; i + 4 <= nv; i += 4) {
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
-        const VT vv = V[(long long)(i + u) * vstride + t], yy = y[(long long)(i + u) * nb + c];
+        const VT yy = y[(long long)(i + u) * nb + c], vv = vector(i + u, t, yy);
         sr[u] = fma(vv.x, yy.x, fma(-vv.y, yy.y, sr[u]));
         si[u] = fma(vv.x, yy.y, fma(vv.y, yy.x, si[u]));
       }
     }
     for (; i < nv; ++i) {
-      const VT vv = V[(long long)i * vstride + t], yy = y[(long long)i * nb + c];
+      const VT yy = y[(long long)i * nb + c], vv = vector(i, t, yy);
       sr[0] = fma(vv.x, yy.x, fma(-vv.y, yy.y, sr[0]));
       si[0] = fma(vv.x, yy.y, fma(vv.y, yy.x, si[0]));
     }
