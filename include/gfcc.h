@@ -161,6 +161,11 @@ int gfcc_vectors(gfcc_t ctx, const int* orbitals, int norb, int transpose, doubl
  *   A  (optional, host or device): A[w] = -(1/pi) sum_{p in set, p also in q set} Im G_pp(w).
  *   X  (optional, host or device): X[(w*np + p)*ldx ...] complex solutions, ldx >= D.
  *   stats (optional, host).
+ * With a TF32 or BF16 context and a non-null X the solutions themselves are the result, and the error of a column near
+ * a pole is its residual times up to 1/eta: cycles then aim at a tenth of the tolerance instead of half of it, and a
+ * column that meets the tolerance by less than a factor of four gets one more cycle, whose solution replaces it only if
+ * its residual is smaller. G, the residuals and the counts of such a call belong to these solutions and so differ
+ * (within the tolerance) from those of the same call without X.
  * Returns GFCC_ERR_NOT_CONVERGED (outputs still written) if a column hit the cycle cap. */
 int gfcc_solve_full(gfcc_t ctx, const double* omegas, int nw, double eta, const int* orbitals,
                     int np, const int* qorb, int nq, double* G, double* A, double* X, int ldx,

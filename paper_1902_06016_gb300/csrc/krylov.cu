@@ -986,14 +986,14 @@ static void gmres_impl(gfcc_ctx* c, const cplx* Bin, cplx* Xout, cplx* Rout, con
       int orig = map[w];
       double bn = hbn[orig];
       double rel = bn > 0.0 ? hres[w] / bn : 0.0;
-      GFCC_CHECK(std::isfinite(rel), GFCC_ERR_NONFINITE, "solve: non-finite residual (singular shift?)");
-      if (polished[orig]) {
+      if (polished[orig]) {   // (a residual that is not finite is not smaller: the solution in hand stays)
         if (rel < st.relres[orig]) {
           st.relres[orig] = rel;
           done.push_back(w);
         }
         continue;
       }
+      GFCC_CHECK(std::isfinite(rel), GFCC_ERR_NONFINITE, "solve: non-finite residual (singular shift?)");
       st.relres[orig] = rel;
       if (rel <= tol || cycle == max_cycles) {
         done.push_back(w);
