@@ -310,8 +310,8 @@ __device__ __forceinline__ cplx cdiv_newton(cplx x, cplx p) {
 // it alone reads and writes), and the rows still to come arrive by cp.async EF_RING - 1 steps ahead. The
 // chain of a step is the pivot of its owner thread (an FP64 division) and one barrier; everything else
 // (two FP64 multiply-adds per column, the split to double-float) is in its shadow. RING = false (rows too
-// long for shared memory) reads each row when it is needed and carries the row in global memory (the
-// tail of the frequency's dU block).
+// long for shared memory) reads each row when it is needed and carries the row in global memory (m + np
+// entries per frequency of EvalScratch::rows).
 constexpr int EF_T = 128, EF_RING = 4;
 template <bool RING>
 __global__ void __launch_bounds__(EF_T) eval_factor_kernel(EvalArgs a, int w0, cplx* __restrict__ rows) {
@@ -1535,7 +1535,7 @@ void mor_eval(gfcc_ctx* c, const double* omegas_host, int nw, cplx* G_dev, doubl
 
 // Initial guesses for new frequencies: x0_p(w) = S yhat_p(w) with (w - i eta + Hhat) yhat_p = bhat_p.
 // Hhat is reduced to Hessenberg form H = P^H Hhat P by Householder reflections (recorded), each
-// frequency is the shifted Hessenberg solve of eval_solve_kernel, yhat = P y_H applies the reflections
+// frequency is a shifted Hessenberg solve (launch_eval_solve), yhat = P y_H applies the reflections
 // in reverse order, and X0 = S yhat is one complex GEMM. X0: [D][nw np] batch-minor (column w np + p).
 void mor_extrapolate(gfcc_ctx* c, const double* omegas_host, int nw, cplx* X0) {
   MorState& ms = c->mor;

@@ -382,9 +382,9 @@ __device__ __forceinline__ long long split_sum(const int* __restrict__ p, int zs
   return sum;
 }
 
-// One diagonal of a column chunk (Np real columns): its split sums, weighted by scale = 2^(-9d), are
+// One diagonal of a column chunk (Np real columns): its split sums, weighted by scale = 2^(-bits d), are
 // added to the FP64 accumulator acc[m][n'] (MODE 0; first: acc is set), or, on the last diagonal, added
-// to acc, scaled by 2^(ea[m] + eb[n'] - 16) and written to a real (MODE 1) or complex (MODE 2) output.
+// to acc, scaled by 2^(ea[m] + eb[n'] - 2 (bits - 1)) and written to a real (MODE 1) or complex (MODE 2) output.
 // One thread per element, or (WARP) one warp for outputs too small to occupy the GPU that have many K
 // splits. Only the last diagonal needs the (m, n) of an element; 32-bit division when it fits.
 template <typename I>

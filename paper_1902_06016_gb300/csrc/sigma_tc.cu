@@ -1,7 +1,9 @@
 // Low-precision sigma on the tcgen05 tensor cores, for the inner (Krylov) steps of the iterative
 // refinement: every GEMM-shaped term of the sigma runs as one tc_gemm launch with bf16 or tf32
-// operands and FP32 accumulation; the Fock diagonal, the shift and the small 1h-1h block are applied
-// in FP64 in the final combine. The residuals that decide convergence always use the FP64 sigma.
+// operands and FP32 accumulation. On FP64 vectors (gfcc_sigma) the Fock diagonal, the shift and the small 1h-1h
+// block are applied in FP64 in the final combine; on the FP32 Krylov basis in FP32 (the sum of shift and diagonal of
+// the preconditioner from pairs of FP32 numbers, precond.cuh; the 1h-1h block with the down operand). The residuals that
+// decide convergence always use the FP64 sigma.
 //
 //   up:   [Xe ; Y1'] ((v+o) x 2nb) = [Vt ; A12] ((v+o) x Pv) . r2          (split-K over Pv)
 //   oooo: C2[(pij,a)][(c,r)]       = Woo (P x P) . r2 arranged [(a,c,r)][pmn]
@@ -379,9 +381,6 @@ __global__ void __launch_bounds__(256) combine_f32_kernel(const float2* __restri
   }
 }
 
-// ring: U[(j*nb + c)*2 + r][m*v + e] = r_mj^e (component r), K padded
-// oooo: B[(a*nb + c)*2 + r][pmn] = X2[(pmn*v + a)][c].r
-// up: B[c*2 + r][kk] = X2[kk][c].r  (kk = pmn*v + f)
 // sum split-K partials: out[i] = sum_z part[z*stride + i]
 __global__ void reduce_splits_kernel(const float* __restrict__ part, int zs, long long stride, long long n,
                                      float* __restrict__ out) {
