@@ -430,7 +430,11 @@ void build_operator(gfcc_ctx* c, const HostInputs& in) {
   // W_mnij
   Tensor Wmnij("mnij", {o, o, o, o});
   perm(v_oooo->as("mnij"), 1.0, 0.0, Wmnij.as("mnij"), s);
-  {  // P(ij) t_j^e <mn||ie>
+  // P(ij) t_j^e <mn||ie>: one product antisymmetrised after, or two when another o^4 array would be above 4 GB
+  if ((double)o * o * o * o * sizeof(double) > (double)(4LL << 30)) {
+    contract(1.0, t1->as("je"), v_ooov->as("mnie"), 1.0, Wmnij.as("mnij"), s);
+    contract(-1.0, t1->as("ie"), v_ooov->as("mnje"), 1.0, Wmnij.as("mnij"), s);
+  } else {
     Tensor Z("mnij", {o, o, o, o});
     contract(1.0, t1->as("je"), v_ooov->as("mnie"), 0.0, Z.as("mnij"), s);
     perm(Z.as("mnij"), 1.0, 1.0, Wmnij.as("mnij"), s);
