@@ -386,7 +386,7 @@ std::unique_ptr<HbarCommon> build_common(const HostInputs& in, int o, int v, cud
     h->oovvP = std::make_unique<Tensor>("mnt", std::vector<int>{o, o, V});
     pack_last<true>(tau, (long long)o * o, v, *h->tauP, s);
     pack_last(*v_oovv, (long long)o * o, v, *h->oovvP, s);
-    contract(1.0, h->tauP->as("int"), h->oovvP->as("mnt"), 1.0, Fmi.as("mi"), s);
+    contract(1.0, h->tauP->as("int"), h->oovvP->as("mnt"), 1.0, Fmi.as("mi"), s, 2.0);
   }
   add_diag_kernel<<<(o + 255) / 256, 256, 0, s>>>(Fmi.p(), o, h->eps->p(), 1.0);
   GFCC_LAUNCH_CHECK();
@@ -395,7 +395,7 @@ std::unique_ptr<HbarCommon> build_common(const HostInputs& in, int o, int v, cud
     Tensor tp("paf", {P, v, v}), vp("pef", {P, v, v});
     take_pairs<true>(tau, o, (long long)v * v, tp, s);
     take_pairs(*v_oovv, o, (long long)v * v, vp, s);
-    contract(-1.0, tp.as("paf"), vp.as("pef"), 1.0, Fae.as("ae"), s);
+    contract(-1.0, tp.as("paf"), vp.as("pef"), 1.0, Fae.as("ae"), s, 2.0);
   }
   add_diag_kernel<<<(v + 255) / 256, 256, 0, s>>>(Fae.p(), v, h->eps->p() + o, 1.0);
   GFCC_LAUNCH_CHECK();
@@ -448,7 +448,7 @@ void build_operator(gfcc_ctx* c, const HostInputs& in) {
     Tensor vPP("qt", {P, V}), R("qp", {P, P});
     take_pairs(*hc->tauP, o, V, *tauPP, s);
     take_pairs(*hc->oovvP, o, V, vPP, s);
-    contract(1.0, vPP.as("qt"), tauPP->as("pt"), 0.0, R.as("qp"), s);
+    contract(1.0, vPP.as("qt"), tauPP->as("pt"), 0.0, R.as("qp"), s, 8.0);
     add_pair_pairs_kernel<<<grid_for((long long)o * o * o * o), 256, 0, s>>>(R.p(), o, Wmnij.p());
     GFCC_LAUNCH_CHECK();
     GFCC_CUDA(cudaStreamSynchronize(s));   // R is released here
@@ -469,7 +469,7 @@ void build_operator(gfcc_ctx* c, const HostInputs& in) {
   if (V > 0) {   // 1/2 <mb||ef> tau_ij^ef over e < f, i < j: a quarter of the multiply-adds
     Tensor vP("mbt", {o, v, V}), R("mbp", {o, v, P});
     pack_last(*v_ovvv, (long long)o * v, v, vP, s);
-    contract(1.0, vP.as("mbt"), tauPP->as("pt"), 0.0, R.as("mbp"), s);
+    contract(1.0, vP.as("mbt"), tauPP->as("pt"), 0.0, R.as("mbp"), s, 4.0);
     add_pairs_kernel<<<grid_for((long long)o * v * o * o), 256, 0, s>>>(R.p(), (long long)o * v, o, Wmbij.p());
     GFCC_LAUNCH_CHECK();
     GFCC_CUDA(cudaStreamSynchronize(s));

@@ -185,7 +185,7 @@ TV Tensor::as(const std::string& l) const {
   return TV{buf.p, l, dims};
 }
 
-void contract(double alpha, const TV& A, const TV& B, double beta, const TV& C, cudaStream_t s) {
+void contract(double alpha, const TV& A, const TV& B, double beta, const TV& C, cudaStream_t s, double packed) {
   const std::string &la = A.l, &lb = B.l, &lc = C.l;
   std::map<char, int> size;
   auto reg = [&](const std::string& l, const std::vector<int>& d) {
@@ -233,10 +233,12 @@ void contract(double alpha, const TV& A, const TV& B, double beta, const TV& C, 
   // which the tests use to exercise this path at small sizes). The digits keep 62 bits below a row's largest element:
   // closer to 64 bits than FP64 sums where a row is of one magnitude, but an element more than 2^9 below its row's
   // largest keeps fewer than its 53 bits, and small operators, whose contractions are all below this, stay free of that.
-  // (A line at 3e7 gains 10 ms of 375 in the whole method at o = 30, v = 130, and 0.3 of 75 in the build at o = 42, v = 186.)
+  // A sum over packed pairs counts with the multiply-adds of the sum it stands for: it had the digits before it was
+  // packed, with 55 bits. (A line at 3e7 gains about 3 % of the whole method at o = 30, v = 130, and 12 % of the gradient
+  // at o = 19, v = 67.)
   double min_macs = 5e8;
   if (const char* env = getenv("GFCC_OZ_MIN_MACS")) min_macs = atof(env);
-  if ((double)M * (double)N * (double)K >= min_macs && M >= 16 && N >= 16) {
+  if (packed * (double)M * (double)N * (double)K >= min_macs && M >= 16 && N >= 16) {
     // FP64-accurate GEMM from exact f16 slices on the tensor cores (7 slices: FP64-level accuracy)
     const double* Aop2 = A.p;
     std::vector<int> pa2 = perm_of(la, Ml + Kl);

@@ -27,7 +27,8 @@ struct Tensor {
 };
 
 // C = alpha * sum A B + beta * C over the labels missing from C (no batch labels).
-void contract(double alpha, const TV& A, const TV& B, double beta, const TV& C, cudaStream_t s);
+// packed: how many times fewer multiply-adds it has than the sum over full index ranges that it stands for.
+void contract(double alpha, const TV& A, const TV& B, double beta, const TV& C, cudaStream_t s, double packed = 1.0);
 // dst = alpha * src + beta * dst, matching axes by label
 void perm(const TV& src, double alpha, double beta, const TV& dst, cudaStream_t s);
 
