@@ -45,6 +45,7 @@ struct Args {
   T* C; long long scm, scn, bsc;
   T alpha, beta;
   int ksplit = 1, kchunk = 0;   // split-K: blockIdx.z = batch * ksplit + split, partials in C
+  int split_k = 256;            // least K of a split (see GemmDesc)
 };
 
 // 256 threads: thread (tx, ty) in a 16x16 grid owns rows ty + 16*i and columns tx + 16*j.
@@ -269,8 +270,8 @@ void launch(Args<T> a, int batch, cudaStream_t s) {
   // too few tiles to fill 152 SMs and a long K: split K, then reduce the partial tiles
   const long long tiles = (long long)grid.x * grid.y * batch;
   int ksplit = 1;
-  if (tiles < 2 * 152 && a.K >= 1024) {
-    ksplit = (int)std::min<long long>((2 * 152 + tiles - 1) / tiles, a.K / 256);
+  if (tiles < 2 * 152 && a.K >= 4 * a.split_k) {
+    ksplit = (int)std::min<long long>((2 * 152 + tiles - 1) / tiles, a.K / a.split_k);
     ksplit = std::max(1, std::min(ksplit, 65535 / std::max(batch, 1)));
   }
   GFCC_CHECK((long long)batch * ksplit <= 65535, GFCC_ERR_ARG, "gemm batch too large");
@@ -311,6 +312,7 @@ void launch(Args<T> a, int batch, cudaStream_t s) {
 void dgemm(const GemmDesc& d, cudaStream_t s) {
   Args<double> a{d.M, d.N, d.K, d.A, d.sam, d.sak, d.bsa, false, d.B, d.sbk, d.sbn, d.bsb, false,
                  d.C, d.scm, d.scn, d.bsc, d.alpha, d.beta};
+  a.split_k = d.split_k;
   launch(a, d.batch, s);
 }
 
@@ -336,8 +338,9 @@ void zgemm(const ZGemmDesc& d, cudaStream_t s) {
 }
 
 void dgemm_rm(int M, int N, int K, double alpha, const double* A, int lda, bool transA,
-              const double* B, int ldb, bool transB, double beta, double* C, int ldc, cudaStream_t s) {
+              const double* B, int ldb, bool transB, double beta, double* C, int ldc, cudaStream_t s, int split_k) {
   GemmDesc g;
+  g.split_k = split_k;
   g.M = M; g.N = N; g.K = K;
   g.A = A; g.sam = transA ? 1 : lda; g.sak = transA ? lda : 1;
   g.B = B; g.sbk = transB ? 1 : ldb; g.sbn = transB ? ldb : 1;

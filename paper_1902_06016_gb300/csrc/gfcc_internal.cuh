@@ -308,6 +308,7 @@ struct GemmDesc {
   const double* B = nullptr; long long sbk = 0, sbn = 0, bsb = 0;
   double* C = nullptr; long long scm = 0, scn = 0, bsc = 0;
   double alpha = 1.0, beta = 0.0;
+  int split_k = 256;   // K is split, in parts of at least this, from four times this on when the tiles are few
 };
 void dgemm(const GemmDesc& g, cudaStream_t s);
 
@@ -342,7 +343,8 @@ void green_grad_t2_core(gfcc_ctx* c, int nw, const std::vector<int>& porb, const
 
 // row-major contiguous helpers
 void dgemm_rm(int M, int N, int K, double alpha, const double* A, int lda, bool transA,
-              const double* B, int ldb, bool transB, double beta, double* C, int ldc, cudaStream_t s);
+              const double* B, int ldb, bool transB, double beta, double* C, int ldc, cudaStream_t s,
+              int split_k = 256);
 
 // ---- tensor.cu ---------------------------------------------------------------------------------
 // dst = alpha * permute(src) + beta * dst for up to 6-D tensors (row-major);

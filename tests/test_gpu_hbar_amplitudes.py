@@ -20,7 +20,7 @@ def torch():
 
 
 @pytest.mark.parametrize("sector", ["ip", "ea"])
-@pytest.mark.parametrize("o,v,seed", [(2, 1, 9), (2, 2, 9), (3, 5, 11), (5, 4, 12), (7, 13, 103)])
+@pytest.mark.parametrize("o,v,seed", [(2, 1, 9), (2, 2, 9), (3, 5, 11), (5, 4, 12), (7, 13, 103), (4, 24, 13), (3, 37, 14)])
 def test_sigma_with_any_doubles(torch, sector, o, v, seed):
     from paper_1902_06016_gb300 import Context
     if sector == "ea" and v < 2:
