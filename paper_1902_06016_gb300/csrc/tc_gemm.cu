@@ -376,15 +376,15 @@ __global__ void __launch_bounds__(EXACT ? 320 : 192, 1)
                   }
                   *reinterpret_cast<float4*>(p + j) = v;
                 }
+              } else if (beta) {   // two loops: one with the test inside took twice the time (130 columns: up 9.4 us
+                                   // instead of 4.7, down 33 instead of 21)
+#pragma unroll
+                for (int j = 0; j < 32; ++j)
+                  if (gcol + j < N) p[j] += nk == 0 ? 0.f : __uint_as_float(r[j]);
               } else {
 #pragma unroll
-                for (int j = 0; j < 32; ++j) {
-                  if (gcol + j < N) {
-                    float v = nk == 0 ? 0.f : __uint_as_float(r[j]);
-                    if (beta) v += p[j];
-                    p[j] = v;
-                  }
-                }
+                for (int j = 0; j < 32; ++j)
+                  if (gcol + j < N) p[j] = nk == 0 ? 0.f : __uint_as_float(r[j]);
               }
             }
           }
