@@ -319,12 +319,13 @@ void dgemm(const GemmDesc& d, cudaStream_t s) {
 void zgemm(const ZGemmDesc& d, cudaStream_t s) {
   // Complex products of some size (the subspace projections of the reduced model, its evaluation) go to the
   // exact-slice tensor-core GEMM: 6 slices (53 bits per row) for the large ones, 7 (62 bits) for those whose extra
-  // slice costs little. 270 x 30 x 56,580: 8.3 ms on the FP64 pipe. The operands are unit vectors and coefficients in
-  // an orthonormal basis, whose products count by their norm: the digits' rounding (2^-62 of the largest entries for
-  // each term) is below that of FP64 sums unless two columns hardly overlap (sum of |s||z| below about 2^-9), where it is
-  // still 2^-62 of the columns' own size. A product that would be slow there (a billion
-  // multiply-adds, 8 ms at best) takes the scratch it needs; a smaller or shorter one stays on the FP64 pipe, which needs
-  // none, when memory is short.
+  // slice costs little. 270 x 30 x 56,580: 8.3 ms on the FP64 pipe. (On FP64 below 1e9 multiply-adds the whole method at
+  // o = 30, v = 130 takes 448 ms instead of 385.) Their operands are unit vectors and coefficients in an orthonormal basis,
+  // which carry the rounding of its orthonormalisation, 2^-48 of a column, and whose products count by their norm: the digits'
+  // rounding (2^-62 of the largest entries for each term) is below that of FP64 sums unless two columns hardly overlap (sum
+  // of |s||z| below about 2^-9), where it is still 2^-62 of the columns' own size. A product that would be slow on FP64 (a
+  // billion multiply-adds, 8 ms at best) takes the scratch it needs; a smaller or shorter one stays on the FP64 pipe, which
+  // needs none, when memory is short.
   const double macs = (double)d.M * (double)d.N * (double)d.K;
   const int ns = macs >= 1e9 ? 6 : 7;
   if (d.batch == 1 && macs >= oz_min_macs() && d.M >= 16 && d.N >= 1 && d.K >= 64 &&
